@@ -307,18 +307,39 @@ __global__ void df_dots_kernel(int64_t n, int p, const float2* A0, const float2*
   }
 }
 
-__global__ void df_dots_final_kernel(int nb, const float2* part, double* out) {
-  if (threadIdx.x != 0) return;
+// Fixed-order final sums over the nb blocks' partials, one warp: lane l adds
+// the partials l, l + 32, ... in ascending order and the lanes are folded in
+// a butterfly. One thread adding them all (a dependent df64 chain per
+// partial) took 72-77 us at 608 partials and 15 us at 152; this takes 3 us.
+__device__ __forceinline__ void final_sums(int nb, const float2* part, int stride, const float* mx, int mstride,
+                                           double* out, bool with_max) {
+  const int lane = threadIdx.x & 31;
   float2 t0 = make_float2(0.f, 0.f), t1 = make_float2(0.f, 0.f);
   float m = 0.f;
-  for (int b = 0; b < nb; ++b) {
-    t0 = df_add(t0, part[3 * b]);
-    t1 = df_add(t1, part[3 * b + 1]);
-    m = fmaxf(m, part[3 * b + 2].x);
+#pragma unroll 4
+  for (int b = lane; b < nb; b += 32) {
+    t0 = df_add(t0, part[(size_t)stride * b]);
+    t1 = df_add(t1, part[(size_t)stride * b + 1]);
+    if (with_max) m = fmaxf(m, mx[(size_t)mstride * b]);
   }
-  out[0] = df_to_double(t0);
-  out[1] = df_to_double(t1);
-  out[2] = (double)m;
+  // both partners of an exchange form the sum in the same operand order, so
+  // every lane ends with the same value
+  for (int o = 16; o > 0; o >>= 1) {
+    const float2 u0 = shfl_df(t0, o), u1 = shfl_df(t1, o);
+    const bool up = (lane & o) != 0;
+    t0 = up ? df_add(u0, t0) : df_add(t0, u0);
+    t1 = up ? df_add(u1, t1) : df_add(t1, u1);
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  }
+  if (lane == 0) {
+    out[0] = df_to_double(t0);
+    out[1] = df_to_double(t1);
+    if (with_max) out[2] = (double)m;
+  }
+}
+
+__global__ void df_dots_final_kernel(int nb, const float2* part, double* out) {
+  final_sums(nb, part, 3, &part[2].x, 6, out, true);
 }
 
 gsi_status df_dots(int64_t n, int p, const float2* A0, const float2* B0, const float2* A1,
@@ -364,19 +385,7 @@ gsi_status df_combine3(int64_t count, float2 a, const float2* W, float2 b, const
 }
 
 __global__ void df_sum_parts_kernel(int nparts, const float2* parts, double* out, const float* rinf) {
-  if (threadIdx.x != 0) return;
-  float2 t0 = make_float2(0.f, 0.f), t1 = make_float2(0.f, 0.f);
-  float m = 0.f;
-  // unrolled so that several partials are in flight at once (same order)
-#pragma unroll 8
-  for (int b = 0; b < nparts; ++b) {
-    t0 = df_add(t0, parts[2 * b]);
-    t1 = df_add(t1, parts[2 * b + 1]);
-    if (rinf) m = fmaxf(m, rinf[b]);
-  }
-  out[0] = df_to_double(t0);
-  out[1] = df_to_double(t1);
-  if (rinf) out[2] = (double)m;
+  final_sums(nparts, parts, 2, rinf, 1, out, rinf != nullptr);
 }
 
 gsi_status df_sum_parts(int nparts, const float2* parts, double* out, cudaStream_t st,

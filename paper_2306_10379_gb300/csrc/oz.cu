@@ -1093,7 +1093,7 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool va
 template <bool SYM>
 __global__ void __launch_bounds__(TG_THREADS, 1)
 oz_gram_tc_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const float2* __restrict__ V,
-                  int vec16, float2* part, int nbj, int tri) {
+                  int vec16, float2* part, int nbj, int tri, int ec) {
   using Geo = TgGeom<SYM>;
   // the 64 x 64 output block of this CTA: U's columns 64 bi .., V's 64 bj ..
   // (blockIdx.y over the nbi x nbj blocks, or with tri over the upper
@@ -1112,7 +1112,9 @@ oz_gram_tc_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const f
   }
   const int cu0 = 64 * bi, cv0 = 64 * bj;
   const int wu = min(64, p - cu0), wv = min(64, q - cv0);  // live columns of the block
-  constexpr int EC = Geo::EC, SK = Geo::SK, NSUB = EC / SK, RAWR = Geo::RAWR, NG = Geo::NG;
+  // chunks of ec <= EC rows; V's raw rows start at row EC of the stage
+  constexpr int EC = Geo::EC, SK = Geo::SK, RAWR = Geo::RAWR, NG = Geo::NG;
+  const int NSUB = ec / SK;
   constexpr uint32_t TG_DBUF = Geo::DBUF;
   constexpr uint32_t plane = 64u * SK * 2;  // one digit plane: 64 columns x SK rows, bf16
   extern __shared__ __align__(16) unsigned char tg_smem[];
@@ -1165,30 +1167,32 @@ oz_gram_tc_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const f
 #pragma unroll
   for (int e = 0; e < 16; ++e) res[e] = make_float2(0.f, 0.f);
   bool failed = false;
-  const int64_t nchunks = (n + EC - 1) / EC;
+  const int64_t nchunks = (n + ec - 1) / ec;
 
   // raw rows of chunk ch (workers): U rows (256, or 160 then V's 160),
   // zero-filled outside the matrix
   auto stage = [&](int64_t ch) {
-    const int64_t r0 = ch * EC;
+    const int64_t r0 = ch * ec;
     if (vec16) {
       for (int e = tid; e < RAWR * 32; e += TG_WORKERS) {
         const int row = e >> 5, c = 2 * (e & 31);
         const bool isv = !SYM && row >= EC;
-        const int64_t R = r0 + (isv ? row - EC : row);
+        const int lr = isv ? row - EC : row;
+        const int64_t R = r0 + lr;
         const int ld = isv ? q : p;
         const float2* src = (isv ? V + cv0 : U + cu0);
-        const bool ok = R < n && c < (isv ? wv : wu);
+        const bool ok = lr < ec && R < n && c < (isv ? wv : wu);
         cp_async16(raw + row * TG_RS + c, src + (ok ? R * ld + c : 0), ok);
       }
     } else {
       for (int e = tid; e < RAWR * 64; e += TG_WORKERS) {
         const int row = e >> 6, c = e & 63;
         const bool isv = !SYM && row >= EC;
-        const int64_t R = r0 + (isv ? row - EC : row);
+        const int lr = isv ? row - EC : row;
+        const int64_t R = r0 + lr;
         const int ld = isv ? q : p;
         const float2* src = (isv ? V + cv0 : U + cu0);
-        const bool ok = R < n && c < (isv ? wv : wu);
+        const bool ok = lr < ec && R < n && c < (isv ? wv : wu);
         cp_async8(raw + row * TG_RS + c, src + (ok ? R * ld + c : 0), ok);
       }
     }
@@ -1200,7 +1204,7 @@ oz_gram_tc_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const f
   // current chunk's sub-chunk has been cut, so that the copies spread over
   // the chunk instead of queueing at its end
   auto stage_sub = [&](int64_t ch, int sub) {
-    const int64_t r0 = ch * EC + sub * SK;
+    const int64_t r0 = ch * ec + sub * SK;
     if (vec16) {
       for (int e = tid; e < 2 * SK * 32 / (SYM ? 2 : 1); e += TG_WORKERS) {
         const int rr = e >> 5, c = 2 * (e & 31);
@@ -1440,15 +1444,13 @@ constexpr int TR_THREADS = TR_WORKERS + 96;  // + the issuing warp + two maxima 
 constexpr int TR_BAR_COUNT = TR_WORKERS + 32;
 template <bool SYM, int NDT = ND>
 struct TrGeom {
-  static constexpr int EC = SYM ? 512 : 384;       // exponent chunk rows
+  static constexpr int EC = SYM ? 512 : 384;       // most rows of an exponent chunk
   static constexpr int SK = SYM ? 32 : 16;         // sub-chunk rows
-  static constexpr int NSUB = EC / SK;             // sub-chunks per chunk
   static constexpr int NB = 3;                     // digit buffers
   static constexpr int NR = 4;                     // raw slots (staging NR - 1 sub-chunks ahead)
   static constexpr int MSW = SYM ? 3 : 4;          // maxima slots per maxima warp
   static constexpr int MS = 2 * MSW;
   static constexpr int MB = SYM ? 16 : 8;          // rows per operand in one maxima slot
-  static constexpr int NMB = EC / MB;              // maxima batches per chunk
   static constexpr uint32_t PLANE = 64u * SK * 2;  // one digit plane: 64 columns x SK rows, bf16
   // U == V: NDT planes and a zero pad plane; U != V: NDT planes of U, NDT of V
   static constexpr uint32_t DBUF = (uint32_t)(SYM ? NDT + 1 : 2 * NDT) * PLANE;
@@ -1500,10 +1502,14 @@ __device__ __forceinline__ bool bar1_or(bool v) {
   return r != 0;
 }
 
-template <bool SYM, int NDT>
+// FULL: chunks of the geometry's whole length (large n), a compile-time
+// constant: with a run-time length the row counters cost the U != V kernel
+// 6% at 128^3 (968 -> 1031 us), so the other instantiation serves only the
+// sizes whose chunks are shorter.
+template <bool SYM, int NDT, bool FULL>
 __global__ void __launch_bounds__(TR_THREADS, 1)
 oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const float2* __restrict__ V,
-                       float2* part, int nbj, int tri) {
+                       float2* part, int nbj, int tri, int ec) {
   using Geo = TrGeom<SYM, NDT>;
   int bi = 0, bj = (int)blockIdx.y;
   if (tri) {
@@ -1519,9 +1525,11 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
   }
   const int cu0 = 64 * bi, cv0 = 64 * bj;
   const int wu = min(64, p - cu0), wv = min(64, q - cv0);  // live columns (even: p, q even)
-  constexpr int EC = Geo::EC, SK = Geo::SK, NSUB = Geo::NSUB, NB = Geo::NB, NR = Geo::NR;
-  constexpr int MS = Geo::MS, MSW = Geo::MSW, MB = Geo::MB, NMB = Geo::NMB;
-  static_assert(NMB % 2 == 0, "the maxima warps take alternate batches");
+  constexpr int SK = Geo::SK, NB = Geo::NB, NR = Geo::NR;
+  constexpr int MS = Geo::MS, MSW = Geo::MSW, MB = Geo::MB;
+  static_assert(Geo::EC % SK == 0 && SK % (2 * MB) == 0, "chunks are whole sub-chunks; the maxima warps take alternate batches");
+  const int EC = FULL ? Geo::EC : ec;
+  const int NSUB = EC / SK, NMB = EC / MB;  // sub-chunks and maxima batches per chunk
   constexpr uint32_t plane = Geo::PLANE, DBUF = Geo::DBUF;
   extern __shared__ __align__(16) unsigned char tr_smem[];
   float2* raw = reinterpret_cast<float2*>(tr_smem);  // NR slots of 32 rows
@@ -1556,7 +1564,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
   }
   const int nchunks = (int)((n + EC - 1) / EC);  // n < 2^34 (checked by the caller)
   const int nmy = (int)blockIdx.x < nchunks ? (nchunks - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-  const int G = nmy * NSUB;
+  const int G = nmy * NSUB;  // sub-chunks of this CTA
   const uint32_t mbase = smem_addr(mbar), msbase = smem_addr(mbar + NB + 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -1577,16 +1585,37 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
     const int total = nmy * NMB / 2;  // this warp's batches
     const bool contU = wu == p, contV = SYM ? contU : wv == q;
     const int strU = contU ? p : 64, strV = contV ? q : 64;
-    auto batch_rows = [&](int t, int64_t& R0) {  // first row of this warp's t-th batch
-      const int gb = 2 * t + mw;
-      const int j = gb / NMB, b = gb - j * NMB;
-      R0 = ((int64_t)blockIdx.x + (int64_t)j * gridDim.x) * EC + (int64_t)b * MB;
+    // first rows of this warp's next batch to copy and to reduce, carried
+    // along (a division per batch by the run-time chunk length cost the
+    // U != V kernel 8%: these two warps pace the others)
+    const int64_t skip = (int64_t)(gridDim.x - 1) * EC;  // from a chunk's end to this CTA's next
+    struct Walk {
+      int64_t R0;
+      int b;
+    };
+    auto advance = [&](Walk& w) {
+      w.R0 += 2 * MB;
+      w.b += 2;
+      if (w.b >= NMB) {
+        w.b = mw;
+        w.R0 += skip;
+      }
+    };
+    Walk wi{(int64_t)blockIdx.x * EC + mw * MB, mw}, wd = wi;
+    auto row_of = [&](int t, Walk& w) {  // first row of this warp's t-th batch (t ascending)
+      if (FULL) {
+        const int gb = 2 * t + mw;
+        const int j = gb / NMB, b = gb - j * NMB;
+        return ((int64_t)blockIdx.x + (int64_t)j * gridDim.x) * EC + (int64_t)b * MB;
+      }
+      const int64_t R0 = w.R0;
+      advance(w);
+      return R0;
     };
     auto slot_of = [&](int t) { return mslot + (size_t)(mw * MSW + t % MSW) * 16 * 64; };
     auto bar_of = [&](int t) { return msbase + 8u * (uint32_t)(mw * MSW + t % MSW); };
     auto issue = [&](int t) {
-      int64_t R0;
-      batch_rows(t, R0);
+      const int64_t R0 = row_of(t, wi);
       const int64_t left = n - R0;
       const int nv = left <= 0 ? 0 : (left < MB ? (int)left : MB);
       float2* sl = slot_of(t);
@@ -1649,9 +1678,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
             break;
           }
           done_t = t + 1;
-          int64_t R0;
-          batch_rows(t, R0);
-          const int64_t left = n - R0;  // cells i % MB below it are live
+          const int64_t left = n - row_of(t, wd);  // cells i % MB below it are live
           const float2* sl = slot_of(t) + 2 * lane;
           if (left >= MB && lu && (SYM || lv)) {
             float4 v[16];
@@ -1747,9 +1774,21 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
     const float2* sA = U + cu0 + sc + (int64_t)sr * ldA;
     const float2* sB = SYM ? U + cu0 + sc + (int64_t)(sr + 16) * ldA : V + cv0 + sc + (int64_t)sr * ldB;
     const int64_t rA0 = sr, rB0 = SYM ? sr + 16 : sr;
+    // sub-chunks are staged in order: their first row is carried along
+    int64_t st_r0 = (int64_t)blockIdx.x * EC;
+    int st_s = 0;
     auto stage_sub = [&](int g) {
       if (g < G) {
-        const int64_t r0 = (int64_t)((int)blockIdx.x + (g / NSUB) * (int)gridDim.x) * EC + (g % NSUB) * SK;
+        int64_t r0 = st_r0;
+        if (FULL) {
+          r0 = (int64_t)((int)blockIdx.x + (g / NSUB) * (int)gridDim.x) * EC + (g % NSUB) * SK;
+        } else {
+          st_r0 += SK;
+          if (++st_s == NSUB) {
+            st_s = 0;
+            st_r0 += (int64_t)(gridDim.x - 1) * EC;
+          }
+        }
         float2* slot = raw + (size_t)(g % NR) * (32 * TG_RS) + sr * TG_RS + sc;
         const bool okA = sokA && r0 + rA0 < n, okB = sokB && r0 + rB0 < n;
         cp_async16(slot, okA ? sA + r0 * ldA : U, okA);
@@ -1781,9 +1820,15 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
     }
     __syncthreads();  // the maxima warps have written chunk 0's exponents
     float scut = worker ? exp2i(7 - Ex[(isv ? 64 : 0) + ic]) : 0.f;
+    int k = 0, s = -1;
     for (int g = 0; g < G; ++g) {
-      const int k = g / NSUB;
-      const int s = g - k * NSUB;
+      if (FULL) {
+        k = g / NSUB;
+        s = g - k * NSUB;
+      } else if (++s == NSUB) {
+        s = 0;
+        ++k;
+      }
       const int buf = g % NB;
       const int es = k & 1;
       if (!failed) {
@@ -1923,57 +1968,91 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
   __syncthreads();
 }
 
-// Fixed-order sum of the per-block partials into G (float64, p x q); the
-// symmetric case fills the lower triangle from the upper one.
-__global__ void oz_gram_reduce_kernel(int p, int q, int nsplit, int nblk, int sym, int nbj,
-                                      const float2* part, double* G) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= p * q) return;
-  int i = e / q, j = e - i * q;
-  int si = i, sj = j;
-  if (sym && i > j) {
-    si = j;
-    sj = i;
-  }
-  int bi = si / 64, bj = sj / 64;
-  int b;
-  if (sym) {
-    b = 0;
-    for (int r = 0; r < bi; ++r) b += nbj - r;
-    b += bj - bi;
-  } else {
-    b = bi * nbj + bj;
-  }
-  int ii = si - bi * 64, jj = sj - bj * 64;
-  if (sym && bi == bj && (ii / 16) > (jj / 16)) {  // lower warp tile inside a diagonal block
-    int t = ii;
-    ii = jj;
-    jj = t;
-  }
+// Fixed-order sums of the per-block partials. A block is 32 entries x
+// RED_GROUPS groups: warp g adds the splits k = g, g + RED_GROUPS, ... in
+// ascending order (lanes on consecutive entries, four loads in flight), and
+// the group sums are added in group order. One thread per entry instead had
+// a chain of 152 dependent df64 additions (20 float operations each) and
+// only p q / 256 blocks: 22-24 us for any p, q at 152 splits, against 3-4 us.
+constexpr int RED_GROUPS = 8;
+
+template <class Src>
+__device__ __forceinline__ float2 red_groups(int nsplit, Src src, float2 (*sm)[33]) {
+  const int lane = threadIdx.x & 31, grp = threadIdx.x >> 5;
   float2 s = make_float2(0.f, 0.f);
-  // unrolled so that several partials are in flight at once (same order)
-#pragma unroll 8
-  for (int k = 0; k < nsplit; ++k) s = df_add(s, part[((size_t)k * nblk + b) * 4096 + ii * 64 + jj]);
-  G[e] = df_to_double(s);
+#pragma unroll 4
+  for (int k = grp; k < nsplit; k += RED_GROUPS) s = df_add(s, src(k));
+  __syncthreads();
+  sm[grp][lane] = s;
+  __syncthreads();
+  float2 t = sm[0][lane];
+  for (int g = 1; g < RED_GROUPS; ++g) t = df_add(t, sm[g][lane]);
+  return t;  // the same in every group
+}
+
+// G (float64, p x q) from the partials; the symmetric case fills the lower
+// triangle from the upper one. sym2: U != V but U^T V symmetric in exact
+// arithmetic (p == q): G = (G + G^T) / 2, both entries summed here, which
+// saves the symmetrising launch that followed.
+__global__ void __launch_bounds__(32 * RED_GROUPS)
+oz_gram_reduce_kernel(int p, int q, int nsplit, int nblk, int sym, int sym2, int nbj, const float2* part,
+                      double* G) {
+  __shared__ float2 sm[RED_GROUPS][33];
+  const int e = blockIdx.x * 32 + (threadIdx.x & 31);
+  const bool live = e < p * q;
+  const int i = live ? e / q : 0, j = live ? e - i * q : 0;
+  auto at = [&](int r, int c) {
+    int si = r, sj = c;
+    if (sym && r > c) {
+      si = c;
+      sj = r;
+    }
+    const int bi = si / 64, bj = sj / 64;
+    int b;
+    if (sym) {
+      b = 0;
+      for (int z = 0; z < bi; ++z) b += nbj - z;
+      b += bj - bi;
+    } else {
+      b = bi * nbj + bj;
+    }
+    int ii = si - bi * 64, jj = sj - bj * 64;
+    if (sym && bi == bj && (ii / 16) > (jj / 16)) {  // lower warp tile inside a diagonal block
+      const int t = ii;
+      ii = jj;
+      jj = t;
+    }
+    return part + (size_t)b * 4096 + ii * 64 + jj;
+  };
+  const float2* P = at(i, j);
+  const size_t stride = (size_t)nblk * 4096;
+  double v = df_to_double(red_groups(nsplit, [&](int k) { return P[k * stride]; }, sm));
+  if (sym2) {
+    const float2* Pt = at(j, i);
+    const double w = df_to_double(red_groups(nsplit, [&](int k) { return Pt[k * stride]; }, sm));
+    v = i <= j ? 0.5 * (v + w) : 0.5 * (w + v);
+  }
+  if (live && threadIdx.x < 32) G[e] = v;
 }
 
 // The same for a symmetric Gram whose upper-triangle blocks (bi <= bj, row by
 // row) were computed in full by the tcgen05 kernel: entry (i, j) is read
 // from the upper triangle, so G is exactly symmetric.
-__global__ void oz_gram_reduce_tri_kernel(int p, int nsplit, int nblk, int nbj, const float2* part, double* G) {
-  int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= p * p) return;
-  const int i = e / p, j = e - i * p;
+__global__ void __launch_bounds__(32 * RED_GROUPS)
+oz_gram_reduce_tri_kernel(int p, int nsplit, int nblk, int nbj, const float2* part, double* G) {
+  __shared__ float2 sm[RED_GROUPS][33];
+  const int e = blockIdx.x * 32 + (threadIdx.x & 31);
+  const bool live = e < p * p;
+  const int i = live ? e / p : 0, j = live ? e - i * p : 0;
   const int si = min(i, j), sj = max(i, j);
   const int bi = si / 64, bj = sj / 64;
   int b = 0;
   for (int r = 0; r < bi; ++r) b += nbj - r;
   b += bj - bi;
-  const int ii = si - bi * 64, jj = sj - bj * 64;
-  float2 s = make_float2(0.f, 0.f);
-#pragma unroll 8
-  for (int k = 0; k < nsplit; ++k) s = df_add(s, part[((size_t)k * nblk + b) * 4096 + ii * 64 + jj]);
-  G[e] = df_to_double(s);
+  const float2* P = part + (size_t)b * 4096 + (si - bi * 64) * 64 + (sj - bj * 64);
+  const size_t stride = (size_t)nblk * 4096;
+  const float2 t = red_groups(nsplit, [&](int k) { return P[k * stride]; }, sm);
+  if (live && threadIdx.x < 32) G[e] = df_to_double(t);
 }
 
 // ---------------------------------------------------------------------------
@@ -2128,9 +2207,26 @@ int oz_gram_blocks(int p, int q, bool sym) {
   return sym ? nbi * (nbi + 1) / 2 : nbi * nbj;
 }
 
+constexpr int GRAM_MIN_ROWS = 32;  // fewest rows worth a split of their own
+
+// Rows of an exponent chunk for n rows over ns CTAs: a multiple of `unit`
+// rows, at most `most`, such that every CTA gets the same number of chunks.
+// A CTA's time is its sub-chunks in a row (about 1.1-2 us each) after the
+// maxima of its first chunk, so at small n full chunks left most SMs idle:
+// n = 1024 ran on 3 CTAs of 24 sub-chunks (p = 8: U^T V 48.9 us, U^T U 35.0
+// us; with this rule 32 CTAs, 13.1 and 11.4 us), n = 35,000 on 92 (p = 16:
+// 49.2 -> 36.9, 35.3 -> 23.1 us). Equal chunk counts also even out the large
+// sizes. Shorter chunks only make the digit grid finer.
+static int gram_chunk_rows(int64_t n, int ns, int unit, int most) {
+  const int64_t per = (n + ns - 1) / ns;             // rows a CTA
+  const int64_t k = std::max<int64_t>(1, (per + most - 1) / most);  // chunks a CTA
+  const int64_t rows = (per + k - 1) / k;
+  return (int)std::min<int64_t>(most, std::max<int64_t>(unit, (rows + unit - 1) / unit * unit));
+}
+
 int oz_gram_splits(int64_t n, int p, int q, bool sym) {
   int nb = oz_gram_blocks(p, q, sym);
-  int64_t chunks = (n + GR_KC - 1) / GR_KC;
+  int64_t chunks = (n + GRAM_MIN_ROWS - 1) / GRAM_MIN_ROWS;
   int s = std::max(1, sm_count() / nb);
   return (int)std::max<int64_t>(1, std::min<int64_t>(s, chunks));
 }
@@ -2155,9 +2251,9 @@ __global__ void oz_gram_reduce_df_kernel(int p, int q, int nsplit, int nbj, cons
 }
 
 gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bool sym, double* G,
-                   float2* scratch, cudaStream_t st, int nd, float2* Gdf, int reserve_sms) {
+                   float2* scratch, cudaStream_t st, int nd, float2* Gdf, int reserve_sms, bool sym2) {
   if (p < 1 || q < 1 || q > 128 || (sym && (p != q || Gdf)) || (nd != 3 && nd != ND) ||
-      (!G && !Gdf) || (p > 128 && !Gdf))
+      (!G && !Gdf) || (p > 128 && !Gdf) || (sym2 && (sym || p != q || Gdf)))
     return GSI_ERR_ARG;
   const int nbj = (q + 63) / 64;
   const int nblk = oz_gram_blocks(p, q, sym);
@@ -2178,18 +2274,24 @@ gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bo
     tri = sym && !one;
     const bool ksym = sym && one;
     const size_t tsm = oz_gram_tc_ring_smem(ksym, nd);
-    auto kern = nd == 3 ? (ksym ? oz_gram_tc_ring_kernel<true, 3> : oz_gram_tc_ring_kernel<false, 3>)
-                        : (ksym ? oz_gram_tc_ring_kernel<true, ND> : oz_gram_tc_ring_kernel<false, ND>);
+    // (3 digits: always full chunks, whose exponents set those products' errors)
+    const int most = ksym ? TrGeom<true>::EC : TrGeom<false>::EC;
+    const int ec = nd == ND ? gram_chunk_rows(n, ns, ksym ? TrGeom<true>::SK : TrGeom<false>::SK, most) : most;
+    auto kern = ec == most ? (ksym ? oz_gram_tc_ring_kernel<true, ND, true> : oz_gram_tc_ring_kernel<false, ND, true>)
+                           : (ksym ? oz_gram_tc_ring_kernel<true, ND, false> : oz_gram_tc_ring_kernel<false, ND, false>);
+    if (nd == 3) kern = ksym ? oz_gram_tc_ring_kernel<true, 3, true> : oz_gram_tc_ring_kernel<false, 3, true>;
     GSI_CUDA_TRY(ensure_dyn_smem((const void*)kern, (int)tsm));
     kern<<<dim3(ns, one ? 1 : nblk), TR_THREADS, tsm, st>>>(n, p, q, U, V, scratch, one ? 1 : nbj,
-                                                            tri ? 1 : 0);
+                                                            tri ? 1 : 0, ec);
     GSI_LAUNCH_CHECK();
   } else if (nd == ND && p <= 64 && q <= 64 && tp != 1) {
     // one 64 x 64 output block; every partial entry is written
     const size_t tsm = oz_gram_tc_smem(sym);
     auto kern = sym ? oz_gram_tc_kernel<true> : oz_gram_tc_kernel<false>;
     GSI_CUDA_TRY(ensure_dyn_smem((const void*)kern, (int)tsm));
-    kern<<<ns, TG_THREADS, tsm, st>>>(n, p, q, U, V, vec16 ? 1 : 0, scratch, 1, 0);
+    const int ec = sym ? gram_chunk_rows(n, ns, 2 * TgGeom<true>::SK, TgGeom<true>::EC)
+                       : gram_chunk_rows(n, ns, 2 * TgGeom<false>::SK, TgGeom<false>::EC);
+    kern<<<ns, TG_THREADS, tsm, st>>>(n, p, q, U, V, vec16 ? 1 : 0, scratch, 1, 0, ec);
     GSI_LAUNCH_CHECK();
   } else if (nd == ND && tp != 1) {
     // several 64 x 64 output blocks (p or q > 64), one per blockIdx.y, each
@@ -2198,8 +2300,9 @@ gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bo
     tri = sym;
     const size_t tsm = oz_gram_tc_smem(false);
     GSI_CUDA_TRY(ensure_dyn_smem((const void*)oz_gram_tc_kernel<false>, (int)tsm));
+    const int ec = gram_chunk_rows(n, ns, 2 * TgGeom<false>::SK, TgGeom<false>::EC);
     oz_gram_tc_kernel<false><<<dim3(ns, nblk), TG_THREADS, tsm, st>>>(n, p, q, U, V, vec16 ? 1 : 0, scratch, nbj,
-                                                                     tri ? 1 : 0);
+                                                                     tri ? 1 : 0, ec);
     GSI_LAUNCH_CHECK();
   } else {
     size_t smem = oz_gram_smem(nd);
@@ -2212,10 +2315,10 @@ gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bo
   if (Gdf) {
     oz_gram_reduce_df_kernel<<<ceil_div((int64_t)p * q, 256), 256, 0, st>>>(p, q, ns, nbj, scratch, Gdf);
   } else if (tri) {
-    oz_gram_reduce_tri_kernel<<<ceil_div(p * q, 256), 256, 0, st>>>(p, ns, nblk, nbj, scratch, G);
+    oz_gram_reduce_tri_kernel<<<ceil_div(p * q, 32), 32 * RED_GROUPS, 0, st>>>(p, ns, nblk, nbj, scratch, G);
   } else {
-    oz_gram_reduce_kernel<<<ceil_div(p * q, 256), 256, 0, st>>>(p, q, ns, nblk, sym ? 1 : 0, nbj,
-                                                                scratch, G);
+    oz_gram_reduce_kernel<<<ceil_div(p * q, 32), 32 * RED_GROUPS, 0, st>>>(p, q, ns, nblk, sym ? 1 : 0,
+                                                                           sym2 ? 1 : 0, nbj, scratch, G);
   }
   GSI_LAUNCH_CHECK();
   return GSI_OK;

@@ -302,11 +302,7 @@ gsi_status op_gram(gsi_ctx* c, const void* U, const void* V, bool sym, double* G
   gsi_status s;
   if (c->emu) {
     s = oz_gram(c->n, c->p, c->p, (const float2*)U, (const float2*)V, sym && U == V, G,
-                c->oz_gram_ws, c->st, 7, nullptr, c->gram_reserve);
-    if (s == GSI_OK && sym && U != V) {
-      symmetrize_kernel<<<ceil_div(c->p * c->p, 256), 256, 0, c->st>>>(c->p, G);
-      note_launch();
-    }
+                c->oz_gram_ws, c->st, 7, nullptr, c->gram_reserve, sym && U != V);
   } else {
     s = gram(c->n, c->p, c->p, (const double*)U, (const double*)V, G, c->gram_ws, c->st);
     if (s == GSI_OK && sym) {
