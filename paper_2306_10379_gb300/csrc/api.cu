@@ -5,6 +5,7 @@
 
 #include "blas_f64.cuh"
 #include "oz.cuh"
+#include "small_df.cuh"
 
 using namespace gsi;
 
@@ -75,7 +76,19 @@ gsi_status gsi_linesearch(int32_t p, const double* C, const double* B, const dou
   ScratchGuard g(st);
   if (precision == GSI_PREC_DF64) {
     GSI_CUDA_TRY(cudaMallocAsync(&g.ptr, small_df_scratch_bytes(p), st));
-    return small_step_df(0, p, C, B, Gam, Z, XX, XD, M, out, g.ptr, st);
+    PpArgs a{};
+    a.mode = 0;
+    a.p = p;
+    a.C = {nullptr, C, 1};
+    a.B = {nullptr, B, 1};
+    a.Gam = {nullptr, Gam, 1};
+    a.Z = {nullptr, Z, 1};
+    a.XX = {nullptr, XX, 1};
+    a.XD = {nullptr, XD, 0};
+    a.M = M;
+    a.out = out;
+    a.gws = (float2*)g.ptr;
+    return small_step_df(a, true, st);
   }
   GSI_CUDA_TRY(cudaMallocAsync(&g.ptr, small_scratch_doubles(p) * sizeof(double), st));
   return small_step(0, p, C, B, Gam, Z, XX, XD, M, out, (double*)g.ptr, st);

@@ -34,7 +34,7 @@
 #include "common.cuh"
 #include "df.cuh"
 #include "oz.cuh"
-#include "small_df_dev.cuh"
+#include "pp_dev.cuh"
 
 namespace gsi {
 namespace {
@@ -608,35 +608,55 @@ __global__ void __launch_bounds__(BT) b_retract_kernel(BDev d, int32_t mode) {
 }
 
 // ---- the p x p step, one block per problem ------------------------------------
-// The step of the single-problem df64 path (float32 Jacobi refined to df64,
-// Alg. 3 in float64, M = S^{-1/2} by the first-order expansion in the
-// eigenbasis), run by one block per problem on its reduced Grams.
+// The step of the single-problem df64 path (pp_dev.cuh), run by one block per
+// problem on its reduced Grams.
 // mode 0 (step problems): X^T D = (I - X^T X)(C + beta K); the step t and
 //   M; K_next = M (X^T D + t D^T D); the recompute decision.
 // mode 1 (F_START): M = (X^T X)^{-1/2}.
 // mode 2 (F_START): Rayleigh-Ritz, C' = U diag(theta) U^T, theta descending,
 //   M = U.
+using BPp16 = PpCfg<BS, 16, 1, 1, 1, 1, 1>;
+using BPp32 = PpCfg<BS, 32, 4, 1, 1, 1, 1>;
+
 __global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
   const int i = blockIdx.x;
   const int32_t mask = mode == 0 ? F_STEP : F_START;
   if (!(d.st[i].flags & mask)) return;
   extern __shared__ __align__(16) unsigned char sm_dyn[];
-  __shared__ double red[BS / 32];
-  __shared__ int flag;
-  __shared__ double sh_t;
+  __shared__ PpSh sh;
   __shared__ double outs[16];
   __shared__ int order[PMAX];
   const int tid = threadIdx.x;
   const BProb pr = d.prob[i];
   const int p = pr.p, q = p * p;
-  SdWs w = sd_carve(sm_dyn, p);
   double* M = d.Mm + pr.ppoff;
   double* XD = d.XDm + pr.ppoff;
-  const double* C = d.Cm + pr.ppoff;
   const double* G4 = d.G4 + (int64_t)NG * pr.ppoff;  // D^T D, D^T W, D^T R, X^T X
+  PpArgs a{};
+  a.mode = mode;
+  a.p = p;
+  a.B = {nullptr, G4, 0};
+  a.M = M;
+  a.theta = XD;
+  a.out = outs;
+  if (mode == 0) {
+    a.C = {nullptr, d.Cm + pr.ppoff, 0};
+    a.Gam = {nullptr, G4 + q, 0};
+    a.Z = {nullptr, d.cg ? G4 + 2 * q : G4, 0};
+    a.XX = {nullptr, G4 + 3 * q, 0};
+    a.K = {nullptr, d.Km + pr.ppoff, 0};
+    a.beta = d.st[i].beta;
+    a.Kd = d.cg ? d.Km + pr.ppoff : nullptr;
+  }
+  if (p <= 16) {
+    PpCtx<BPp16> c = pp_ctx<BPp16>(sm_dyn, &sh, p, nullptr);
+    pp_body<BPp16>(a, c);
+  } else {
+    PpCtx<BPp32> c = pp_ctx<BPp32>(sm_dyn, &sh, p, nullptr);
+    pp_body<BPp32>(a, c);
+  }
+  __syncthreads();
   if (mode == 1) {
-    small_df_body(1, p, nullptr, G4, nullptr, nullptr, nullptr, nullptr, M, outs, w, red, &flag, &sh_t);
-    __syncthreads();
     if (tid == 0 && outs[3] != 0.0) {
       d.st[i].status = GSI_ERR_BREAKDOWN;
       d.st[i].flags = 0;
@@ -644,20 +664,18 @@ __global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
     return;
   }
   if (mode == 2) {
-    small_df_body(2, p, nullptr, G4, nullptr, nullptr, nullptr, XD, M, outs, w, red, &flag, &sh_t);
-    __syncthreads();
     if (tid == 0) {
       for (int k = 0; k < p; ++k) order[k] = k;
-      for (int a = 0; a < p; ++a) {  // selection sort, descending
-        int best = a;
-        for (int c = a + 1; c < p; ++c)
+      for (int z = 0; z < p; ++z) {  // selection sort, descending
+        int best = z;
+        for (int c = z + 1; c < p; ++c)
           if (XD[order[c]] > XD[order[best]]) best = c;
-        const int tmp = order[a];
-        order[a] = order[best];
+        const int tmp = order[z];
+        order[z] = order[best];
         order[best] = tmp;
       }
     }
-    double* tmp = reinterpret_cast<double*>(w.Td);  // q doubles of scratch
+    double* tmp = reinterpret_cast<double*>(sm_dyn);  // q doubles of scratch
     for (int e = tid; e < q; e += BS) tmp[e] = M[e];
     __syncthreads();
     for (int k = tid; k < p; k += BS) d.theta[pr.ppoff + k] = XD[order[k]];
@@ -667,22 +685,6 @@ __global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
     }
     return;
   }
-  const double beta_used = d.st[i].beta;
-  const double* Bm = G4;
-  const double* XX = G4 + 3 * q;
-  double* G2 = reinterpret_cast<double*>(w.Ud);  // q doubles of scratch
-  for (int e = tid; e < q; e += BS)
-    G2[e] = beta_used != 0.0 ? C[e] + beta_used * d.Km[pr.ppoff + e] : C[e];
-  __syncthreads();
-  for (int e = tid; e < q; e += BS) {
-    const int r = e / p, c = e - r * p;
-    double s = 0.0;
-    for (int k = 0; k < p; ++k) s = fma(XX[r * p + k], G2[k * p + c], s);
-    XD[e] = G2[e] - s;
-  }
-  __syncthreads();
-  small_df_body(0, p, C, Bm, G4 + q, d.cg ? G4 + 2 * q : Bm, XX, XD, M, outs, w, red, &flag, &sh_t);
-  __syncthreads();
   const double t = outs[0];
   if (!isfinite(t) || outs[3] != 0.0) {
     if (tid == 0) {
@@ -690,17 +692,6 @@ __global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
       d.st[i].flags = 0;
     }
     return;
-  }
-  if (d.cg) {  // K_next = M (X^T D + t D^T D)
-    double* T = reinterpret_cast<double*>(w.Ud);
-    for (int e = tid; e < q; e += BS) T[e] = XD[e] + t * Bm[e];
-    __syncthreads();
-    for (int e = tid; e < q; e += BS) {
-      const int r = e / p, c = e - r * p;
-      double s = 0.0;
-      for (int k = 0; k < p; ++k) s = fma(M[r * p + k], T[k * p + c], s);
-      d.Km[pr.ppoff + e] = s;
-    }
   }
   if (tid == 0) {
     BState s = d.st[i];
@@ -1315,7 +1306,7 @@ gsi_status gsi_batched_create(int32_t nprob, const int32_t* n, const int32_t* p,
                                cudaMemcpyHostToDevice)));
   CK(cuda_status_ok(cudaMemset(b->Km, 0, (size_t)pp * sizeof(double))));
   {
-    b->small_smem = sd_bytes(pmax);
+    b->small_smem = pp_smem(pmax, 1);
     CK(cuda_status_ok(cudaFuncSetAttribute(b_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)b->small_smem)));
   }

@@ -1996,7 +1996,7 @@ __device__ __forceinline__ float2 red_groups(int nsplit, Src src, float2 (*sm)[3
 // saves the symmetrising launch that followed.
 __global__ void __launch_bounds__(32 * RED_GROUPS)
 oz_gram_reduce_kernel(int p, int q, int nsplit, int nblk, int sym, int sym2, int nbj, const float2* part,
-                      double* G) {
+                      double* G, float2* Gf) {
   __shared__ float2 sm[RED_GROUPS][33];
   const int e = blockIdx.x * 32 + (threadIdx.x & 31);
   const bool live = e < p * q;
@@ -2032,14 +2032,17 @@ oz_gram_reduce_kernel(int p, int q, int nsplit, int nblk, int sym, int sym2, int
     const double w = df_to_double(red_groups(nsplit, [&](int k) { return Pt[k * stride]; }, sm));
     v = i <= j ? 0.5 * (v + w) : 0.5 * (w + v);
   }
-  if (live && threadIdx.x < 32) G[e] = v;
+  if (live && threadIdx.x < 32) {
+    G[e] = v;
+    if (Gf) Gf[e] = df_from_double(v);
+  }
 }
 
 // The same for a symmetric Gram whose upper-triangle blocks (bi <= bj, row by
 // row) were computed in full by the tcgen05 kernel: entry (i, j) is read
 // from the upper triangle, so G is exactly symmetric.
 __global__ void __launch_bounds__(32 * RED_GROUPS)
-oz_gram_reduce_tri_kernel(int p, int nsplit, int nblk, int nbj, const float2* part, double* G) {
+oz_gram_reduce_tri_kernel(int p, int nsplit, int nblk, int nbj, const float2* part, double* G, float2* Gf) {
   __shared__ float2 sm[RED_GROUPS][33];
   const int e = blockIdx.x * 32 + (threadIdx.x & 31);
   const bool live = e < p * p;
@@ -2052,7 +2055,10 @@ oz_gram_reduce_tri_kernel(int p, int nsplit, int nblk, int nbj, const float2* pa
   const float2* P = part + (size_t)b * 4096 + (si - bi * 64) * 64 + (sj - bj * 64);
   const size_t stride = (size_t)nblk * 4096;
   const float2 t = red_groups(nsplit, [&](int k) { return P[k * stride]; }, sm);
-  if (live && threadIdx.x < 32) G[e] = df_to_double(t);
+  if (live && threadIdx.x < 32) {
+    G[e] = df_to_double(t);
+    if (Gf) Gf[e] = t;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -2251,7 +2257,7 @@ __global__ void oz_gram_reduce_df_kernel(int p, int q, int nsplit, int nbj, cons
 }
 
 gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bool sym, double* G,
-                   float2* scratch, cudaStream_t st, int nd, float2* Gdf, int reserve_sms, bool sym2) {
+                   float2* scratch, cudaStream_t st, int nd, float2* Gdf, int reserve_sms, bool sym2, float2* Gf) {
   if (p < 1 || q < 1 || q > 128 || (sym && (p != q || Gdf)) || (nd != 3 && nd != ND) ||
       (!G && !Gdf) || (p > 128 && !Gdf) || (sym2 && (sym || p != q || Gdf)))
     return GSI_ERR_ARG;
@@ -2315,10 +2321,10 @@ gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bo
   if (Gdf) {
     oz_gram_reduce_df_kernel<<<ceil_div((int64_t)p * q, 256), 256, 0, st>>>(p, q, ns, nbj, scratch, Gdf);
   } else if (tri) {
-    oz_gram_reduce_tri_kernel<<<ceil_div(p * q, 32), 32 * RED_GROUPS, 0, st>>>(p, ns, nblk, nbj, scratch, G);
+    oz_gram_reduce_tri_kernel<<<ceil_div(p * q, 32), 32 * RED_GROUPS, 0, st>>>(p, ns, nblk, nbj, scratch, G, Gf);
   } else {
     oz_gram_reduce_kernel<<<ceil_div(p * q, 32), 32 * RED_GROUPS, 0, st>>>(p, q, ns, nblk, sym ? 1 : 0,
-                                                                           sym2 ? 1 : 0, nbj, scratch, G);
+                                                                           sym2 ? 1 : 0, nbj, scratch, G, Gf);
   }
   GSI_LAUNCH_CHECK();
   return GSI_OK;

@@ -53,10 +53,10 @@ size_t oz_gram_scratch_bytes(int64_t n, int p, int q, bool sym);
 // the dense apply A X = A^T X.
 // reserve_sms: SMs left free for work running alongside on another stream.
 // sym2 (U != V, p == q, G only): U^T V is symmetric in exact arithmetic (D^T A D);
-// G = (U^T V + (U^T V)^T) / 2.
+// G = (U^T V + (U^T V)^T) / 2. Gf: the same G in df64 as well (p x q), or null.
 gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bool sym, double* G,
                    float2* scratch, cudaStream_t st, int nd = 7, float2* Gdf = nullptr,
-                   int reserve_sms = 0, bool sym2 = false);
+                   int reserve_sms = 0, bool sym2 = false, float2* Gf = nullptr);
 
 // Bounded waits of the tcgen05 kernels: polls allowed to a wait on a batch of
 // products (limit < 0: the default, 2^24); a wait that runs out drains the

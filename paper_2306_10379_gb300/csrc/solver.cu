@@ -30,6 +30,7 @@
 #include "blas_f64.cuh"
 #include "df.cuh"
 #include "oz.cuh"
+#include "small_df.cuh"
 
 namespace gsi {
 
@@ -139,6 +140,7 @@ struct gsi_ctx {
   void *X = nullptr, *Y = nullptr, *R = nullptr, *Rp = nullptr, *D = nullptr, *P = nullptr,
        *W = nullptr, *Xn = nullptr, *Yn = nullptr;
   double* pp = nullptr;  // p x p matrices
+  float2* ppf = nullptr;  // their df64 copies (same offsets), written by the Grams and the p x p step
   double *Cm, *Bm, *Gm, *Zm, *XXm, *XDm, *Km, *Mm, *Gm2, *out, *dout;
   double *Tm, *Fm;  // p x p scratch of gsi_get_basis, which no iteration reads
   double* gram_ws = nullptr;
@@ -149,13 +151,15 @@ struct gsi_ctx {
   bool rinf_fused = false;   // the last block product also left max_r sum_j |R[r,j]| in dout[2]
   double* dots_ws = nullptr;
   double* small_ws = nullptr;
-  // the eigenbasis of D^T D runs on a second stream while the other
-  // line-search Grams run on st (one SM left to it); V and the diagonal pass
-  // through eig_ws
+  // the eigenbasis of D^T D runs on st while the other line-search Grams run
+  // on a second stream and leave SMs to it; V and the diagonal pass through
+  // eig_ws
   cudaStream_t st2 = nullptr;
   cudaEvent_t ev_b = nullptr, ev_e = nullptr;
   void* eig_ws = nullptr;
-  int gram_reserve = 0;  // SMs the next Grams leave free
+  cudaStream_t gst = nullptr;  // the stream of the next Grams
+  int gram_reserve = 0;        // SMs they leave free
+  bool eig_cluster = false;    // 32 < p <= 64: the eigenbasis on a cluster of CTAs
   double* host = nullptr;  // pinned readback buffer
   // LOBCG comparator: p x p workspace, masks of the kept columns of the
   // second and third basis blocks, and the eigensolver's scratch for 3p x 3p
@@ -205,16 +209,16 @@ cudaEvent_t pool_get(gsi_ctx* c) {
   return e;
 }
 
-void prof_begin(gsi_ctx* c) {
+void prof_begin(gsi_ctx* c, cudaStream_t st = nullptr) {
   if (!c->prof) return;
   c->cur = pool_get(c);
-  cudaEventRecord(c->cur, c->st);
+  cudaEventRecord(c->cur, st ? st : c->st);
 }
 
-void prof_end(gsi_ctx* c, int k, double bytes, double flops) {
+void prof_end(gsi_ctx* c, int k, double bytes, double flops, cudaStream_t st = nullptr) {
   if (!c->prof || !c->cur) return;
   cudaEvent_t e = pool_get(c);
-  cudaEventRecord(e, c->st);
+  cudaEventRecord(e, st ? st : c->st);
   c->pending.push_back({k, c->cur, e});
   c->cur = nullptr;
   c->cls[k].launches++;
@@ -297,20 +301,27 @@ gsi_status op_matvec(gsi_ctx* c, const void* in, void* outp, bool accurate = tru
   return s;
 }
 
+// the df64 copy that goes with a p x p matrix of the context, or null
+float2* pp_df(gsi_ctx* c, const double* G) {
+  const size_t q = (size_t)c->p * c->p;
+  return c->ppf && G >= c->pp && G < c->pp + 11 * q ? c->ppf + (G - c->pp) : nullptr;
+}
+
 gsi_status op_gram(gsi_ctx* c, const void* U, const void* V, bool sym, double* G) {
-  prof_begin(c);
+  cudaStream_t st = c->gst ? c->gst : c->st;
+  prof_begin(c, st);
   gsi_status s;
   if (c->emu) {
     s = oz_gram(c->n, c->p, c->p, (const float2*)U, (const float2*)V, sym && U == V, G,
-                c->oz_gram_ws, c->st, 7, nullptr, c->gram_reserve, sym && U != V);
+                c->oz_gram_ws, st, 7, nullptr, c->gram_reserve, sym && U != V, pp_df(c, G));
   } else {
-    s = gram(c->n, c->p, c->p, (const double*)U, (const double*)V, G, c->gram_ws, c->st);
+    s = gram(c->n, c->p, c->p, (const double*)U, (const double*)V, G, c->gram_ws, st);
     if (s == GSI_OK && sym) {
-      symmetrize_kernel<<<ceil_div(c->p * c->p, 256), 256, 0, c->st>>>(c->p, G);
+      symmetrize_kernel<<<ceil_div(c->p * c->p, 256), 256, 0, st>>>(c->p, G);
       note_launch();
     }
   }
-  prof_end(c, GSI_K_GRAM, (U == V ? 1 : 2) * blk_bytes(c), 2.0 * c->n * c->p * c->p);
+  prof_end(c, GSI_K_GRAM, (U == V ? 1 : 2) * blk_bytes(c), 2.0 * c->n * c->p * c->p, st);
   return s;
 }
 
@@ -376,10 +387,45 @@ gsi_status op_rowinf(gsi_ctx* c, const void* Rb) {
   return s;
 }
 
+// a p x p input of the df64 step: the df64 copy where there is one
+PpMat pp_in(gsi_ctx* c, const double* G) {
+  float2* f = pp_df(c, G);
+  return f ? PpMat{f, nullptr, 0} : PpMat{nullptr, G, 1};
+}
+
+// The df64 p x p step (PpArgs, pp_dev.cuh): mode 1 with B; mode 2 with B,
+// eigenvectors into Mout, eigenvalues into theta; mode 3 with B; mode 4 with
+// C, B, Gm, Zp, XX and K (X^T D = (I - XX)(C + beta K) formed inside), K_next
+// into Km for CG.
+gsi_status op_pp(gsi_ctx* c, int mode, const double* B, const double* Zp, double beta, bool want_k,
+                 double* Mout = nullptr, double* theta = nullptr) {
+  PpArgs a{};
+  a.mode = mode;
+  a.p = c->p;
+  a.B = pp_in(c, B);
+  if (mode == 4) {
+    a.C = pp_in(c, c->Cm);
+    a.Gam = pp_in(c, c->Gm);
+    a.Z = pp_in(c, Zp);
+    a.XX = pp_in(c, c->XXm);
+    a.K = pp_in(c, c->Km);
+    a.beta = beta;
+    if (want_k) {
+      a.Kd = c->Km;
+      a.Kf = pp_df(c, c->Km);
+    }
+  }
+  a.M = Mout ? Mout : c->Mm;
+  a.theta = theta;
+  a.eig = (float2*)c->eig_ws;
+  a.out = c->out;
+  a.gws = (float2*)c->small_ws;
+  return small_step_df(a, mode == 3 ? c->eig_cluster : true, c->st);
+}
+
 gsi_status op_small(gsi_ctx* c, int mode, const double* B, const double* Zp) {
   prof_begin(c);
-  gsi_status s = c->emu ? small_step_df(mode, c->p, c->Cm, B, c->Gm, Zp, c->XXm, c->XDm, c->Mm,
-                                        c->out, c->small_ws, c->st, c->eig_ws)
+  gsi_status s = c->emu ? op_pp(c, mode, B, Zp, 0.0, false)
                         : small_step(mode, c->p, c->Cm, B, c->Gm, Zp, c->XXm, c->XDm, c->Mm, c->out,
                                      c->small_ws, c->st);
   prof_end(c, GSI_K_SMALL, 0.0, 0.0);
@@ -476,15 +522,16 @@ gsi_status iterate(gsi_ctx* c, bool* stop) {
   }
   GSI_TRY(op_matvec(c, Dp, c->W, false));
   GSI_TRY(op_gram(c, Dp, Dp, true, c->Bm));
-  // the eigenbasis of B = D^T D on the second stream, alongside the Grams below
+  // the eigenbasis of B = D^T D alongside the Grams below: it goes first on
+  // st, so that its CTAs are placed before the Grams (second stream, after
+  // the event) fill the remaining SMs
   const bool split = c->st2 != nullptr;
   if (split) {
     GSI_CUDA_TRY(cudaEventRecord(c->ev_b, c->st));
+    GSI_TRY(op_pp(c, 3, c->Bm, nullptr, 0.0, false));
     GSI_CUDA_TRY(cudaStreamWaitEvent(c->st2, c->ev_b, 0));
-    GSI_TRY(small_step_df(3, c->p, nullptr, c->Bm, nullptr, nullptr, nullptr, nullptr, nullptr, c->out,
-                          c->small_ws, c->st2, c->eig_ws));
-    GSI_CUDA_TRY(cudaEventRecord(c->ev_e, c->st2));
-    c->gram_reserve = 1;
+    c->gst = c->st2;
+    c->gram_reserve = c->p > 64 || c->eig_cluster ? 8 : 1;
   }
   gsi_status gs = op_gram(c, Dp, c->W, true, c->Gm);
   const double* Zp = c->Bm;
@@ -494,15 +541,25 @@ gsi_status iterate(gsi_ctx* c, bool* stop) {
   }
   if (gs == GSI_OK) gs = op_gram(c, c->X, c->X, true, c->XXm);
   c->gram_reserve = 0;
-  if (split) GSI_CUDA_TRY(cudaStreamWaitEvent(c->st, c->ev_e, 0));
+  c->gst = nullptr;
+  if (split) {
+    GSI_CUDA_TRY(cudaEventRecord(c->ev_e, c->st2));
+    GSI_CUDA_TRY(cudaStreamWaitEvent(c->st, c->ev_e, 0));
+  }
   GSI_TRY(gs);
   // X^T D in closed form from the measured X^T X: X^T R = (I - X^T X) C and
   // X^T P = K give X^T D = (I - X^T X)(C + b K) (b = 0 for SD and restarts)
-  prof_begin(c);
-  GSI_TRY(pp_axpby(c->p, 1.0, c->Cm, beta_used, beta_used != 0.0 ? c->Km : nullptr, c->Gm2, c->st));
-  GSI_TRY(pp_gemm(c->p, -1.0, c->XXm, c->Gm2, 1.0, c->Gm2, c->XDm, c->st));
-  prof_end(c, GSI_K_SMALL, 0.0, 0.0);
-  GSI_TRY(op_small(c, split ? 4 : 0, c->Bm, Zp));
+  if (split) {
+    prof_begin(c);
+    GSI_TRY(op_pp(c, 4, c->Bm, Zp, beta_used, cg));
+    prof_end(c, GSI_K_SMALL, 0.0, 0.0);
+  } else {
+    prof_begin(c);
+    GSI_TRY(pp_axpby(c->p, 1.0, c->Cm, beta_used, beta_used != 0.0 ? c->Km : nullptr, c->Gm2, c->st));
+    GSI_TRY(pp_gemm(c->p, -1.0, c->XXm, c->Gm2, 1.0, c->Gm2, c->XDm, c->st));
+    prof_end(c, GSI_K_SMALL, 0.0, 0.0);
+    GSI_TRY(op_small(c, 0, c->Bm, Zp));
+  }
   GSI_TRY(readback(c, c->out, 5));
   const double t = c->host[0];
   c->last_t = t;
@@ -510,7 +567,7 @@ gsi_status iterate(gsi_ctx* c, bool* stop) {
   if (c->host[3] != 0.0) return GSI_ERR_BREAKDOWN;
   if (!isfinite(t)) return GSI_ERR_NONFINITE;
   const double bmax = c->host[4];
-  if (cg) {
+  if (cg && !split) {
     // next step's K = X_new^T D = M (X^T D + t D^T D)
     prof_begin(c);
     GSI_TRY(pp_axpby(c->p, 1.0, c->XDm, t, c->Bm, c->Gm2, c->st));
@@ -576,8 +633,7 @@ gsi_status iterate_cheb(gsi_ctx* c, bool* stop) {
   GSI_TRY(op_gram(c, c->X, c->Y, true, c->Cm));
   prof_begin(c);
   if (c->emu) {
-    GSI_TRY(small_step_df(2, p, nullptr, c->Cm, nullptr, nullptr, nullptr, c->XDm, c->Bm, c->out,
-                          c->small_ws, c->st));
+    GSI_TRY(op_pp(c, 2, c->Cm, nullptr, 0.0, false, c->Bm, c->XDm));
   } else {
     GSI_TRY(small_eig(p, c->Cm, c->XDm, c->Bm, c->small_ws, c->st));
   }
@@ -1128,6 +1184,12 @@ gsi_status gsi_create(const gsi_matrix* A, int32_t p, const double* X0, int32_t 
     CK(dev_alloc(c, (void**)&c->small_ws, std::max(small_scratch_doubles(p) * sizeof(double),
                                                    small_df_scratch_bytes(p))));
     if (c->emu) {
+      CK(dev_alloc(c, (void**)&c->ppf, 11 * q * sizeof(float2)));
+      // 32 < p <= 64: on one CTA the eigenbasis hides behind the three Grams
+      // beside it where those take as long (p = 64: about 0.4 ms on one CTA;
+      // the Grams 0.3 ms at n = 250,000, 2.5 ms at n = 2,097,152); below,
+      // eight CTAs shorten it
+      c->eig_cluster = p > 32 && n < 250000;
       CK(dev_alloc(c, &c->eig_ws, (size_t)(q + p) * sizeof(float2)));
       CK(cuda_status_ok(cudaStreamCreateWithFlags(&c->st2, cudaStreamNonBlocking)));
       CK(cuda_status_ok(cudaEventCreateWithFlags(&c->ev_b, cudaEventDisableTiming)));
