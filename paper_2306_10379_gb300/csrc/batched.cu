@@ -615,15 +615,13 @@ __global__ void __launch_bounds__(BT) b_retract_kernel(BDev d, int32_t mode) {
 // mode 1 (F_START): M = (X^T X)^{-1/2}.
 // mode 2 (F_START): Rayleigh-Ritz, C' = U diag(theta) U^T, theta descending,
 //   M = U.
-using BPp16 = PpCfg<BS, 16, 1, 1, 1, 1, 1>;
-using BPp32 = PpCfg<BS, 32, 4, 1, 1, 1, 1>;
+using BPp16 = PpCfg<BS, 16, 1, 1, 1, 8, 1, 1, 1>;
+using BPp32 = PpCfg<BS, 32, 4, 1, 1, 16, 2, 2, 1>;
 
 __global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
   const int i = blockIdx.x;
   const int32_t mask = mode == 0 ? F_STEP : F_START;
   if (!(d.st[i].flags & mask)) return;
-  extern __shared__ __align__(16) unsigned char sm_dyn[];
-  __shared__ PpSh sh;
   __shared__ double outs[16];
   __shared__ int order[PMAX];
   const int tid = threadIdx.x;
@@ -649,10 +647,10 @@ __global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
     a.Kd = d.cg ? d.Km + pr.ppoff : nullptr;
   }
   if (p <= 16) {
-    PpCtx<BPp16> c = pp_ctx<BPp16>(sm_dyn, &sh, p, nullptr);
+    PpCtx<BPp16> c = pp_ctx<BPp16>(p, nullptr);
     pp_body<BPp16>(a, c);
   } else {
-    PpCtx<BPp32> c = pp_ctx<BPp32>(sm_dyn, &sh, p, nullptr);
+    PpCtx<BPp32> c = pp_ctx<BPp32>(p, nullptr);
     pp_body<BPp32>(a, c);
   }
   __syncthreads();
@@ -675,7 +673,7 @@ __global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
         order[best] = tmp;
       }
     }
-    double* tmp = reinterpret_cast<double*>(sm_dyn);  // q doubles of scratch
+    double* tmp = reinterpret_cast<double*>(pp_sm);  // q doubles of scratch
     for (int e = tid; e < q; e += BS) tmp[e] = M[e];
     __syncthreads();
     for (int k = tid; k < p; k += BS) d.theta[pr.ppoff + k] = XD[order[k]];

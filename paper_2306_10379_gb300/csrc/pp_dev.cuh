@@ -10,14 +10,18 @@
 // df64 Jacobi sweeps this trades the serial rounds of ~400 float operations a
 // 2 x 2 block for df64 products, which have no chain between rounds.
 //
-// Layout of the work. A Jacobi round is one barrier for the angles (one
-// thread per rotation), one for the 2 x 2 blocks of J^T A J (one thread per
-// unordered pair of rotations: A is symmetric, both halves are stored); the
-// update of V by a round's rotations runs beside the next round's angles.
+// Layout of the work. The sweeps are a chain of p - 1 rounds each, so a
+// round is kept short: AW warps (1, 2 or 8) work on A alone, every lane
+// computes the angle of its own rotation, 2 x 2 blocks take their partner's
+// by shuffle, and A is double-buffered, which leaves one barrier among those
+// warps per round. The rotations go to a log; V is a chain per row only, and
+// is formed from a sweep's log by the other warps (ranks, for NC > 1) while
+// the next sweep runs. For p > 64 the angles pass through shared memory (two
+// barriers a round).
 // Products give every thread a TR x TC register tile. With NC > 1 CTAs the
 // matrices live in global memory (L2), each CTA forms p / NC rows of every
-// product from copies in its shared memory, and rank 0 alone runs the
-// sweeps; the CTAs meet at cluster barriers.
+// product from copies in its shared memory, rank 0 runs the sweeps and the
+// other ranks form V; the CTAs meet at cluster barriers.
 #pragma once
 #include <math.h>
 
@@ -27,12 +31,17 @@
 namespace gsi {
 
 // Block shape: NT threads; a group of CL lanes covers TC CL columns of a
-// product (NCG such column blocks), the groups its rows, TR each. MI: 2 x 2
-// blocks a thread holds in a Jacobi round (half (half - 1) / 2 of them).
-template <int NT_, int CL_, int TR_, int TC_, int NCG_, int MI_, int NC_>
+// product (NCG such column blocks), the groups its rows, TR each. Jacobi:
+// AW warps work on A; a segment of SEG lanes holds one rotation per lane
+// (SEG = 64: p > 64), IL 2 x 2 blocks a lane: the blocks of rotations k and
+// k + d, 1 <= d <= half / 2, half <= SEG rotations a round.
+template <int NT_, int CL_, int TR_, int TC_, int NCG_, int SEG_, int AW_, int IL_, int NC_>
 struct PpCfg {
-  static constexpr int NT = NT_, CL = CL_, TR = TR_, TC = TC_, NCG = NCG_, MI = MI_, NC = NC_;
+  static constexpr int NT = NT_, CL = CL_, TR = TR_, TC = TC_, NCG = NCG_, NC = NC_;
   static constexpr int NG = NT / CL, RG = NG / NCG;
+  static constexpr int SEG = SEG_, AW = AW_, IL = IL_;
+  static_assert(SEG == 64 || (32 / SEG) * AW * IL * 2 >= SEG, "every pair of rotations has a lane");
+  static_assert(SEG == 64 ? NC > 1 : NC > 1 || NT / 32 > AW, "V needs warps (or ranks) of its own");
 };
 
 struct PpMat {  // a p x p input: df64, or float64 (then symmetrised where sym is set)
@@ -54,44 +63,66 @@ struct PpArgs {
   double* theta;  // mode 2: eigenvalues
   float2* eig;    // modes 3, 4: V (p x p), then the diagonal of V^T B V
   double* out;    // 16 doubles: t, phi, evaluations, status, max beta, cycle counts and sweeps
-  float2* gws;    // NC > 1: 4 p x p matrices and PP_CTL float2 of global scratch
+  float2* gws;    // NC > 1: pp_gws_bytes(p) of global scratch
 };
-constexpr int PP_CTL = 1024 + 64;  // float2: partial dots of up to 8 ranks, then the control words
+constexpr int PP_CTL = 1024 + 64;  // float2: control words, then the partial dots of up to 8 ranks
 
 struct PpSh {  // small tables, shared memory
   double al[128], be[128], ga[128], ze[128], sv[128];
-  float2 lam[130];
-  float2 cs[2][64];
+  float2 lam[2][130];
+  float2 cs[64];
   float red[32];
   double t;
   int flag, ctl;
 };
 
+// All dynamic shared memory of a kernel that runs this code: PpSh first, then
+// the matrices. Everything is addressed as pp_sm + offset, so that the
+// compiler sees shared accesses: pointers kept in a context struct became
+// generic ones, and the loads of a Jacobi round's chain took twice as long.
+extern __shared__ __align__(16) unsigned char pp_sm[];
+__device__ __forceinline__ PpSh* pp_sh() { return reinterpret_cast<PpSh*>(pp_sm); }
+
 template <class P>
 struct PpCtx {
-  int p, ld, tid, cl, g, rank, r0, r1;
-  float2 *Bd, *Vd, *Td, *Ud;  // p x p df64, rows ld apart (shared memory; global for NC > 1)
-  float *Af, *Vf;             // Jacobi matrices, rows lda apart (shared memory)
-  int lda;
-  float2 *sX, *sY;            // NC > 1: the strip of X and the whole Y of a product
-  float2* ctl;                // NC > 1: control words in global memory
-  PpSh* sh;
+  int p, ld, tid, cl, g, rank, r0, r1, lda;
+  // offsets: df64 matrices (rows ld apart) and the two logs of a sweep's
+  // rotations in float2 units of pp_sm (NC = 1) or gws (NC > 1); the Jacobi
+  // matrices (rows lda apart) in floats of pp_sm; for NC > 1 the staged Y and
+  // strip of X of a product in float2 of pp_sm, the control words in gws
+  int Bd, Vd, Td, Ud, log0, log1, Af, A2, Vf, sX, sY, ctl;
+  float2* gws;
+  __device__ __forceinline__ float2* mat(int o) const {
+    if constexpr (P::NC == 1) return reinterpret_cast<float2*>(pp_sm) + o;
+    else return gws + o;
+  }
+  __device__ __forceinline__ float2 ldm(int o) const {
+    if constexpr (P::NC == 1) return reinterpret_cast<float2*>(pp_sm)[o];
+    else return __ldcg(gws + o);
+  }
 };
+__device__ __forceinline__ float* pp_sf(int o) { return reinterpret_cast<float*>(pp_sm) + o; }
+__device__ __forceinline__ float2* pp_s2(int o) { return reinterpret_cast<float2*>(pp_sm) + o; }
 
 __host__ __device__ inline int pp_lda(int p) { return (p + 31) / 32 * 32; }
 __host__ __device__ inline size_t pp_al(size_t b) { return (b + 15) & ~(size_t)15; }
-// dynamic shared memory: NC = 1: four df64 matrices and the two Jacobi
-// matrices; NC > 1: staged Y (the Jacobi matrices share its space), strip of
-// X, float32 copy of E
+__host__ __device__ inline size_t pp_log_len(int p) {  // rotations of a sweep
+  const size_t m = (p + 1) & ~1;
+  return (m - 1) * (m / 2);
+}
+// dynamic shared memory: NC = 1: four df64 matrices, the Jacobi matrices A
+// (two buffers) and V, two logs; NC > 1: staged Y (V or a log share its
+// space), strip of X, A or a float32 copy of E, A's second buffer (p <= 64)
 inline size_t pp_smem(int p, int nc) {
   const size_t ld = p | 1, m = (p + 1) & ~1, lda = pp_lda((int)m);
-  const size_t jac = 2 * pp_al(m * lda * sizeof(float));
-  if (nc == 1) return 4 * pp_al((size_t)p * ld * sizeof(float2)) + jac;
+  const size_t jac = pp_al(m * lda * sizeof(float));
+  const size_t sh = pp_al(sizeof(PpSh));
+  if (nc == 1)
+    return sh + 4 * pp_al((size_t)p * ld * sizeof(float2)) + 3 * jac + 2 * pp_al(pp_log_len(p) * sizeof(float2));
   const size_t sy = pp_al((size_t)p * ld * sizeof(float2));
-  return (sy > jac ? sy : jac) + pp_al((size_t)((p + nc - 1) / nc) * ld * sizeof(float2)) +
-         pp_al(m * lda * sizeof(float));
+  return sh + (sy > jac ? sy : jac) + pp_al((size_t)((p + nc - 1) / nc) * ld * sizeof(float2)) + (p > 64 ? 1 : 2) * jac;
 }
-inline size_t pp_gws_bytes(int p) { return (4 * (size_t)p * p + PP_CTL) * sizeof(float2); }
+inline size_t pp_gws_bytes(int p) { return (4 * (size_t)p * p + PP_CTL + 2 * pp_log_len(p)) * sizeof(float2); }
 
 template <class P>
 __device__ __forceinline__ void pp_sync() {
@@ -103,62 +134,60 @@ __device__ __forceinline__ void pp_sync() {
 }
 
 template <class P>
-__device__ __forceinline__ float2 pp_ld(const float2* p) {
-  if constexpr (P::NC == 1) return *p;
-  else return __ldcg(p);
-}
-
-template <class P>
-__device__ PpCtx<P> pp_ctx(unsigned char* sm, PpSh* sh, int p, float2* gws) {
+__device__ __forceinline__ PpCtx<P> pp_ctx(int p, float2* gws) {
   PpCtx<P> c;
   c.p = p;
+  c.gws = gws;
   c.tid = threadIdx.x;
   c.cl = c.tid % P::CL;
   c.g = c.tid / P::CL;
-  c.sh = sh;
   const int m = (p + 1) & ~1;
   c.lda = pp_lda(m);
-  unsigned char* cur = sm;
-  auto take = [&](size_t b) {
-    unsigned char* r = cur;
-    cur += pp_al(b);
+  int cur = (int)pp_al(sizeof(PpSh));
+  auto take = [&](int bytes) {
+    const int r = cur;
+    cur += (bytes + 15) & ~15;
     return r;
   };
+  const int jac = m * c.lda * 4, len = (m - 1) * (m / 2);
   if constexpr (P::NC == 1) {
     c.rank = 0;
     c.r0 = 0;
     c.r1 = p;
     c.ld = p | 1;
-    const size_t mb = (size_t)p * c.ld * sizeof(float2);
-    c.Bd = (float2*)take(mb);
-    c.Vd = (float2*)take(mb);
-    c.Td = (float2*)take(mb);
-    c.Ud = (float2*)take(mb);
-    c.Af = (float*)take((size_t)m * c.lda * sizeof(float));
-    c.Vf = (float*)take((size_t)m * c.lda * sizeof(float));
-    c.sX = c.sY = c.ctl = nullptr;
+    const int mb = p * c.ld * 8;
+    c.Bd = take(mb) / 8;
+    c.Vd = take(mb) / 8;
+    c.Td = take(mb) / 8;
+    c.Ud = take(mb) / 8;
+    c.Af = take(jac) / 4;
+    c.A2 = take(jac) / 4;
+    c.Vf = take(jac) / 4;
+    c.log0 = take(len * 8) / 8;
+    c.log1 = take(len * 8) / 8;
+    c.sX = c.sY = c.ctl = 0;
   } else {
     uint32_t rk;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rk));
     c.rank = (int)rk;
-    const int rs = (p + P::NC - 1) / P::NC;
+    const int rs = (p + P::NC - 1) / P::NC, q = p * p;
     c.r0 = min(p, c.rank * rs);
     c.r1 = min(p, c.r0 + rs);
     c.ld = p;
-    const size_t q = (size_t)p * p;
-    c.Bd = gws;
-    c.Vd = gws + q;
-    c.Td = gws + 2 * q;
-    c.Ud = gws + 3 * q;
-    c.ctl = gws + 4 * q;
-    const size_t jac = pp_al((size_t)m * c.lda * sizeof(float));
-    const size_t sy = pp_al((size_t)p * (p | 1) * sizeof(float2));
-    unsigned char* y = take(sy > 2 * jac ? sy : 2 * jac);
-    c.sY = (float2*)y;
-    c.Vf = (float*)(y + jac);
-    c.sX = (float2*)take((size_t)rs * (p | 1) * sizeof(float2));
+    c.Bd = 0;
+    c.Vd = q;
+    c.Td = 2 * q;
+    c.Ud = 3 * q;
+    c.ctl = 4 * q;
+    c.log0 = c.ctl + PP_CTL;
+    c.log1 = c.log0 + len;
+    const int y = take(max(p * (p | 1) * 8, jac));
+    c.sY = y / 8;
+    c.Vf = y / 4;  // rank 0: the first-order correction K
+    c.sX = take(rs * (p | 1) * 8) / 8;
     // the Jacobi matrix of rank 0 and every rank's copy of E share this
-    c.Af = (float*)take((size_t)m * c.lda * sizeof(float));
+    c.Af = take(jac) / 4;
+    c.A2 = P::SEG == 64 ? 0 : take(jac) / 4;
   }
   return c;
 }
@@ -181,45 +210,44 @@ __device__ __forceinline__ void pp_mac(float& sh, float& se, float2 a, float2 b)
   se = __fadd_rn(se, __fadd_rn(t.y, __fmaf_rn(a.x, b.y, __fmaf_rn(a.y, b.x, pe))));
 }
 
-// Rows r0..r1 of X' Y', X' = X^T if tx, Y' = Y^T if ty. With dots null:
-// Out = (Add +) X' Y' - dsub I. With dots: dots[g p + j] += sum over this
+// Rows r0..r1 of X' Y', X' = X^T if tx, Y' = Y^T if ty (matrices by offset,
+// -1: none). Without dots: Out = (Add +) X' Y' - dsub I. With dots (in
+// shared memory): dots[g p + j] += sum over this
 // group's rows i of Vdot[i, j] (X' Y')[i, j] (df64 pairs, one row of dots per
 // row group). The caller synchronises before and after. One copy of the code
 // serves every product of a step (the instruction cache is cold at each
 // launch).
 template <class P>
-__device__ __noinline__ void pp_mm(const PpCtx<P>& c, const float2* X, bool tx, const float2* Y, bool ty,
-                                   float2* Out, const float2* Add, float dsub, const float2* Vdot = nullptr,
-                                   float2* dots = nullptr) {
-  const int p = c.p, rows = c.r1 - c.r0;
+__device__ __noinline__ void pp_mm_fn(int p, float2* gws, int X, bool tx, int Y, bool ty, int Out, int Add, float dsub,
+                                      int Vdot, int dots) {
+  const PpCtx<P> c = pp_ctx<P>(p, gws);
+  const int rows = c.r1 - c.r0;
   const float2 *xs, *ys;
   int xi, xk, yk, yj;
   if constexpr (P::NC == 1) {
-    xs = X;
-    ys = Y;
+    xs = pp_s2(X);
+    ys = pp_s2(Y);
     xi = tx ? 1 : c.ld;
     xk = tx ? c.ld : 1;
     yk = ty ? 1 : c.ld;
     yj = ty ? c.ld : 1;
   } else {
     const int ls = p | 1;
+    float2 *const sY = pp_s2(c.sY), *const sX = pp_s2(c.sX);
     for (int k = c.g; k < p; k += P::NG)
-      for (int j = c.cl; j < p; j += P::CL) {
-        const float2 v = __ldcg(Y + k * p + j);
-        c.sY[ty ? j * ls + k : k * ls + j] = v;
-      }
+      for (int j = c.cl; j < p; j += P::CL) sY[ty ? j * ls + k : k * ls + j] = c.ldm(Y + k * p + j);
     if (tx) {
       for (int e = c.tid; e < rows * p; e += P::NT) {
         const int k = e / rows, i = e - k * rows;
-        c.sX[i * ls + k] = __ldcg(X + k * p + c.r0 + i);
+        sX[i * ls + k] = c.ldm(X + k * p + c.r0 + i);
       }
     } else {
       for (int i = c.g; i < rows; i += P::NG)
-        for (int k = c.cl; k < p; k += P::CL) c.sX[i * ls + k] = __ldcg(X + (c.r0 + i) * p + k);
+        for (int k = c.cl; k < p; k += P::CL) sX[i * ls + k] = c.ldm(X + (c.r0 + i) * p + k);
     }
     __syncthreads();
-    xs = c.sX;
-    ys = c.sY;
+    xs = sX;
+    ys = sY;
     xi = ls;
     xk = 1;
     yk = ls;
@@ -261,28 +289,35 @@ __device__ __noinline__ void pp_mm(const PpCtx<P>& c, const float2* X, bool tx, 
         const int i = c.r0 + i0 + s, j = jb + t * P::CL;
         if (i0 + s < rows && j < p) {
           float2 v = fast_two_sum(h[s][t], e[s][t]);
-          if (dots) {
-            pp_mac(dacc[t].x, dacc[t].y, pp_ld<P>(Vdot + i * c.ld + j), v);
+          if (dots >= 0) {
+            pp_mac(dacc[t].x, dacc[t].y, c.ldm(Vdot + i * c.ld + j), v);
           } else {
             if (i == j && dsub != 0.f) v = df_add_f(v, -dsub);
-            if (Add) v = df_add(pp_ld<P>(Add + i * c.ld + j), v);
-            Out[i * c.ld + j] = v;
+            if (Add >= 0) v = df_add(c.ldm(Add + i * c.ld + j), v);
+            c.mat(Out)[i * c.ld + j] = v;
           }
         }
       }
   }
-  if (dots) {
+  if (dots >= 0) {
 #pragma unroll
     for (int t = 0; t < P::TC; ++t) {
       const int j = jb + t * P::CL;
-      if (j < p) dots[rg * p + j] = fast_two_sum(dacc[t].x, dacc[t].y);
+      if (j < p) pp_s2(dots)[rg * p + j] = fast_two_sum(dacc[t].x, dacc[t].y);
     }
   }
 }
 
+template <class P>
+__device__ __forceinline__ void pp_mm(const PpCtx<P>& c, int X, bool tx, int Y, bool ty, int Out, int Add = -1,
+                                      float dsub = 0.f, int Vdot = -1, int dots = -1) {
+  pp_mm_fn<P>(c.p, c.gws, X, tx, Y, ty, Out, Add, dsub, Vdot, dots);
+}
+
 // sum over the block (float32, fixed order), the same in every thread
 template <class P>
-__device__ float pp_bsum(PpSh* sh, float v) {
+__device__ float pp_bsum(float v) {
+  PpSh* const sh = pp_sh();
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   __syncthreads();
   if ((threadIdx.x & 31) == 0) sh->red[threadIdx.x >> 5] = v;
@@ -294,7 +329,8 @@ __device__ float pp_bsum(PpSh* sh, float v) {
 }
 
 template <class P>
-__device__ float pp_bmax(PpSh* sh, float v) {
+__device__ float pp_bmax(float v) {
+  PpSh* const sh = pp_sh();
   for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
   __syncthreads();
   if ((threadIdx.x & 31) == 0) sh->red[threadIdx.x >> 5] = v;
@@ -319,22 +355,145 @@ __device__ __forceinline__ void pp_pair(int r, int k, int m1, int& a, int& b) {
   }
 }
 
-// Jacobi sweeps in float32 by one CTA on the symmetric m x m matrix A (m = p
-// rounded up to even; the dummy row and column of an odd p are zero and stay
-// so), rotations gathered in V (p rows) on the right, until the squared
-// off-diagonal mass is at most `stop`. DELTA: A holds only the off-diagonal
-// part (zero diagonal) and lam the df64 diagonal.
+// The angle of one rotation: t = tan, (c, s). DELTA: pivot f and the df64
+// diagonal entries la, lb; otherwise the diagonal is la.x, lb.x. IEEE
+// division and square root for DELTA, whose angles' errors are what a pass
+// leaves behind.
+template <bool DELTA>
+__device__ __forceinline__ float2 pp_angle(float f, float2 la, float2 lb, float& t) {
+  const float b2 = 2.f * f;
+  t = 0.f;
+  if (DELTA) {
+    const float2 dd = df_add(lb, pp_neg(la));
+    const float d = __fadd_rn(dd.x, dd.y);
+    const float q = __fsqrt_rn(__fmaf_rn(d, d, b2 * b2));
+    if (q > 0.f) t = __fdiv_rn(d >= 0.f ? b2 : -b2, fabsf(d) + q);
+  } else {
+    const float d = lb.x - la.x;
+    const float q2 = __fmaf_rn(d, d, b2 * b2);
+    if (q2 > 0.f) t = __fdividef(d >= 0.f ? b2 : -b2, fabsf(d) + q2 * rsqrtf(q2));
+  }
+  const float q = __fmaf_rn(t, t, 1.f);
+  float cc = rsqrtf(q);
+  cc = cc * __fmaf_rn(-0.5f * q, cc * cc, 1.5f);  // one Newton step: c^2 + s^2 = 1 to rounding
+  return make_float2(cc, t * cc);
+}
+
+// 2 x 2 block z = J_k^T x J_l
+__device__ __forceinline__ void pp_rot2(float2 wk, float2 wl, const float x[4], float z[4]) {
+  const float y00 = wl.x * x[0] - wl.y * x[1], y01 = wl.y * x[0] + wl.x * x[1];
+  const float y10 = wl.x * x[2] - wl.y * x[3], y11 = wl.y * x[2] + wl.x * x[3];
+  z[0] = wk.x * y00 - wk.y * y10;
+  z[2] = wk.y * y00 + wk.x * y10;
+  z[1] = wk.x * y01 - wk.y * y11;
+  z[3] = wk.y * y01 + wk.x * y11;
+}
+
+// One sweep over A (symmetric m x m, m even; the dummy row and column of an
+// odd p are zero and stay so) by the first AW warps of the CTA, p <= 64; the
+// result is in `An` after an odd number of rounds. DELTA: A holds only the
+// off-diagonal part and lam[lp] the df64 diagonal (lam[lp ^ 1] on return).
+// A, An: offsets of the two buffers.
 template <class P, bool DELTA>
-__device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop) {
-  const int p = c.p, lda = c.lda, tid = c.tid;
-  const int m = (p + 1) & ~1, half = m / 2, m1 = m - 1;
-  float* const A = c.Af;
-  float* const V = c.Vf;
-  float2* const lam = c.sh->lam;
-  const int items = half * (half - 1) / 2;
-  int ik[P::MI], il[P::MI];
+__device__ void pp_sweep(const PpCtx<P>& c, int Ao, int Ano, int lp, int log) {
+  constexpr int SEG = P::SEG, NSEG = 32 / SEG;
+  const int lda = c.lda, m = (c.p + 1) & ~1, half = m / 2, m1 = m - 1;
+  const int lane = c.tid & 31, w = c.tid >> 5, seg = lane / SEG, k = lane % SEG;
+  const bool own = k < half, lead = own && w == 0 && seg == 0;
+  int a = own ? k : 0, b = own ? (k == 0 ? m1 : m1 - k) : 0;  // round 0's pair
+  int src[P::IL];
+  bool live[P::IL];
 #pragma unroll
-  for (int z = 0; z < P::MI; ++z) {
+  for (int z = 0; z < P::IL; ++z) {
+    const int d = 1 + ((z * P::AW + w) * NSEG + seg);
+    live[z] = own && 2 * d <= half && !(2 * d == half && k >= d);
+    int l = k + d;
+    l -= l >= half ? half : 0;
+    src[z] = live[z] ? seg * SEG + l : lane;
+  }
+  for (int r = 0; r < m1; ++r) {
+    float *const A = pp_sf(Ao), *const An = pp_sf(Ano);
+    float2 *const lam = pp_sh()->lam[lp], *const lamn = pp_sh()->lam[lp ^ 1];
+    const int ra = a * lda, rb = b * lda;
+    const float f = own ? A[ra + b] : 0.f;
+    float2 la = make_float2(0.f, 0.f), lb = la;
+    if (DELTA) {
+      la = lam[a];
+      lb = lam[b];
+    } else if (own) {
+      la.x = A[ra + a];
+      lb.x = A[rb + b];
+    }
+    float x[P::IL][4];
+    int al[P::IL], bl[P::IL];
+#pragma unroll
+    for (int z = 0; z < P::IL; ++z) {
+      al[z] = __shfl_sync(0xffffffffu, a, src[z]);
+      bl[z] = __shfl_sync(0xffffffffu, b, src[z]);
+      if (live[z]) {
+        x[z][0] = A[ra + al[z]];
+        x[z][1] = A[ra + bl[z]];
+        x[z][2] = A[rb + al[z]];
+        x[z][3] = A[rb + bl[z]];
+      } else {
+        x[z][0] = x[z][1] = x[z][2] = x[z][3] = 0.f;
+      }
+    }
+    float t;
+    const float2 cs = pp_angle<DELTA>(f, la, lb, t);
+    if (lead) {
+      c.mat(log)[r * half + k] = cs;
+      const float d = t * f;
+      if (DELTA) {
+        lamn[a] = df_add_f(la, -d);
+        lamn[b] = df_add_f(lb, d);
+      } else {
+        An[ra + a] = la.x - d;
+        An[rb + b] = lb.x + d;
+      }
+      An[ra + b] = 0.f;
+      An[rb + a] = 0.f;
+    }
+#pragma unroll
+    for (int z = 0; z < P::IL; ++z) {
+      const float2 wl = make_float2(__shfl_sync(0xffffffffu, cs.x, src[z]), __shfl_sync(0xffffffffu, cs.y, src[z]));
+      float y[4];
+      pp_rot2(cs, wl, x[z], y);
+      if (live[z]) {
+        const int rl = al[z] * lda, sl = bl[z] * lda;
+        An[ra + al[z]] = y[0];
+        An[ra + bl[z]] = y[1];
+        An[rb + al[z]] = y[2];
+        An[rb + bl[z]] = y[3];
+        An[rl + a] = y[0];
+        An[sl + a] = y[1];
+        An[rl + b] = y[2];
+        An[sl + b] = y[3];
+      }
+    }
+    // both indices of a pair advance by one modulo m - 1 (slot 0 keeps m - 1)
+    a = a + 1 == m1 ? 0 : a + 1;
+    if (k != 0) b = b + 1 == m1 ? 0 : b + 1;
+    const int u = Ao;
+    Ao = Ano;
+    Ano = u;
+    lp ^= 1;
+    if constexpr (P::AW == 1) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"n"(P::AW * 32) : "memory");
+  }
+}
+
+// The same for p > 64 by the whole CTA, A in place: half threads form the
+// angles, then every unordered pair of rotations is one thread's block.
+template <class P, bool DELTA>
+__device__ void pp_sweep_wide(const PpCtx<P>& c, int log) {
+  float* const A = pp_sf(c.Af);
+  float2* const lam = pp_sh()->lam[0];
+  const int lda = c.lda, tid = c.tid, m = (c.p + 1) & ~1, half = m / 2, m1 = m - 1;
+  const int items = half * (half - 1) / 2;
+  int ik[P::IL], il[P::IL];
+#pragma unroll
+  for (int z = 0; z < P::IL; ++z) {
     const int e = tid + z * P::NT;
     ik[z] = -1;
     il[z] = 0;
@@ -345,87 +504,164 @@ __device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop) {
       il[z] -= il[z] >= half ? half : 0;
     }
   }
-  auto update_v = [&](int r, const float2* cs) {
-    for (int l = c.cl; l < half; l += P::CL) {
+  for (int r = 0; r < m1; ++r) {
+    if (tid < half) {
       int a, b;
-      pp_pair(r, l, m1, a, b);
-      const float2 w = cs[l];
-      for (int row = c.g; row < p; row += P::NG) {
-        const float x = V[row * lda + a], y = V[row * lda + b];
-        V[row * lda + a] = w.x * x - w.y * y;
-        V[row * lda + b] = w.y * x + w.x * y;
+      pp_pair(r, tid, m1, a, b);
+      const int ra = a * lda, rb = b * lda;
+      const float f = A[ra + b];
+      float2 la, lb;
+      if (DELTA) {
+        la = lam[a];
+        lb = lam[b];
+      } else {
+        la = make_float2(A[ra + a], 0.f);
+        lb = make_float2(A[rb + b], 0.f);
       }
+      float t;
+      const float2 cs = pp_angle<DELTA>(f, la, lb, t);
+      pp_sh()->cs[tid] = cs;
+      c.mat(log)[r * half + tid] = cs;
+      const float d = t * f;
+      if (DELTA) {
+        lam[a] = df_add_f(la, -d);
+        lam[b] = df_add_f(lb, d);
+      } else {
+        A[ra + a] = la.x - d;
+        A[rb + b] = lb.x + d;
+      }
+      A[ra + b] = 0.f;
+      A[rb + a] = 0.f;
     }
-  };
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    float off = 0.f;
-    for (int i = c.g; i < p; i += P::NG)
-      for (int j = c.cl; j < p; j += P::CL)
-        if (i != j) off += A[i * lda + j] * A[i * lda + j];
-    off = pp_bsum<P>(c.sh, off);
-    if (!(off > stop)) break;
-    for (int r = 0; r < m1; ++r) {
-      float2* const cs = c.sh->cs[r & 1];
-      if (tid < half) {
-        int a, b;
-        pp_pair(r, tid, m1, a, b);
-        const float f = A[a * lda + b];
-        float t = 0.f;
-        if (DELTA) {
-          const float2 la = lam[a], lb = lam[b];
-          const float2 dd = df_add(lb, pp_neg(la));
-          const float d = __fadd_rn(dd.x, dd.y), b2 = 2.f * f;
-          const float q = __fsqrt_rn(__fmaf_rn(d, d, b2 * b2));
-          if (q > 0.f) t = __fdiv_rn(d >= 0.f ? b2 : -b2, fabsf(d) + q);
-          const float x = t * f;
-          lam[a] = df_add_f(la, -x);
-          lam[b] = df_add_f(lb, x);
-        } else {
-          const float aa = A[a * lda + a], ab = A[b * lda + b];
-          const float d = ab - aa, b2 = 2.f * f;
-          const float q2 = __fmaf_rn(d, d, b2 * b2);
-          if (q2 > 0.f) t = __fdividef(d >= 0.f ? b2 : -b2, fabsf(d) + q2 * rsqrtf(q2));
-          const float x = t * f;
-          A[a * lda + a] = aa - x;
-          A[b * lda + b] = ab + x;
-        }
-        A[a * lda + b] = 0.f;
-        A[b * lda + a] = 0.f;
-        const float q = __fmaf_rn(t, t, 1.f);
-        float cc = rsqrtf(q);
-        cc = cc * __fmaf_rn(-0.5f * q, cc * cc, 1.5f);  // one Newton step: c^2 + s^2 = 1 to rounding
-        cs[tid] = make_float2(cc, t * cc);
-      }
-      if (r > 0) update_v(r - 1, c.sh->cs[(r - 1) & 1]);
-      __syncthreads();
-#pragma unroll
-      for (int z = 0; z < P::MI; ++z) {
-        if (ik[z] >= 0) {
-          int ak, bk, al, bl;
-          pp_pair(r, ik[z], m1, ak, bk);
-          pp_pair(r, il[z], m1, al, bl);
-          const float2 wk = cs[ik[z]], wl = cs[il[z]];
-          const float x00 = A[ak * lda + al], x01 = A[ak * lda + bl];
-          const float x10 = A[bk * lda + al], x11 = A[bk * lda + bl];
-          const float y00 = wl.x * x00 - wl.y * x01, y01 = wl.y * x00 + wl.x * x01;
-          const float y10 = wl.x * x10 - wl.y * x11, y11 = wl.y * x10 + wl.x * x11;
-          const float z00 = wk.x * y00 - wk.y * y10, z10 = wk.y * y00 + wk.x * y10;
-          const float z01 = wk.x * y01 - wk.y * y11, z11 = wk.y * y01 + wk.x * y11;
-          A[ak * lda + al] = z00;
-          A[ak * lda + bl] = z01;
-          A[bk * lda + al] = z10;
-          A[bk * lda + bl] = z11;
-          A[al * lda + ak] = z00;
-          A[bl * lda + ak] = z01;
-          A[al * lda + bk] = z10;
-          A[bl * lda + bk] = z11;
-        }
-      }
-      __syncthreads();
-    }
-    update_v(m1 - 1, c.sh->cs[(m1 - 1) & 1]);
     __syncthreads();
+#pragma unroll
+    for (int z = 0; z < P::IL; ++z) {
+      if (ik[z] >= 0) {
+        int ak, bk, al, bl;
+        pp_pair(r, ik[z], m1, ak, bk);
+        pp_pair(r, il[z], m1, al, bl);
+        const int ra = ak * lda, rb = bk * lda, rl = al * lda, sl = bl * lda;
+        const float x[4] = {A[ra + al], A[ra + bl], A[rb + al], A[rb + bl]};
+        float y[4];
+        pp_rot2(pp_sh()->cs[ik[z]], pp_sh()->cs[il[z]], x, y);
+        A[ra + al] = y[0];
+        A[ra + bl] = y[1];
+        A[rb + al] = y[2];
+        A[rb + bl] = y[3];
+        A[rl + ak] = y[0];
+        A[sl + ak] = y[1];
+        A[rl + bk] = y[2];
+        A[sl + bk] = y[3];
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// rows [0, rows) of V (ldv apart; offsets of V and of the log in shared
+// memory) times the rotations of a sweep's log, by nw
+// warps (this one is w of them): a row belongs to one segment of lanes
+template <class P>
+__device__ void pp_apply_log(int p, int Vo, int ldv, int rows, int logo, int w, int nw) {
+  float* const V = pp_sf(Vo);
+  const float2* const log = pp_s2(logo);
+  constexpr int SEG = P::SEG > 32 ? 32 : P::SEG, NSEG = 32 / SEG, LL = P::SEG / SEG;  // rotations a lane
+  const int m = (p + 1) & ~1, half = m / 2, m1 = m - 1;
+  const int lane = threadIdx.x & 31, seg = lane / SEG;
+  for (int r = 0; r < m1; ++r) {
+#pragma unroll
+    for (int z = 0; z < LL; ++z) {
+      const int l = lane % SEG + z * SEG;
+      if (l < half) {
+        int a, b;
+        pp_pair(r, l, m1, a, b);
+        const float2 cs = log[r * half + l];
+#pragma unroll 4
+        for (int row = w * NSEG + seg; row < rows; row += nw * NSEG) {
+          float* const v = V + row * ldv;
+          const float x = v[a], y = v[b];
+          v[a] = cs.x * x - cs.y * y;
+          v[b] = cs.y * x + cs.x * y;
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// rows of V of this rank for NC > 1 (rank 0 runs the sweeps and has none)
+template <class P>
+__device__ __forceinline__ void pp_vrows(const PpCtx<P>& c, int& v0, int& v1) {
+  constexpr int VR = P::NC > 1 ? P::NC - 1 : 1;
+  const int per = (c.p + VR - 1) / VR;
+  v0 = c.rank == 0 ? 0 : min(c.p, (c.rank - 1) * per);
+  v1 = c.rank == 0 ? 0 : min(c.p, v0 + per);
+}
+
+// Float32 Jacobi sweeps on c.Af until the squared off-diagonal mass is at most
+// `stop` (rank 0's value), the rotations gathered in V: c.Vf (NC = 1) or the
+// ranks' rows in c.sX. A and lam[0] are synchronised on entry, V on exit.
+// Returns the sweeps (rank 0; the others 0 or not 0).
+template <class P, bool DELTA>
+__device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop) {
+  const int p = c.p, lda = c.lda, m = (p + 1) & ~1;
+  int A = c.Af, An = c.A2, lp = 0;
+  const int w = c.tid >> 5;
+  int v0 = 0, v1 = p, V = c.Vf, ldv = lda;
+  if constexpr (P::NC > 1) {
+    pp_vrows(c, v0, v1);
+    V = 2 * c.sX;
+    ldv = m;
+  }
+  for (int e = c.tid; e < (v1 - v0) * ldv; e += P::NT) {
+    const int i = e / ldv, j = e - i * ldv;
+    pp_sf(V)[e] = v0 + i == j ? 1.f : 0.f;
+  }
+  __syncthreads();
+  int sweep = 0;
+  for (;; ++sweep) {
+    bool go = true;
+    const int log = sweep & 1 ? c.log1 : c.log0, prev = sweep & 1 ? c.log0 : c.log1;
+    if (c.rank == 0) {
+      const float* const a = pp_sf(A);
+      float off = 0.f;
+      for (int i = c.g; i < p; i += P::NG)
+        for (int j = c.cl; j < p; j += P::CL)
+          if (i != j) off += a[i * lda + j] * a[i * lda + j];
+      off = pp_bsum<P>(off);
+      go = sweep < max_sweeps && off > stop;
+      if constexpr (P::SEG == 64) {
+        if (go) pp_sweep_wide<P, DELTA>(c, log);
+      } else {
+        if (w < P::AW) {
+          if (go) pp_sweep<P, DELTA>(c, A, An, lp, log);
+        } else if (P::NC == 1 && sweep > 0) {
+          pp_apply_log<P>(p, V, ldv, p, prev, w - P::AW, P::NT / 32 - P::AW);
+        }
+        const int u = A;  // m - 1 rounds: odd
+        A = An;
+        An = u;
+        lp ^= 1;
+      }
+    }
+    if constexpr (P::NC == 1) {
+      __syncthreads();
+      if (!go) break;
+    } else {
+      float2* const word = c.gws + c.ctl + 4 + (sweep & 1);
+      if (c.rank == 0 && c.tid == 0) *word = make_float2(go ? 1.f : 0.f, 0.f);
+      pp_sync<P>();
+      if (c.rank == 0) {
+        if (!go) break;
+      } else {
+        if (__ldcg(&word->x) == 0.f) break;
+        const int len = (int)pp_log_len(p);
+        for (int e = c.tid; e < len; e += P::NT) pp_s2(c.sY)[e] = c.ldm(log + e);
+        __syncthreads();
+        pp_apply_log<P>(p, V, ldv, v1 - v0, c.sY, w, P::NT / 32);
+        __syncthreads();
+      }
+    }
   }
   return sweep;
 }
@@ -434,20 +670,20 @@ __device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop) {
 // V comes from float32 rotations): Out = V + V G, G = -E/2 + 3/8 E^2, E^2 in
 // float32. T is scratch; V is not changed. Synchronised on entry and exit.
 template <class P>
-__device__ void pp_orth(const PpCtx<P>& c, const float2* V, float2* T, float2* Out) {
-  pp_mm(c, V, true, V, false, T, (const float2*)nullptr, 1.f);  // E
+__device__ void pp_orth(const PpCtx<P>& c, int V, int T, int Out) {
+  pp_mm(c, V, true, V, false, T, -1, 1.f);  // E
   pp_sync<P>();
   for (int i = c.g; i < c.p; i += P::NG)
-    for (int j = c.cl; j < c.p; j += P::CL) c.Af[i * c.lda + j] = pp_ld<P>(T + i * c.ld + j).x;
+    for (int j = c.cl; j < c.p; j += P::CL) pp_sf(c.Af)[i * c.lda + j] = c.ldm(T + i * c.ld + j).x;
   __syncthreads();
   pp_each(c, [&](int i, int j) {
     float s = 0.f;
-    for (int k = 0; k < c.p; ++k) s = fmaf(c.Af[i * c.lda + k], c.Af[k * c.lda + j], s);
-    const float2 e = T[i * c.ld + j];
-    T[i * c.ld + j] = df_add_f(make_float2(-0.5f * e.x, -0.5f * e.y), 0.375f * s);
+    for (int k = 0; k < c.p; ++k) s = fmaf(pp_sf(c.Af)[i * c.lda + k], pp_sf(c.Af)[k * c.lda + j], s);
+    const float2 e = c.mat(T)[i * c.ld + j];
+    c.mat(T)[i * c.ld + j] = df_add_f(make_float2(-0.5f * e.x, -0.5f * e.y), 0.375f * s);
   });
   pp_sync<P>();
-  pp_mm(c, V, false, T, false, Out, V, 0.f);
+  pp_mm(c, V, false, T, false, Out, V);
   pp_sync<P>();
 }
 
@@ -458,135 +694,135 @@ __device__ void pp_orth(const PpCtx<P>& c, const float2* V, float2* T, float2* O
 template <class P>
 __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
   const int p = c.p, lda = c.lda, m = (p + 1) & ~1;
-  PpSh* sh = c.sh;
+  PpSh* const sh = pp_sh();
   const long long c0 = clock64();
   float sc = 1.f;  // a power of two that brings max |B| near 1 (rank 0)
-  int s32 = 0, s_delta = 0;
-  auto identity_v = [&]() {
-    for (int i = c.g; i < p; i += P::NG)
-      for (int j = c.cl; j < m; j += P::CL) c.Vf[i * lda + j] = i == j ? 1.f : 0.f;
-  };
-  // V of the sweeps into a df64 matrix, and a control word for the other ranks
-  auto publish = [&](float2* V, int word) {
-    if (c.rank == 0) {
-      for (int i = c.g; i < p; i += P::NG)
-        for (int j = c.cl; j < p; j += P::CL) V[i * c.ld + j] = make_float2(c.Vf[i * lda + j], 0.f);
-      if (c.tid == 0) {
-        sh->ctl = word;
-        if (P::NC > 1) c.ctl[0] = make_float2(__int_as_float(word), 0.f);
-      }
+  int s32 = 0, s_delta = 0;  // sweeps
+  // a control word of rank 0 to all ranks, and into a df64 matrix: nothing
+  // (what = 0), the gathered rotations (1) or rank 0's c.Vf (2)
+  auto publish = [&](int Vo, int word, int what) {
+    float2* const V = c.mat(Vo);
+    if (what == 0) {
+    } else if (P::NC == 1 || what == 2) {
+      if (c.rank == 0)
+        for (int i = c.g; i < p; i += P::NG)
+          for (int j = c.cl; j < p; j += P::CL) V[i * c.ld + j] = make_float2(pp_sf(c.Vf)[i * lda + j], 0.f);
+    } else {
+      int v0, v1;
+      pp_vrows(c, v0, v1);
+      const float* const sv = pp_sf(2 * c.sX);
+      for (int i = v0 + c.g; i < v1; i += P::NG)
+        for (int j = c.cl; j < p; j += P::CL) V[i * c.ld + j] = make_float2(sv[(i - v0) * m + j], 0.f);
+    }
+    if (c.rank == 0 && c.tid == 0) {
+      sh->ctl = word;
+      if (P::NC > 1) c.gws[c.ctl] = make_float2(__int_as_float(word), 0.f);
     }
     pp_sync<P>();
-    return P::NC == 1 ? sh->ctl : __float_as_int(__ldcg(&c.ctl[0].x));
+    return P::NC == 1 ? sh->ctl : __float_as_int(__ldcg(&c.gws[c.ctl].x));
   };
+  float tot0 = 0.f;
   if (c.rank == 0) {
-    float mx = 0.f, tot = 0.f;
+    float mx = 0.f;
     for (int i = c.g; i < p; i += P::NG)
-      for (int j = c.cl; j < p; j += P::CL) mx = fmaxf(mx, fabsf(pp_ld<P>(c.Bd + i * c.ld + j).x));
-    mx = pp_bmax<P>(sh, mx);
+      for (int j = c.cl; j < p; j += P::CL) mx = fmaxf(mx, fabsf(c.ldm(c.Bd + i * c.ld + j).x));
+    mx = pp_bmax<P>(mx);
     const int ex = ((__float_as_int(mx) >> 23) & 255) - 127;
     if (mx > 0.f && ex <= 127) sc = exp2i(max(-126, min(126, -ex)));
     for (int i = c.g; i < m; i += P::NG)
       for (int j = c.cl; j < m; j += P::CL) {
-        const float v = i < p && j < p ? pp_ld<P>(c.Bd + i * c.ld + j).x * sc : 0.f;
-        c.Af[i * lda + j] = v;
-        tot += v * v;
+        const float v = i < p && j < p ? c.ldm(c.Bd + i * c.ld + j).x * sc : 0.f;
+        pp_sf(c.Af)[i * lda + j] = v;
+        tot0 += v * v;
       }
-    identity_v();
-    tot = pp_bsum<P>(sh, tot);  // (its barriers also publish A and V)
-    __syncthreads();
-    // down to ~1e-5 relative off-diagonal mass, above float32's rounding floor
-    s32 = pp_jacobi<P, false>(c, 12, 1e-10f * tot);
+    tot0 = pp_bsum<P>(tot0);  // (its barriers also publish A)
   }
-  const bool rotated = publish(c.Td, s32 > 0) != 0;
+  // down to ~1e-5 relative off-diagonal mass, above float32's rounding floor
+  s32 = pp_jacobi<P, false>(c, 12, 1e-10f * tot0);
+  const bool rotated = publish(c.Td, s32 > 0, 1) != 0;
   const long long c1 = clock64();
   if (rotated) {
     pp_orth(c, c.Td, c.Ud, c.Vd);
-    pp_mm(c, c.Bd, false, c.Vd, false, c.Td, (const float2*)nullptr, 0.f);
+    pp_mm(c, c.Bd, false, c.Vd, false, c.Td);
     pp_sync<P>();
-    pp_mm(c, c.Vd, true, c.Td, false, c.Ud, (const float2*)nullptr, 0.f);
+    pp_mm(c, c.Vd, true, c.Td, false, c.Ud);
   } else {
     pp_each(c, [&](int i, int j) {
-      c.Vd[i * c.ld + j] = make_float2(i == j ? 1.f : 0.f, 0.f);
-      c.Ud[i * c.ld + j] = c.Bd[i * c.ld + j];
+      c.mat(c.Vd)[i * c.ld + j] = make_float2(i == j ? 1.f : 0.f, 0.f);
+      c.mat(c.Ud)[i * c.ld + j] = c.mat(c.Bd)[i * c.ld + j];
     });
   }
   pp_sync<P>();
   const long long c2 = clock64();
   for (int pass = 0; pass < 3; ++pass) {
     int word = 0;  // 0: done, 1: rotations in Td, 2: first-order correction in Td
+    float stop = 0.f;
     if (c.rank == 0) {
       // F scaled by 2^30 so that squares of entries at 1e-15 stay in range
       constexpr float UP = 1073741824.f;
       float off = 0.f, tot = 0.f;
+      float2* const lam = sh->lam[0];
       for (int i = c.g; i < m; i += P::NG)
         for (int j = c.cl; j < m; j += P::CL) {
-          float2 u = i < p && j < p ? pp_ld<P>(c.Ud + i * c.ld + j) : make_float2(0.f, 0.f);
+          float2 u = i < p && j < p ? c.ldm(c.Ud + i * c.ld + j) : make_float2(0.f, 0.f);
           u = make_float2(u.x * sc, u.y * sc);
           tot += u.x * u.x;
           if (i == j) {
-            sh->lam[i] = make_float2(u.x * UP, u.y * UP);
-            c.Af[i * lda + j] = 0.f;
+            lam[i] = make_float2(u.x * UP, u.y * UP);
+            pp_sf(c.Af)[i * lda + j] = 0.f;
           } else {
             off += u.x * u.x;
-            c.Af[i * lda + j] = u.x * UP;
+            pp_sf(c.Af)[i * lda + j] = u.x * UP;
           }
         }
-      tot = pp_bsum<P>(sh, tot);
-      off = pp_bsum<P>(sh, off);
-      identity_v();
-      __syncthreads();
+      tot = pp_bsum<P>(tot);
+      off = pp_bsum<P>(off);
+      stop = 1e-30f * tot * UP * UP;
       if (off > 1e-27f * tot) {
-        float kmax = 1.f;
+        word = 1;
         if (first_order && pass > 0) {
           // largest rotation angle F_ij / (lambda_j - lambda_i): below 1e-8
           // the rotations are I + K to working accuracy. K is made exactly
           // skew from the upper half of F: the halves differ by rounding,
           // which over a small gap would leave V off orthogonal
-          kmax = 0.f;
+          float kmax = 0.f;
           for (int i = c.g; i < p; i += P::NG)
             for (int j = c.cl; j < p; j += P::CL)
               if (i < j) {
-                const float2 d = df_add(sh->lam[j], pp_neg(sh->lam[i]));
-                const float f = c.Af[i * lda + j];
+                const float2 d = df_add(lam[j], pp_neg(lam[i]));
+                const float f = pp_sf(c.Af)[i * lda + j];
                 const float k = f == 0.f ? 0.f : f / d.x;
-                c.Vf[i * lda + j] = k;
-                c.Vf[j * lda + i] = -k;
+                pp_sf(c.Vf)[i * lda + j] = k;
+                pp_sf(c.Vf)[j * lda + i] = -k;
                 kmax = fmaxf(kmax, fabsf(k) <= 1.f ? fabsf(k) : 1.f);
+              } else if (i == j) {
+                pp_sf(c.Vf)[i * lda + i] = 0.f;
               }
-          kmax = pp_bmax<P>(sh, kmax);
-        }
-        if (kmax <= 1e-8f) {
-          for (int i = c.g; i < p; i += P::NG)
-            if (c.cl == 0) c.Vf[i * lda + i] = 0.f;
-          __syncthreads();
-          word = 2;
-        } else {
-          if (first_order && pass > 0) {
-            identity_v();
-            __syncthreads();
-          }
-          s_delta += pp_jacobi<P, true>(c, 8, 1e-30f * tot * UP * UP);
-          word = 1;
+          kmax = pp_bmax<P>(kmax);
+          if (kmax <= 1e-8f) word = 2;
         }
       }
     }
-    word = publish(c.Td, word);
+    word = publish(c.Td, word, word == 2 ? 2 : 0);
+    if (word == 1) {
+      s_delta += pp_jacobi<P, true>(c, 8, stop);
+      publish(c.Td, 1, 1);
+    }
     if (word == 0) break;
     if (word == 2) {  // V += V K
-      pp_mm(c, c.Vd, false, c.Td, false, c.Bd, c.Vd, 0.f);
+      pp_mm(c, c.Vd, false, c.Td, false, c.Bd, c.Vd);
       pp_sync<P>();
-      pp_each(c, [&](int i, int j) { c.Vd[i * c.ld + j] = c.Bd[i * c.ld + j]; });
+      pp_each(c, [&](int i, int j) { c.mat(c.Vd)[i * c.ld + j] = c.mat(c.Bd)[i * c.ld + j]; });
       pp_sync<P>();
       break;
     }
     // V <- orth(V W), U = V^T B V
-    pp_mm(c, c.Vd, false, c.Td, false, c.Ud, (const float2*)nullptr, 0.f);
+    pp_mm(c, c.Vd, false, c.Td, false, c.Ud);
     pp_sync<P>();
     pp_orth(c, c.Ud, c.Td, c.Vd);
-    pp_mm(c, c.Bd, false, c.Vd, false, c.Td, (const float2*)nullptr, 0.f);
+    pp_mm(c, c.Bd, false, c.Vd, false, c.Td);
     pp_sync<P>();
-    pp_mm(c, c.Vd, true, c.Td, false, c.Ud, (const float2*)nullptr, 0.f);
+    pp_mm(c, c.Vd, true, c.Td, false, c.Ud);
     pp_sync<P>();
   }
   if (c.rank == 0 && c.tid == 0 && diag) {
@@ -604,12 +840,12 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
 // taken in float32.
 template <class P>
 __device__ void pp_inv_sqrt(const PpCtx<P>& c, double* M) {
-  PpSh* sh = c.sh;
+  PpSh* const sh = pp_sh();
   const int p = c.p;
   if (c.tid < 32) {
     double mx = 0.0;
     for (int i = c.tid; i < p; i += 32) {
-      const double s = df_to_double(pp_ld<P>(c.Ud + i * c.ld + i));
+      const double s = df_to_double(c.ldm(c.Ud + i * c.ld + i));
       sh->be[i] = s;
       mx = fmax(mx, s);
     }
@@ -632,23 +868,24 @@ __device__ void pp_inv_sqrt(const PpCtx<P>& c, double* M) {
       v = df_from_double(1.0 / sh->sv[i]);
     } else {
       const float ri = (float)sh->sv[i], rj = (float)sh->sv[j];
-      const float2 f = c.Ud[i * c.ld + j];
+      const float2 f = c.mat(c.Ud)[i * c.ld + j];
       v = make_float2(-((__fadd_rn(f.x, f.y) / ri) / rj) / (ri + rj), 0.f);
     }
-    c.Ud[i * c.ld + j] = v;
+    c.mat(c.Ud)[i * c.ld + j] = v;
   });
   pp_sync<P>();
-  pp_mm(c, c.Vd, false, c.Ud, false, c.Td, (const float2*)nullptr, 0.f);  // V N
+  pp_mm(c, c.Vd, false, c.Ud, false, c.Td);  // V N
   pp_sync<P>();
-  pp_mm(c, c.Td, false, c.Vd, true, c.Ud, (const float2*)nullptr, 0.f);   // (V N) V^T
+  pp_mm(c, c.Td, false, c.Vd, true, c.Ud);   // (V N) V^T
   pp_sync<P>();
-  pp_each(c, [&](int i, int j) { M[i * p + j] = df_to_double(c.Ud[i * c.ld + j]); });
+  pp_each(c, [&](int i, int j) { M[i * p + j] = df_to_double(c.mat(c.Ud)[i * c.ld + j]); });
 }
 
 // this CTA's rows of an input into a df64 matrix
 template <class P, class F>
-__device__ __forceinline__ void pp_load(const PpCtx<P>& c, const PpMat& a, float2* dst, F f) {
+__device__ __forceinline__ void pp_load(const PpCtx<P>& c, const PpMat& a, int dsto, F f) {
   const int p = c.p;
+  float2* const dst = c.mat(dsto);
   pp_each(c, [&](int i, int j) {
     float2 v;
     if (a.f) v = a.f[i * p + j];
@@ -752,6 +989,12 @@ __device__ __forceinline__ float2 pp_brent(const PpModel<MC>& md, float2 a, floa
   return b;
 }
 
+// the search in float64 throughout, where the scaled model does not serve
+static __device__ __noinline__ double pp_step_length_f64(int p, int* ev) {
+  const PpSh* const sh = pp_sh();
+  return get_mu_warp(p, sh->al, sh->be, sh->ga, sh->ze, ev);
+}
+
 // The step of get_mu_warp (alg3.cuh: bracket from the branch roots xi_i, the
 // right end doubled from xi_min, Brent on phi'), one warp. The bracket ends
 // come in float64; the evaluations of the search run in df64 on a scaled
@@ -762,8 +1005,9 @@ __device__ __forceinline__ float2 pp_brent(const PpModel<MC>& md, float2 a, floa
 // leaves float32's range or the Newton step is not small, the float64
 // search runs instead.
 template <int MC>
-__device__ __noinline__ double pp_step_length(int p, const double* al, const double* be, const double* ga,
-                                              const double* ze, int* ev) {
+__device__ __noinline__ double pp_step_length(int p, int* ev_out) {
+  const double *const al = pp_sh()->al, *const be = pp_sh()->be, *const ga = pp_sh()->ga, *const ze = pp_sh()->ze;
+  int evs = 0, *const ev = &evs;
   const int lane = threadIdx.x & 31;
   double sb = 0.0, bmax = 0.0, zmax = 0.0, dmax = 0.0;
   for (int i = lane; i < p; i += 32) {
@@ -793,7 +1037,7 @@ __device__ __noinline__ double pp_step_length(int p, const double* al, const dou
     dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
     cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
   }
-  *ev = 0;
+  *ev_out = 0;
   if (cnt == 0) return 0.0;
   // t = T tau with T = min(1/sqrt(max beta), max|zeta| / max|delta|), values
   // over Sz = max|zeta|, each rounded down to a power of two
@@ -802,7 +1046,7 @@ __device__ __noinline__ double pp_step_length(int p, const double* al, const dou
   const int eT = T > 0.0 && isfinite(T) ? ilogb(T) : 1 << 20, eZ = zmax > 0.0 && isfinite(zmax) ? ilogb(zmax) : 1 << 20;
   const double lo_s = abs(eT) < 900 ? scalbn(xmin, -eT) : 0.0;
   const bool scaled = abs(eT) < 900 && abs(eZ) < 900 && lo_s > 1e-9 && lo_s < 1e9;
-  if (!scaled) return get_mu_warp(p, al, be, ga, ze, ev);
+  if (!scaled) return pp_step_length_f64(p, ev_out);
   PpModel<MC> md;
   md.cnt = 0;
 #pragma unroll
@@ -827,7 +1071,10 @@ __device__ __noinline__ double pp_step_length(int p, const double* al, const dou
     lo = make_float2(0.f, 0.f);
     flo = pp_dphi(md, lo);
     ++*ev;
-    if (flo.x >= 0.f) return 0.0;
+    if (flo.x >= 0.f) {
+      *ev_out = evs;
+      return 0.0;
+    }
     hi = xmn;
     fhi = fa;
   } else {
@@ -835,7 +1082,7 @@ __device__ __noinline__ double pp_step_length(int p, const double* al, const dou
     flo = fhi = fa;
     int k = 0;
     while (fhi.x < 0.f) {
-      if (k >= 64 || hi.x > 1e18f) return get_mu_warp(p, al, be, ga, ze, ev);
+      if (k >= 64 || hi.x > 1e18f) return pp_step_length_f64(p, ev_out);
       float2 nxt = make_float2(2.f * hi.x, 2.f * hi.y);
       if (df_less(hi, xmx) && df_less(xmx, nxt)) nxt = xmx;
       lo = hi;
@@ -862,7 +1109,8 @@ __device__ __noinline__ double pp_step_length(int p, const double* al, const dou
   const double f = dphi_warp(t, p, al, be, ga, ze);
   ++*ev;
   const double corr = scalbn(f / (double)sl, eT - eZ);
-  if (!(fabs(corr) <= 1e-9 * t)) return get_mu_warp(p, al, be, ga, ze, ev);
+  if (!(fabs(corr) <= 1e-9 * t)) return pp_step_length_f64(p, ev_out);
+  *ev_out = evs;
   return t - corr;
 }
 
@@ -872,20 +1120,21 @@ __device__ __noinline__ double pp_step_length(int p, const double* al, const dou
 template <class P>
 __device__ void pp_diag(const PpCtx<P>& c, double* d) {
   const int p = c.p;
-  float2* part = reinterpret_cast<float2*>(c.Af);
-  pp_mm(c, c.Ud, false, c.Vd, false, (float2*)nullptr, (const float2*)nullptr, 0.f, c.Vd, part);
+  float2* const part = pp_s2(c.Af / 2);
+  pp_mm(c, c.Ud, false, c.Vd, false, -1, -1, 0.f, c.Vd, c.Af / 2);
   __syncthreads();
   for (int j = c.tid; j < p; j += P::NT) {
     float2 s = part[j];
     for (int g = 1; g < P::RG; ++g) s = df_add(s, part[g * p + j]);
     if constexpr (P::NC == 1) d[j] = df_to_double(s);
-    else c.ctl[64 + c.rank * 128 + j] = s;
+    else c.gws[c.ctl + 64 + c.rank * 128 + j] = s;
   }
   pp_sync<P>();
   if constexpr (P::NC > 1) {
     for (int j = c.tid; j < p; j += P::NT) {
-      float2 s = __ldcg(c.ctl + 64 + j);
-      for (int g = 1; g < P::NC; ++g) s = df_add(s, __ldcg(c.ctl + 64 + g * 128 + j));
+      const float2* const pd = c.gws + c.ctl + 64 + j;
+      float2 s = __ldcg(pd);
+      for (int g = 1; g < P::NC; ++g) s = df_add(s, __ldcg(pd + g * 128));
       d[j] = df_to_double(s);
     }
     pp_sync<P>();
@@ -900,13 +1149,13 @@ __device__ void pp_diag(const PpCtx<P>& c, double* d) {
 template <class P>
 __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
   const int p = c.p;
-  PpSh* sh = c.sh;
+  PpSh* const sh = pp_sh();
   double* out = a.out;
   const bool lead = c.rank == 0 && c.tid == 0;
   const long long t0 = clock64();
   auto same = [](int, int, float2 v) { return v; };
   if (a.mode == 4) {
-    pp_each(c, [&](int i, int j) { c.Vd[i * c.ld + j] = a.eig[i * p + j]; });
+    pp_each(c, [&](int i, int j) { c.mat(c.Vd)[i * c.ld + j] = a.eig[i * p + j]; });
     for (int i = c.tid; i < p; i += P::NT) sh->be[i] = fmax(df_to_double(a.eig[p * p + i]), 0.0);
     __syncthreads();
   } else {
@@ -915,23 +1164,23 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
     pp_eig(c, a.mode != 1, out + 8);
     if (a.mode == 0) {
       for (int i = c.tid; i < p; i += P::NT)
-        sh->be[i] = fmax(df_to_double(pp_ld<P>(c.Ud + i * c.ld + i)), 0.0);
+        sh->be[i] = fmax(df_to_double(c.ldm(c.Ud + i * c.ld + i)), 0.0);
       __syncthreads();
     }
   }
   const long long t1 = clock64();
   if (a.mode == 3) {
     pp_each(c, [&](int i, int j) {
-      a.eig[i * p + j] = c.Vd[i * c.ld + j];
-      if (i == j) a.eig[p * p + i] = c.Ud[i * c.ld + i];
+      a.eig[i * p + j] = c.mat(c.Vd)[i * c.ld + j];
+      if (i == j) a.eig[p * p + i] = c.mat(c.Ud)[i * c.ld + i];
     });
     if (lead) out[5] = (double)(t1 - t0);
     return;
   }
   if (a.mode == 2) {
     pp_each(c, [&](int i, int j) {
-      a.M[i * p + j] = df_to_double(c.Vd[i * c.ld + j]);
-      if (i == j) a.theta[i] = df_to_double(c.Ud[i * c.ld + i]);
+      a.M[i * p + j] = df_to_double(c.mat(c.Vd)[i * c.ld + j]);
+      if (i == j) a.theta[i] = df_to_double(c.mat(c.Ud)[i * c.ld + i]);
     });
     if (lead) out[3] = 0.0;
     return;
@@ -971,21 +1220,21 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
       return df_add(v, df_mul(bt, k));
     });
     pp_sync<P>();
-    pp_mm(c, c.Ud, false, c.Td, false, c.Bd, (const float2*)nullptr, 0.f);
+    pp_mm(c, c.Ud, false, c.Td, false, c.Bd);
   }
   pp_sync<P>();
   const long long t2 = clock64();
   if (c.tid < 32) {
     if (c.rank == 0) {
       int ev = 0;
-      const double t = pp_step_length<(P::CL * P::TC * P::NCG + 31) / 32>(p, sh->al, sh->be, sh->ga, sh->ze, &ev);
+      const double t = pp_step_length<(P::CL * P::TC * P::NCG + 31) / 32>(p, &ev);
       double bmax = 0.0;
       for (int i = c.tid; i < p; i += 32) bmax = fmax(bmax, sh->be[i]);
       for (int o = 16; o > 0; o >>= 1) bmax = fmax(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
       const double ph = phi_model_warp(t, p, sh->al, sh->be, sh->ga, sh->ze);
       if (c.tid == 0) {
         sh->t = t;
-        if (P::NC > 1) *reinterpret_cast<double*>(c.ctl + 2) = t;
+        if (P::NC > 1) *reinterpret_cast<double*>(c.gws + c.ctl + 2) = t;
         out[0] = t;
         out[1] = ph;
         out[2] = (double)ev;
@@ -994,7 +1243,7 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
     }
   }
   pp_sync<P>();
-  const double t = P::NC == 1 ? sh->t : __ldcg(reinterpret_cast<const double*>(c.ctl + 2));
+  const double t = P::NC == 1 ? sh->t : __ldcg(reinterpret_cast<const double*>(c.gws + c.ctl + 2));
   const long long t3 = clock64();
   // S' = V^T S V with S = XX + t (XD + XD^T) + t^2 B
   const float2 td = df_from_double(t), tt = df_from_double(t * t);
@@ -1003,25 +1252,25 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
                : df_from_double(g.sym ? 0.5 * (g.d[i * p + j] + g.d[j * p + i]) : g.d[i * p + j]);
   };
   pp_load(c, a.XX, c.Ud, [&](int i, int j, float2 v) {
-    const float2 xd = df_add(pp_ld<P>(c.Bd + i * c.ld + j), pp_ld<P>(c.Bd + j * c.ld + i));
+    const float2 xd = df_add(c.ldm(c.Bd + i * c.ld + j), c.ldm(c.Bd + j * c.ld + i));
     return df_add(df_add(v, df_mul(td, xd)), df_mul(tt, elem(a.B, i, j)));
   });
   pp_sync<P>();
-  pp_mm(c, c.Ud, false, c.Vd, false, c.Td, (const float2*)nullptr, 0.f);
+  pp_mm(c, c.Ud, false, c.Vd, false, c.Td);
   pp_sync<P>();
-  pp_mm(c, c.Vd, true, c.Td, false, c.Ud, (const float2*)nullptr, 0.f);
+  pp_mm(c, c.Vd, true, c.Td, false, c.Ud);
   pp_sync<P>();
   pp_inv_sqrt(c, a.M);
   if (lead) out[3] = (double)sh->flag;
   if (a.Kd) {  // K_next = X_new^T D = M (X^T D + t D^T D)
     pp_each(c, [&](int i, int j) {
-      c.Td[i * c.ld + j] = df_add(c.Bd[i * c.ld + j], df_mul(td, elem(a.B, i, j)));
+      c.mat(c.Td)[i * c.ld + j] = df_add(c.mat(c.Bd)[i * c.ld + j], df_mul(td, elem(a.B, i, j)));
     });
     pp_sync<P>();
-    pp_mm(c, c.Ud, false, c.Td, false, c.Bd, (const float2*)nullptr, 0.f);
+    pp_mm(c, c.Ud, false, c.Td, false, c.Bd);
     pp_sync<P>();
     pp_each(c, [&](int i, int j) {
-      const float2 v = c.Bd[i * c.ld + j];
+      const float2 v = c.mat(c.Bd)[i * c.ld + j];
       a.Kd[i * p + j] = df_to_double(v);
       if (a.Kf) a.Kf[i * p + j] = v;
     });
