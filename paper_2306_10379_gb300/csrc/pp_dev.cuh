@@ -52,6 +52,7 @@ struct PpMat {  // a p x p input: df64, or float64 (then symmetrised where sym i
 
 struct PpArgs {
   int mode, p;
+  int scale_b;  // mode 3, float64 B: divided by a power of two near max |B| (B may leave float32's range)
   // B = D^T D (modes 0, 3) or the matrix itself (modes 1, 2); C = X^T A X,
   // Gam = D^T W, Z = D^T R, XX = X^T X; XD = X^T D, or null pointers: formed
   // here as (I - XX)(C + beta K)
@@ -1159,7 +1160,18 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
     for (int i = c.tid; i < p; i += P::NT) sh->be[i] = fmax(df_to_double(a.eig[p * p + i]), 0.0);
     __syncthreads();
   } else {
-    pp_load(c, a.B, c.Bd, same);
+    if (a.scale_b) {
+      float ex = 0.f;  // largest biased exponent
+      for (int e = c.tid; e < p * p; e += P::NT) ex = fmaxf(ex, (float)((__double2hiint(a.B.d[e]) >> 20) & 0x7ff));
+      ex = pp_bmax<P>(ex);
+      const int k = ex < 2047.f ? max(1, 2046 - (int)ex) : 1023;
+      const double sb = __hiloint2double(k << 20, 0);
+      pp_each(c, [&](int i, int j) {
+        c.mat(c.Bd)[i * c.ld + j] = df_from_double(0.5 * (sb * a.B.d[i * p + j]) + 0.5 * (sb * a.B.d[j * p + i]));
+      });
+    } else {
+      pp_load(c, a.B, c.Bd, same);
+    }
     pp_sync<P>();
     pp_eig(c, a.mode != 1, out + 8);
     if (a.mode == 0) {
