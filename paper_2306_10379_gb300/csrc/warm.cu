@@ -17,11 +17,10 @@
 #include <vector>
 
 #include "common.cuh"
+#include "df.cuh"
 
 namespace gsi {
 namespace {
-
-constexpr int GBM = 64, GBN = 64, GBK = 32, GPAD = 8;
 
 __device__ __forceinline__ void mma_bf16_16816(float c[4], const uint32_t a[4], const uint32_t b[2]) {
   asm volatile(
@@ -31,91 +30,152 @@ __device__ __forceinline__ void mma_bf16_16816(float c[4], const uint32_t a[4], 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
+__device__ __forceinline__ void cp_bytes16(float* smem, const float* gmem, int bytes) {
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(bytes));
+}
+__device__ __forceinline__ void cp_float(float* smem, const float* gmem, bool valid) {
+  const uint32_t sa = (uint32_t)__cvta_generic_to_shared(smem);
+  const int sz = valid ? 4 : 0;
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(sa), "l"(gmem), "r"(sz));
+}
+
+// How an operand X(i, k) = X[i si + k sk] is staged: along k (sk == 1) or along
+// i (si == 1) in 16-byte pieces where base and rows are 16-byte aligned,
+// element by element otherwise.
+enum : int { G_K16 = 0, G_I16 = 1, G_ANY = 2 };
+
+constexpr int GBK = 32;  // columns of a stage
+
+// A stage of T rows x GBK: [i][k] (row stride GBK + 4), or for G_I16 [k][i]
+// (row stride T + 8); both leave the fragment reads free of bank conflicts.
+template <int T>
+struct GStage {
+  static constexpr int KS = GBK + 4, IS = T + 8;
+  static constexpr int FLOATS = T * KS > GBK * IS ? T * KS : GBK * IS;
+};
+
+template <int T, int NTH>
+__device__ __forceinline__ void g_stage(float* dst, const float* __restrict__ X, int64_t si, int64_t sk, int mode,
+                                        int i0, int imax, int k0, int kmax) {
+  if (mode == G_K16) {
+#pragma unroll
+    for (int e = threadIdx.x; e < T * (GBK / 4); e += NTH) {
+      const int i = e / (GBK / 4), k = 4 * (e % (GBK / 4));
+      const int left = i0 + i < imax ? min(4, kmax - (k0 + k)) : 0;
+      cp_bytes16(dst + i * GStage<T>::KS + k, left > 0 ? X + (i0 + i) * si + k0 + k : X, left > 0 ? 4 * left : 0);
+    }
+  } else if (mode == G_I16) {
+#pragma unroll
+    for (int e = threadIdx.x; e < GBK * (T / 4); e += NTH) {
+      const int k = e / (T / 4), i = 4 * (e % (T / 4));
+      const int left = k0 + k < kmax ? min(4, imax - (i0 + i)) : 0;
+      cp_bytes16(dst + k * GStage<T>::IS + i, left > 0 ? X + (k0 + k) * sk + i0 + i : X, left > 0 ? 4 * left : 0);
+    }
+  } else {
+    for (int e = threadIdx.x; e < T * GBK; e += NTH) {
+      // consecutive threads walk the operand's contiguous index
+      const int i = si == 1 ? e % T : e / GBK, k = si == 1 ? e / T : e % GBK;
+      const bool ok = i0 + i < imax && k0 + k < kmax;
+      cp_float(dst + i * GStage<T>::KS + k, ok ? X + (i0 + i) * si + (k0 + k) * sk : X, ok);
+    }
+  }
+}
+
+// the bfloat16 pair (k, k + 1) of row i of a stage
+template <int T>
+__device__ __forceinline__ uint32_t g_pair(const float* st, int mode, int i, int k) {
+  float x, y;
+  if (mode == G_I16) {
+    x = st[k * GStage<T>::IS + i];
+    y = st[(k + 1) * GStage<T>::IS + i];
+  } else {
+    const float2 v = *reinterpret_cast<const float2*>(st + i * GStage<T>::KS + k);
+    x = v.x;
+    y = v.y;
+  }
+  const __nv_bfloat162 b = __floats2bfloat162_rn(x, y);
+  return *reinterpret_cast<const uint32_t*>(&b);
+}
+
 // C[i][j] = alpha sum_k A(i,k) B(k,j) + beta C[i][j] (+ bias[j]); then, if
 // mask: C = 0 where mask[i][j] <= 0; if relu: C = max(C, 0). A(i,k) =
 // A[i*sai + k*sak], B(k,j) = B[k*sbk + j*sbj]; operands rounded to
-// bfloat16 (nearest even) when staged, products summed in float32.
-// Block 64 x 64, 4 warps of 32 x 32, K steps of 32.
+// bfloat16 (nearest even), products summed in float32, k ascending by 16 as
+// one accumulation per output whatever the tile.
+// Block T x T, 4 warps of T/2 x T/2. The products are few (batch 64): what
+// bounds them is the operands' way from memory, so float32 stages of 32
+// columns come through NST cp.async buffers, NST - 1 ahead, and are rounded
+// when a fragment is read. With one synchronous stage at a time a step of K
+// cost a memory latency: 64 x 256 x 256 33 us (now 5 us), 64 x 32768 x 512
+// (67 MB of weights) 255 us (now 48 us). T = 32 where T = 64 leaves SMs idle.
+template <int T>
 __global__ void __launch_bounds__(128) gemm_bf16_kernel(int M, int N, int K, const float* __restrict__ A,
-                                                        int64_t sai, int64_t sak, const float* __restrict__ B,
-                                                        int64_t sbk, int64_t sbj, float* __restrict__ C,
-                                                        int64_t ldc, float alpha, float beta,
-                                                        const float* __restrict__ bias,
+                                                        int64_t sai, int64_t sak, int modeA,
+                                                        const float* __restrict__ B, int64_t sbk, int64_t sbj,
+                                                        int modeB, float* __restrict__ C, int64_t ldc, float alpha,
+                                                        float beta, const float* __restrict__ bias,
                                                         const float* __restrict__ mask, int relu) {
-  __shared__ __align__(16) __nv_bfloat16 As[GBM][GBK + GPAD];
-  __shared__ __align__(16) __nv_bfloat16 Bs[GBN][GBK + GPAD];
+  constexpr int NST = 4, W = T / 2, MI = W / 16, NI = W / 8, SF = GStage<T>::FLOATS;
+  extern __shared__ __align__(16) float g_sm[];  // NST stages of A, then of B
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int wm = warp >> 1, wn = warp & 1, g = lane >> 2, t = lane & 3;
-  const int m0 = blockIdx.y * GBM, n0 = blockIdx.x * GBN;
-  float acc[2][4][4];
+  const int m0 = blockIdx.y * T, n0 = blockIdx.x * T;
+  float acc[MI][NI][4];
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+  for (int a = 0; a < MI; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
+    for (int b = 0; b < NI; ++b)
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += GBK) {
-    // stage 64 x 32 of A (rows i, columns k) and 32 x 64 of B as [j][k]
-    // consecutive threads walk the operand's contiguous index
-    for (int e = tid; e < GBM * GBK; e += 128) {
-      int i, k;
-      if (sai == 1) {
-        i = e % GBM;
-        k = e / GBM;
-      } else {
-        i = e / GBK;
-        k = e - i * GBK;
-      }
-      const int gi = m0 + i, gk = k0 + k;
-      const float v = (gi < M && gk < K) ? A[gi * sai + gk * sak] : 0.f;
-      As[i][k] = __float2bfloat16_rn(v);
+  const int ns = (K + GBK - 1) / GBK;
+  auto stage = [&](int s) {
+    if (s < ns) {
+      g_stage<T, 128>(g_sm + (s % NST) * SF, A, sai, sak, modeA, m0, M, s * GBK, K);
+      g_stage<T, 128>(g_sm + (NST + s % NST) * SF, B, sbj, sbk, modeB, n0, N, s * GBK, K);
     }
-    for (int e = tid; e < GBN * GBK; e += 128) {
-      int j, k;
-      if (sbj == 1) {
-        j = e % GBN;
-        k = e / GBN;
-      } else {
-        j = e / GBK;
-        k = e - j * GBK;
-      }
-      const int gj = n0 + j, gk = k0 + k;
-      const float v = (gj < N && gk < K) ? B[gk * sbk + gj * sbj] : 0.f;
-      Bs[j][k] = __float2bfloat16_rn(v);
-    }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+#pragma unroll
+  for (int s = 0; s < NST - 1; ++s) stage(s);
+  for (int s = 0; s < ns; ++s) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(NST - 2) : "memory");
+    __syncthreads();  // stage s has landed; stage s - 1 is free
+    stage(s + NST - 1);
+    const float* as = g_sm + (s % NST) * SF;
+    const float* bs = g_sm + (NST + s % NST) * SF;
 #pragma unroll
     for (int kk = 0; kk < GBK; kk += 16) {
-      uint32_t af[2][4], bfr[4][2];
+      uint32_t af[MI][4], bfr[NI][2];
 #pragma unroll
-      for (int mi = 0; mi < 2; ++mi) {
-        const int r = wm * 32 + mi * 16 + g;
-        af[mi][0] = *reinterpret_cast<const uint32_t*>(&As[r][kk + 2 * t]);
-        af[mi][1] = *reinterpret_cast<const uint32_t*>(&As[r + 8][kk + 2 * t]);
-        af[mi][2] = *reinterpret_cast<const uint32_t*>(&As[r][kk + 2 * t + 8]);
-        af[mi][3] = *reinterpret_cast<const uint32_t*>(&As[r + 8][kk + 2 * t + 8]);
+      for (int mi = 0; mi < MI; ++mi) {
+        const int r = wm * W + mi * 16 + g;
+        af[mi][0] = g_pair<T>(as, modeA, r, kk + 2 * t);
+        af[mi][1] = g_pair<T>(as, modeA, r + 8, kk + 2 * t);
+        af[mi][2] = g_pair<T>(as, modeA, r, kk + 2 * t + 8);
+        af[mi][3] = g_pair<T>(as, modeA, r + 8, kk + 2 * t + 8);
       }
 #pragma unroll
-      for (int ni = 0; ni < 4; ++ni) {
-        const int c = wn * 32 + ni * 8 + g;
-        bfr[ni][0] = *reinterpret_cast<const uint32_t*>(&Bs[c][kk + 2 * t]);
-        bfr[ni][1] = *reinterpret_cast<const uint32_t*>(&Bs[c][kk + 2 * t + 8]);
+      for (int ni = 0; ni < NI; ++ni) {
+        const int c = wn * W + ni * 8 + g;
+        bfr[ni][0] = g_pair<T>(bs, modeB, c, kk + 2 * t);
+        bfr[ni][1] = g_pair<T>(bs, modeB, c, kk + 2 * t + 8);
       }
 #pragma unroll
-      for (int mi = 0; mi < 2; ++mi)
+      for (int mi = 0; mi < MI; ++mi)
 #pragma unroll
-        for (int ni = 0; ni < 4; ++ni) mma_bf16_16816(acc[mi][ni], af[mi], bfr[ni]);
+        for (int ni = 0; ni < NI; ++ni) mma_bf16_16816(acc[mi][ni], af[mi], bfr[ni]);
     }
-    __syncthreads();
   }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
 #pragma unroll
-  for (int mi = 0; mi < 2; ++mi) {
+  for (int mi = 0; mi < MI; ++mi) {
 #pragma unroll
-    for (int ni = 0; ni < 4; ++ni) {
+    for (int ni = 0; ni < NI; ++ni) {
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        const int i = m0 + wm * 32 + mi * 16 + g + (r >= 2 ? 8 : 0);
-        const int j = n0 + wn * 32 + ni * 8 + 2 * t + (r & 1);
+        const int i = m0 + wm * W + mi * 16 + g + (r >= 2 ? 8 : 0);
+        const int j = n0 + wn * W + ni * 8 + 2 * t + (r & 1);
         if (i >= M || j >= N) continue;
         const int64_t o = (int64_t)i * ldc + j;
         float v = alpha * acc[mi][ni][r];
@@ -219,109 +279,207 @@ __global__ void restrict_kernel(int nc, int nf, int p, int batch, const double* 
   Bt[idx] = (float)v;
 }
 
-// One block per sample s: with C = C[s] (m x p), Bt = Bt[s] (m x p),
+// The loss and its gradient, per sample s with C = C[s], Bt = Bt[s] (m x p):
 //   SC = S C; N = C^T SC (symmetrised); G = Bt^T C; Q = G^T G;
 //   loss[s] = p - tr(N^{-1} Q);
 //   dC[s] = gscale * (-2) [Bt (G N^{-1}) - SC (N^{-1} Q N^{-1})].
 // Long sums in float32 over 32-row chunks, chunk sums and the p x p algebra
 // in float64 (N^{-1} from its Cholesky factor). A non-positive pivot gives
-// loss = NaN and dC = 0. Dynamic shared memory: 5 p^2 doubles + 2 p^2 floats.
+// loss = NaN and dC = 0.
+// Three launches: the row work (SC, N, G; then dC) goes over blocks of WR rows
+// of every sample, only the algebra takes one block per sample. One block
+// per sample for everything left half of the SMs idle and read every operand
+// of the Grams from memory twice per multiply-add: 64 samples, m = 1024,
+// p = 32 1,207 us (now 82 + 113 + 28 us; the algebra, a chain on the
+// float64 pipe, is what is left).
 constexpr int WT = 256;
+constexpr int WR = 128;  // rows of a block, a multiple of 32
+constexpr int WNZ = 1536;  // entries of S staged per block (bilinear elements: 9 a row)
 
-__global__ void __launch_bounds__(WT) warm_loss_kernel(int m, int p, const int64_t* __restrict__ Srp,
+// acc += a x with a split in two floats: float64-class in float32 arithmetic
+__device__ __forceinline__ void w_mac(float& h, float& e, float2 a, float x) {
+  const float p = __fmul_rn(a.x, x);
+  const float pe = __fmaf_rn(a.x, x, -p);
+  const float2 t = two_sum(h, p);
+  h = t.x;
+  e = __fadd_rn(e, __fadd_rn(t.y, __fmaf_rn(a.y, x, pe)));
+}
+
+__global__ void __launch_bounds__(WT) warm_gram_kernel(int m, int p, const int64_t* __restrict__ Srp,
                                                        const int32_t* __restrict__ Sci,
                                                        const double* __restrict__ Sv,
                                                        const float* __restrict__ Call,
-                                                       const float* __restrict__ Btall,
-                                                       float* __restrict__ SCall, double* __restrict__ loss,
-                                                       float* __restrict__ dCall, float gscale) {
+                                                       const float* __restrict__ Btall, float* __restrict__ SCall,
+                                                       double* __restrict__ part) {
+  extern __shared__ __align__(16) float w_rows[];  // WR rows of C, SC and Bt, row stride pp
+  // the block's rows of S, its values split in two floats once (a float64
+  // conversion for every value and column took half of the kernel's time);
+  // rows beyond WNZ entries are read from memory
+  __shared__ float2 sval[WNZ];
+  __shared__ int32_t scol[WNZ];
+  const int tid = threadIdx.x, pp = (p + 3) & ~3, q = p * p;
+  float *cs = w_rows, *ss = cs + WR * pp, *bs = ss + WR * pp;
+  const int64_t off = (int64_t)blockIdx.y * m * p;
+  const float* C = Call + off;
+  const int r0 = blockIdx.x * WR, nr = min(WR, m - r0);
+  const int64_t k0 = Srp[r0], kn = min((int64_t)WNZ, Srp[r0 + nr] - k0);
+  for (int k = tid; k < kn; k += WT) {
+    sval[k] = df_from_double(Sv[k0 + k]);
+    scol[k] = Sci[k0 + k];
+  }
+  __syncthreads();
+  for (int e = tid; e < WR * pp; e += WT) {
+    const int r = e / pp, c = e - r * pp;
+    const bool ok = r < nr && c < p;
+    float h = 0.f, l = 0.f;
+    if (ok) {
+      const int64_t kb = Srp[r0 + r] - k0, ke = Srp[r0 + r + 1] - k0;
+      int64_t k = kb;
+#pragma unroll 3
+      for (; k < min(ke, kn); ++k) w_mac(h, l, sval[k], C[(int64_t)scol[k] * p + c]);
+      for (; k < ke; ++k) w_mac(h, l, df_from_double(Sv[k0 + k]), C[(int64_t)Sci[k0 + k] * p + c]);
+    }
+    const float sc = h + l;
+    cs[e] = ok ? C[(int64_t)(r0 + r) * p + c] : 0.f;
+    bs[e] = ok ? Btall[off + (int64_t)(r0 + r) * p + c] : 0.f;
+    ss[e] = sc;
+    if (ok) SCall[off + (int64_t)(r0 + r) * p + c] = sc;
+  }
+  __syncthreads();
+  // N = C^T SC and G = Bt^T C: a thread forms 4 x 2 entries
+  const int ti = pp / 4, tj = (p + 1) / 2;
+  double* out = part + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 2 * q;
+  for (int w = tid; w < 2 * ti * tj; w += WT) {
+    const int which = w / (ti * tj), rem = w - which * ti * tj, i = 4 * (rem / tj), j = 2 * (rem % tj);
+    const float* U = (which == 0 ? cs : bs) + i;
+    const float* V = (which == 0 ? ss : cs) + j;
+    double tot[4][2] = {};
+    for (int b0 = 0; b0 < nr; b0 += 32) {
+      float a[4][2] = {};
+      const int b1 = min(nr, b0 + 32);
+#pragma unroll 4
+      for (int r = b0; r < b1; ++r) {
+        const float4 u = *reinterpret_cast<const float4*>(U + r * pp);
+        const float2 v = *reinterpret_cast<const float2*>(V + r * pp);
+        a[0][0] = fmaf(u.x, v.x, a[0][0]);
+        a[0][1] = fmaf(u.x, v.y, a[0][1]);
+        a[1][0] = fmaf(u.y, v.x, a[1][0]);
+        a[1][1] = fmaf(u.y, v.y, a[1][1]);
+        a[2][0] = fmaf(u.z, v.x, a[2][0]);
+        a[2][1] = fmaf(u.z, v.y, a[2][1]);
+        a[3][0] = fmaf(u.w, v.x, a[3][0]);
+        a[3][1] = fmaf(u.w, v.y, a[3][1]);
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) tot[x][y] += (double)a[x][y];
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < 2; ++y)
+        if (i + x < p && j + y < p) out[which * q + (i + x) * p + j + y] = tot[x][y];
+  }
+}
+
+// 1/sqrt(d) in float64 from a float32 seed: the pipe's own root and division
+// are serial chains of many slow operations
+__device__ __forceinline__ double w_rsqrt(double d) {
+  const int ex = ((__double2hiint(d) >> 20) & 0x7ff) - 1023;
+  const int h = ex >= 0 ? ex / 2 : -((1 - ex) / 2);              // floor(ex / 2)
+  const double sc = __hiloint2double((1023 - 2 * h) << 20, 0);   // d sc in [1, 4)
+  const double x = d * sc;
+  double y = (double)rsqrtf((float)x);
+  y = y * fma(-0.5 * x, y * y, 1.5);
+  y = y * fma(-0.5 * x, y * y, 1.5);
+  return y * __hiloint2double((1023 - h) << 20, 0);
+}
+
+// Dynamic shared memory: 5 p^2 + p doubles. A1 = G N^{-1} and A2 = N^{-1} Q
+// N^{-1} (float32, 2 p^2 per sample) are NaN where N is not positive definite.
+__global__ void __launch_bounds__(WT) warm_alg_kernel(int p, int nblk, const double* __restrict__ part,
+                                                      double* __restrict__ loss, float* __restrict__ Aall) {
   extern __shared__ __align__(16) double wsm[];
   __shared__ int bad;
-  __shared__ double trace;
+  __shared__ double trw[WT / 32];
   const int s = blockIdx.x, tid = threadIdx.x, q = p * p;
-  const int64_t off = (int64_t)s * m * p;
-  const float* C = Call + off;
-  const float* Bt = Btall + off;
-  float* SC = SCall + off;
-  float* dC = dCall + off;
   double* Nm = wsm;       // N, then its Cholesky factor L (lower)
-  double* Gm = Nm + q;    // G, then G N^{-1}
+  double* Gm = Nm + q;    // G
   double* Qm = Gm + q;    // Q
   double* Ni = Qm + q;    // L^{-1}, then N^{-1}
   double* Tm = Ni + q;    // scratch
-  float* A1 = reinterpret_cast<float*>(Tm + q);  // G N^{-1}
-  float* A2 = A1 + q;                            // N^{-1} Q N^{-1}
+  double* dinv = Tm + q;  // 1 / L_kk
+  float* A1 = Aall + (size_t)s * 2 * q;
+  float* A2 = A1 + q;
   if (tid == 0) bad = 0;
-  // SC = S C
-  for (int e = tid; e < m * p; e += WT) {
-    const int r = e / p, c = e - r * p;
-    double a = 0.0;
-    for (int64_t k = Srp[r]; k < Srp[r + 1]; ++k) a += Sv[k] * (double)C[(int64_t)Sci[k] * p + c];
-    SC[e] = (float)a;
-  }
-  __syncthreads();
-  // N = C^T SC and G = Bt^T C
   for (int e = tid; e < 2 * q; e += WT) {
-    const int which = e / q, rem = e - which * q, i = rem / p, j = rem - i * p;
-    const float* U = which == 0 ? C : Bt;
-    const float* V = which == 0 ? SC : C;
-    double tot = 0.0;
-    for (int r0 = 0; r0 < m; r0 += 32) {
-      float a = 0.f;
-      const int r1 = min(m, r0 + 32);
-      for (int r = r0; r < r1; ++r) a = fmaf(U[(int64_t)r * p + i], V[(int64_t)r * p + j], a);
-      tot += (double)a;
-    }
-    (which == 0 ? Nm : Gm)[rem] = tot;
+    double t = 0.0;
+    for (int b = 0; b < nblk; ++b) t += part[((size_t)s * nblk + b) * 2 * q + e];
+    (e < q ? Tm : Gm - q)[e] = t;
   }
   __syncthreads();
   for (int e = tid; e < q; e += WT) {  // symmetrise N; Q = G^T G
     const int i = e / p, j = e - i * p;
-    double a = 0.0;
-    for (int k = 0; k < p; ++k) a = fma(Gm[k * p + i], Gm[k * p + j], a);
-    Qm[e] = a;
-    Tm[e] = 0.5 * (Nm[e] + Nm[j * p + i]);
+    Nm[e] = 0.5 * (Tm[e] + Tm[j * p + i]);
+    if (j >= i) {
+      double a = 0.0;
+      for (int k = 0; k < p; ++k) a = fma(Gm[k * p + i], Gm[k * p + j], a);
+      Qm[e] = a;
+      Qm[j * p + i] = a;
+    }
   }
-  __syncthreads();
-  for (int e = tid; e < q; e += WT) Nm[e] = Tm[e];
   __syncthreads();
   // Cholesky N = L L^T (right-looking, column k by the block)
   for (int k = 0; k < p; ++k) {
+    const double d = Nm[k * p + k];
+    const bool ok = d > 0.0 && isfinite(d);
+    const double inv = ok ? w_rsqrt(d) : 1.0;
+    __syncthreads();
     if (tid == 0) {
-      const double d = Nm[k * p + k];
-      if (!(d > 0.0) || !isfinite(d)) bad = 1;
-      Nm[k * p + k] = d > 0.0 ? sqrt(d) : 1.0;
+      if (!ok) bad = 1;
+      dinv[k] = inv;
     }
+    for (int i = k + 1 + tid; i < p; i += WT) Nm[i * p + k] *= inv;
     __syncthreads();
-    const double lkk = Nm[k * p + k];
-    for (int i = k + 1 + tid; i < p; i += WT) Nm[i * p + k] /= lkk;
-    __syncthreads();
-    for (int e = tid; e < (p - k - 1) * (p - k - 1); e += WT) {
-      const int i = k + 1 + e / (p - k - 1), j = k + 1 + e % (p - k - 1);
+    const int w = p - k - 1;
+    for (int e = tid; e < w * w; e += WT) {
+      const int i = k + 1 + e / w, j = k + 1 + e % w;
       if (j <= i) Nm[i * p + j] -= Nm[i * p + k] * Nm[j * p + k];
     }
     __syncthreads();
   }
-  // L^{-1} by forward substitution, one column per thread
-  for (int c = tid; c < p; c += WT) {
+  // L^{-1} by forward substitution, four lanes per column (their partial sums
+  // are folded in a fixed order)
+  for (int c = tid >> 2; c < (p + 7) / 8 * 8; c += WT / 4) {
+    const int l4 = tid & 3;
     for (int i = 0; i < p; ++i) {
-      double v = (i == c) ? 1.0 : 0.0;
-      for (int k = c; k < i; ++k) v -= Nm[i * p + k] * Ni[k * p + c];
-      Ni[i * p + c] = i < c ? 0.0 : v / Nm[i * p + i];
+      double v = 0.0;
+      if (c < p)
+        for (int k = c + l4; k < i; k += 4) v = fma(Nm[i * p + k], Ni[k * p + c], v);
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      if (l4 == 0 && c < p) Ni[i * p + c] = i < c ? 0.0 : ((i == c ? 1.0 : 0.0) - v) * dinv[i];
+      __syncwarp();
     }
   }
   __syncthreads();
   // N^{-1} = L^{-T} L^{-1}
   for (int e = tid; e < q; e += WT) {
     const int i = e / p, j = e - i * p;
-    double a = 0.0;
-    for (int k = max(i, j); k < p; ++k) a = fma(Ni[k * p + i], Ni[k * p + j], a);
-    Tm[e] = a;
+    if (j >= i) {
+      double a = 0.0;
+      for (int k = j; k < p; ++k) a = fma(Ni[k * p + i], Ni[k * p + j], a);
+      Tm[e] = a;
+      Tm[j * p + i] = a;
+    }
   }
   __syncthreads();
   for (int e = tid; e < q; e += WT) Ni[e] = Tm[e];
   __syncthreads();
-  // T = N^{-1} Q; G <- G N^{-1} (into A1 as float)
+  const bool ok = !bad;
+  // T = N^{-1} Q; A1 = G N^{-1}
+  double tr = 0.0;
   for (int e = tid; e < q; e += WT) {
     const int i = e / p, j = e - i * p;
     double a = 0.0, b = 0.0;
@@ -330,35 +488,85 @@ __global__ void __launch_bounds__(WT) warm_loss_kernel(int m, int p, const int64
       b = fma(Gm[i * p + k], Ni[k * p + j], b);
     }
     Tm[e] = a;
-    A1[e] = (float)b;
+    A1[e] = ok ? (float)b : NAN;
+    if (i == j) tr += a;
   }
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  if ((tid & 31) == 0) trw[tid >> 5] = tr;
   __syncthreads();
-  if (tid == 0) {
-    double tr = 0.0;
-    for (int k = 0; k < p; ++k) tr += Tm[k * p + k];
-    trace = tr;
-  }
-  // A2 = T N^{-1}
+  // A2 = T N^{-1} (symmetric)
   for (int e = tid; e < q; e += WT) {
     const int i = e / p, j = e - i * p;
-    double a = 0.0;
-    for (int k = 0; k < p; ++k) a = fma(Tm[i * p + k], Ni[k * p + j], a);
-    A2[e] = (float)a;
+    if (j >= i) {
+      double a = 0.0;
+      for (int k = 0; k < p; ++k) a = fma(Tm[i * p + k], Ni[k * p + j], a);
+      A2[e] = ok ? (float)a : NAN;
+      A2[j * p + i] = ok ? (float)a : NAN;
+    }
   }
-  __syncthreads();
-  const bool ok = !bad;
-  if (tid == 0) loss[s] = ok ? (double)p - trace : NAN;
-  const float sc = -2.f * gscale;
-  for (int e = tid; e < m * p; e += WT) {
-    const int r = e / p, c = e - r * p;
-    float a = 0.f;
-    for (int k = 0; k < p; ++k) a = fmaf(Bt[(int64_t)r * p + k], A1[k * p + c], a);
-    for (int k = 0; k < p; ++k) a = fmaf(-SC[(int64_t)r * p + k], A2[k * p + c], a);
-    dC[e] = ok ? sc * a : 0.f;
+  if (tid == 0) {
+    double t = 0.0;
+    for (int w = 0; w < WT / 32; ++w) t += trw[w];
+    loss[s] = ok ? (double)p - t : NAN;
   }
 }
 
-size_t warm_smem(int p) { return (size_t)5 * p * p * sizeof(double) + (size_t)2 * p * p * sizeof(float); }
+__global__ void __launch_bounds__(WT) warm_dc_kernel(int m, int p, const float* __restrict__ Btall,
+                                                     const float* __restrict__ SCall,
+                                                     const float* __restrict__ Aall, const double* __restrict__ loss,
+                                                     float* __restrict__ dCall, float sc) {
+  extern __shared__ __align__(16) float w_sm[];  // A1, A2, then 32 rows of Bt and SC at a time
+  const int tid = threadIdx.x, q = p * p;
+  float *a1 = w_sm, *a2 = a1 + q, *bt = a2 + q, *st = bt + 32 * p;
+  const float* A = Aall + (size_t)blockIdx.y * 2 * q;
+  for (int e = tid; e < 2 * q; e += WT) a1[e] = A[e];
+  const bool ok = !isnan(loss[blockIdx.y]);
+  const int64_t off = (int64_t)blockIdx.y * m * p;
+  const int r0 = blockIdx.x * WR, r1 = min(m, r0 + WR);
+  for (int b0 = r0; b0 < r1; b0 += 32) {
+    const int cnt = min(32, r1 - b0) * p;
+    __syncthreads();
+    for (int e = tid; e < cnt; e += WT) {
+      bt[e] = Btall[off + (int64_t)b0 * p + e];
+      st[e] = SCall[off + (int64_t)b0 * p + e];
+    }
+    __syncthreads();
+    // a thread forms 4 rows of one column: each value of A1, A2 read serves four
+    const int RG = WT / p, c = tid % p, rows = min(32, r1 - b0);
+    if (tid < RG * p)
+      for (int r = tid / p; r < rows; r += 4 * RG) {
+        int o[4];
+        float a[4];
+#pragma unroll
+        for (int z = 0; z < 4; ++z) {
+          o[z] = min(r + z * RG, rows - 1) * p;
+          a[z] = 0.f;
+        }
+        for (int k = 0; k < p; ++k) {
+          const float v = a1[k * p + c];
+#pragma unroll
+          for (int z = 0; z < 4; ++z) a[z] = fmaf(bt[o[z] + k], v, a[z]);
+        }
+        for (int k = 0; k < p; ++k) {
+          const float v = a2[k * p + c];
+#pragma unroll
+          for (int z = 0; z < 4; ++z) a[z] = fmaf(-st[o[z] + k], v, a[z]);
+        }
+#pragma unroll
+        for (int z = 0; z < 4; ++z)
+          if (r + z * RG < rows) dCall[off + (int64_t)b0 * p + o[z] + c] = ok ? sc * a[z] : 0.f;
+      }
+  }
+}
+
+size_t warm_alg_smem(int p) { return ((size_t)5 * p * p + p) * sizeof(double); }
+size_t warm_gram_smem(int p) { return (size_t)3 * WR * ((p + 3) & ~3) * sizeof(float); }
+size_t warm_dc_smem(int p) { return ((size_t)2 * p * p + 64 * p) * sizeof(float); }
+// partial Grams (float64), then A1 and A2 of every sample
+size_t warm_ws_bytes(int batch, int m, int p) {
+  const size_t nblk = (m + WR - 1) / WR, q = (size_t)p * p;
+  return (size_t)batch * (nblk * 2 * q * sizeof(double) + 2 * q * sizeof(float));
+}
 
 }  // namespace
 }  // namespace gsi
@@ -373,6 +581,8 @@ struct gsi_mlp {
   float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
   float *h1 = nullptr, *h2 = nullptr, *out = nullptr, *d1 = nullptr, *d2 = nullptr, *dout_buf = nullptr;
   float* sc_buf = nullptr;
+  void* loss_ws = nullptr;  // scratch of the loss, sized for the largest (batch, m, p) so far
+  size_t loss_ws_bytes = 0;
   double* loss = nullptr;
   double* hloss = nullptr;  // pinned
   std::vector<void*> allocs;
@@ -392,9 +602,22 @@ gsi_status gemm(cudaStream_t st, int M, int N, int K, const float* A, int64_t sa
                 const float* B, int64_t sbk, int64_t sbj, float* C, int64_t ldc, float alpha, float beta,
                 const float* bias, const float* mask, int relu) {
   if (M <= 0 || N <= 0) return GSI_OK;
-  dim3 grid((unsigned)((N + GBN - 1) / GBN), (unsigned)((M + GBM - 1) / GBM));
-  gemm_bf16_kernel<<<grid, 128, 0, st>>>(M, N, K, A, sai, sak, B, sbk, sbj, C, ldc, alpha, beta, bias,
-                                         mask, relu);
+  auto mode = [](const float* X, int64_t si, int64_t sk) {
+    if (((uintptr_t)X & 15) != 0) return (int)G_ANY;
+    if (sk == 1 && (si & 3) == 0) return (int)G_K16;
+    if (si == 1 && (sk & 3) == 0) return (int)G_I16;
+    return (int)G_ANY;
+  };
+  const int ma = mode(A, sai, sak), mb = mode(B, sbj, sbk);
+  // 64 x 64 tiles read each operand least often; with fewer of them than SMs
+  // the 32 x 32 ones spread the reads over four times as many
+  const bool big = (int64_t)((N + 63) / 64) * ((M + 63) / 64) >= sm_count();
+  const int T = big ? 64 : 32;
+  const size_t sm = (size_t)8 * (big ? GStage<64>::FLOATS : GStage<32>::FLOATS) * sizeof(float);
+  dim3 grid((unsigned)((N + T - 1) / T), (unsigned)((M + T - 1) / T));
+  auto kern = big ? gemm_bf16_kernel<64> : gemm_bf16_kernel<32>;
+  GSI_CUDA_TRY(ensure_dyn_smem((const void*)kern, (int)sm));
+  kern<<<grid, 128, sm, st>>>(M, N, K, A, sai, sak, ma, B, sbk, sbj, mb, C, ldc, alpha, beta, bias, mask, relu);
   GSI_LAUNCH_CHECK();
   return GSI_OK;
 }
@@ -449,15 +672,31 @@ gsi_status mlp_adam(gsi_mlp* n, double lr, double b1, double b2, double eps) {
   return GSI_OK;
 }
 
+// ws: warm_ws_bytes(batch, m, p) bytes of device memory
 gsi_status loss_grad(int batch, int m, int p, const int64_t* Srp, const int32_t* Sci, const double* Sv,
                      const float* C, const float* Bt, float* SC, double* loss, float* dC, float gscale,
-                     cudaStream_t st) {
+                     void* ws, cudaStream_t st) {
   if (batch <= 0) return GSI_OK;
-  const size_t sm = warm_smem(p);  // <= 196 KB for p <= 64; with the static part above 48 KB from p = 32
-  if (sm >= 32 * 1024)
-    GSI_CUDA_TRY(cudaFuncSetAttribute(warm_loss_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  warm_loss_kernel<<<batch, WT, sm, st>>>(m, p, Srp, Sci, Sv, C, Bt, SC, loss, dC, gscale);
-  GSI_LAUNCH_CHECK();
+  const int nblk = (m + WR - 1) / WR;
+  double* part = reinterpret_cast<double*>(ws);
+  float* A = reinterpret_cast<float*>(part + (size_t)batch * nblk * 2 * p * p);
+  GSI_CUDA_TRY(ensure_dyn_smem((const void*)warm_gram_kernel, (int)warm_gram_smem(p)));
+  GSI_CUDA_TRY(ensure_dyn_smem((const void*)warm_alg_kernel, (int)warm_alg_smem(p)));
+  GSI_CUDA_TRY(ensure_dyn_smem((const void*)warm_dc_kernel, (int)warm_dc_smem(p)));
+  // samples go in the grid's second dimension, at most 65,535 at a time
+  for (int b0 = 0; b0 < batch; b0 += 65535) {
+    const int nb = std::min(batch - b0, 65535);
+    const size_t o = (size_t)b0 * m * p;
+    double* pt = part + (size_t)b0 * nblk * 2 * p * p;
+    float* Ab = A + (size_t)b0 * 2 * p * p;
+    warm_gram_kernel<<<dim3(nblk, nb), WT, warm_gram_smem(p), st>>>(m, p, Srp, Sci, Sv, C + o, Bt + o, SC + o, pt);
+    GSI_LAUNCH_CHECK();
+    warm_alg_kernel<<<nb, WT, warm_alg_smem(p), st>>>(p, nblk, pt, loss + b0, Ab);
+    GSI_LAUNCH_CHECK();
+    warm_dc_kernel<<<dim3(nblk, nb), WT, warm_dc_smem(p), st>>>(m, p, Bt + o, SC + o, Ab, loss + b0, dC + o,
+                                                               -2.f * gscale);
+    GSI_LAUNCH_CHECK();
+  }
   return GSI_OK;
 }
 
@@ -473,6 +712,7 @@ gsi_status gsi_mlp_destroy(gsi_mlp* n) {
   if (!n) return GSI_ERR_ARG;
   if (n->st) cudaStreamSynchronize(n->st);
   for (void* p : n->allocs) cudaFree(p);
+  if (n->loss_ws) cudaFree(n->loss_ws);
   if (n->hloss) cudaFreeHost(n->hloss);
   delete n;
   return GSI_OK;
@@ -552,8 +792,12 @@ gsi_status gsi_warm_loss_grad(int32_t batch, int32_t m, int32_t p, const int64_t
   if (batch < 1 || m < 1 || p < 1 || p > 64 || !S_rowptr || !S_colidx || !S_val || !C || !Bt ||
       !SC_scratch || !loss || !dC)
     return GSI_ERR_ARG;
-  return loss_grad(batch, m, p, S_rowptr, S_colidx, S_val, C, Bt, SC_scratch, loss, dC, gscale,
-                   (cudaStream_t)stream);
+  cudaStream_t st = (cudaStream_t)stream;
+  void* ws = nullptr;
+  GSI_CUDA_TRY(cudaMallocAsync(&ws, warm_ws_bytes(batch, m, p), st));
+  const gsi_status s = loss_grad(batch, m, p, S_rowptr, S_colidx, S_val, C, Bt, SC_scratch, loss, dC, gscale, ws, st);
+  GSI_CUDA_TRY(cudaFreeAsync(ws, st));
+  return s;
 }
 
 gsi_status gsi_warm_train_step(gsi_mlp* n, int32_t batch, const float* x, int32_t m, int32_t p,
@@ -561,9 +805,29 @@ gsi_status gsi_warm_train_step(gsi_mlp* n, int32_t batch, const float* x, int32_
                                const float* Bt, double lr, double* mean_loss) {
   if (!n || !x || !Bt || batch < 1 || batch > n->max_batch || p < 1 || p > 64 || (int64_t)m * p != n->dout)
     return GSI_ERR_ARG;
+  const size_t need = warm_ws_bytes(batch, m, p);
+  void *ws = n->loss_ws, *tmp = nullptr;
+  if (need > n->loss_ws_bytes) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    GSI_CUDA_TRY(cudaStreamIsCapturing(n->st, &cap));
+    if (cap != cudaStreamCaptureStatusNone) {  // recorded: a buffer of the graph's own
+      GSI_CUDA_TRY(cudaMallocAsync(&tmp, need, n->st));
+      ws = tmp;
+    } else {  // kept for later steps; grown on the first of a size
+      GSI_CUDA_TRY(cudaStreamSynchronize(n->st));
+      if (n->loss_ws) cudaFree(n->loss_ws);
+      n->loss_ws = nullptr;
+      n->loss_ws_bytes = 0;
+      const cudaError_t e = cudaMalloc(&n->loss_ws, need);
+      if (e != cudaSuccess) return cuda_status(e);
+      n->loss_ws_bytes = need;
+      ws = n->loss_ws;
+    }
+  }
   GSI_TRY(mlp_forward(n, batch, x, n->out));
   GSI_TRY(loss_grad(batch, m, p, S_rowptr, S_colidx, S_val, n->out, Bt, n->sc_buf, n->loss, n->dout_buf,
-                    1.f / batch, n->st));
+                    1.f / batch, ws, n->st));
+  if (tmp) GSI_CUDA_TRY(cudaFreeAsync(tmp, n->st));
   GSI_TRY(mlp_backward(n, batch, x, n->dout_buf));
   GSI_TRY(mlp_adam(n, lr, 0.9, 0.999, 1e-8));
   if (mean_loss) {
