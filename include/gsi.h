@@ -404,10 +404,12 @@ gsi_status gsi_oz_gram(int64_t n, int32_t p, int32_t q, const float* U, const fl
                        int32_t sym, double* G, void* stream);
 
 /* Dense block matvec W = A X for a symmetric n x n A (df64, row-major),
- * computed as A^T X with the contraction over n cut into 64-row chunks, each
- * chunk's digit products exact on the tensor cores. nd = 7: float64-class;
- * nd = 3: bf16-level products (the mixed-precision iterations). X and W are
- * n x p df64 (p <= 128). Uses temporary device memory (stream-ordered). */
+ * computed as A^T X with the contraction over n cut into chunks, each chunk's
+ * digit products exact on the tensor cores. nd = 7: float64-class (160-row
+ * chunks; 64 on tensor path 1); nd = 3: bf16-level products (the mixed-precision
+ * iterations; 384-row chunks for 16-byte aligned blocks of even width, else
+ * 64). X and W are n x p df64 (p <= 128). Uses temporary device memory
+ * (stream-ordered). */
 gsi_status gsi_oz_dense_apply(int64_t n, int32_t p, const float* A, const float* X, float* W,
                               int32_t nd, void* stream);
 
@@ -432,9 +434,9 @@ gsi_status gsi_oz_gram_noalloc(int64_t n, int32_t p, int32_t q, const float* U, 
                                int32_t sym, double* G, void* stream);
 
 /* Which tensor-core kernels the digit-split products use: 0 (default) and 2
- * the tcgen05 kernels wherever they apply (7-digit Grams of any p, q and
- * the 7-digit dense apply, one CTA per 64 x 64 output block; 3-digit Grams
- * and the 3-digit dense apply on 16-byte aligned blocks of even width;
+ * the tcgen05 kernels wherever they apply (7-digit Grams of any p, q, one
+ * CTA per 64 x 64 output block; 3-digit Grams on 16-byte aligned blocks of
+ * even width; the dense apply, 128 rows of W per CTA;
  * 7-digit block products of any p <= 128, the contraction cut into slices
  * of at most 64 for p > 64), 1 the mma.sync kernels everywhere (they also
  * serve the remaining 3-digit products). Block products with p <= 64 are

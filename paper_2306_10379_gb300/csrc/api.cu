@@ -158,6 +158,14 @@ gsi_status gsi_oz_dense_apply(int64_t n, int32_t p, const float* A, const float*
   if (n < 1 || p < 1 || p > 128 || !A || !X || !W || (nd != 3 && nd != 7)) return GSI_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   ScratchGuard g(st);
+  if (tensor_path() != 1) {
+    const int EC = oz_dense_chunk(n, p, nd, (((uintptr_t)A | (uintptr_t)X) & 15) == 0);
+    const size_t eb = (oz_colexp_bytes(n, EC) + 255) / 256 * 256;
+    GSI_CUDA_TRY(cudaMallocAsync(&g.ptr, eb + oz_dense_scratch_bytes(n, p, nd, EC), st));
+    GSI_TRY(oz_colexp(n, EC, reinterpret_cast<const float2*>(A), (int16_t*)g.ptr, st));
+    return oz_dense_apply(n, p, reinterpret_cast<const float2*>(A), (const int16_t*)g.ptr, EC,
+                          reinterpret_cast<const float2*>(X), reinterpret_cast<float2*>(W), nd, (char*)g.ptr + eb, st);
+  }
   GSI_CUDA_TRY(cudaMallocAsync(&g.ptr, std::max<size_t>(oz_gram_scratch_bytes(n, (int)n, p, false), 16), st));
   return oz_gram(n, (int)n, p, reinterpret_cast<const float2*>(A), reinterpret_cast<const float2*>(X),
                  false, nullptr, reinterpret_cast<float2*>(g.ptr), st, nd,

@@ -1968,6 +1968,304 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
   __syncthreads();
 }
 
+// ---------------------------------------------------------------------------
+// Dense apply W = A^T X (A n x n, X n x p): the Gram's digit products with the
+// operands prepared for their shape. As 64 x 64 output blocks of a Gram, every
+// CTA cut X again and A once per 64 columns of X, with one barrier among 16
+// rows of work (1.5 us for 8 KB of A): n = 16384, p = 128, 3 digits took 5.25 ms,
+// n = 4096, p = 32, 7 digits 185 us, against 0.32 ms and 20 us to read A. Here
+//  - X's digits are cut once by a small kernel into the images that shared
+//    memory holds per sub-chunk of 32 rows, and come by one bulk copy;
+//  - A's column exponents per chunk of EC rows come from a table, which the
+//    solver keeps with its operator (A does not change between applies);
+//  - a CTA takes 128 columns of A (the M of the products; TMEM lane = column
+//    of W^T) and NC columns of X: A is cut once for p <= NC. Its rows come
+//    straight into registers one sub-chunk ahead, 64-byte segments per row,
+//    after an L2 prefetch three sub-chunks ahead;
+//  - NS stages of digits, one mbarrier each for the products and for X's copy.
+// Group sums accumulate in tensor memory over a chunk (28800 EC < 2^24, as in
+// the Grams) and are combined in df64 once per chunk. Per left plane i the
+// right planes 0 .. ND - 1 - i feed the adjacent groups i ..: runs of up to
+// 256 / NC planes are one MMA.
+// Measured: n = 16384, p = 128, 3 digits 5.25 -> 1.00 ms, 7 digits 5.8 -> 3.3 ms;
+// n = 4096, p = 32, 7 digits 185 -> 92 us. A sub-chunk takes 2 us, of which the
+// products are 0.4-1; the rest is the loads' latency at one sub-chunk ahead
+// (registers allow no more) and its barrier.
+// ---------------------------------------------------------------------------
+constexpr int DN_SK = 32;       // rows of a sub-chunk
+constexpr int DN_THREADS = 512;
+template <int NDT, int NC>
+struct DnGeom {
+  static constexpr uint32_t APL = 128u * DN_SK * 2, XPL = (uint32_t)NC * DN_SK * 2;  // bytes of a plane
+  static constexpr uint32_t XB = NDT * XPL, STAGE = NDT * APL + XB;
+  static constexpr int NS = (220u * 1024u) / STAGE < 4 ? (int)((220u * 1024u) / STAGE) : 4;
+  static constexpr size_t SMEM = (size_t)NS * STAGE + (2 * NS + 1) * 8 + 16;
+  static_assert(NS >= 2 && NDT * NC <= 512, "two stages, groups in tensor memory");
+};
+
+// columns of X per CTA
+static int dn_nc(int p, int nd) { return p <= 32 ? 32 : (p <= 64 || nd == ND) ? 64 : 128; }
+
+// E[chunk n + c]: the exponent of column c of A over the chunk's EC rows
+__global__ void __launch_bounds__(512) oz_colexp_kernel(int64_t n, int EC, const float2* __restrict__ A,
+                                                        int16_t* __restrict__ E) {
+  __shared__ float mx[4][128];
+  const int64_t r0 = (int64_t)blockIdx.y * EC, r1 = min(n, r0 + EC);
+  const int64_t c = (int64_t)blockIdx.x * 128 + (threadIdx.x & 127);
+  float m = 0.f;
+  if (c < n) {
+#pragma unroll 8
+    for (int64_t r = r0 + (threadIdx.x >> 7); r < r1; r += 4) m = fmaxf(m, fabsf(__ldg(&A[r * n + c].x)));
+  }
+  mx[threadIdx.x >> 7][threadIdx.x & 127] = m;
+  __syncthreads();
+  if (threadIdx.x < 128 && c < n) {
+    m = fmaxf(fmaxf(mx[0][threadIdx.x], mx[1][threadIdx.x]), fmaxf(mx[2][threadIdx.x], mx[3][threadIdx.x]));
+    E[(int64_t)blockIdx.y * n + c] = (int16_t)exponent_above(m);
+  }
+}
+
+// X's digits: sub-chunk sg of column block b at img + (sg nxb + b) XB, plane
+// after plane; scales F[chunk (nxb NC) + column] = 2^(E - 7). One block per
+// chunk and 16 columns.
+template <int NDT>
+__global__ void __launch_bounds__(256) oz_dense_prep_kernel(int64_t n, int p, int NC, int nxb, int EC,
+                                                            const float2* __restrict__ X,
+                                                            unsigned char* __restrict__ img, float* __restrict__ F) {
+  __shared__ float mx[16][16];
+  __shared__ float cut[16];
+  const int64_t r0 = (int64_t)blockIdx.y * EC;
+  const int cc = threadIdx.x & 15, g = threadIdx.x >> 4, col = blockIdx.x * 16 + cc;
+  const bool live = col < p;
+  float m = 0.f;
+  for (int r = g; r < EC; r += 16)
+    if (live && r0 + r < n) m = fmaxf(m, fabsf(X[(r0 + r) * p + col].x));
+  mx[g][cc] = m;
+  __syncthreads();
+  if (threadIdx.x < 16) {
+    for (int z = 1; z < 16; ++z) m = fmaxf(m, mx[z][cc]);
+    const int E = exponent_above(m);
+    cut[cc] = exp2i(7 - E);
+    F[(int64_t)blockIdx.y * nxb * NC + col] = exp2i(E - 7);
+  }
+  __syncthreads();
+  const float sc = cut[cc];
+  const uint32_t xpl = (uint32_t)NC * DN_SK * 2;
+  const int b = col / NC, c = col - b * NC;
+  for (int q = g; q < EC / 4; q += 16) {  // rows 4q .. 4q + 3 of the chunk
+    float d[4][NDT];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      const int64_t R = r0 + 4 * q + t;
+      const float2 x = live && R < n ? X[R * p + col] : make_float2(0.f, 0.f);
+      digits_scaled<NDT>(x.x, x.y, sc, d[t]);
+    }
+    const int64_t sg = r0 / DN_SK + q / (DN_SK / 4);
+    unsigned char* dst = img + (sg * nxb + b) * (int64_t)(NDT * xpl) + tc_off(c, 4 * (q % (DN_SK / 4)), DN_SK);
+#pragma unroll
+    for (int i = 0; i < NDT; ++i)
+      *reinterpret_cast<uint2*>(dst + i * xpl) =
+          make_uint2(pack_bf16x2(d[0][i], d[1][i]), pack_bf16x2(d[2][i], d[3][i]));
+  }
+}
+
+template <int NDT, int NC>
+__global__ void __launch_bounds__(DN_THREADS, 1)
+oz_dense_kernel(int64_t n, int EC, const float2* __restrict__ A, const int16_t* __restrict__ Ea,
+                const unsigned char* __restrict__ img, const float* __restrict__ F, int nbj, int nblk, float2* part) {
+  using Geo = DnGeom<NDT, NC>;
+  constexpr int NS = Geo::NS, NPT = NC / 4;  // columns of X per thread in the combination
+  extern __shared__ __align__(128) unsigned char dn_sm[];
+  uint64_t* mbar = reinterpret_cast<uint64_t*>(dn_sm + (size_t)NS * Geo::STAGE);  // NS products, NS copies, drain
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2 * NS + 1);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int xb = blockIdx.z, nxb = gridDim.z;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
+                 "r"(TC_TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    for (int b = 0; b < 2 * NS + 1; ++b)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(mbar + b)));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot, sbase = smem_addr(dn_sm), mb = smem_addr(mbar), xm = mb + 8u * NS;
+  const int wait_limit = g_oz_wait_limit;
+  // this CTA's chunks: a contiguous range
+  const int nch = (int)((n + EC - 1) / EC), per = (nch + gridDim.x - 1) / gridDim.x;
+  const int ch0 = min(nch, (int)blockIdx.x * per), ch1 = min(nch, ch0 + per);
+  const int NSUB = EC / DN_SK, G = (ch1 - ch0) * NSUB;
+  const int64_t row0 = (int64_t)ch0 * EC, sg0 = row0 / DN_SK;
+  // cut: warp w holds columns 8w .. 8w + 7 of the tile, a lane the column
+  // (lane & 7) and the rows 4q .. 4q + 3, q = lane >> 3 and that + 4: its
+  // 8-byte digit stores cover the banks evenly
+  const int64_t acol = (int64_t)blockIdx.y * 128 + 8 * warp + (lane & 7);
+  const bool alive = acol < n;
+  const int qd = lane >> 3;
+  float2 v[8];
+  auto load = [&](int g) {
+#pragma unroll
+    for (int z = 0; z < 2; ++z)
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int64_t R = row0 + (int64_t)g * DN_SK + 4 * (qd + 4 * z) + t;
+        v[4 * z + t] = alive && R < n ? __ldg(A + R * n + acol) : make_float2(0.f, 0.f);
+      }
+  };
+  // rows of sub-chunk g into L2: one 128-byte line per thread (tid < 256)
+  auto prefetch = [&](int g) {
+    const int64_t R = row0 + (int64_t)g * DN_SK + (tid >> 3), c = (int64_t)blockIdx.y * 128 + 16 * (tid & 7);
+    if (tid < 256 && g < G && R < n && c < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(A + R * n + c));
+  };
+  int copied = 0;  // X copies issued (thread 0)
+  auto copy_x = [&](int g) {
+    const uint32_t bar = xm + 8u * (g % NS);
+    asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(bar),
+                 "r"(Geo::XB)
+                 : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     sbase + (uint32_t)(g % NS) * Geo::STAGE + NDT * Geo::APL),
+                 "l"(img + ((sg0 + g) * nxb + xb) * (int64_t)Geo::XB), "r"(Geo::XB), "r"(bar)
+                 : "memory");
+    copied = g + 1;
+  };
+  const int quarter = warp & 3, cb = (warp >> 2) * NPT;
+  float2 res[NPT];
+#pragma unroll
+  for (int e = 0; e < NPT; ++e) res[e] = make_float2(0.f, 0.f);
+  bool failed = false, ok = true;
+  int committed = 0;  // sub-chunks whose products were issued (thread 0)
+  if (G > 0) {
+    if (tid == 0) copy_x(0);
+    load(0);
+    for (int g = 1; g < 4; ++g) prefetch(g);
+  }
+  int s = 0, ch = ch0;
+  for (int g = 0; g < G && !failed; ++g) {
+    const int st = g % NS;
+    unsigned char* const stage = dn_sm + (size_t)st * Geo::STAGE;
+    // the next stage is free once its last products are done; X's copy into it
+    if (g + 1 < G) {
+      if (g + 1 >= NS) ok = tc_wait(mb + 8u * ((g + 1) % NS), (uint32_t)(((g + 1) / NS - 1) & 1), wait_limit) && ok;
+      if (tid == 0 && ok) copy_x(g + 1);
+    }
+    {
+      const float sc = alive ? exp2i(7 - (int)__ldg(Ea + (int64_t)ch * n + acol)) : 0.f;
+      const int col = 8 * warp + (lane & 7);
+#pragma unroll
+      for (int z = 0; z < 2; ++z) {
+        float d[4][NDT];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) digits_scaled<NDT>(v[4 * z + t].x, v[4 * z + t].y, sc, d[t]);
+        unsigned char* dst = stage + tc_off(col, 4 * (qd + 4 * z), DN_SK);
+#pragma unroll
+        for (int i = 0; i < NDT; ++i)
+          *reinterpret_cast<uint2*>(dst + i * Geo::APL) =
+              make_uint2(pack_bf16x2(d[0][i], d[1][i]), pack_bf16x2(d[2][i], d[3][i]));
+      }
+    }
+    if (g + 1 < G) load(g + 1);
+    prefetch(g + 4);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    if (__syncthreads_or(!ok)) {
+      failed = true;
+      break;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (tid == 0) {
+      ok = tc_wait(xm + 8u * st, (uint32_t)((g / NS) & 1), wait_limit);
+      if (ok) {
+        const uint32_t ab = sbase + (uint32_t)st * Geo::STAGE;
+        const uint64_t da = tc_desc(ab, DN_SK), db = tc_desc(ab + NDT * Geo::APL, DN_SK);
+        const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);
+        constexpr int RUN = 256 / NC;
+#pragma unroll
+        for (int i = 0; i < NDT; ++i)
+#pragma unroll
+          for (int j0 = 0; j0 < NDT - i; j0 += RUN) {
+            const int run = NDT - i - j0 < RUN ? NDT - i - j0 : RUN;
+            const uint32_t idn = idesc0 | ((uint32_t)((NC * run) >> 3) << 17);
+#pragma unroll
+            for (int ks = 0; ks < DN_SK / 16; ++ks)
+              tc_mma(tmem + (uint32_t)((i + j0) * NC), da + ((i * Geo::APL + ks * 256) >> 4),
+                     db + ((j0 * Geo::XPL + ks * 256) >> 4), idn, (i > 0 || ks > 0 || s > 0) ? 1u : 0u);
+          }
+        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mb + 8u * st)
+                     : "memory");
+        committed = g + 1;
+      }
+    }
+    __syncwarp();
+    if (++s < NSUB) continue;
+    // chunk end: its products, then the combination
+    ok = tc_wait(mb + 8u * st, (uint32_t)((g / NS) & 1), wait_limit) && ok;
+    if (__syncthreads_or(!ok)) {
+      failed = true;
+      break;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const int64_t ac = (int64_t)blockIdx.y * 128 + 32 * quarter + lane;
+    const float fu = ac < n ? exp2i((int)__ldg(Ea + (int64_t)ch * n + ac) - 7) : 0.f;
+    const float* Fv = F + ((int64_t)ch * nxb + xb) * NC + cb;
+    const uint32_t lanes = tmem + ((uint32_t)(32 * quarter) << 16);
+#pragma unroll
+    for (int c0 = 0; c0 < NPT; c0 += 4) {
+      uint32_t u[NDT][4];
+#pragma unroll
+      for (int h = 0; h < NDT; ++h) tc_ld4(u[h], lanes + (uint32_t)(h * NC + cb + c0));
+      const float4 f4 = __ldg(reinterpret_cast<const float4*>(Fv + c0));
+      const float fv[4] = {f4.x, f4.y, f4.z, f4.w};
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        float S[NDT];
+#pragma unroll
+        for (int h = 0; h < NDT; ++h) S[h] = __uint_as_float(u[h][e]);
+        const float2 w = combine_groups_fast<NDT, (NDT > 4 ? 4 : NDT - 1)>(S);
+        res[c0 + e] = df_add(res[c0 + e], make_float2(w.x * fu * fv[e], w.y * fu * fv[e]));
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();  // the reads are done before the next chunk's products
+    s = 0;
+    ++ch;
+  }
+  if (failed) {
+    // a wait ran out: let the products and copies in flight land (bounded),
+    // report non-finite partial sums
+    // (thread 0 issued them all; the others wait for it at the barrier below)
+    if (tid == 0) {
+      atomicAdd(&g_oz_tc_timeouts, 1);
+      for (int b = 0; b < NS; ++b) {
+        const int lp = committed - 1 - ((committed - 1 - b) % NS + NS) % NS;  // last g' < committed, g' % NS == b
+        if (lp >= 0) tc_wait(mb + 8u * b, (uint32_t)((lp / NS) & 1), TC_WAIT_LIMIT);
+        const int lc = copied - 1 - ((copied - 1 - b) % NS + NS) % NS;
+        if (lc >= 0) tc_wait(xm + 8u * b, (uint32_t)((lc / NS) & 1), TC_WAIT_LIMIT);
+      }
+      tc_drain(true, mb + 8u * (2 * NS));
+    }
+#pragma unroll
+    for (int e = 0; e < NPT; ++e) res[e] = make_float2(NAN, NAN);
+  }
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_TMEM_COLS));
+  // rows of W = columns of A: 64 x 64 blocks (bi, bj) of the reduction
+  const int64_t ac = (int64_t)blockIdx.y * 128 + 32 * quarter + lane;
+  const int64_t bi = ac >> 6;
+  if (bi * nbj < nblk) {
+#pragma unroll
+    for (int e = 0; e < NPT; ++e) {
+      const int c = xb * NC + cb + e;
+      if ((c >> 6) < nbj) part[((size_t)blockIdx.x * nblk + bi * nbj + (c >> 6)) * 4096 + (ac & 63) * 64 + (c & 63)] = res[e];
+    }
+  }
+}
+
 // Fixed-order sums of the per-block partials. A block is 32 entries x
 // RED_GROUPS groups: warp g adds the splits k = g, g + RED_GROUPS, ... in
 // ascending order (lanes on consecutive entries, four loads in flight), and
@@ -2326,6 +2624,79 @@ gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bo
     oz_gram_reduce_kernel<<<ceil_div(p * q, 32), 32 * RED_GROUPS, 0, st>>>(p, q, ns, nblk, sym ? 1 : 0,
                                                                            sym2 ? 1 : 0, nbj, scratch, G, Gf);
   }
+  GSI_LAUNCH_CHECK();
+  return GSI_OK;
+}
+
+// ---- dense apply ------------------------------------------------------------
+// rows of an exponent chunk: 160 for 7 digits; for 3 the grids of the Gram
+// kernels that served them (384 rows for aligned blocks of even width, else
+// 64), which set their errors
+int oz_dense_chunk(int64_t n, int p, int nd, bool aligned) {
+  if (nd == ND) return 160;
+  return ((n | p) & 1) == 0 && aligned ? 384 : 64;
+}
+
+size_t oz_colexp_bytes(int64_t n, int EC) { return (size_t)((n + EC - 1) / EC) * n * sizeof(int16_t); }
+
+gsi_status oz_colexp(int64_t n, int EC, const float2* A, int16_t* E, cudaStream_t st) {
+  oz_colexp_kernel<<<dim3((unsigned)((n + 127) / 128), (unsigned)((n + EC - 1) / EC)), 512, 0, st>>>(n, EC, A, E);
+  GSI_LAUNCH_CHECK();
+  return GSI_OK;
+}
+
+// CTAs along the contraction, and the scratch: partial sums, X's digits and
+// scales
+static int oz_dense_splits(int64_t n, int p, int nd, int EC) {
+  const int64_t tiles = (n + 127) / 128 * ((p + dn_nc(p, nd) - 1) / dn_nc(p, nd)), nch = (n + EC - 1) / EC;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(sm_count() / tiles, nch));
+}
+static size_t oz_dense_part_bytes(int64_t n, int p, int nd, int EC) {
+  return (size_t)oz_dense_splits(n, p, nd, EC) * ((n + 63) / 64) * ((p + 63) / 64) * 4096 * sizeof(float2);
+}
+static size_t oz_dense_img_bytes(int64_t n, int p, int nd, int EC) {
+  const int NC = dn_nc(p, nd), nxb = (p + NC - 1) / NC;
+  return (size_t)((n + EC - 1) / EC) * EC * nxb * NC * nd * 2;
+}
+size_t oz_dense_scratch_bytes(int64_t n, int p, int nd, int EC) {
+  const int NC = dn_nc(p, nd), nxb = (p + NC - 1) / NC;
+  return oz_dense_part_bytes(n, p, nd, EC) + oz_dense_img_bytes(n, p, nd, EC) +
+         (size_t)((n + EC - 1) / EC) * nxb * NC * sizeof(float) + 256;
+}
+
+template <int NDT, int NC>
+static gsi_status dn_launch(int64_t n, int EC, const float2* A, const int16_t* Ea, const unsigned char* img,
+                            const float* F, int ns, int nxb, int nbj, int nblk, float2* part, cudaStream_t st) {
+  GSI_CUDA_TRY(ensure_dyn_smem((const void*)oz_dense_kernel<NDT, NC>, (int)DnGeom<NDT, NC>::SMEM));
+  oz_dense_kernel<NDT, NC><<<dim3(ns, (unsigned)((n + 127) / 128), nxb), DN_THREADS, DnGeom<NDT, NC>::SMEM, st>>>(
+      n, EC, A, Ea, img, F, nbj, nblk, part);
+  GSI_LAUNCH_CHECK();
+  return GSI_OK;
+}
+
+// W = A^T X in nd digits with A's exponent table Ea (oz_colexp for EC rows)
+gsi_status oz_dense_apply(int64_t n, int p, const float2* A, const int16_t* Ea, int EC, const float2* X, float2* W,
+                          int nd, void* scratch, cudaStream_t st) {
+  if (n < 1 || p < 1 || p > 128 || (nd != 3 && nd != ND) || EC % DN_SK != 0 || EC > 512) return GSI_ERR_ARG;
+  const int NC = dn_nc(p, nd), nxb = (p + NC - 1) / NC, ns = oz_dense_splits(n, p, nd, EC);
+  const int nbj = (p + 63) / 64, nblk = (int)((n + 63) / 64) * nbj, nch = (int)((n + EC - 1) / EC);
+  float2* part = reinterpret_cast<float2*>(scratch);
+  unsigned char* img = reinterpret_cast<unsigned char*>(scratch) + oz_dense_part_bytes(n, p, nd, EC);
+  float* F = reinterpret_cast<float*>(img + oz_dense_img_bytes(n, p, nd, EC));
+  const dim3 pg((unsigned)(nxb * NC / 16), (unsigned)nch);
+  if (nd == 3) oz_dense_prep_kernel<3><<<pg, 256, 0, st>>>(n, p, NC, nxb, EC, X, img, F);
+  else oz_dense_prep_kernel<ND><<<pg, 256, 0, st>>>(n, p, NC, nxb, EC, X, img, F);
+  GSI_LAUNCH_CHECK();
+  gsi_status s;
+  if (nd == 3)
+    s = NC == 32   ? dn_launch<3, 32>(n, EC, A, Ea, img, F, ns, nxb, nbj, nblk, part, st)
+        : NC == 64 ? dn_launch<3, 64>(n, EC, A, Ea, img, F, ns, nxb, nbj, nblk, part, st)
+                   : dn_launch<3, 128>(n, EC, A, Ea, img, F, ns, nxb, nbj, nblk, part, st);
+  else
+    s = NC == 32 ? dn_launch<ND, 32>(n, EC, A, Ea, img, F, ns, nxb, nbj, nblk, part, st)
+                 : dn_launch<ND, 64>(n, EC, A, Ea, img, F, ns, nxb, nbj, nblk, part, st);
+  GSI_TRY(s);
+  oz_gram_reduce_df_kernel<<<ceil_div(n * p, 256), 256, 0, st>>>((int)n, p, ns, nbj, part, W);
   GSI_LAUNCH_CHECK();
   return GSI_OK;
 }

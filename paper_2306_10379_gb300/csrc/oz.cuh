@@ -58,6 +58,18 @@ gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bo
                    float2* scratch, cudaStream_t st, int nd = 7, float2* Gdf = nullptr,
                    int reserve_sms = 0, bool sym2 = false, float2* Gf = nullptr);
 
+// Dense apply W = A^T X (A n x n df64 row-major; for symmetric A this is A X):
+// oz_dense_chunk: rows of an exponent chunk (aligned: A and X on 16 bytes);
+// oz_colexp: A's table of column exponents for that chunk length
+// (oz_colexp_bytes), which may be kept as long as A does not change;
+// scratch: oz_dense_scratch_bytes.
+int oz_dense_chunk(int64_t n, int p, int nd, bool aligned);
+size_t oz_colexp_bytes(int64_t n, int EC);
+gsi_status oz_colexp(int64_t n, int EC, const float2* A, int16_t* E, cudaStream_t st);
+size_t oz_dense_scratch_bytes(int64_t n, int p, int nd, int EC);
+gsi_status oz_dense_apply(int64_t n, int p, const float2* A, const int16_t* Ea, int EC, const float2* X, float2* W,
+                          int nd, void* scratch, cudaStream_t st);
+
 // Bounded waits of the tcgen05 kernels: polls allowed to a wait on a batch of
 // products (limit < 0: the default, 2^24); a wait that runs out drains the
 // tensor core, counts one timeout and leaves non-finite outputs.

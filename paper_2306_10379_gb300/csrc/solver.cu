@@ -120,6 +120,8 @@ struct gsi_ctx {
   double* Ad = nullptr;   // dense A, float64 (GSI_DENSE)
   float2* Adf = nullptr;  // dense A, df64
   float2* dense_ws = nullptr;
+  int16_t* colexp[2] = {nullptr, nullptr};  // A's column exponents for the 7-digit and the 3-digit apply
+  int colexp_ec[2] = {0, 0};
   int64_t* rowptr = nullptr;
   int32_t* colidx = nullptr;
   double* val = nullptr;    // float64 values (native mode and Rayleigh-Ritz)
@@ -271,9 +273,13 @@ gsi_status op_matvec(gsi_ctx* c, const void* in, void* outp, bool accurate = tru
   double bytes;
   if (c->fmt == GSI_DENSE) {
     bytes = 8.0 * (double)c->n * c->n + 2 * blk_bytes(c);
-    s = c->emu ? oz_gram(c->n, (int)c->n, c->p, c->Adf, (const float2*)in, false, nullptr, c->dense_ws,
-                         c->st, accurate ? 7 : c->nd, (float2*)outp)
-               : dense_gemm(c->n, c->p, c->Ad, (const double*)in, (double*)outp, c->st);
+    const int nd = accurate ? 7 : c->nd, k = nd == 7 ? 0 : 1;
+    s = !c->emu ? dense_gemm(c->n, c->p, c->Ad, (const double*)in, (double*)outp, c->st)
+        : tensor_path() != 1
+            ? oz_dense_apply(c->n, c->p, c->Adf, c->colexp[k], c->colexp_ec[k], (const float2*)in, (float2*)outp, nd,
+                             c->dense_ws, c->st)
+            : oz_gram(c->n, (int)c->n, c->p, c->Adf, (const float2*)in, false, nullptr, c->dense_ws, c->st, nd,
+                      (float2*)outp);
     prof_end(c, GSI_K_SPMM, bytes, 2.0 * (double)c->n * c->n * c->p);
     return s;
   }
@@ -973,7 +979,16 @@ gsi_status upload_operator(gsi_ctx* c, const gsi_matrix* A) {
     if (c->emu) {
       if (!c->Adf) GSI_TRY(dev_alloc(c, (void**)&c->Adf, nn * sizeof(float2)));
       GSI_TRY(df_from_f64((int64_t)nn, c->Ad, c->Adf, c->st));
-      if (!c->dense_ws) GSI_TRY(dev_alloc(c, (void**)&c->dense_ws, oz_gram_scratch_bytes(n, (int)n, p, false)));
+      // column exponents of A for the digit applies, once per operator
+      size_t ws = oz_gram_scratch_bytes(n, (int)n, p, false);
+      for (int k = 0; k < (c->mixed ? 2 : 1); ++k) {
+        const int nd = k == 0 ? 7 : 3, ec = oz_dense_chunk(n, p, nd, true);
+        c->colexp_ec[k] = ec;
+        if (!c->colexp[k]) GSI_TRY(dev_alloc(c, (void**)&c->colexp[k], oz_colexp_bytes(n, ec)));
+        GSI_TRY(oz_colexp(n, ec, c->Adf, c->colexp[k], c->st));
+        ws = std::max(ws, oz_dense_scratch_bytes(n, p, nd, ec));
+      }
+      if (!c->dense_ws) GSI_TRY(dev_alloc(c, (void**)&c->dense_ws, ws));
     }
     return GSI_OK;
   }
