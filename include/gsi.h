@@ -435,11 +435,9 @@ gsi_status gsi_oz_gram_noalloc(int64_t n, int32_t p, int32_t q, const float* U, 
 
 /* Which tensor-core kernels the digit-split products use: 0 (default) and 2
  * the tcgen05 kernels wherever they apply (7-digit Grams of any p, q, one
- * CTA per 64 x 64 output block; 3-digit Grams on 16-byte aligned blocks of
- * even width; the dense apply, 128 rows of W per CTA;
+ * CTA per 64 x 64 output block; the dense apply, 128 rows of W per CTA;
  * 7-digit block products of any p <= 128, the contraction cut into slices
- * of at most 64 for p > 64), 1 the mma.sync kernels everywhere (they also
- * serve the remaining 3-digit products). Block products with p <= 64 are
+ * of at most 64 for p > 64), 1 the mma.sync kernels everywhere. Block products with p <= 64 are
  * identical on both (same digits, exact integer digit-pair sums, same
  * combination order); for p > 64 the tcgen05 slices take their own digit
  * exponents and are summed in df64, so the two agree to df64 rounding but

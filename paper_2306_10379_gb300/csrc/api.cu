@@ -79,6 +79,7 @@ gsi_status gsi_linesearch(int32_t p, const double* C, const double* B, const dou
     PpArgs a{};
     a.mode = 0;
     a.p = p;
+    a.want_phi = 1;
     a.C = {nullptr, C, 1};
     a.B = {nullptr, B, 1};
     a.Gam = {nullptr, Gam, 1};

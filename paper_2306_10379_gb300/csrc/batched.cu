@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(BT) b_retract_kernel(BDev d, int32_t mode) {
 using BPp16 = PpCfg<BS, 16, 1, 1, 1, 8, 1, 1, 1>;
 using BPp32 = PpCfg<BS, 32, 4, 1, 1, 16, 2, 2, 1>;
 
-__global__ void __launch_bounds__(BS) b_small_kernel(BDev d, int32_t mode) {
+__global__ void __launch_bounds__(BS, 2) b_small_kernel(BDev d, int32_t mode) {
   const int i = blockIdx.x;
   const int32_t mask = mode == 0 ? F_STEP : F_START;
   if (!(d.st[i].flags & mask)) return;

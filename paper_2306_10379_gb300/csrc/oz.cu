@@ -1410,7 +1410,7 @@ oz_gram_tc_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const f
 
 // ---------------------------------------------------------------------------
 // oz_gram_tc_ring_kernel: the tcgen05 Gram for 16-byte aligned blocks of even
-// width (one 64 x 64 output block per blockIdx.y, as oz_gram_tc_kernel).
+// width and at most 64 columns.
 //
 // The kernel above stages a whole exponent chunk raw, which fills shared
 // memory and leaves room for two digit buffers only; its sub-chunk loop then
@@ -1442,7 +1442,7 @@ oz_gram_tc_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const f
 constexpr int TR_WORKERS = 512;
 constexpr int TR_THREADS = TR_WORKERS + 96;  // + the issuing warp + two maxima warps
 constexpr int TR_BAR_COUNT = TR_WORKERS + 32;
-template <bool SYM, int NDT = ND>
+template <bool SYM>
 struct TrGeom {
   static constexpr int EC = SYM ? 512 : 384;       // most rows of an exponent chunk
   static constexpr int SK = SYM ? 32 : 16;         // sub-chunk rows
@@ -1452,8 +1452,8 @@ struct TrGeom {
   static constexpr int MS = 2 * MSW;
   static constexpr int MB = SYM ? 16 : 8;          // rows per operand in one maxima slot
   static constexpr uint32_t PLANE = 64u * SK * 2;  // one digit plane: 64 columns x SK rows, bf16
-  // U == V: NDT planes and a zero pad plane; U != V: NDT planes of U, NDT of V
-  static constexpr uint32_t DBUF = (uint32_t)(SYM ? NDT + 1 : 2 * NDT) * PLANE;
+  // U == V: ND planes and a zero pad plane; U != V: ND planes of U, ND of V
+  static constexpr uint32_t DBUF = (uint32_t)(SYM ? ND + 1 : 2 * ND) * PLANE;
   static constexpr size_t RAW_SLOT = (size_t)32 * TG_RS * sizeof(float2);
   static constexpr size_t MSLOT = (size_t)16 * 64 * sizeof(float2);  // 16 rows of 64 df64
   // raw slots, digit buffers, maxima slots, exponents and scales [2][128]
@@ -1470,10 +1470,7 @@ static_assert(TrGeom<false>::NR * TrGeom<false>::RAW_SLOT >= 64 * 65 * sizeof(fl
                   TrGeom<true>::NR * TrGeom<true>::RAW_SLOT >= 64 * 65 * sizeof(float2),
               "final stage fits the raw ring");
 
-size_t oz_gram_tc_ring_smem(bool sym, int nd) {
-  return nd == 3 ? (sym ? TrGeom<true, 3>::smem() : TrGeom<false, 3>::smem())
-                 : (sym ? TrGeom<true>::smem() : TrGeom<false>::smem());
-}
+size_t oz_gram_tc_ring_smem(bool sym) { return sym ? TrGeom<true>::smem() : TrGeom<false>::smem(); }
 
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() {
@@ -1506,25 +1503,11 @@ __device__ __forceinline__ bool bar1_or(bool v) {
 // constant: with a run-time length the row counters cost the U != V kernel
 // 6% at 128^3 (968 -> 1031 us), so the other instantiation serves only the
 // sizes whose chunks are shorter.
-template <bool SYM, int NDT, bool FULL>
+template <bool SYM, bool FULL>
 __global__ void __launch_bounds__(TR_THREADS, 1)
 oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, const float2* __restrict__ V,
-                       float2* part, int nbj, int tri, int ec) {
-  using Geo = TrGeom<SYM, NDT>;
-  int bi = 0, bj = (int)blockIdx.y;
-  if (tri) {
-    int y = (int)blockIdx.y;
-    while (y >= nbj - bi) {
-      y -= nbj - bi;
-      ++bi;
-    }
-    bj = bi + y;
-  } else {
-    bi = (int)blockIdx.y / nbj;
-    bj = (int)blockIdx.y - bi * nbj;
-  }
-  const int cu0 = 64 * bi, cv0 = 64 * bj;
-  const int wu = min(64, p - cu0), wv = min(64, q - cv0);  // live columns (even: p, q even)
+                       float2* part, int ec) {
+  using Geo = TrGeom<SYM>;
   constexpr int SK = Geo::SK, NB = Geo::NB, NR = Geo::NR;
   constexpr int MS = Geo::MS, MSW = Geo::MSW, MB = Geo::MB;
   static_assert(Geo::EC % SK == 0 && SK % (2 * MB) == 0, "chunks are whole sub-chunks; the maxima warps take alternate batches");
@@ -1548,7 +1531,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
   if (SYM && worker)
     for (int e = tid; e < NB * (int)(plane / 16); e += TR_WORKERS) {
       const int b = e / (int)(plane / 16), o = e - b * (int)(plane / 16);
-      *reinterpret_cast<uint4*>(dig + b * DBUF + NDT * plane + 16 * o) = make_uint4(0u, 0u, 0u, 0u);
+      *reinterpret_cast<uint4*>(dig + b * DBUF + ND * plane + 16 * o) = make_uint4(0u, 0u, 0u, 0u);
     }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tslot)),
@@ -1578,13 +1561,10 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
     // chunk j: cells 0..MB-1 hold U's rows, cells MB..15 V's (U != V). The
     // warps take alternate batches (b % 2 == mw; NMB is even), each through
     // its own ring of MSW slots, and merge their maxima once per chunk.
-    // Where the block spans whole rows (64 columns or fewer), a batch's rows
-    // are contiguous: one copy per operand, rows ld apart in the slot;
-    // otherwise one copy per row, rows 64 apart (the copy engine's cost per
-    // copy made 16 copies of 512 B per batch the bottleneck).
+    // A batch's rows are contiguous: one copy per operand, rows p (q) apart in
+    // the slot (the copy engine's cost per copy made 16 copies of 512 B per
+    // batch the bottleneck).
     const int total = nmy * NMB / 2;  // this warp's batches
-    const bool contU = wu == p, contV = SYM ? contU : wv == q;
-    const int strU = contU ? p : 64, strV = contV ? q : 64;
     // first rows of this warp's next batch to copy and to reduce, carried
     // along (a division per batch by the run-time chunk length cost the
     // U != V kernel 8%: these two warps pace the others)
@@ -1622,28 +1602,14 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
       uint32_t bytes = 0;
       const float2* src = U;
       float2* dst = sl;
-      if (contU) {
-        if (lane == 0 && nv > 0) {
-          bytes = (uint32_t)nv * (uint32_t)p * 8u;
-          src = U + (size_t)R0 * p;
-        }
-      } else if (lane < MB && lane < nv) {
-        bytes = (uint32_t)wu * 8u;
-        src = U + (size_t)(R0 + lane) * p + cu0;
-        dst = sl + lane * 64;
+      if (lane == 0 && nv > 0) {
+        bytes = (uint32_t)nv * (uint32_t)p * 8u;
+        src = U + (size_t)R0 * p;
       }
-      if (!SYM) {
-        if (contV) {
-          if (lane == 16 && nv > 0) {
-            bytes = (uint32_t)nv * (uint32_t)q * 8u;
-            src = V + (size_t)R0 * q;
-            dst = sl + MB * 64;
-          }
-        } else if (lane >= 16 && lane < 16 + MB && lane - 16 < nv) {
-          bytes = (uint32_t)wv * 8u;
-          src = V + (size_t)(R0 + lane - 16) * q + cv0;
-          dst = sl + (MB + lane - 16) * 64;
-        }
+      if (!SYM && lane == 16 && nv > 0) {
+        bytes = (uint32_t)nv * (uint32_t)q * 8u;
+        src = V + (size_t)R0 * q;
+        dst = sl + MB * 64;
       }
       const uint32_t tot = __reduce_add_sync(0xffffffffu, bytes);
       const uint32_t mb = bar_of(t);
@@ -1659,7 +1625,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
             "l"(src), "r"(bytes), "r"(mb)
             : "memory");
     };
-    const bool lu = 2 * lane < wu, lv = 2 * lane < wv;
+    const bool lu = 2 * lane < p, lv = 2 * lane < q;
     float mu0 = 0.f, mu1 = 0.f, mv0 = 0.f, mv1 = 0.f;  // columns 2 lane, 2 lane + 1 of U and V
     bool dead = false;
     int issued_t = 0, done_t = 0;
@@ -1685,7 +1651,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const bool isvc = !SYM && i >= MB;
-              v[i] = *reinterpret_cast<const float4*>(sl + (isvc ? MB * 64 + (i - MB) * strV : i * strU));
+              v[i] = *reinterpret_cast<const float4*>(sl + (isvc ? MB * 64 + (i - MB) * q : i * p));
             }
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
@@ -1704,7 +1670,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
               const int li = isvc ? i - MB : i;
               if (li < left && (isvc ? lv : lu)) {
                 const float4 v =
-                    *reinterpret_cast<const float4*>(sl + (isvc ? MB * 64 + li * strV : li * strU));
+                    *reinterpret_cast<const float4*>(sl + (isvc ? MB * 64 + li * q : li * p));
                 if (isvc) {
                   mv0 = fmaxf(mv0, fabsf(v.x));
                   mv1 = fmaxf(mv1, fabsf(v.z));
@@ -1769,10 +1735,10 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
     // c, c + 1 (c = 2 (tid % 32)), one 16-byte copy each; raw row r + 16 is
     // U's row r + 16 (U == V) or V's row r (U != V)
     const int sr = tid >> 5, sc = 2 * (tid & 31);
-    const bool sokA = sc < wu, sokB = sc < (SYM ? wu : wv);
+    const bool sokA = sc < p, sokB = sc < q;
     const int ldA = p, ldB = SYM ? p : q;
-    const float2* sA = U + cu0 + sc + (int64_t)sr * ldA;
-    const float2* sB = SYM ? U + cu0 + sc + (int64_t)(sr + 16) * ldA : V + cv0 + sc + (int64_t)sr * ldB;
+    const float2* sA = U + sc + (int64_t)sr * ldA;
+    const float2* sB = SYM ? U + sc + (int64_t)(sr + 16) * ldA : V + sc + (int64_t)sr * ldB;
     const int64_t rA0 = sr, rB0 = SYM ? sr + 16 : sr;
     // sub-chunks are staged in order: their first row is carried along
     int64_t st_r0 = (int64_t)blockIdx.x * EC;
@@ -1811,7 +1777,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
     const int ic = 8 * ((loc >> 5) & 7) + (lane & 7);
     const int iq = 2 * (((lane >> 4) & 1) + 2 * (loc >> 8)) + ((lane >> 3) & 1);
     const int irow = (isv ? SK : 0) + 4 * iq;
-    const uint32_t doff = (isv ? NDT * plane : 0) + tc_off(ic, 4 * iq, SK);
+    const uint32_t doff = (isv ? ND * plane : 0) + tc_off(ic, 4 * iq, SK);
     bool failed = false;
     int issued = 0;  // sub-chunks whose products were issued (the same in every thread)
     if (worker) {
@@ -1839,14 +1805,14 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
           if (ok) {
             const float2* slot = raw + (size_t)(g % NR) * (32 * TG_RS) + irow * TG_RS + ic;
             unsigned char* dst = dig + buf * DBUF + doff;
-            float d[4][NDT];
+            float d[4][ND];
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
               const float2 x = slot[t * TG_RS];
-              digits_scaled<NDT>(x.x, x.y, scut, d[t]);
+              digits_scaled<ND>(x.x, x.y, scut, d[t]);
             }
 #pragma unroll
-            for (int i = 0; i < NDT; ++i)
+            for (int i = 0; i < ND; ++i)
               *reinterpret_cast<uint2*>(dst + i * plane) =
                   make_uint2(pack_bf16x2(d[0][i], d[1][i]), pack_bf16x2(d[2][i], d[3][i]));
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1864,15 +1830,15 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           if (issuer) {
             if (lane == 0) {
-              const uint32_t ab = dbase + buf * DBUF, bb = SYM ? ab : ab + NDT * plane;
+              const uint32_t ab = dbase + buf * DBUF, bb = SYM ? ab : ab + ND * plane;
               const uint64_t da = tc_desc(ab, SK), db = tc_desc(bb, SK);
               const uint32_t acc0 = s > 0 ? 1u : 0u;
               const uint32_t idesc0 = idesc & ~(0x3Fu << 17);
 #pragma unroll
               for (int m = 0; m < 4; ++m)
 #pragma unroll
-                for (int j0 = 0; j0 < NDT - 2 * m; j0 += 4) {
-                  const int run = (NDT - 2 * m - j0) < 4 ? (NDT - 2 * m - j0) : 4;
+                for (int j0 = 0; j0 < ND - 2 * m; j0 += 4) {
+                  const int run = (ND - 2 * m - j0) < 4 ? (ND - 2 * m - j0) : 4;
                   const uint32_t idn = idesc0 | ((uint32_t)((64 * run) >> 3) << 17);
 #pragma unroll
                   for (int ks = 0; ks < SK / 16; ++ks)
@@ -1904,20 +1870,20 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
           const uint32_t lanes = tmem + ((uint32_t)(32 * quarter) << 16);
 #pragma unroll
           for (int c0 = 0; c0 < 16; c0 += 4) {
-            uint32_t v[NDT][4];
+            uint32_t v[ND][4];
 #pragma unroll
-            for (int h = 0; h < NDT; ++h)
-              if (top || h < NDT - 1) tc_ld4(v[h], lanes + (uint32_t)(h * 64 + cb + c0));
+            for (int h = 0; h < ND; ++h)
+              if (top || h < ND - 1) tc_ld4(v[h], lanes + (uint32_t)(h * 64 + cb + c0));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-              float S[NDT];
+              float S[ND];
 #pragma unroll
-              for (int h = 0; h < NDT; ++h) S[h] = __uint_as_float(v[h][e]);
+              for (int h = 0; h < ND; ++h) S[h] = __uint_as_float(v[h][e]);
               // top: groups 0..6 (even digits of U); bottom: groups 1..6
               // (odd digits), block h holding group h + 1
-              const float2 w = top ? combine_groups_fast<NDT, (NDT > 4 ? 4 : NDT - 1)>(S)
-                                   : combine_groups_fast<NDT - 1, (NDT > 4 ? 3 : NDT - 2)>(S);
+              const float2 w = top ? combine_groups_fast<ND, (ND > 4 ? 4 : ND - 1)>(S)
+                                   : combine_groups_fast<ND - 1, (ND > 4 ? 3 : ND - 2)>(S);
               const float fv = Fv[c0 + e];
               res[c0 + e] = df_add(res[c0 + e], make_float2(w.x * fu * fv, w.y * fu * fv));
             }
@@ -1957,7 +1923,7 @@ oz_gram_tc_ring_kernel(int64_t n, int p, int q, const float2* __restrict__ U, co
     }
     __syncthreads();
     if (worker && top) {
-      float2* out = part + ((size_t)blockIdx.x * gridDim.y + blockIdx.y) * 4096;
+      float2* out = part + (size_t)blockIdx.x * 4096;
 #pragma unroll
       for (int e = 0; e < 16; ++e) out[arow * 64 + cb + e] = df_add(res[e], st[arow * 65 + cb + e]);
     }
@@ -2567,26 +2533,20 @@ gsi_status oz_gram(int64_t n, int p, int q, const float2* U, const float2* V, bo
   // 16-byte copies need even row lengths and 16-byte aligned bases
   const bool vec16 = ((p | q) & 1) == 0 && ((uintptr_t)U & 15) == 0 && ((uintptr_t)V & 15) == 0;
   bool tri = false;  // symmetric Gram from full upper-triangle blocks
-  // 16-byte aligned blocks of even width: the kernel with the maxima warps
-  // (it counts its sub-chunks in 32 bits: n < 2^34). Its maxima warps copy
-  // a batch's rows in one piece where the block spans whole rows (p, q <=
-  // 64); 64-column blocks of wider matrices take one copy per row, where the
-  // whole-chunk kernel is as fast for 7 digits, so those stay with it.
-  const bool ring = tp != 1 && vec16 && n < ((int64_t)1 << 34) && ((p <= 64 && q <= 64) || nd == 3);
+  // 16-byte aligned blocks of even width and at most 64 columns: the kernel
+  // with the maxima warps (it counts its sub-chunks in 32 bits: n < 2^34),
+  // which copy a batch's whole rows in one piece; wider blocks, where a
+  // 64-column block takes one copy per row, stay with the whole-chunk kernel,
+  // which is as fast there.
+  const bool ring = tp != 1 && nd == ND && vec16 && n < ((int64_t)1 << 34) && p <= 64 && q <= 64;
   if (ring) {
-    const bool one = p <= 64 && q <= 64;
-    tri = sym && !one;
-    const bool ksym = sym && one;
-    const size_t tsm = oz_gram_tc_ring_smem(ksym, nd);
-    // (3 digits: always full chunks, whose exponents set those products' errors)
-    const int most = ksym ? TrGeom<true>::EC : TrGeom<false>::EC;
-    const int ec = nd == ND ? gram_chunk_rows(n, ns, ksym ? TrGeom<true>::SK : TrGeom<false>::SK, most) : most;
-    auto kern = ec == most ? (ksym ? oz_gram_tc_ring_kernel<true, ND, true> : oz_gram_tc_ring_kernel<false, ND, true>)
-                           : (ksym ? oz_gram_tc_ring_kernel<true, ND, false> : oz_gram_tc_ring_kernel<false, ND, false>);
-    if (nd == 3) kern = ksym ? oz_gram_tc_ring_kernel<true, 3, true> : oz_gram_tc_ring_kernel<false, 3, true>;
+    const size_t tsm = oz_gram_tc_ring_smem(sym);
+    const int most = sym ? TrGeom<true>::EC : TrGeom<false>::EC;
+    const int ec = gram_chunk_rows(n, ns, sym ? TrGeom<true>::SK : TrGeom<false>::SK, most);
+    auto kern = ec == most ? (sym ? oz_gram_tc_ring_kernel<true, true> : oz_gram_tc_ring_kernel<false, true>)
+                           : (sym ? oz_gram_tc_ring_kernel<true, false> : oz_gram_tc_ring_kernel<false, false>);
     GSI_CUDA_TRY(ensure_dyn_smem((const void*)kern, (int)tsm));
-    kern<<<dim3(ns, one ? 1 : nblk), TR_THREADS, tsm, st>>>(n, p, q, U, V, scratch, one ? 1 : nbj,
-                                                            tri ? 1 : 0, ec);
+    kern<<<ns, TR_THREADS, tsm, st>>>(n, p, q, U, V, scratch, ec);
     GSI_LAUNCH_CHECK();
   } else if (nd == ND && p <= 64 && q <= 64 && tp != 1) {
     // one 64 x 64 output block; every partial entry is written

@@ -39,6 +39,7 @@ template <int NT_, int CL_, int TR_, int TC_, int NCG_, int SEG_, int AW_, int I
 struct PpCfg {
   static constexpr int NT = NT_, CL = CL_, TR = TR_, TC = TC_, NCG = NCG_, NC = NC_;
   static constexpr int NG = NT / CL, RG = NG / NCG;
+  static_assert(RG <= 16, "pp_jac_bytes");
   static constexpr int SEG = SEG_, AW = AW_, IL = IL_;
   static_assert(SEG == 64 || (32 / SEG) * AW * IL * 2 >= SEG, "every pair of rotations has a lane");
   static_assert(SEG == 64 ? NC > 1 : NC > 1 || NT / 32 > AW, "V needs warps (or ranks) of its own");
@@ -52,6 +53,7 @@ struct PpMat {  // a p x p input: df64, or float64 (then symmetrised where sym i
 
 struct PpArgs {
   int mode, p;
+  int want_phi;  // mode 0: out[1] = phi(t)
   int scale_b;  // mode 3, float64 B: divided by a power of two near max |B| (B may leave float32's range)
   // B = D^T D (modes 0, 3) or the matrix itself (modes 1, 2); C = X^T A X,
   // Gam = D^T W, Z = D^T R, XX = X^T X; XD = X^T D, or null pointers: formed
@@ -70,6 +72,7 @@ constexpr int PP_CTL = 1024 + 64;  // float2: control words, then the partial do
 
 struct PpSh {  // small tables, shared memory
   double al[128], be[128], ga[128], ze[128], sv[128];
+  float2 alf[128], bef[128], gaf[128], zef[128];  // the same in df64
   float2 lam[2][130];
   float2 cs[64];
   float red[32];
@@ -105,7 +108,17 @@ struct PpCtx {
 __device__ __forceinline__ float* pp_sf(int o) { return reinterpret_cast<float*>(pp_sm) + o; }
 __device__ __forceinline__ float2* pp_s2(int o) { return reinterpret_cast<float2*>(pp_sm) + o; }
 
-__host__ __device__ inline int pp_lda(int p) { return (p + 31) / 32 * 32; }
+// row stride of the Jacobi matrices for m columns: rows and columns of a
+// round's blocks advance together over the lanes, so that for m > 32 a
+// multiple of 32 spreads them over the banks, and for the two or four
+// segments of a smaller m an odd stride
+__host__ __device__ inline int pp_lda(int m) { return m <= 32 ? m + 1 : (m + 31) / 32 * 32; }
+// bytes of a Jacobi matrix; the first also holds the dot products' partial
+// sums (up to 16 row groups of p df64 values, pp_diag)
+__host__ __device__ inline int pp_jac_bytes(int p) {
+  const int m = (p + 1) & ~1, a = m * pp_lda(m) * (int)sizeof(float), b = 16 * p * (int)sizeof(float2);
+  return ((a > b ? a : b) + 15) & ~15;
+}
 __host__ __device__ inline size_t pp_al(size_t b) { return (b + 15) & ~(size_t)15; }
 __host__ __device__ inline size_t pp_log_len(int p) {  // rotations of a sweep
   const size_t m = (p + 1) & ~1;
@@ -115,8 +128,7 @@ __host__ __device__ inline size_t pp_log_len(int p) {  // rotations of a sweep
 // (two buffers) and V, two logs; NC > 1: staged Y (V or a log share its
 // space), strip of X, A or a float32 copy of E, A's second buffer (p <= 64)
 inline size_t pp_smem(int p, int nc) {
-  const size_t ld = p | 1, m = (p + 1) & ~1, lda = pp_lda((int)m);
-  const size_t jac = pp_al(m * lda * sizeof(float));
+  const size_t ld = p | 1, jac = pp_jac_bytes(p);
   const size_t sh = pp_al(sizeof(PpSh));
   if (nc == 1)
     return sh + 4 * pp_al((size_t)p * ld * sizeof(float2)) + 3 * jac + 2 * pp_al(pp_log_len(p) * sizeof(float2));
@@ -150,7 +162,7 @@ __device__ __forceinline__ PpCtx<P> pp_ctx(int p, float2* gws) {
     cur += (bytes + 15) & ~15;
     return r;
   };
-  const int jac = m * c.lda * 4, len = (m - 1) * (m / 2);
+  const int jac = pp_jac_bytes(p), len = (m - 1) * (m / 2);
   if constexpr (P::NC == 1) {
     c.rank = 0;
     c.r0 = 0;
@@ -356,28 +368,34 @@ __device__ __forceinline__ void pp_pair(int r, int k, int m1, int& a, int& b) {
   }
 }
 
-// The angle of one rotation: t = tan, (c, s). DELTA: pivot f and the df64
-// diagonal entries la, lb; otherwise the diagonal is la.x, lb.x. IEEE
-// division and square root for DELTA, whose angles' errors are what a pass
-// leaves behind.
+__device__ __forceinline__ float pp_rsqrt(float x) {  // 1/sqrt(x), one Newton step on the approximation
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y * __fmaf_rn(-0.5f * x, y * y, 1.5f);
+}
+
+// The rotation of a pivot f with diagonal entries la, lb (DELTA: df64;
+// otherwise la.x, lb.x): returns (c, s), t = s / c. From cos 2 theta =
+// |d| / sqrt(d^2 + 4 f^2), d = lb - la: c^2 = (1 + cos 2 theta) / 2 and
+// s = f / (sqrt(d^2 + 4 f^2) c), a chain of two reciprocal roots (a division,
+// a root and a reciprocal root took half of a round).
 template <bool DELTA>
 __device__ __forceinline__ float2 pp_angle(float f, float2 la, float2 lb, float& t) {
-  const float b2 = 2.f * f;
-  t = 0.f;
+  float d;
   if (DELTA) {
     const float2 dd = df_add(lb, pp_neg(la));
-    const float d = __fadd_rn(dd.x, dd.y);
-    const float q = __fsqrt_rn(__fmaf_rn(d, d, b2 * b2));
-    if (q > 0.f) t = __fdiv_rn(d >= 0.f ? b2 : -b2, fabsf(d) + q);
+    d = __fadd_rn(dd.x, dd.y);
   } else {
-    const float d = lb.x - la.x;
-    const float q2 = __fmaf_rn(d, d, b2 * b2);
-    if (q2 > 0.f) t = __fdividef(d >= 0.f ? b2 : -b2, fabsf(d) + q2 * rsqrtf(q2));
+    d = lb.x - la.x;
   }
-  const float q = __fmaf_rn(t, t, 1.f);
-  float cc = rsqrtf(q);
-  cc = cc * __fmaf_rn(-0.5f * q, cc * cc, 1.5f);  // one Newton step: c^2 + s^2 = 1 to rounding
-  return make_float2(cc, t * cc);
+  const float b2 = 2.f * f, q2 = __fmaf_rn(d, d, b2 * b2);
+  const bool rot = q2 >= 1.17549435e-38f;  // else d and f are zero, or far below the matrix's rounding
+  const float h = pp_rsqrt(rot ? q2 : 1.f);
+  const float c2 = __fmaf_rn(0.5f * fabsf(d), h, 0.5f);
+  const float rc = pp_rsqrt(c2);
+  const float sn = (d >= 0.f ? f : -f) * h * rc;
+  t = rot ? sn * rc : 0.f;
+  return rot ? make_float2(c2 * rc, sn) : make_float2(1.f, 0.f);
 }
 
 // 2 x 2 block z = J_k^T x J_l
@@ -402,8 +420,8 @@ __device__ void pp_sweep(const PpCtx<P>& c, int Ao, int Ano, int lp, int log) {
   const int lane = c.tid & 31, w = c.tid >> 5, seg = lane / SEG, k = lane % SEG;
   const bool own = k < half, lead = own && w == 0 && seg == 0;
   int a = own ? k : 0, b = own ? (k == 0 ? m1 : m1 - k) : 0;  // round 0's pair
-  int src[P::IL];
-  bool live[P::IL];
+  int src[P::IL], al[P::IL], bl[P::IL];  // the partner's lane and pair
+  bool live[P::IL], l0[P::IL];
 #pragma unroll
   for (int z = 0; z < P::IL; ++z) {
     const int d = 1 + ((z * P::AW + w) * NSEG + seg);
@@ -411,6 +429,9 @@ __device__ void pp_sweep(const PpCtx<P>& c, int Ao, int Ano, int lp, int log) {
     int l = k + d;
     l -= l >= half ? half : 0;
     src[z] = live[z] ? seg * SEG + l : lane;
+    al[z] = live[z] ? l : 0;
+    l0[z] = l == 0;
+    bl[z] = live[z] ? (l == 0 ? m1 : m1 - l) : 0;
   }
   for (int r = 0; r < m1; ++r) {
     float *const A = pp_sf(Ao), *const An = pp_sf(Ano);
@@ -426,11 +447,8 @@ __device__ void pp_sweep(const PpCtx<P>& c, int Ao, int Ano, int lp, int log) {
       lb.x = A[rb + b];
     }
     float x[P::IL][4];
-    int al[P::IL], bl[P::IL];
 #pragma unroll
     for (int z = 0; z < P::IL; ++z) {
-      al[z] = __shfl_sync(0xffffffffu, a, src[z]);
-      bl[z] = __shfl_sync(0xffffffffu, b, src[z]);
       if (live[z]) {
         x[z][0] = A[ra + al[z]];
         x[z][1] = A[ra + bl[z]];
@@ -475,6 +493,11 @@ __device__ void pp_sweep(const PpCtx<P>& c, int Ao, int Ano, int lp, int log) {
     // both indices of a pair advance by one modulo m - 1 (slot 0 keeps m - 1)
     a = a + 1 == m1 ? 0 : a + 1;
     if (k != 0) b = b + 1 == m1 ? 0 : b + 1;
+#pragma unroll
+    for (int z = 0; z < P::IL; ++z) {
+      al[z] = al[z] + 1 == m1 ? 0 : al[z] + 1;
+      if (!l0[z]) bl[z] = bl[z] + 1 == m1 ? 0 : bl[z] + 1;
+    }
     const int u = Ao;
     Ao = Ano;
     Ano = u;
@@ -569,21 +592,39 @@ __device__ void pp_apply_log(int p, int Vo, int ldv, int rows, int logo, int w, 
   constexpr int SEG = P::SEG > 32 ? 32 : P::SEG, NSEG = 32 / SEG, LL = P::SEG / SEG;  // rotations a lane
   const int m = (p + 1) & ~1, half = m / 2, m1 = m - 1;
   const int lane = threadIdx.x & 31, seg = lane / SEG;
+  int a[LL], b[LL];
+#pragma unroll
+  for (int z = 0; z < LL; ++z) {
+    const int l = lane % SEG + z * SEG;
+    a[z] = l;
+    b[z] = l == 0 ? m1 : m1 - l;
+  }
   for (int r = 0; r < m1; ++r) {
 #pragma unroll
     for (int z = 0; z < LL; ++z) {
       const int l = lane % SEG + z * SEG;
       if (l < half) {
-        int a, b;
-        pp_pair(r, l, m1, a, b);
         const float2 cs = log[r * half + l];
-#pragma unroll 4
-        for (int row = w * NSEG + seg; row < rows; row += nw * NSEG) {
-          float* const v = V + row * ldv;
-          const float x = v[a], y = v[b];
-          v[a] = cs.x * x - cs.y * y;
-          v[b] = cs.y * x + cs.x * y;
+        // four rows in flight: their loads before any of their stores
+        for (int row = w * NSEG + seg; row < rows; row += 4 * nw * NSEG) {
+          float x[4], y[4];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int rr = min(row + u * nw * NSEG, rows - 1);
+            x[u] = V[rr * ldv + a[z]];
+            y[u] = V[rr * ldv + b[z]];
+          }
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            const int rr = row + u * nw * NSEG;
+            if (rr < rows) {
+              V[rr * ldv + a[z]] = cs.x * x[u] - cs.y * y[u];
+              V[rr * ldv + b[z]] = cs.y * x[u] + cs.x * y[u];
+            }
+          }
         }
+        a[z] = a[z] + 1 == m1 ? 0 : a[z] + 1;
+        if (l != 0) b[z] = b[z] + 1 == m1 ? 0 : b[z] + 1;
       }
     }
     __syncwarp();
@@ -996,75 +1037,95 @@ static __device__ __noinline__ double pp_step_length_f64(int p, int* ev) {
   return get_mu_warp(p, sh->al, sh->be, sh->ga, sh->ze, ev);
 }
 
+__device__ __forceinline__ float2 df_sqrt(float2 a) {  // a >= 0
+  if (!(a.x > 0.f)) return make_float2(0.f, 0.f);
+  const float y = __fsqrt_rn(a.x), y2 = __fmul_rn(y, y);
+  const float2 r = df_add(a, make_float2(-y2, -__fmaf_rn(y, y, -y2)));
+  return fast_two_sum(y, __fdiv_rn(__fadd_rn(r.x, r.y), 2.f * y));
+}
+__device__ __forceinline__ float2 df_scale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
+// a 2^e for |e| beyond a float's exponent
+__device__ __forceinline__ float2 df_ldexp(float2 a, int e) { return make_float2(ldexpf(a.x, e), ldexpf(a.y, e)); }
+
 // The step of get_mu_warp (alg3.cuh: bracket from the branch roots xi_i, the
-// right end doubled from xi_min, Brent on phi'), one warp. The bracket ends
-// come in float64; the evaluations of the search run in df64 on a scaled
-// model (a float64 evaluation is a chain of ~25 operations on a pipe with
-// 1/64 of the float32 rate, ~5,000 cycles an evaluation); the root is then
-// corrected by one Newton step from a float64 evaluation of phi', which
-// leaves it as accurate as a search in float64. Where the scaled model
-// leaves float32's range or the Newton step is not small, the float64
-// search runs instead.
+// right end doubled from xi_min, Brent on phi'), one warp. The search runs in
+// df64 on a model scaled by powers of two (a float64 evaluation is a chain of
+// ~25 operations on a pipe with 1/64 of the float32 rate, ~5,000 cycles an
+// evaluation); the root is then corrected by one Newton step from a float64
+// evaluation of phi', which leaves it as accurate as a search in float64.
+// Where the scaled model leaves float32's range or the Newton step is not
+// small, the float64 search runs instead.
 template <int MC>
 __device__ __noinline__ double pp_step_length(int p, int* ev_out) {
-  const double *const al = pp_sh()->al, *const be = pp_sh()->be, *const ga = pp_sh()->ga, *const ze = pp_sh()->ze;
+  const PpSh* const sh = pp_sh();
   int evs = 0, *const ev = &evs;
   const int lane = threadIdx.x & 31;
-  double sb = 0.0, bmax = 0.0, zmax = 0.0, dmax = 0.0;
-  for (int i = lane; i < p; i += 32) {
-    sb += be[i];
-    bmax = fmax(bmax, be[i]);
-    zmax = fmax(zmax, fabs(ze[i]));
-    dmax = fmax(dmax, fabs(ga[i] - al[i] * be[i]));
-  }
-  sb = warp_sum(sb);
-  double xmin = INFINITY, xmax = -INFINITY;
-  int cnt = 0;
-  for (int i = lane; i < p; i += 32) {
-    const double b = be[i], z = ze[i];
-    if (!(b > ALG3_EPS * sb) || !(z > 0.0)) continue;
-    const double d = ga[i] - al[i] * b;
-    const double disc = sqrt(d * d + 4.0 * b * z * z);
-    const double xi = (d < 0.0) ? 2.0 * z / (-d + disc) : (d + disc) / (2.0 * b * z);
-    xmin = fmin(xmin, xi);
-    xmax = fmax(xmax, xi);
-    ++cnt;
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    xmin = fmin(xmin, __shfl_xor_sync(0xffffffffu, xmin, o));
-    xmax = fmax(xmax, __shfl_xor_sync(0xffffffffu, xmax, o));
-    bmax = fmax(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
-    zmax = fmax(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
-    dmax = fmax(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
-    cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-  }
-  *ev_out = 0;
-  if (cnt == 0) return 0.0;
-  // t = T tau with T = min(1/sqrt(max beta), max|zeta| / max|delta|), values
-  // over Sz = max|zeta|, each rounded down to a power of two
-  double T = 1.0 / sqrt(bmax);
-  if (dmax > 0.0) T = fmin(T, zmax / dmax);
-  const int eT = T > 0.0 && isfinite(T) ? ilogb(T) : 1 << 20, eZ = zmax > 0.0 && isfinite(zmax) ? ilogb(zmax) : 1 << 20;
-  const double lo_s = abs(eT) < 900 ? scalbn(xmin, -eT) : 0.0;
-  const bool scaled = abs(eT) < 900 && abs(eZ) < 900 && lo_s > 1e-9 && lo_s < 1e9;
-  if (!scaled) return pp_step_length_f64(p, ev_out);
   PpModel<MC> md;
+  float sb = 0.f, bmax = 0.f, zmax = 0.f, dmax = 0.f;
   md.cnt = 0;
 #pragma unroll
   for (int u = 0; u < MC; ++u) {
     const int i = lane + 32 * u;
+    md.z[u] = md.dl[u] = md.b[u] = make_float2(0.f, 0.f);
     if (i < p) {
-      const double b = scalbn(be[i], 2 * eT), z = scalbn(ze[i], -eZ);
-      md.z[u] = df_from_double(z);
-      md.b[u] = df_from_double(b);
-      md.bz[u] = df_from_double(b * z);
-      md.dl[u] = df_from_double(scalbn(ga[i] - al[i] * be[i], eT - eZ));
+      md.b[u] = sh->bef[i];
+      md.z[u] = sh->zef[i];
+      md.dl[u] = df_add(sh->gaf[i], pp_neg(df_mul(sh->alf[i], md.b[u])));
       md.cnt = u + 1;
+      sb += md.b[u].x;
+      bmax = fmaxf(bmax, md.b[u].x);
+      zmax = fmaxf(zmax, fabsf(md.z[u].x));
+      dmax = fmaxf(dmax, fabsf(md.dl[u].x));
     }
   }
-  const double hmax = scalbn(xmax, -eT);
-  const float2 xmn = df_from_double(lo_s);
-  const float2 xmx = hmax < 1e30 ? df_from_double(hmax) : make_float2(1e30f, 0.f);
+  for (int o = 16; o > 0; o >>= 1) {
+    sb += __shfl_xor_sync(0xffffffffu, sb, o);
+    bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
+    zmax = fmaxf(zmax, __shfl_xor_sync(0xffffffffu, zmax, o));
+    dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+  }
+  sb = __shfl_sync(0xffffffffu, sb, 0);
+  // t = T tau with T = min(1/sqrt(max beta), max|zeta| / max|delta|), values
+  // over Sz = max|zeta|, each rounded down to a power of two
+  const bool range = bmax > 1e-36f && bmax < 1e36f && zmax > 1e-36f && zmax < 1e36f && dmax < 1e36f;
+  int eT = 0, eZ = 0;
+  if (range) {
+    eZ = ilogbf(zmax);
+    eT = -((ilogbf(bmax) + 2) / 2);
+    if (dmax > 0.f) eT = min(eT, eZ - ilogbf(dmax));
+  }
+  // (alpha and gamma enter through delta only, so that an empty bracket and a
+  // model without positive zeta are the same here as in the float64 search)
+  float2 xmn = make_float2(INFINITY, 0.f), xmx = make_float2(0.f, 0.f);
+  bool any = false;
+#pragma unroll
+  for (int u = 0; u < MC; ++u) {
+    const bool use = u < md.cnt && md.b[u].x > (float)ALG3_EPS * sb && md.z[u].x > 0.f;
+    any = any || use;
+    md.b[u] = df_ldexp(md.b[u], 2 * eT);
+    md.z[u] = df_ldexp(md.z[u], -eZ);
+    md.dl[u] = df_ldexp(md.dl[u], eT - eZ);
+    md.bz[u] = df_mul(md.b[u], md.z[u]);
+    if (use) {
+      const float2 d = md.dl[u], z = md.z[u];
+      const float2 disc = df_sqrt(df_add(df_mul(d, d), df_scale(df_mul(md.bz[u], z), 4.f)));
+      float2 xi;
+      if (d.x < 0.f) xi = df_div(df_scale(z, 2.f), df_add(disc, pp_neg(d)));
+      else xi = df_div(df_add(d, disc), df_scale(md.bz[u], 2.f));
+      if (!(xi.x < 1e30f)) xi = make_float2(1e30f, 0.f);  // past the largest step searched, or 2 b z underflowed
+      if (df_less(xi, xmn)) xmn = xi;
+      if (df_less(xmx, xi)) xmx = xi;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const float2 lo = make_float2(__shfl_xor_sync(0xffffffffu, xmn.x, o), __shfl_xor_sync(0xffffffffu, xmn.y, o));
+    const float2 hi = make_float2(__shfl_xor_sync(0xffffffffu, xmx.x, o), __shfl_xor_sync(0xffffffffu, xmx.y, o));
+    if (df_less(lo, xmn)) xmn = lo;
+    if (df_less(xmx, hi)) xmx = hi;
+  }
+  *ev_out = 0;
+  if (!range || !__any_sync(0xffffffffu, any) || !(xmn.x > 1e-9f) || !(xmn.x < 1e9f))
+    return pp_step_length_f64(p, ev_out);
   const float2 fa = pp_dphi(md, xmn);
   ++*ev;
   float2 lo, flo, hi, fhi;
@@ -1072,10 +1133,7 @@ __device__ __noinline__ double pp_step_length(int p, int* ev_out) {
     lo = make_float2(0.f, 0.f);
     flo = pp_dphi(md, lo);
     ++*ev;
-    if (flo.x >= 0.f) {
-      *ev_out = evs;
-      return 0.0;
-    }
+    if (flo.x >= 0.f) return pp_step_length_f64(p, ev_out);
     hi = xmn;
     fhi = fa;
   } else {
@@ -1107,19 +1165,20 @@ __device__ __noinline__ double pp_step_length(int p, int* ev_out) {
     }
   for (int o = 16; o > 0; o >>= 1) sl += __shfl_xor_sync(0xffffffffu, sl, o);
   sl = -__shfl_sync(0xffffffffu, sl, 0);
-  const double f = dphi_warp(t, p, al, be, ga, ze);
+  const double f = dphi_warp(t, p, sh->al, sh->be, sh->ga, sh->ze);
   ++*ev;
-  const double corr = scalbn(f / (double)sl, eT - eZ);
-  if (!(fabs(corr) <= 1e-9 * t)) return pp_step_length_f64(p, ev_out);
+  // phi' over Sz and the slope are of order one; the quotient is the step in tau
+  const float corr = (float)scalbn(f, -eZ) / sl;
+  if (!(fabsf(corr) <= 1e-9f * tau.x)) return pp_step_length_f64(p, ev_out);
   *ev_out = evs;
-  return t - corr;
+  return t - scalbn((double)corr, eT);
 }
 
 // The diagonal of V^T G V (G in c.Ud, V in c.Vd) into d (shared memory of
 // every CTA). The row groups' sums pass through c.Af, the ranks' through the
 // control words. Synchronised on exit.
 template <class P>
-__device__ void pp_diag(const PpCtx<P>& c, double* d) {
+__device__ void pp_diag(const PpCtx<P>& c, double* d, float2* df) {
   const int p = c.p;
   float2* const part = pp_s2(c.Af / 2);
   pp_mm(c, c.Ud, false, c.Vd, false, -1, -1, 0.f, c.Vd, c.Af / 2);
@@ -1127,8 +1186,10 @@ __device__ void pp_diag(const PpCtx<P>& c, double* d) {
   for (int j = c.tid; j < p; j += P::NT) {
     float2 s = part[j];
     for (int g = 1; g < P::RG; ++g) s = df_add(s, part[g * p + j]);
-    if constexpr (P::NC == 1) d[j] = df_to_double(s);
-    else c.gws[c.ctl + 64 + c.rank * 128 + j] = s;
+    if constexpr (P::NC == 1) {
+      d[j] = df_to_double(s);
+      df[j] = s;
+    } else c.gws[c.ctl + 64 + c.rank * 128 + j] = s;
   }
   pp_sync<P>();
   if constexpr (P::NC > 1) {
@@ -1137,6 +1198,7 @@ __device__ void pp_diag(const PpCtx<P>& c, double* d) {
       float2 s = __ldcg(pd);
       for (int g = 1; g < P::NC; ++g) s = df_add(s, __ldcg(pd + g * 128));
       d[j] = df_to_double(s);
+      df[j] = s;
     }
     pp_sync<P>();
   }
@@ -1157,7 +1219,11 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
   auto same = [](int, int, float2 v) { return v; };
   if (a.mode == 4) {
     pp_each(c, [&](int i, int j) { c.mat(c.Vd)[i * c.ld + j] = a.eig[i * p + j]; });
-    for (int i = c.tid; i < p; i += P::NT) sh->be[i] = fmax(df_to_double(a.eig[p * p + i]), 0.0);
+    for (int i = c.tid; i < p; i += P::NT) {
+      const float2 b = a.eig[p * p + i];
+      sh->bef[i] = b.x > 0.f ? b : make_float2(0.f, 0.f);
+      sh->be[i] = df_to_double(sh->bef[i]);
+    }
     __syncthreads();
   } else {
     if (a.scale_b) {
@@ -1175,8 +1241,11 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
     pp_sync<P>();
     pp_eig(c, a.mode != 1, out + 8);
     if (a.mode == 0) {
-      for (int i = c.tid; i < p; i += P::NT)
-        sh->be[i] = fmax(df_to_double(c.ldm(c.Ud + i * c.ld + i)), 0.0);
+      for (int i = c.tid; i < p; i += P::NT) {
+        const float2 b = c.ldm(c.Ud + i * c.ld + i);
+        sh->bef[i] = b.x > 0.f ? b : make_float2(0.f, 0.f);
+        sh->be[i] = df_to_double(sh->bef[i]);
+      }
       __syncthreads();
     }
   }
@@ -1209,13 +1278,13 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
   pp_sync<P>();  // every rank has read the diagonal from Ud
   pp_load(c, a.C, c.Ud, same);
   pp_sync<P>();
-  pp_diag(c, sh->al);
+  pp_diag(c, sh->al, sh->alf);
   pp_load(c, a.Gam, c.Ud, same);
   pp_sync<P>();
-  pp_diag(c, sh->ga);
+  pp_diag(c, sh->ga, sh->gaf);
   pp_load(c, a.Z, c.Ud, same);
   pp_sync<P>();
-  pp_diag(c, sh->ze);
+  pp_diag(c, sh->ze, sh->zef);
   // X^T D = (I - X^T X)(C + beta K) into Bd
   if (a.XD.f || a.XD.d) {
     pp_load(c, a.XD, c.Bd, same);
@@ -1240,17 +1309,22 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
     if (c.rank == 0) {
       int ev = 0;
       const double t = pp_step_length<(P::CL * P::TC * P::NCG + 31) / 32>(p, &ev);
-      double bmax = 0.0;
-      for (int i = c.tid; i < p; i += 32) bmax = fmax(bmax, sh->be[i]);
-      for (int o = 16; o > 0; o >>= 1) bmax = fmax(bmax, __shfl_xor_sync(0xffffffffu, bmax, o));
-      const double ph = phi_model_warp(t, p, sh->al, sh->be, sh->ga, sh->ze);
+      float2 bmax = make_float2(0.f, 0.f);
+      for (int i = c.tid; i < p; i += 32)
+        if (df_less(bmax, sh->bef[i])) bmax = sh->bef[i];
+      for (int o = 16; o > 0; o >>= 1) {
+        const float2 v = make_float2(__shfl_xor_sync(0xffffffffu, bmax.x, o), __shfl_xor_sync(0xffffffffu, bmax.y, o));
+        if (df_less(bmax, v)) bmax = v;
+      }
+      // the model's value is reported to direct callers only
+      const double ph = a.mode == 0 && a.want_phi ? phi_model_warp(t, p, sh->al, sh->be, sh->ga, sh->ze) : 0.0;
       if (c.tid == 0) {
         sh->t = t;
         if (P::NC > 1) *reinterpret_cast<double*>(c.gws + c.ctl + 2) = t;
         out[0] = t;
         out[1] = ph;
         out[2] = (double)ev;
-        out[4] = bmax;
+        out[4] = df_to_double(bmax);
       }
     }
   }

@@ -12,7 +12,7 @@ namespace gsi {
 namespace {
 
 template <class P>
-__global__ void __launch_bounds__(P::NT) pp_kernel(PpArgs a) {
+__global__ void __launch_bounds__(P::NT, 1) pp_kernel(PpArgs a) {
   PpCtx<P> c = pp_ctx<P>(a.p, a.gws);
   pp_body<P>(a, c);
 }
