@@ -616,7 +616,7 @@ __global__ void __launch_bounds__(BT) b_retract_kernel(BDev d, int32_t mode) {
 // mode 2 (F_START): Rayleigh-Ritz, C' = U diag(theta) U^T, theta descending,
 //   M = U.
 using BPp16 = PpCfg<BS, 16, 1, 1, 1, 8, 1, 1, 1>;
-using BPp32 = PpCfg<BS, 32, 4, 1, 1, 16, 2, 2, 1>;
+using BPp32 = PpCfg<BS, 32, 4, 1, 1, 16, 4, 1, 1>;
 
 __global__ void __launch_bounds__(BS, 2) b_small_kernel(BDev d, int32_t mode) {
   const int i = blockIdx.x;

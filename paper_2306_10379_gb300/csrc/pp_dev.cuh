@@ -32,7 +32,8 @@ namespace gsi {
 
 // Block shape: NT threads; a group of CL lanes covers TC CL columns of a
 // product (NCG such column blocks), the groups its rows, TR each. Jacobi:
-// AW warps work on A; a segment of SEG lanes holds one rotation per lane
+// AW warps work on A (p = 64: 687 cycles a round with 16 warps of one block
+// a lane, 934 with 8 of two; p = 32: 689 with 4, 779 with 2); a segment of SEG lanes holds one rotation per lane
 // (SEG = 64: p > 64), IL 2 x 2 blocks a lane: the blocks of rotations k and
 // k + d, 1 <= d <= half / 2, half <= SEG rotations a round.
 template <int NT_, int CL_, int TR_, int TC_, int NCG_, int SEG_, int AW_, int IL_, int NC_>
@@ -42,7 +43,7 @@ struct PpCfg {
   static_assert(RG <= 16, "pp_jac_bytes");
   static constexpr int SEG = SEG_, AW = AW_, IL = IL_;
   static_assert(SEG == 64 || (32 / SEG) * AW * IL * 2 >= SEG, "every pair of rotations has a lane");
-  static_assert(SEG == 64 ? NC > 1 : NC > 1 || NT / 32 > AW, "V needs warps (or ranks) of its own");
+  static_assert(NC > 1 ? NT / 32 >= AW : NT / 32 > AW, "V needs warps (or ranks) of its own");
 };
 
 struct PpMat {  // a p x p input: df64, or float64 (then symmetrised where sym is set)
@@ -108,11 +109,11 @@ struct PpCtx {
 __device__ __forceinline__ float* pp_sf(int o) { return reinterpret_cast<float*>(pp_sm) + o; }
 __device__ __forceinline__ float2* pp_s2(int o) { return reinterpret_cast<float2*>(pp_sm) + o; }
 
-// row stride of the Jacobi matrices for m columns: rows and columns of a
-// round's blocks advance together over the lanes, so that for m > 32 a
-// multiple of 32 spreads them over the banks, and for the two or four
-// segments of a smaller m an odd stride
-__host__ __device__ inline int pp_lda(int m) { return m <= 32 ? m + 1 : (m + 31) / 32 * 32; }
+// Row stride of the Jacobi matrices for m (even) columns. Over the lanes a row
+// index grows by one and a column index grows or falls by one, so the banks
+// of a round's accesses step by lda + 1 or lda - 1: both are odd for the even
+// m itself, and no two lanes of a segment meet.
+__host__ __device__ inline int pp_lda(int m) { return m; }
 // bytes of a Jacobi matrix; the first also holds the dot products' partial
 // sums (up to 16 row groups of p df64 values, pp_diag)
 __host__ __device__ inline int pp_jac_bytes(int p) {

@@ -48,9 +48,9 @@ size_t small_df_scratch_bytes(int p) { return pp_gws_bytes(p); }
 gsi_status small_step_df(const PpArgs& a, bool cluster, cudaStream_t st) {
   if (a.p < 1 || a.p > 128 || ((a.mode == 3 || a.mode == 4) && !a.eig)) return GSI_ERR_ARG;
   if (a.p <= 16) return launch<PpCfg<128, 16, 2, 1, 1, 8, 1, 1, 1>>(a, st);
-  if (a.p <= 32) return launch<PpCfg<256, 32, 4, 1, 1, 16, 2, 2, 1>>(a, st);
+  if (a.p <= 32) return launch<PpCfg<256, 32, 4, 1, 1, 16, 4, 1, 1>>(a, st);
   if (a.p > 64) return launch<PpCfg<512, 32, 2, 2, 2, 64, 16, 4, 8>>(a, st);
-  if (cluster) return launch<PpCfg<512, 32, 1, 1, 2, 32, 8, 2, 8>>(a, st);
+  if (cluster) return launch<PpCfg<512, 32, 1, 1, 2, 32, 16, 1, 8>>(a, st);
   return launch<PpCfg<512, 32, 4, 2, 1, 32, 8, 2, 1>>(a, st);
 }
 
