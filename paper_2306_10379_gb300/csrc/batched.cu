@@ -12,8 +12,7 @@
 // SpMM, retraction) is done by persistent grid-stride kernels over that table;
 // each tile is skipped unless its problem's flags select it. Gram products
 // leave float64 partial sums per tile, summed per problem in tile order
-// (deterministic). The p x p step runs one thread block per problem in
-// float64. Small control kernels (one thread per problem) take the decisions
+// (deterministic). The p x p step runs one thread block per problem. Small control kernels (one thread per problem) take the decisions
 // of the single-problem iteration: stop test, Polak-Ribiere beta, restart,
 // explicit recompute of AX, step counting.
 //
@@ -42,7 +41,6 @@ namespace {
 constexpr int BT = 256;    // threads of the tile kernels
 constexpr int BS = 256;    // threads of the per-problem p x p kernel
 constexpr int PMAX = 32;   // largest block width of a batched problem
-constexpr int RC = 32;     // rows per staged chunk in the Gram kernel
 constexpr int NG = 4;      // Gram products per tile slot
 constexpr int kTileMin = 64;  // fewest rows of a tile
 
@@ -146,116 +144,260 @@ __device__ float bmaxf(float v, float* red) {
   return s;
 }
 
+// ---- sums against an offset ---------------------------------------------------
+// A sum of df64 products whose partial sums are bounded beforehand by 2^k
+// starts at sigma = 1.5 * 2^k instead of 0. Every partial sum S then lies in
+// [2^(k-1), 2.5 * 2^k], so S_new - S is exact, the fma that made S_new has
+// rounded the product to a multiple of S's ulp, and a second fma returns what
+// that rounding left: product and accumulation take 6 float32 operations
+// instead of the 12 of TwoProd + TwoSum (bmac). What the rounding leaves is
+// at most 2^(k-23), and its sum e keeps a further 24 bits. The bound is
+// Hoelder's, max |a| times sum |b|, over few rows: the error grows with their
+// number to the power 3/2, that of all rows with the square root.
+constexpr float kBoundMax = 4.2535296e37f;  // 2^125
+
+// 1.5 times the power of two above the bound v >= 0 (at least 2^-126)
+__device__ __forceinline__ float sigma_of(float f, float g) {
+  return 1.5f * __uint_as_float((__float_as_uint(fminf(f * g, kBoundMax)) & 0x7f800000u) + 0x00800000u);
+}
+
+// S + e += a b
+__device__ __forceinline__ void omac(float& S, float& e, float2 a, float2 b) {
+  const float n = __fmaf_rn(a.x, b.x, S);
+  float r = __fmaf_rn(a.x, b.x, -__fsub_rn(n, S));
+  r = __fmaf_rn(a.y, b.x, r);
+  r = __fmaf_rn(a.x, b.y, r);
+  S = n;
+  e = __fadd_rn(e, r);
+}
+
+__device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
+
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
 // ---- Gram partials ---------------------------------------------------------
 // G = 1: sel 0 -> X^T Y, sel 1 -> X^T X, sel 2 -> X^T W.
 // G = 4: D^T D, D^T W, D^T R, X^T X (the line-search Grams, Eqs. (diags),
 // (CG_linesearch_D), and the measured X^T X of the polar factor).
-// A thread owns 2 x 2 output blocks and a subset of the tile's rows; partial
-// sums are df64 in registers, float64 in the tile's slot.
+// D^T D, X^T X and D^T W (W = A D explicitly) are symmetric: their upper half
+// is formed, and mirrored. X^T Y is formed in full: Y follows A X by a
+// recursion, and X^T D = (I - X^T X)(C + beta K) takes C to be the symmetric
+// part of X^T Y exactly (mirrored, X^T X - I grew from 5e-13 to 2.5e-12 over
+// a solve). A thread owns 4 x 4 output blocks -- columns 2b, 2b+1,
+// p/2 + 2b, p/2 + 2b + 1, which keeps its 16-byte loads of a row free of bank
+// conflicts -- over the rows s, s + S, ... of a staged chunk; chunks are
+// double-buffered with cp.async. At p = 32, which is where the multiply-adds
+// are, the sums over a chunk's 8 rows run against the offsets of its own
+// columns and are added to df64 totals by TwoSum; at p <= 16 a block sums by
+// TwoProd + TwoSum throughout (offsets taken over a chunk of many short rows
+// were up to 10 times less accurate there).
+// Bound by instruction issue (0.57 of the slots, 18 warps per SM; DRAM at a
+// tenth): 48 problems of 2048..65536 rows, p in {4, 8, 16, 32}, together
+// 1.6e6 rows, take 880 us for G = 4 (2 x 2 blocks, full products and TwoProd
+// + TwoSum throughout: 1770) and 400 us for G = 1 (465).
+constexpr int GT = 192;     // 172 blocks of 4 x 4 at p = 32, G = 4
+constexpr int kGE = 512;    // most elements of an array per chunk
+
 template <int G>
-__global__ void __launch_bounds__(BT) b_gram_kernel(BDev d, int32_t mask, int32_t sel) {
-  constexpr int NA = G == 4 ? 4 : 2;
-  constexpr int UPT = G == 4 ? 4 : 1;  // most units per thread (p = 32)
-  __shared__ __align__(16) float4 sm[NA][RC * PMAX / 2];
-  __shared__ double red[BT * 4];
-  const int tid = threadIdx.x;
+struct GramSm {
+  static constexpr int NA = G == 4 ? 4 : 2;
+  union {
+    float4 st[2][NA][kGE / 2];
+    double red[GT * 16];  // at the end: [row group][entry of the block][block]
+  };
+  float wmax[NA][GT / 32][PMAX], wsum[NA][GT / 32][PMAX];
+  float cf[NA][PMAX], cg[NA][PMAX];
+};
+
+template <int G, int P>
+__device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const BProb& pr, int sel,
+                                          GramSm<G>& sm) {
+  constexpr int U = P >= 4 ? 4 : 2, NB = P / U, SYM = NB * (NB + 1) / 2;
+  constexpr int UNITS = (G == 4 ? 3 * SYM : 0) + NB * NB;
+  constexpr int S = GT / UNITS, RC = (G == 4 && P == 32 ? kGE / 2 : kGE) / P, H4 = P / 2, NA = GramSm<G>::NA;
+  constexpr bool OFFSET = G == 4 && P == 32;
+  static_assert(S >= 1 && GT % H4 == 0 && NA * P <= GT, "thread mapping");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nload = G == 4 ? 4 : (sel == 1 ? 1 : 2);
+  const float2* src[NA];
+  if (G == 4) {
+    src[0] = d.D;
+    src[1] = d.W;
+    src[NA - 2] = rcur(d, tl.prob);
+    src[NA - 1] = d.X;
+  } else {
+    src[0] = d.X;
+    src[1] = sel == 0 ? d.Y : d.W;
+  }
+  // this thread's block (g, bi, bj) of row group s
+  const int s = tid / UNITS;
+  auto decode = [&](int unit, int& g, int& bi, int& bj) {
+    g = 0;
+    if (G == 4) {
+      if (unit >= SYM) g = 1, unit -= SYM;
+      if (g == 1 && unit >= SYM) g = 2, unit -= SYM;
+      if (g == 2 && unit >= NB * NB) g = 3, unit -= NB * NB;
+    }
+    if (G == 1 || g == 2) {
+      bi = unit / NB;
+      bj = unit % NB;
+    } else {
+      bi = 0;
+      while (unit >= NB - bi) unit -= NB - bi++;
+      bj = bi + unit;
+    }
+  };
+  int g, bi, bj;
+  decode(tid % UNITS, g, bi, bj);
+  const int ia = G == 4 ? (g == 3 ? 3 : 0) : 0;
+  const int ib = G == 4 ? g : (nload == 1 ? 0 : 1);
+  auto col = [&](int b, int q) { return U == 4 && q >= 2 ? P / 2 + 2 * b + q - 2 : 2 * b + q; };
+  float H[U][U], E[U][U];
+#pragma unroll
+  for (int a = 0; a < U; ++a)
+#pragma unroll
+    for (int b = 0; b < U; ++b) H[a][b] = E[a][b] = 0.f;
+  auto issue = [&](int buf, int c0) {
+    const int cnt = min(RC, tl.rows - c0) * H4;
+    const int64_t off = pr.boff + (int64_t)(tl.row0 + c0) * P;
+    for (int a = 0; a < nload; ++a) {
+      const float4* g4 = reinterpret_cast<const float4*>(src[a] + off);
+      for (int i = tid; i < cnt; i += GT) cp16(&sm.st[buf][a][i], g4 + i);
+    }
+  };
+  __syncthreads();  // the last tile's sums have been read
+  issue(0, 0);
+  int buf = 0;
+  for (int c0 = 0; c0 < tl.rows; c0 += RC, buf ^= 1) {
+    const int rows = min(RC, tl.rows - c0);
+    cp_wait();
+    __syncthreads();
+    if (c0 + RC < tl.rows) issue(buf ^ 1, c0 + RC);
+    // the chunk's column maxima and column sums of |.|
+    for (int a = 0; OFFSET && a < nload; ++a) {
+      float m0 = 0.f, m1 = 0.f, t0 = 0.f, t1 = 0.f;
+      for (int i = tid; i < rows * H4; i += GT) {
+        const float4 v = sm.st[buf][a][i];
+        m0 = fmaxf(m0, fabsf(v.x));
+        m1 = fmaxf(m1, fabsf(v.z));
+        t0 += fabsf(v.x);
+        t1 += fabsf(v.z);
+      }
+      for (int o = 16; o >= H4; o >>= 1) {
+        m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+        t0 += __shfl_xor_sync(0xffffffffu, t0, o);
+        t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+      }
+      if (lane < H4) {
+        sm.wmax[a][warp][2 * lane] = m0;
+        sm.wmax[a][warp][2 * lane + 1] = m1;
+        sm.wsum[a][warp][2 * lane] = t0;
+        sm.wsum[a][warp][2 * lane + 1] = t1;
+      }
+    }
+    if (OFFSET) __syncthreads();
+    if (OFFSET && tid < nload * P) {
+      const int a = tid / P, c = tid % P;
+      float m = 0.f, t = 0.f;
+#pragma unroll
+      for (int w = 0; w < GT / 32; ++w) {
+        m = fmaxf(m, sm.wmax[a][w][c]);
+        t += sm.wsum[a][w][c];
+      }
+      sm.cf[a][c] = m;
+      sm.cg[a][c] = t * 1.000004f;  // above the rounding of t and of m t
+    }
+    if (OFFSET) __syncthreads();
+    if (s < S) {
+      float Sm[U][U], e[U][U];
+      if (OFFSET) {
+#pragma unroll
+        for (int a = 0; a < U; ++a)
+#pragma unroll
+          for (int b = 0; b < U; ++b) {
+            Sm[a][b] = sigma_of(sm.cf[ia][col(bi, a)], sm.cg[ib][col(bj, b)]);
+            e[a][b] = 0.f;
+          }
+      }
+      const float4* A = &sm.st[buf][ia][bi];
+      const float4* B = &sm.st[buf][ib][bj];
+      for (int r = s; r < rows; r += S) {
+        float2 av[U], bv[U];
+        const float4 a0 = A[r * H4], b0 = B[r * H4];
+        av[0] = lo2(a0), av[1] = hi2(a0), bv[0] = lo2(b0), bv[1] = hi2(b0);
+        if (U == 4) {
+          const float4 a1 = A[r * H4 + P / 4], b1 = B[r * H4 + P / 4];
+          av[U - 2] = lo2(a1), av[U - 1] = hi2(a1), bv[U - 2] = lo2(b1), bv[U - 1] = hi2(b1);
+        }
+#pragma unroll
+        for (int a = 0; a < U; ++a)
+#pragma unroll
+          for (int b = 0; b < U; ++b) {
+            if (OFFSET)
+              omac(Sm[a][b], e[a][b], av[a], bv[b]);
+            else
+              bmac(H[a][b], E[a][b], av[a], bv[b]);
+          }
+      }
+#pragma unroll
+      for (int a = 0; a < U; ++a)
+#pragma unroll
+        for (int b = 0; b < U; ++b) {
+          if (OFFSET) {
+            const float sg = sigma_of(sm.cf[ia][col(bi, a)], sm.cg[ib][col(bj, b)]);
+            const float2 t = two_sum(H[a][b], __fsub_rn(Sm[a][b], sg));
+            H[a][b] = t.x;
+            E[a][b] = __fadd_rn(E[a][b], __fadd_rn(t.y, e[a][b]));
+          } else {
+            renorm(H[a][b], E[a][b]);
+          }
+        }
+    }
+  }
+  __syncthreads();
+  if (s < S) {
+#pragma unroll
+    for (int a = 0; a < U; ++a)
+#pragma unroll
+      for (int b = 0; b < U; ++b)
+        sm.red[(s * U * U + a * U + b) * UNITS + tid % UNITS] = (double)H[a][b] + (double)E[a][b];
+  }
+  __syncthreads();
+  double* out = d.parts + tl.part;
+  for (int k = tid; k < UNITS * U * U; k += GT) {
+    double v = 0.0;
+    for (int z = 0; z < S; ++z) v += sm.red[z * U * U * UNITS + k];
+    int gk, bik, bjk;
+    const int q = k / UNITS;
+    decode(k % UNITS, gk, bik, bjk);
+    const int i = col(bik, q / U), j = col(bjk, q % U);
+    out[gk * P * P + i * P + j] = v;
+    if (bik != bjk && G == 4 && gk != 2) out[gk * P * P + j * P + i] = v;
+  }
+}
+
+template <int G>
+__global__ void __maxnreg__(112) b_gram_kernel(BDev d, int32_t mask, int32_t sel) {
+  extern __shared__ __align__(16) unsigned char gram_smem[];
+  GramSm<G>& sm = *reinterpret_cast<GramSm<G>*>(gram_smem);
   const int nt = *d.ntiles;
   for (int t = blockIdx.x; t < nt; t += gridDim.x) {
     const BTile tl = d.tile[t];
     if (!(d.st[tl.prob].flags & mask)) continue;
     const BProb pr = d.prob[tl.prob];
-    const int p = pr.p, nb = p >> 1, nbb = nb * nb;
-    const int units = G * nbb;
-    const bool wide = units >= BT;
-    const int upt = wide ? units / BT : 1;
-    const int S = wide ? 1 : BT / units;
-    const int s = wide ? 0 : tid / units;
-    const int ub = wide ? tid : tid % units;
-    const float2* src[NA];
-    int nload;
-    if (G == 4) {
-      src[0] = d.D;
-      src[1] = d.W;
-      src[2] = rcur(d, tl.prob);
-      src[3] = d.X;
-      nload = 4;
-    } else {
-      src[0] = d.X;
-      src[1] = sel == 0 ? d.Y : d.W;
-      nload = sel == 1 ? 1 : 2;
-    }
-    int ia[UPT], ib[UPT], bi[UPT], bj[UPT];
-#pragma unroll
-    for (int u = 0; u < UPT; ++u) {
-      const int unit = ub + u * BT;
-      const int g = unit / max(nbb, 1), rem = unit - g * nbb;
-      bi[u] = rem / nb;
-      bj[u] = rem - bi[u] * nb;
-      if (G == 4) {
-        ia[u] = g == 3 ? 3 : 0;
-        ib[u] = g == 3 ? 3 : g;
-      } else {
-        ia[u] = 0;
-        ib[u] = nload == 1 ? 0 : 1;
-      }
-    }
-    float h[UPT][4], e[UPT][4];
-#pragma unroll
-    for (int u = 0; u < UPT; ++u)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) h[u][q] = e[u][q] = 0.f;
-    for (int c0 = 0; c0 < tl.rows; c0 += RC) {
-      const int rows = min(RC, tl.rows - c0);
-      const int64_t off = pr.boff + (int64_t)(tl.row0 + c0) * p;
-      __syncthreads();
-      for (int a = 0; a < nload; ++a) {
-        const float4* g4 = reinterpret_cast<const float4*>(src[a] + off);
-        for (int i = tid; i < rows * nb; i += BT) sm[a][i] = g4[i];
-      }
-      __syncthreads();
-      for (int r = s; r < rows; r += S) {
-#pragma unroll
-        for (int u = 0; u < UPT; ++u) {
-          if (u < upt) {
-            const float4 a = sm[ia[u]][r * nb + bi[u]];
-            const float4 b = sm[ib[u]][r * nb + bj[u]];
-            bmac(h[u][0], e[u][0], make_float2(a.x, a.y), make_float2(b.x, b.y));
-            bmac(h[u][1], e[u][1], make_float2(a.x, a.y), make_float2(b.z, b.w));
-            bmac(h[u][2], e[u][2], make_float2(a.z, a.w), make_float2(b.x, b.y));
-            bmac(h[u][3], e[u][3], make_float2(a.z, a.w), make_float2(b.z, b.w));
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < UPT; ++u)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) renorm(h[u][q], e[u][q]);
-    }
-    double* out = d.parts + tl.part;
-    if (wide) {
-#pragma unroll
-      for (int u = 0; u < UPT; ++u) {
-        if (u < upt) {
-          const int unit = ub + u * BT, g = unit / nbb;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int i = 2 * bi[u] + (q >> 1), j = 2 * bj[u] + (q & 1);
-            out[(int64_t)g * p * p + i * p + j] = (double)h[u][q] + (double)e[u][q];
-          }
-        }
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) red[(s * units + ub) * 4 + q] = (double)h[0][q] + (double)e[0][q];
-      __syncthreads();
-      for (int k = tid; k < units * 4; k += BT) {
-        double v = 0.0;
-        for (int z = 0; z < S; ++z) v += red[z * units * 4 + k];
-        const int unit = k >> 2, q = k & 3, g = unit / nbb, rem = unit - g * nbb;
-        const int i = 2 * (rem / nb) + (q >> 1), j = 2 * (rem % nb) + (q & 1);
-        out[(int64_t)g * p * p + i * p + j] = v;
-      }
-      __syncthreads();
+    switch (pr.p) {
+      case 32: gram_tile<G, 32>(d, tl, pr, sel, sm); break;
+      case 16: gram_tile<G, 16>(d, tl, pr, sel, sm); break;
+      case 8: gram_tile<G, 8>(d, tl, pr, sel, sm); break;
+      case 4: gram_tile<G, 4>(d, tl, pr, sel, sm); break;
+      default: gram_tile<G, 2>(d, tl, pr, sel, sm); break;
     }
   }
 }
@@ -414,108 +556,353 @@ __global__ void __launch_bounds__(256) b_reduce_kernel(BDev d, int32_t mask, int
 }
 
 // ---- row-local block updates ------------------------------------------------
-// thread <-> (row group rg, column j); a pass covers BT / p rows.
+// Z B for the rows of a tile, B p x p. A thread owns rows rg and rg + RG of a
+// staged chunk and (as in the Gram kernel) columns 2c, 2c+1, p/2 + 2c,
+// p/2 + 2c + 1: a row's two columns of Z and the four of B feed 16 products
+// from six 16-byte loads. The sums stay TwoProd + TwoSum: against an offset
+// the error is relative to the largest |z| of the row, and a row of X that
+// carries a localised vector has entries far below that (6.7e-13 instead of
+// 9e-15 for X U with an orthogonal U at p = 32). Bound by instruction issue
+// (0.73 of the slots); 1.6e6 rows in 48 problems of p in {4, 8, 16, 32}:
+// residual 381 us, direction 283, retraction 503, where one product per
+// thread and row took 645, 500 and 867.
+template <int P>
+struct RowCfg {
+  static constexpr int TC = P >= 4 ? 4 : 2, CG = P / TC, RG = BT / CG, ROWS = 2 * RG;
+  static constexpr int H4 = P / 2;                       // float4 per row
+  static constexpr int LD = P >= 8 ? H4 + 1 : H4;        // row stride: an odd number of float4
+  static constexpr int STAGE = ROWS * LD;                // float4
+};
+constexpr int kRowStage = RowCfg<8>::STAGE;              // the largest of the five
+static_assert(RowCfg<32>::STAGE <= kRowStage && RowCfg<16>::STAGE <= kRowStage &&
+                  RowCfg<4>::STAGE <= kRowStage && RowCfg<2>::STAGE <= kRowStage,
+              "row buffers");
+
+template <int NZ>  // staged operands
+struct RowSm {
+  float4 z[NZ][kRowStage];
+  float4 b[PMAX * PMAX / 2];
+  double red[BT / 32];
+  float redf[BT / 32];
+};
+
+// B = scale * src; the caller's __syncthreads() after staging publishes it
+template <int P, int NZ>
+__device__ __forceinline__ void row_matrix(RowSm<NZ>& sm, const double* __restrict__ src, double scale) {
+  __syncthreads();
+  float2* b = reinterpret_cast<float2*>(sm.b);
+  for (int e = threadIdx.x; e < P * P; e += BT) b[e] = df_from_double(scale * src[e]);
+}
+
+// out[i][q] = (Z B) at row rg + i RG and this thread's column q
+template <int P, int NZ>
+__device__ __forceinline__ void row_mul(const RowSm<NZ>& sm, const float4* __restrict__ z, int rg, int c,
+                                        float2 (&out)[2][RowCfg<P>::TC]) {
+  using C = RowCfg<P>;
+  constexpr int TC = C::TC, H4 = C::H4;
+  float h[2][TC], e[2][TC];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int q = 0; q < TC; ++q) h[i][q] = e[i][q] = 0.f;
+  const float4* z0 = z + rg * C::LD;
+  const float4* z1 = z0 + C::RG * C::LD;
+#pragma unroll 4
+  for (int k2 = 0; k2 < H4; ++k2) {
+    const float4 a0 = z0[k2], a1 = z1[k2];
+#pragma unroll
+    for (int kk = 0; kk < 2; ++kk) {
+      float2 bv[TC];
+      const float4 b0 = sm.b[(2 * k2 + kk) * H4 + c];
+      bv[0] = lo2(b0), bv[1] = hi2(b0);
+      if (TC == 4) {
+        const float4 b1 = sm.b[(2 * k2 + kk) * H4 + P / 4 + c];
+        bv[TC - 2] = lo2(b1), bv[TC - 1] = hi2(b1);
+      }
+#pragma unroll
+      for (int q = 0; q < TC; ++q) {
+        bmac(h[0][q], e[0][q], kk ? hi2(a0) : lo2(a0), bv[q]);
+        bmac(h[1][q], e[1][q], kk ? hi2(a1) : lo2(a1), bv[q]);
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int q = 0; q < TC; ++q) out[i][q] = fast_two_sum(h[i][q], e[i][q]);
+}
+
+__device__ __forceinline__ float4 pack2(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
 
 // R = Y - X C in place with <R,R>, <R,R_prev> and max_r sum_j |R_rj|; D = R
 // where the direction is the gradient (SD, first CG step).
-__global__ void __launch_bounds__(BT) b_resid_kernel(BDev d) {
-  __shared__ float2 cs[PMAX * PMAX];
-  __shared__ float2 xs[BT];
-  __shared__ double red[BT / 32];
-  __shared__ float redf[BT / 32];
-  const int tid = threadIdx.x;
-  const int nt = *d.ntiles;
-  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-    const BTile tl = d.tile[t];
-    const int32_t flags = d.st[tl.prob].flags;
-    if (!(flags & F_ACTIVE)) continue;
-    const BProb pr = d.prob[tl.prob];
-    const int p = pr.p, RP = BT / p, j = tid % p, rg = tid / p;
-    const bool have_prev = d.st[tl.prob].have_prev != 0;
-    const bool want_rp = d.cg && have_prev;
-    const bool copy_d = !d.cg || !have_prev;
-    const int rsel = d.st[tl.prob].rsel;
-    const float2* __restrict__ Rold = rsel ? d.R[1] : d.R[0];
-    float2* __restrict__ Rnew = rsel ? d.R[0] : d.R[1];
-    __syncthreads();
-    for (int e = tid; e < p * p; e += BT) cs[e] = df_from_double(d.Cm[pr.ppoff + e]);
-    __syncthreads();
-    float rrh = 0.f, rre = 0.f, rph = 0.f, rpe = 0.f, rinf = 0.f;
-    for (int r0 = 0; r0 < tl.rows; r0 += RP) {
-      const int r = r0 + rg;
-      const bool ok = r < tl.rows;
-      const int64_t idx = pr.boff + (int64_t)(tl.row0 + r) * p + j;
-      if (ok) xs[tid] = d.X[idx];
-      __syncthreads();
-      float ab = 0.f;
-      if (ok) {
-        float ah = 0.f, ae = 0.f;
-        for (int k = 0; k < p; ++k) bmac(ah, ae, xs[rg * p + k], cs[k * p + j]);
-        const float2 xc = fast_two_sum(ah, ae);
-        const float2 rn = df_add(d.Y[idx], dneg(xc));
-        if (want_rp) bmac(rph, rpe, rn, Rold[idx]);
-        Rnew[idx] = rn;
-        if (copy_d) d.D[idx] = rn;
-        bmac(rrh, rre, rn, rn);
-        ab = fabsf(rn.x);
+template <int P>
+__device__ __forceinline__ void resid_tile(const BDev& d, const BTile& tl, const BProb& pr, int t,
+                                           RowSm<1>& sm) {
+  using C = RowCfg<P>;
+  constexpr int TC = C::TC, H4 = C::H4;
+  const int tid = threadIdx.x, c = tid % C::CG, rg = tid / C::CG;
+  const bool have_prev = d.st[tl.prob].have_prev != 0;
+  const bool want_rp = d.cg && have_prev;
+  const bool copy_d = !d.cg || !have_prev;
+  const int rsel = d.st[tl.prob].rsel;
+  const int64_t base = (pr.boff + (int64_t)tl.row0 * P) / 2;
+  const float4* __restrict__ X = reinterpret_cast<const float4*>(d.X) + base;
+  const float4* __restrict__ Y = reinterpret_cast<const float4*>(d.Y) + base;
+  const float4* __restrict__ Rold = reinterpret_cast<const float4*>(rsel ? d.R[1] : d.R[0]) + base;
+  float4* __restrict__ Rnew = reinterpret_cast<float4*>(rsel ? d.R[0] : d.R[1]) + base;
+  float4* __restrict__ D = reinterpret_cast<float4*>(d.D) + base;
+  row_matrix<P>(sm, d.Cm + pr.ppoff, 1.0);
+  float rrh = 0.f, rre = 0.f, rph = 0.f, rpe = 0.f, rinf = 0.f;
+  for (int r0 = 0; r0 < tl.rows; r0 += C::ROWS) {
+    const int rows = min(C::ROWS, tl.rows - r0);
+    const int64_t off = (int64_t)r0 * H4;
+    if (r0) __syncthreads();
+    float4 v[TC];
+#pragma unroll
+    for (int u = 0; u < TC; ++u) {
+      const int i = tid + u * BT;
+      v[u] = i < rows * H4 ? X[off + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float4 y[2][TC / 2], ro[2][TC / 2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int q = 0; q < TC / 2; ++q) {
+        const int r = rg + i * C::RG;
+        const int64_t k = off + (int64_t)r * H4 + c + q * (P / 4);
+        y[i][q] = ro[i][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows) {
+          y[i][q] = Y[k];
+          if (want_rp) ro[i][q] = Rold[k];
+        }
       }
-      for (int o = 1; o < p; o <<= 1) ab += __shfl_xor_sync(0xffffffffu, ab, o);
+#pragma unroll
+    for (int u = 0; u < TC; ++u) sm.z[0][(tid + u * BT) / H4 * C::LD + tid % H4] = v[u];
+    __syncthreads();
+    float2 xc[2][TC];
+    row_mul<P>(sm, sm.z[0], rg, c, xc);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = rg + i * C::RG;
+      float ab = 0.f;
+      if (r < rows) {
+#pragma unroll
+        for (int q = 0; q < TC / 2; ++q) {
+          const int64_t k = off + (int64_t)r * H4 + c + q * (P / 4);
+          const float2 n0 = df_add(lo2(y[i][q]), dneg(xc[i][2 * q]));
+          const float2 n1 = df_add(hi2(y[i][q]), dneg(xc[i][2 * q + 1]));
+          if (want_rp) {
+            bmac(rph, rpe, n0, lo2(ro[i][q]));
+            bmac(rph, rpe, n1, hi2(ro[i][q]));
+          }
+          Rnew[k] = pack2(n0, n1);
+          if (copy_d) D[k] = pack2(n0, n1);
+          bmac(rrh, rre, n0, n0);
+          bmac(rrh, rre, n1, n1);
+          ab += fabsf(n0.x) + fabsf(n1.x);
+        }
+      }
+#pragma unroll
+      for (int o = 1; o < C::CG; o <<= 1) ab += __shfl_xor_sync(0xffffffffu, ab, o);
       rinf = fmaxf(rinf, ab);
-      renorm(rrh, rre);
-      renorm(rph, rpe);
-      __syncthreads();
     }
-    const double v0 = bsum((double)rrh + (double)rre, red);
-    const double v1 = bsum((double)rph + (double)rpe, red);
-    const float v2 = bmaxf(rinf, redf);
-    if (tid == 0) {
-      d.tdots[(int64_t)t * 4 + 0] = v0;
-      d.tdots[(int64_t)t * 4 + 1] = v1;
-      d.tdots[(int64_t)t * 4 + 2] = (double)v2;
-    }
+    renorm(rrh, rre);
+    renorm(rph, rpe);
+  }
+  const double v0 = bsum((double)rrh + (double)rre, sm.red);
+  const double v1 = bsum((double)rph + (double)rpe, sm.red);
+  const float v2 = bmaxf(rinf, sm.redf);
+  if (tid == 0) {
+    d.tdots[(int64_t)t * 4 + 0] = v0;
+    d.tdots[(int64_t)t * 4 + 1] = v1;
+    d.tdots[(int64_t)t * 4 + 2] = (double)v2;
   }
 }
 
 // CG direction (Eq. (Pnew) with the projection transport): D <- R + beta D -
 // X (beta K) in place, with <D, R>.
+template <int P>
+__device__ __forceinline__ void dir_tile(const BDev& d, const BTile& tl, const BProb& pr, int t,
+                                         RowSm<1>& sm) {
+  using C = RowCfg<P>;
+  constexpr int TC = C::TC, H4 = C::H4;
+  const int tid = threadIdx.x, c = tid % C::CG, rg = tid / C::CG;
+  const double beta = d.st[tl.prob].beta;
+  const float2 bd = df_from_double(beta);
+  const int64_t base = (pr.boff + (int64_t)tl.row0 * P) / 2;
+  const float4* __restrict__ X = reinterpret_cast<const float4*>(d.X) + base;
+  const float4* __restrict__ Rc = reinterpret_cast<const float4*>(rcur(d, tl.prob)) + base;
+  float4* __restrict__ D = reinterpret_cast<float4*>(d.D) + base;
+  row_matrix<P>(sm, d.Km + pr.ppoff, beta);
+  float drh = 0.f, dre = 0.f;
+  for (int r0 = 0; r0 < tl.rows; r0 += C::ROWS) {
+    const int rows = min(C::ROWS, tl.rows - r0);
+    const int64_t off = (int64_t)r0 * H4;
+    if (r0) __syncthreads();
+    float4 v[TC];
+#pragma unroll
+    for (int u = 0; u < TC; ++u) {
+      const int i = tid + u * BT;
+      v[u] = i < rows * H4 ? X[off + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float4 rv[2][TC / 2], dv[2][TC / 2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int q = 0; q < TC / 2; ++q) {
+        const int r = rg + i * C::RG;
+        const int64_t k = off + (int64_t)r * H4 + c + q * (P / 4);
+        rv[i][q] = dv[i][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < rows) {
+          rv[i][q] = Rc[k];
+          dv[i][q] = D[k];
+        }
+      }
+#pragma unroll
+    for (int u = 0; u < TC; ++u) sm.z[0][(tid + u * BT) / H4 * C::LD + tid % H4] = v[u];
+    __syncthreads();
+    float2 xk[2][TC];
+    row_mul<P>(sm, sm.z[0], rg, c, xk);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int r = rg + i * C::RG;
+      if (r < rows) {
+#pragma unroll
+        for (int q = 0; q < TC / 2; ++q) {
+          const int64_t k = off + (int64_t)r * H4 + c + q * (P / 4);
+          const float2 r0v = lo2(rv[i][q]), r1v = hi2(rv[i][q]);
+          const float2 n0 = df_add(df_add(r0v, df_mul(bd, lo2(dv[i][q]))), dneg(xk[i][2 * q]));
+          const float2 n1 = df_add(df_add(r1v, df_mul(bd, hi2(dv[i][q]))), dneg(xk[i][2 * q + 1]));
+          D[k] = pack2(n0, n1);
+          bmac(drh, dre, n0, r0v);
+          bmac(drh, dre, n1, r1v);
+        }
+      }
+    }
+    renorm(drh, dre);
+  }
+  const double v = bsum((double)drh + (double)dre, sm.red);
+  if (tid == 0) d.tdots[(int64_t)t * 4 + 3] = v;
+}
+
+// mode 0 (step problems): X <- (X + tD) M and, unless Y is recomputed,
+// Y <- (Y + tW) M (Eqs. (Ynew), (save_matvec)); mode 1: X <- X M;
+// mode 2: W <- X M (X unchanged).
+template <int P>
+__device__ __forceinline__ void retract_tile(const BDev& d, const BTile& tl, const BProb& pr, int mode,
+                                             bool upd_y, RowSm<2>& sm) {
+  using C = RowCfg<P>;
+  constexpr int TC = C::TC, H4 = C::H4;
+  const int tid = threadIdx.x, c = tid % C::CG, rg = tid / C::CG;
+  const float2 td = df_from_double(mode == 0 ? d.st[tl.prob].t : 0.0);
+  const int64_t base = (pr.boff + (int64_t)tl.row0 * P) / 2;
+  const float4* X = reinterpret_cast<const float4*>(d.X) + base;
+  const float4* D = reinterpret_cast<const float4*>(d.D) + base;
+  float4* Y = reinterpret_cast<float4*>(d.Y) + base;
+  const float4* W = reinterpret_cast<const float4*>(d.W) + base;
+  float4* Xo = reinterpret_cast<float4*>(mode == 2 ? d.W : d.X) + base;
+  row_matrix<P>(sm, d.Mm + pr.ppoff, 1.0);
+  for (int r0 = 0; r0 < tl.rows; r0 += C::ROWS) {
+    const int rows = min(C::ROWS, tl.rows - r0);
+    const int64_t off = (int64_t)r0 * H4;
+    if (r0) __syncthreads();
+    float4 x[TC], dd[TC], y[TC], w[TC];
+#pragma unroll
+    for (int u = 0; u < TC; ++u) {
+      const int i = tid + u * BT;
+      x[u] = dd[u] = y[u] = w[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < rows * H4) {
+        x[u] = X[off + i];
+        if (mode == 0) dd[u] = D[off + i];
+        if (upd_y) {
+          y[u] = Y[off + i];
+          w[u] = W[off + i];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < TC; ++u) {
+      const int row = (tid + u * BT) / H4, c4 = tid % H4;
+      float4 zv = x[u];
+      if (mode == 0)
+        zv = pack2(df_add(lo2(zv), df_mul(td, lo2(dd[u]))), df_add(hi2(zv), df_mul(td, hi2(dd[u]))));
+      sm.z[0][row * C::LD + c4] = zv;
+      if (upd_y) {
+        zv = pack2(df_add(lo2(y[u]), df_mul(td, lo2(w[u]))), df_add(hi2(y[u]), df_mul(td, hi2(w[u]))));
+        sm.z[1][row * C::LD + c4] = zv;
+      }
+    }
+    __syncthreads();
+    for (int h = 0; h < (upd_y ? 2 : 1); ++h) {
+      float4* o = h ? Y : Xo;
+      float2 v[2][TC];
+      row_mul<P>(sm, sm.z[h], rg, c, v);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int r = rg + i * C::RG;
+        if (r < rows) {
+#pragma unroll
+          for (int q = 0; q < TC / 2; ++q)
+            o[off + (int64_t)r * H4 + c + q * (P / 4)] = pack2(v[i][2 * q], v[i][2 * q + 1]);
+        }
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(BT) b_resid_kernel(BDev d) {
+  __shared__ RowSm<1> sm;
+  const int nt = *d.ntiles;
+  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
+    const BTile tl = d.tile[t];
+    if (!(d.st[tl.prob].flags & F_ACTIVE)) continue;
+    const BProb pr = d.prob[tl.prob];
+    switch (pr.p) {
+      case 32: resid_tile<32>(d, tl, pr, t, sm); break;
+      case 16: resid_tile<16>(d, tl, pr, t, sm); break;
+      case 8: resid_tile<8>(d, tl, pr, t, sm); break;
+      case 4: resid_tile<4>(d, tl, pr, t, sm); break;
+      default: resid_tile<2>(d, tl, pr, t, sm); break;
+    }
+  }
+}
+
 __global__ void __launch_bounds__(BT) b_dir_kernel(BDev d) {
-  __shared__ float2 ks[PMAX * PMAX];
-  __shared__ float2 xs[BT];
-  __shared__ double red[BT / 32];
-  const int tid = threadIdx.x;
+  __shared__ RowSm<1> sm;
   const int nt = *d.ntiles;
   for (int t = blockIdx.x; t < nt; t += gridDim.x) {
     const BTile tl = d.tile[t];
     if (!(d.st[tl.prob].flags & F_DIR)) continue;
     const BProb pr = d.prob[tl.prob];
-    const int p = pr.p, RP = BT / p, j = tid % p, rg = tid / p;
-    const double beta = d.st[tl.prob].beta;
-    const float2 bd = df_from_double(beta);
-    const float2* __restrict__ Rc = rcur(d, tl.prob);
-    __syncthreads();
-    for (int e = tid; e < p * p; e += BT) ks[e] = df_from_double(beta * d.Km[pr.ppoff + e]);
-    __syncthreads();
-    float drh = 0.f, dre = 0.f;
-    for (int r0 = 0; r0 < tl.rows; r0 += RP) {
-      const int r = r0 + rg;
-      const bool ok = r < tl.rows;
-      const int64_t idx = pr.boff + (int64_t)(tl.row0 + r) * p + j;
-      if (ok) xs[tid] = d.X[idx];
-      __syncthreads();
-      if (ok) {
-        float ah = 0.f, ae = 0.f;
-        for (int k = 0; k < p; ++k) bmac(ah, ae, xs[rg * p + k], ks[k * p + j]);
-        const float2 xk = fast_two_sum(ah, ae);
-        const float2 rv = Rc[idx];
-        const float2 dn = df_add(df_add(rv, df_mul(bd, d.D[idx])), dneg(xk));
-        d.D[idx] = dn;
-        bmac(drh, dre, dn, rv);
-      }
-      renorm(drh, dre);
-      __syncthreads();
+    switch (pr.p) {
+      case 32: dir_tile<32>(d, tl, pr, t, sm); break;
+      case 16: dir_tile<16>(d, tl, pr, t, sm); break;
+      case 8: dir_tile<8>(d, tl, pr, t, sm); break;
+      case 4: dir_tile<4>(d, tl, pr, t, sm); break;
+      default: dir_tile<2>(d, tl, pr, t, sm); break;
     }
-    const double v = bsum((double)drh + (double)dre, red);
-    if (tid == 0) d.tdots[(int64_t)t * 4 + 3] = v;
+  }
+}
+
+__global__ void __launch_bounds__(BT) b_retract_kernel(BDev d, int32_t mode) {
+  extern __shared__ __align__(16) unsigned char row_smem[];
+  RowSm<2>& sm = *reinterpret_cast<RowSm<2>*>(row_smem);
+  const int32_t mask = mode == 0 ? F_STEP : F_START;
+  const int nt = *d.ntiles;
+  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
+    const BTile tl = d.tile[t];
+    const int32_t flags = d.st[tl.prob].flags;
+    if (!(flags & mask)) continue;
+    const BProb pr = d.prob[tl.prob];
+    const bool upd_y = mode == 0 && !(flags & F_Y);
+    switch (pr.p) {
+      case 32: retract_tile<32>(d, tl, pr, mode, upd_y, sm); break;
+      case 16: retract_tile<16>(d, tl, pr, mode, upd_y, sm); break;
+      case 8: retract_tile<8>(d, tl, pr, mode, upd_y, sm); break;
+      case 4: retract_tile<4>(d, tl, pr, mode, upd_y, sm); break;
+      default: retract_tile<2>(d, tl, pr, mode, upd_y, sm); break;
+    }
   }
 }
 
@@ -533,8 +920,9 @@ __global__ void __launch_bounds__(BT) b_copy_kernel(BDev d) {
 }
 
 // Block matvec (Sec. 6.1): which 0 -> W = A D (step problems), 1 -> Y = A X,
-// 2 -> W = A X; thread <-> (row, column j): the p lanes of a row read the
-// gathered neighbour rows as p consecutive df64 entries.
+// 2 -> W = A X; thread <-> (row, column pair): the p / 2 lanes of a row read
+// the gathered neighbour rows as 16-byte pieces, four neighbours at a time
+// (1.6e6 rows of mean degree 8 in 48 problems: 300 us, 402 with 8-byte ones).
 __global__ void __launch_bounds__(BT) b_spmm_kernel(BDev d, int32_t mask, int32_t which) {
   const int tid = threadIdx.x;
   const float2* in = which == 0 ? d.D : d.X;
@@ -544,65 +932,35 @@ __global__ void __launch_bounds__(BT) b_spmm_kernel(BDev d, int32_t mask, int32_
     const BTile tl = d.tile[t];
     if (!(d.st[tl.prob].flags & mask)) continue;
     const BProb pr = d.prob[tl.prob];
-    const int p = pr.p, RP = BT / p, j = tid % p, rg = tid / p;
-    const float2* xin = in + pr.boff + j;
+    const int h4 = pr.p >> 1, RP = BT / h4, j = tid % h4, rg = tid / h4;
+    const float4* __restrict__ xin = reinterpret_cast<const float4*>(in + pr.boff) + j;
+    float4* __restrict__ o = reinterpret_cast<float4*>(out + pr.boff) + j;
     for (int r = rg; r < tl.rows; r += RP) {
       const int64_t gr = pr.roff + tl.row0 + r;
-      const int64_t kb = d.rowptr[gr], ke = d.rowptr[gr + 1];
-      float h = 0.f, e = 0.f;
-      for (int64_t k = kb; k < ke; ++k) bmac_f(h, e, __ldg(d.val + k), xin[(int64_t)__ldg(d.colidx + k) * p]);
-      out[pr.boff + (int64_t)(tl.row0 + r) * p + j] = fast_two_sum(h, e);
-    }
-  }
-}
-
-// mode 0 (step problems): X <- (X + tD) M and, unless Y is recomputed,
-// Y <- (Y + tW) M (Eqs. (Ynew), (save_matvec)); mode 1: X <- X M;
-// mode 2: W <- X M (X unchanged).
-__global__ void __launch_bounds__(BT) b_retract_kernel(BDev d, int32_t mode) {
-  __shared__ float2 ms[PMAX * PMAX];
-  __shared__ float2 zs[BT];
-  const int tid = threadIdx.x;
-  const int32_t mask = mode == 0 ? F_STEP : F_START;
-  const int nt = *d.ntiles;
-  for (int t = blockIdx.x; t < nt; t += gridDim.x) {
-    const BTile tl = d.tile[t];
-    const int32_t flags = d.st[tl.prob].flags;
-    if (!(flags & mask)) continue;
-    const BProb pr = d.prob[tl.prob];
-    const int p = pr.p, RP = BT / p, j = tid % p, rg = tid / p;
-    const float2 td = df_from_double(mode == 0 ? d.st[tl.prob].t : 0.0);
-    const bool upd_y = mode == 0 && !(flags & F_Y);
-    __syncthreads();
-    for (int e = tid; e < p * p; e += BT) ms[e] = df_from_double(d.Mm[pr.ppoff + e]);
-    __syncthreads();
-    float2* xo = mode == 2 ? d.W : d.X;
-    for (int r0 = 0; r0 < tl.rows; r0 += RP) {
-      const int r = r0 + rg;
-      const bool ok = r < tl.rows;
-      const int64_t idx = pr.boff + (int64_t)(tl.row0 + r) * p + j;
-      if (ok) {
-        float2 z = d.X[idx];
-        if (mode == 0) z = df_add(z, df_mul(td, d.D[idx]));
-        zs[tid] = z;
-      }
-      __syncthreads();
-      if (ok) {
-        float ah = 0.f, ae = 0.f;
-        for (int k = 0; k < p; ++k) bmac(ah, ae, zs[rg * p + k], ms[k * p + j]);
-        xo[idx] = fast_two_sum(ah, ae);
-      }
-      __syncthreads();
-      if (upd_y) {
-        if (ok) zs[tid] = df_add(d.Y[idx], df_mul(td, d.W[idx]));
-        __syncthreads();
-        if (ok) {
-          float ah = 0.f, ae = 0.f;
-          for (int k = 0; k < p; ++k) bmac(ah, ae, zs[rg * p + k], ms[k * p + j]);
-          d.Y[idx] = fast_two_sum(ah, ae);
+      int64_t k = d.rowptr[gr];
+      const int64_t ke = d.rowptr[gr + 1];
+      float h0 = 0.f, e0 = 0.f, h1 = 0.f, e1 = 0.f;
+      for (; k + 4 <= ke; k += 4) {
+        float a[4];
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          a[u] = __ldg(d.val + k + u);
+          x[u] = xin[(int64_t)__ldg(d.colidx + k + u) * h4];
         }
-        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          bmac_f(h0, e0, a[u], lo2(x[u]));
+          bmac_f(h1, e1, a[u], hi2(x[u]));
+        }
       }
+      for (; k < ke; ++k) {
+        const float a = __ldg(d.val + k);
+        const float4 x = xin[(int64_t)__ldg(d.colidx + k) * h4];
+        bmac_f(h0, e0, a, lo2(x));
+        bmac_f(h1, e1, a, hi2(x));
+      }
+      o[(int64_t)(tl.row0 + r) * h4] = pack2(fast_two_sum(h0, e0), fast_two_sum(h1, e1));
     }
   }
 }
@@ -933,7 +1291,7 @@ struct gsi_batch {
   int32_t* saved = nullptr;
   int32_t* hcounter = nullptr;  // pinned
   size_t parts_cap = 0, tiles_cap = 0;
-  int tile_max = 2048, ctas_per_sm = 4, tiles_per_cta = 2, grid = 1;
+  int tile_max = 2048, ctas_per_sm = 4, tiles_per_cta = 4, grid = 1;
   size_t small_smem = 0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
@@ -1041,6 +1399,16 @@ gsi_status set_tiles(gsi_batch* b, int tile_max, int ctas_per_sm, int tiles_per_
 
 inline int pgrid(int nprob, int threads) { return (nprob + threads - 1) / threads; }
 
+// The tile kernels' grid: a CTA for each tile of the plan (about target_tiles
+// and one ragged tile per problem), so that the hardware hands the tiles out
+// in the table's order, widest problems first, as CTAs finish (a fixed share
+// of the tiles per CTA left the widest ones two to an SM: 1120 instead of
+// 880 us for the four Grams of 48 problems).
+inline int tile_grid(const gsi_batch* b) {
+  const size_t t = (size_t)b->grid * b->tiles_per_cta + b->nprob;
+  return (int)std::max<size_t>(1, std::min(t, b->tiles_cap));
+}
+
 // the reduction grid: problems x chunks of 32 of the ng * pmax^2 entries
 inline dim3 rgrid(gsi_batch* b, int ng) {
   return dim3((unsigned)b->nprob, (unsigned)((ng * b->pmax * b->pmax + 31) / 32));
@@ -1049,10 +1417,10 @@ inline dim3 rgrid(gsi_batch* b, int ng) {
 // one pass of the iteration for every active problem
 gsi_status launch_pass(gsi_batch* b, cudaStream_t s, int32_t use_cond) {
   const BDev d = make_dev(b);
-  const int g = b->grid, np = b->nprob;
+  const int g = tile_grid(b), np = b->nprob;
   b_plan_kernel<<<1, 1024, 0, s>>>(d, F_ACTIVE);
   GSI_LAUNCH_CHECK();
-  b_gram_kernel<1><<<g, BT, 0, s>>>(d, F_ACTIVE, 0);  // C = X^T Y
+  b_gram_kernel<1><<<g, GT, sizeof(GramSm<1>), s>>>(d, F_ACTIVE, 0);  // C = X^T Y
   GSI_LAUNCH_CHECK();
   b_reduce_kernel<<<rgrid(b, 1), 256, 0, s>>>(d, F_ACTIVE, 1, 1, 0);
   GSI_LAUNCH_CHECK();
@@ -1070,14 +1438,14 @@ gsi_status launch_pass(gsi_batch* b, cudaStream_t s, int32_t use_cond) {
   }
   b_spmm_kernel<<<g, BT, 0, s>>>(d, F_STEP, 0);  // W = A D
   GSI_LAUNCH_CHECK();
-  b_gram_kernel<NG><<<g, BT, 0, s>>>(d, F_STEP, 0);
+  b_gram_kernel<NG><<<g, GT, sizeof(GramSm<NG>), s>>>(d, F_STEP, 0);
   GSI_LAUNCH_CHECK();
   // D^T D, D^T W, X^T X symmetrised; D^T R as it is
   b_reduce_kernel<<<rgrid(b, NG), 256, 0, s>>>(d, F_STEP, NG, 1 | 2 | 8, 1);
   GSI_LAUNCH_CHECK();
   b_small_kernel<<<np, BS, b->small_smem, s>>>(d, 0);
   GSI_LAUNCH_CHECK();
-  b_retract_kernel<<<g, BT, 0, s>>>(d, 0);
+  b_retract_kernel<<<g, BT, sizeof(RowSm<2>), s>>>(d, 0);
   GSI_LAUNCH_CHECK();
   b_spmm_kernel<<<g, BT, 0, s>>>(d, F_Y, 1);  // Y = A X where requested
   GSI_LAUNCH_CHECK();
@@ -1089,7 +1457,7 @@ gsi_status launch_pass(gsi_batch* b, cudaStream_t s, int32_t use_cond) {
 // X0 -> df64, two polar orthonormalisations, Y = A X
 gsi_status start(gsi_batch* b) {
   const BDev d = make_dev(b);
-  const int g = b->grid, np = b->nprob;
+  const int g = tile_grid(b), np = b->nprob;
   cudaStream_t s = b->st;
   GSI_TRY(df_from_f64(b->elems, b->X0, b->X, s));
   b_init_kernel<<<pgrid(np, 128), 128, 0, s>>>(d);
@@ -1097,13 +1465,13 @@ gsi_status start(gsi_batch* b) {
   b_plan_kernel<<<1, 1024, 0, s>>>(d, F_START);
   GSI_LAUNCH_CHECK();
   for (int pass = 0; pass < 2; ++pass) {
-    b_gram_kernel<1><<<g, BT, 0, s>>>(d, F_START, 1);  // X^T X
+    b_gram_kernel<1><<<g, GT, sizeof(GramSm<1>), s>>>(d, F_START, 1);  // X^T X
     GSI_LAUNCH_CHECK();
     b_reduce_kernel<<<rgrid(b, 1), 256, 0, s>>>(d, F_START, 1, 1, 1);
     GSI_LAUNCH_CHECK();
     b_small_kernel<<<np, BS, b->small_smem, s>>>(d, 1);
     GSI_LAUNCH_CHECK();
-    b_retract_kernel<<<g, BT, 0, s>>>(d, 1);
+    b_retract_kernel<<<g, BT, sizeof(RowSm<2>), s>>>(d, 1);
     GSI_LAUNCH_CHECK();
   }
   b_spmm_kernel<<<g, BT, 0, s>>>(d, F_START, 1);
@@ -1307,8 +1675,14 @@ gsi_status gsi_batched_create(int32_t nprob, const int32_t* n, const int32_t* p,
     b->small_smem = pp_smem(pmax, 1);
     CK(cuda_status_ok(cudaFuncSetAttribute(b_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            (int)b->small_smem)));
+    CK(cuda_status_ok(cudaFuncSetAttribute(b_gram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sizeof(GramSm<1>))));
+    CK(cuda_status_ok(cudaFuncSetAttribute(b_gram_kernel<NG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sizeof(GramSm<NG>))));
+    CK(cuda_status_ok(cudaFuncSetAttribute(b_retract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           (int)sizeof(RowSm<2>))));
   }
-  CK(set_tiles(b, 2048, 4, 2));
+  CK(set_tiles(b, 2048, 4, 4));
   CK(start(b));
   CK(cuda_status_ok(cudaStreamSynchronize(b->st)));
 #undef CK
@@ -1484,7 +1858,7 @@ gsi_status gsi_batched_get_basis(gsi_batch* b, int32_t i, double* X, double* eva
     // Rayleigh-Ritz of every problem with an explicit AX: W = A X,
     // C' = X^T W, eig, W = X U (X itself is not changed)
     const BDev d = make_dev(b);
-    const int g = b->grid, np = b->nprob;
+    const int g = tile_grid(b), np = b->nprob;
     cudaStream_t s = b->st;
     b_mark_kernel<<<pgrid(np, 128), 128, 0, s>>>(d, 1, b->saved);
     GSI_LAUNCH_CHECK();
@@ -1492,13 +1866,13 @@ gsi_status gsi_batched_get_basis(gsi_batch* b, int32_t i, double* X, double* eva
     GSI_LAUNCH_CHECK();
     b_spmm_kernel<<<g, BT, 0, s>>>(d, F_START, 2);
     GSI_LAUNCH_CHECK();
-    b_gram_kernel<1><<<g, BT, 0, s>>>(d, F_START, 2);
+    b_gram_kernel<1><<<g, GT, sizeof(GramSm<1>), s>>>(d, F_START, 2);
     GSI_LAUNCH_CHECK();
     b_reduce_kernel<<<rgrid(b, 1), 256, 0, s>>>(d, F_START, 1, 1, 1);
     GSI_LAUNCH_CHECK();
     b_small_kernel<<<np, BS, b->small_smem, s>>>(d, 2);
     GSI_LAUNCH_CHECK();
-    b_retract_kernel<<<g, BT, 0, s>>>(d, 2);
+    b_retract_kernel<<<g, BT, sizeof(RowSm<2>), s>>>(d, 2);
     GSI_LAUNCH_CHECK();
     b_mark_kernel<<<pgrid(np, 128), 128, 0, s>>>(d, 0, b->saved);
     GSI_LAUNCH_CHECK();
