@@ -718,7 +718,7 @@ __device__ void pp_orth(const PpCtx<P>& c, int V, int T, int Out) {
   pp_sync<P>();
   for (int i = c.g; i < c.p; i += P::NG)
     for (int j = c.cl; j < c.p; j += P::CL) pp_sf(c.Af)[i * c.lda + j] = c.ldm(T + i * c.ld + j).x;
-  __syncthreads();
+  pp_sync<P>();  // every rank has read T before its rows are replaced
   pp_each(c, [&](int i, int j) {
     float s = 0.f;
     for (int k = 0; k < c.p; ++k) s = fmaf(pp_sf(c.Af)[i * c.lda + k], pp_sf(c.Af)[k * c.lda + j], s);
