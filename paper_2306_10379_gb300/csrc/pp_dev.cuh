@@ -642,11 +642,12 @@ __device__ __forceinline__ void pp_vrows(const PpCtx<P>& c, int& v0, int& v1) {
 }
 
 // Float32 Jacobi sweeps on c.Af until the squared off-diagonal mass is at most
-// `stop` (rank 0's value), the rotations gathered in V: c.Vf (NC = 1) or the
+// `stop` (rank 0's value), and for one sweep more if it is then above `stop2`;
+// the rotations gathered in V: c.Vf (NC = 1) or the
 // ranks' rows in c.sX. A and lam[0] are synchronised on entry, V on exit.
 // Returns the sweeps (rank 0; the others 0 or not 0).
 template <class P, bool DELTA>
-__device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop) {
+__device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop, float stop2) {
   const int p = c.p, lda = c.lda, m = (p + 1) & ~1;
   int A = c.Af, An = c.A2, lp = 0;
   const int w = c.tid >> 5;
@@ -662,6 +663,7 @@ __device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop) {
   }
   __syncthreads();
   int sweep = 0;
+  bool reached = false;
   for (;; ++sweep) {
     bool go = true;
     const int log = sweep & 1 ? c.log1 : c.log0, prev = sweep & 1 ? c.log0 : c.log1;
@@ -672,7 +674,8 @@ __device__ int pp_jacobi(const PpCtx<P>& c, int max_sweeps, float stop) {
         for (int j = c.cl; j < p; j += P::CL)
           if (i != j) off += a[i * lda + j] * a[i * lda + j];
       off = pp_bsum<P>(off);
-      go = sweep < max_sweeps && off > stop;
+      go = sweep < max_sweeps && (off > stop || (!reached && off > stop2));
+      reached = off <= stop;
       if constexpr (P::SEG == 64) {
         if (go) pp_sweep_wide<P, DELTA>(c, log);
       } else {
@@ -780,8 +783,12 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
       }
     tot0 = pp_bsum<P>(tot0);  // (its barriers also publish A)
   }
-  // down to ~1e-5 relative off-diagonal mass, above float32's rounding floor
-  s32 = pp_jacobi<P, false>(c, 12, 1e-10f * tot0);
+  // down to ~1e-5 relative off-diagonal mass, above float32's rounding floor;
+  // past p = 16 one sweep more brings the off-diagonal part to that floor,
+  // where the gaps of most spectra leave the rest to the corrections below (at
+  // p = 64 an extra sweep and three corrections take less than two sweeps
+  // there, the orthogonalisation after them and one correction)
+  s32 = pp_jacobi<P, false>(c, 12, 1e-10f * tot0, p > 16 ? 3e-13f * tot0 : tot0);
   const bool rotated = publish(c.Td, s32 > 0, 1) != 0;
   const long long c1 = clock64();
   if (rotated) {
@@ -797,8 +804,10 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
   }
   pp_sync<P>();
   const long long c2 = clock64();
-  for (int pass = 0; pass < 3; ++pass) {
-    int word = 0;  // 0: done, 1: rotations in Td, 2: first-order correction in Td
+  for (int pass = 0; pass < 4; ++pass) {
+    // 0: done, 1: rotations in Td, 2: the last, first-order correction K in Td,
+    // 3: a skew K in Td, V <- V exp(K), 4: the same, then orthogonalised
+    int word = 0;
     float stop = 0.f;
     if (c.rank == 0) {
       // F scaled by 2^30 so that squares of entries at 1e-15 stay in range
@@ -822,33 +831,39 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
       off = pp_bsum<P>(off);
       stop = 1e-30f * tot * UP * UP;
       if (off > 1e-27f * tot) {
-        word = 1;
-        if (first_order && pass > 0) {
-          // largest rotation angle F_ij / (lambda_j - lambda_i): below 1e-8
-          // the rotations are I + K to working accuracy. K is made exactly
-          // skew from the upper half of F: the halves differ by rounding,
-          // which over a small gap would leave V off orthogonal
-          float kmax = 0.f;
-          for (int i = c.g; i < p; i += P::NG)
-            for (int j = c.cl; j < p; j += P::CL)
-              if (i < j) {
-                const float2 d = df_add(lam[j], pp_neg(lam[i]));
-                const float f = pp_sf(c.Af)[i * lda + j];
-                const float k = f == 0.f ? 0.f : f / d.x;
-                pp_sf(c.Vf)[i * lda + j] = k;
-                pp_sf(c.Vf)[j * lda + i] = -k;
-                kmax = fmaxf(kmax, fabsf(k) <= 1.f ? fabsf(k) : 1.f);
-              } else if (i == j) {
-                pp_sf(c.Vf)[i * lda + i] = 0.f;
-              }
-          kmax = pp_bmax<P>(kmax);
-          if (kmax <= 1e-8f) word = 2;
-        }
+        // K_ij = F_ij / (lambda_j - lambda_i) leaves F of the order |F| |K|,
+        // without a sweep of its m - 1 dependent rounds. Up to |K| = 3e-4,
+        // I + K + K^2 / 2 is orthogonal to |K|^4 / 4 = 2e-15, and float32
+        // carries K^2 to 6e-15.
+        // Up to |K| = 0.1 (single small gaps) the pairs' exact angles and an
+        // orthogonalisation of the result still replace the sweeps.
+        // Angles below 1e-8 are I + K to working accuracy. K is made exactly
+        // skew from the upper half of F: the halves differ by rounding,
+        // which over a small gap would leave V off orthogonal. Small gaps
+        // (clusters, tiny eigenvalues) take the rotations instead.
+        float kmax = 0.f, kf = 0.f;
+        for (int i = c.g; i < p; i += P::NG)
+          for (int j = c.cl; j < p; j += P::CL)
+            if (i < j) {
+              const float2 d = df_add(lam[j], pp_neg(lam[i]));
+              const float f = pp_sf(c.Af)[i * lda + j];
+              float k = f == 0.f ? 0.f : f / d.x;
+              if (fabsf(k) > 1e-4f) k = 0.5f * atanf(2.f * k);
+              pp_sf(c.Vf)[i * lda + j] = k;
+              pp_sf(c.Vf)[j * lda + i] = -k;
+              kmax = fmaxf(kmax, fabsf(k));
+              kf += k * k;
+            } else if (i == j) {
+              pp_sf(c.Vf)[i * lda + i] = 0.f;
+            }
+        kmax = pp_bmax<P>(kmax);
+        kf = pp_bsum<P>(kf);
+        word = first_order && pass > 0 && kmax <= 1e-8f ? 2 : kf <= 1e-7f ? 3 : kf <= 1e-2f ? 4 : 1;
       }
     }
-    word = publish(c.Td, word, word == 2 ? 2 : 0);
+    word = publish(c.Td, word, word >= 2 ? 2 : 0);
     if (word == 1) {
-      s_delta += pp_jacobi<P, true>(c, 8, stop);
+      s_delta += pp_jacobi<P, true>(c, 8, stop, stop);
       publish(c.Td, 1, 1);
     }
     if (word == 0) break;
@@ -859,10 +874,26 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
       pp_sync<P>();
       break;
     }
-    // V <- orth(V W), U = V^T B V
-    pp_mm(c, c.Vd, false, c.Td, false, c.Ud);
+    if (word >= 3) {  // V += V (K + K^2 / 2)
+      for (int i = c.g; i < p; i += P::NG)
+        for (int j = c.cl; j < p; j += P::CL) pp_sf(c.Af)[i * lda + j] = c.ldm(c.Td + i * c.ld + j).x;
+      pp_sync<P>();  // every rank has read Td before its rows are replaced
+      pp_each(c, [&](int i, int j) {
+        float t = 0.f;
+        for (int k = 0; k < p; ++k) t = fmaf(pp_sf(c.Af)[i * lda + k], pp_sf(c.Af)[k * lda + j], t);
+        c.mat(c.Td)[i * c.ld + j] = two_sum(pp_sf(c.Af)[i * lda + j], 0.5f * t);
+      });
+      pp_sync<P>();
+    }
+    pp_mm(c, c.Vd, false, c.Td, false, c.Ud, word >= 3 ? c.Vd : -1);  // or V W
     pp_sync<P>();
-    pp_orth(c, c.Ud, c.Td, c.Vd);
+    if (word == 3) {
+      pp_each(c, [&](int i, int j) { c.mat(c.Vd)[i * c.ld + j] = c.mat(c.Ud)[i * c.ld + j]; });
+      pp_sync<P>();
+    } else {
+      pp_orth(c, c.Ud, c.Td, c.Vd);
+    }
+    // U = V^T B V
     pp_mm(c, c.Bd, false, c.Vd, false, c.Td);
     pp_sync<P>();
     pp_mm(c, c.Vd, true, c.Td, false, c.Ud);
