@@ -355,20 +355,6 @@ __device__ float pp_bmax(float v) {
   return s;
 }
 
-// Round-robin ordering of m (even) indices: in round r slot 0 pairs r with
-// m - 1, slot k pairs r + k and r - k modulo m - 1.
-__device__ __forceinline__ void pp_pair(int r, int k, int m1, int& a, int& b) {
-  if (k == 0) {
-    a = r;
-    b = m1;
-  } else {
-    a = r + k;
-    a -= a >= m1 ? m1 : 0;
-    b = r - k;
-    b += b < 0 ? m1 : 0;
-  }
-}
-
 __device__ __forceinline__ float pp_rsqrt(float x) {  // 1/sqrt(x), one Newton step on the approximation
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -409,6 +395,8 @@ __device__ __forceinline__ void pp_rot2(float2 wk, float2 wl, const float x[4], 
   z[3] = wk.y * y01 + wk.x * y11;
 }
 
+// Round-robin ordering of m (even) indices: in round r slot 0 pairs r with
+// m - 1, slot k pairs r + k and r - k modulo m - 1.
 // One sweep over A (symmetric m x m, m even; the dummy row and column of an
 // odd p are zero and stay so) by the first AW warps of the CTA, p <= 64; the
 // result is in `An` after an odd number of rounds. DELTA: A holds only the
@@ -509,14 +497,18 @@ __device__ void pp_sweep(const PpCtx<P>& c, int Ao, int Ano, int lp, int log) {
 }
 
 // The same for p > 64 by the whole CTA, A in place: half threads form the
-// angles, then every unordered pair of rotations is one thread's block.
+// angles, then every unordered pair of rotations is one thread's block. A
+// thread's pairs advance by one index a round, as in pp_sweep (recomputing
+// them took 2080 cycles a round at p = 128, this takes 1890; loading all of a
+// thread's blocks before the first store 2080 again).
 template <class P, bool DELTA>
 __device__ void pp_sweep_wide(const PpCtx<P>& c, int log) {
-  float* const A = pp_sf(c.Af);
   float2* const lam = pp_sh()->lam[0];
   const int lda = c.lda, tid = c.tid, m = (c.p + 1) & ~1, half = m / 2, m1 = m - 1;
   const int items = half * (half - 1) / 2;
-  int ik[P::IL], il[P::IL];
+  auto next = [&](int x) { return x + 1 == m1 ? 0 : x + 1; };
+  int ta = tid < half ? tid : 0, tb = ta == 0 ? m1 : m1 - ta;  // round 0's pair
+  int ik[P::IL], il[P::IL], ak[P::IL], bk[P::IL], al[P::IL], bl[P::IL];
 #pragma unroll
   for (int z = 0; z < P::IL; ++z) {
     const int e = tid + z * P::NT;
@@ -528,20 +520,23 @@ __device__ void pp_sweep_wide(const PpCtx<P>& c, int log) {
       il[z] = ik[z] + d + 1;
       il[z] -= il[z] >= half ? half : 0;
     }
+    ak[z] = max(ik[z], 0);
+    bk[z] = ak[z] == 0 ? m1 : m1 - ak[z];
+    al[z] = il[z];
+    bl[z] = il[z] == 0 ? m1 : m1 - il[z];
   }
   for (int r = 0; r < m1; ++r) {
+    float* const A = pp_sf(c.Af);
     if (tid < half) {
-      int a, b;
-      pp_pair(r, tid, m1, a, b);
-      const int ra = a * lda, rb = b * lda;
-      const float f = A[ra + b];
+      const int ra = ta * lda, rb = tb * lda;
+      const float f = A[ra + tb];
       float2 la, lb;
       if (DELTA) {
-        la = lam[a];
-        lb = lam[b];
+        la = lam[ta];
+        lb = lam[tb];
       } else {
-        la = make_float2(A[ra + a], 0.f);
-        lb = make_float2(A[rb + b], 0.f);
+        la = make_float2(A[ra + ta], 0.f);
+        lb = make_float2(A[rb + tb], 0.f);
       }
       float t;
       const float2 cs = pp_angle<DELTA>(f, la, lb, t);
@@ -549,34 +544,37 @@ __device__ void pp_sweep_wide(const PpCtx<P>& c, int log) {
       c.mat(log)[r * half + tid] = cs;
       const float d = t * f;
       if (DELTA) {
-        lam[a] = df_add_f(la, -d);
-        lam[b] = df_add_f(lb, d);
+        lam[ta] = df_add_f(la, -d);
+        lam[tb] = df_add_f(lb, d);
       } else {
-        A[ra + a] = la.x - d;
-        A[rb + b] = lb.x + d;
+        A[ra + ta] = la.x - d;
+        A[rb + tb] = lb.x + d;
       }
-      A[ra + b] = 0.f;
-      A[rb + a] = 0.f;
+      A[ra + tb] = 0.f;
+      A[rb + ta] = 0.f;
+      ta = next(ta);
+      if (tid != 0) tb = next(tb);
     }
     __syncthreads();
 #pragma unroll
     for (int z = 0; z < P::IL; ++z) {
       if (ik[z] >= 0) {
-        int ak, bk, al, bl;
-        pp_pair(r, ik[z], m1, ak, bk);
-        pp_pair(r, il[z], m1, al, bl);
-        const int ra = ak * lda, rb = bk * lda, rl = al * lda, sl = bl * lda;
-        const float x[4] = {A[ra + al], A[ra + bl], A[rb + al], A[rb + bl]};
+        const int ra = ak[z] * lda, rb = bk[z] * lda, rl = al[z] * lda, sl = bl[z] * lda;
+        const float x[4] = {A[ra + al[z]], A[ra + bl[z]], A[rb + al[z]], A[rb + bl[z]]};
         float y[4];
         pp_rot2(pp_sh()->cs[ik[z]], pp_sh()->cs[il[z]], x, y);
-        A[ra + al] = y[0];
-        A[ra + bl] = y[1];
-        A[rb + al] = y[2];
-        A[rb + bl] = y[3];
-        A[rl + ak] = y[0];
-        A[sl + ak] = y[1];
-        A[rl + bk] = y[2];
-        A[sl + bk] = y[3];
+        A[ra + al[z]] = y[0];
+        A[ra + bl[z]] = y[1];
+        A[rb + al[z]] = y[2];
+        A[rb + bl[z]] = y[3];
+        A[rl + ak[z]] = y[0];
+        A[sl + ak[z]] = y[1];
+        A[rl + bk[z]] = y[2];
+        A[sl + bk[z]] = y[3];
+        ak[z] = next(ak[z]);
+        if (ik[z] != 0) bk[z] = next(bk[z]);
+        al[z] = next(al[z]);
+        if (il[z] != 0) bl[z] = next(bl[z]);
       }
     }
     __syncthreads();
