@@ -465,7 +465,7 @@ gsi_status gsi_measure_fma_peaks(double* out, void* stream);
  * by Alg. 2 (SD) or Alg. 4 (CG) with the exact line search of Alg. 3 and the
  * recursion of Eq. (save_matvec) -- the same iteration as gsi_solve, with
  * every decision taken on the GPU. Block data are df64; operator entries
- * float32; the p x p step float64. The paper solves one problem at a time;
+ * float32; the p x p step df64. The paper solves one problem at a time;
  * batching is a GPU execution form of the same method. */
 typedef struct gsi_batch gsi_batch;
 
