@@ -3,15 +3,18 @@
 //
 // Eigenbasis of a symmetric B: float32 Jacobi sweeps give V0; V is made
 // orthonormal in df64; then B' = V^T B V = diag(lambda) + F is formed in df64
-// and the small F rotated away by the same float32 Jacobi, which works on F
-// and on df64 differences of lambda, so that its float32 rounding is relative
-// to F: each such pass gains six to seven digits (F 1e-6 -> 1e-13 of ||B||).
-// The rotations of a pass are gathered in one matrix, applied in df64. Against
-// df64 Jacobi sweeps this trades the serial rounds of ~400 float operations a
-// 2 x 2 block for df64 products, which have no chain between rounds.
+// and the small F taken out by V <- V exp(K), K_ij = F_ij / (lambda_j -
+// lambda_i), which squares the relative size of F without a sweep's dependent
+// rounds. Where eigenvalues cluster (|K| > 0.1), F is rotated away by the same
+// float32 Jacobi, which works on F and on df64 differences of lambda, so that
+// its float32 rounding is relative to F: each such pass gains six to seven
+// digits. Either way the correction is one matrix, applied in df64. One step
+// at p = 8 / 32 / 64 / 128: 64 / 174 / 355 / 1330 us; with sweeps instead of
+// the corrections 70 / 195 / 411 / 1728, as one CTA of 1024 threads with df64
+// sweeps and a float64 line search 72 / - / 760 / 6060.
 //
 // Layout of the work. The sweeps are a chain of p - 1 rounds each, so a
-// round is kept short: AW warps (1, 2 or 8) work on A alone, every lane
+// round is kept short: AW warps (1, 4, 8 or 16) work on A alone, every lane
 // computes the angle of its own rotation, 2 x 2 blocks take their partner's
 // by shuffle, and A is double-buffered, which leaves one barrier among those
 // warps per round. The rotations go to a log; V is a chain per row only, and
@@ -33,7 +36,8 @@ namespace gsi {
 // Block shape: NT threads; a group of CL lanes covers TC CL columns of a
 // product (NCG such column blocks), the groups its rows, TR each. Jacobi:
 // AW warps work on A (p = 64: 687 cycles a round with 16 warps of one block
-// a lane, 934 with 8 of two; p = 32: 689 with 4, 779 with 2); a segment of SEG lanes holds one rotation per lane
+// a lane, 934 with 8 of two; p = 32: 689 with 4, 779 with 2; 453 at p = 32
+// with unpadded rows); a segment of SEG lanes holds one rotation per lane
 // (SEG = 64: p > 64), IL 2 x 2 blocks a lane: the blocks of rotations k and
 // k + d, 1 <= d <= half / 2, half <= SEG rotations a round.
 template <int NT_, int CL_, int TR_, int TC_, int NCG_, int SEG_, int AW_, int IL_, int NC_>

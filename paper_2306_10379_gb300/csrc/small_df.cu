@@ -47,6 +47,10 @@ size_t small_df_scratch_bytes(int p) { return pp_gws_bytes(p); }
 
 gsi_status small_step_df(const PpArgs& a, bool cluster, cudaStream_t st) {
   if (a.p < 1 || a.p > 128 || ((a.mode == 3 || a.mode == 4) && !a.eig)) return GSI_ERR_ARG;
+  // one CTA while a product takes fewer cycles than a cluster barrier and the
+  // trip through L2 (p <= 32); a cluster of 8 past p = 64, where the matrices
+  // leave shared memory. Between the two a cluster is the faster one but
+  // holds 8 SMs, which large Grams beside it would miss: the caller decides.
   if (a.p <= 16) return launch<PpCfg<128, 16, 2, 1, 1, 8, 1, 1, 1>>(a, st);
   if (a.p <= 32) return launch<PpCfg<256, 32, 4, 1, 1, 16, 4, 1, 1>>(a, st);
   if (a.p > 64) return launch<PpCfg<512, 32, 2, 2, 2, 64, 16, 4, 8>>(a, st);
