@@ -613,9 +613,9 @@ __device__ void pp_apply_log(int p, int Vo, int ldv, int rows, int logo, int w, 
           float x[4], y[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const int rr = min(row + u * nw * NSEG, rows - 1);
-            x[u] = V[rr * ldv + a[z]];
-            y[u] = V[rr * ldv + b[z]];
+            const int rr = row + u * nw * NSEG;  // other rows belong to other segments
+            x[u] = rr < rows ? V[rr * ldv + a[z]] : 0.f;
+            y[u] = rr < rows ? V[rr * ldv + b[z]] : 0.f;
           }
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
