@@ -365,6 +365,17 @@ gsi_status gsi_linesearch(int32_t p, const double* C, const double* B, const dou
                           const double* Z, const double* XX, const double* XD, double* M,
                           double* out, int32_t precision, void* stream);
 
+/* The df64 p x p part of one iteration as the solver launches it: the
+ * eigenbasis of B in one launch, the rest in a second one, X^T D = (I - XX)
+ * (C + beta K) formed inside (Eq. (Pnew): K = X^T P of the last direction P),
+ * and K_next = M (X^T D + t B). Other inputs and outputs as gsi_linesearch
+ * (phi(t) is not formed). For 32 < p <= 64 the eigenbasis runs on a cluster
+ * of eight thread blocks (cluster != 0) or on one (0), which the solver takes
+ * from 250,000 rows on; other p have one form. */
+gsi_status gsi_pp_step(int32_t p, const double* C, const double* B, const double* Gam, const double* Z,
+                       const double* XX, const double* K, double beta, double* M, double* Knext, double* out,
+                       int32_t cluster, void* stream);
+
 /* Retraction with the AX recursion (Eqs. (Ynew), (save_matvec)):
  * X <- (X + t D) M, Y <- (Y + t W) M, in place. */
 gsi_status gsi_retract(int64_t n, int32_t p, double t, const double* M, double* X,

@@ -95,6 +95,34 @@ gsi_status gsi_linesearch(int32_t p, const double* C, const double* B, const dou
   return small_step(0, p, C, B, Gam, Z, XX, XD, M, out, (double*)g.ptr, st);
 }
 
+gsi_status gsi_pp_step(int32_t p, const double* C, const double* B, const double* Gam, const double* Z,
+                       const double* XX, const double* K, double beta, double* M, double* Knext, double* out,
+                       int32_t cluster, void* stream) {
+  if (p < 1 || p > 128 || !C || !B || !Gam || !Z || !XX || !K || !M || !Knext || !out) return GSI_ERR_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  ScratchGuard g(st);
+  const size_t wb = (small_df_scratch_bytes(p) + 255) / 256 * 256;
+  GSI_CUDA_TRY(cudaMallocAsync(&g.ptr, wb + ((size_t)p * p + p) * sizeof(float2), st));
+  PpArgs a{};
+  a.p = p;
+  a.B = {nullptr, B, 1};
+  a.C = {nullptr, C, 1};
+  a.Gam = {nullptr, Gam, 1};
+  a.Z = {nullptr, Z, 1};
+  a.XX = {nullptr, XX, 1};
+  a.K = {nullptr, K, 0};
+  a.beta = beta;
+  a.M = M;
+  a.Kd = Knext;
+  a.out = out;
+  a.gws = (float2*)g.ptr;
+  a.eig = (float2*)((char*)g.ptr + wb);
+  a.mode = 3;
+  GSI_TRY(small_step_df(a, cluster != 0, st));
+  a.mode = 4;
+  return small_step_df(a, true, st);
+}
+
 gsi_status gsi_retract(int64_t n, int32_t p, double t, const double* M, double* X,
                        const double* D, double* Y, const double* W, void* stream) {
   if (n < 0 || p < 1 || p > 128 || !M || (n > 0 && (!X || !D || !Y || !W))) return GSI_ERR_ARG;

@@ -31,7 +31,7 @@ EXPORTED = [
     "gsi_profile_enable", "gsi_profile_read", "gsi_launch_count", "gsi_oz_dense_apply",
     "gsi_oz_gram_noalloc", "gsi_measure_fma_peaks", "gsi_set_operator", "gsi_set_wait_limit",
     "gsi_device_timeouts", "gsi_create_hermitian", "gsi_get_basis_hermitian", "gsi_csr_to_dia",
-    "gsi_df_spmm_dia",
+    "gsi_df_spmm_dia", "gsi_pp_step",
 ]
 
 
@@ -103,6 +103,7 @@ def _lib():
             "gsi_gram": [i64, i32, i32, vp, vp, vp, vp],
             "gsi_residual": [i64, i32, vp, vp, vp, vp, vp],
             "gsi_linesearch": [i32, vp, vp, vp, vp, vp, vp, vp, vp, i32, vp],
+            "gsi_pp_step": [i32, vp, vp, vp, vp, vp, vp, dbl, vp, vp, vp, i32, vp],
             "gsi_retract": [i64, i32, dbl, vp, vp, vp, vp, vp, vp],
             "gsi_df_spmm_csr": [i64, vp, vp, vp, i32, vp, vp, vp],
             "gsi_oz_gemm": [i64, i32, i32, vp, vp, vp, vp, dbl, dbl, i32, vp, vp, vp, vp, vp],
@@ -274,6 +275,17 @@ def linesearch(C, B, Gam, Z, XX, XD, M, out, precision="df64", stream=None):
                                 _dptr(Z, f, (p, p)), _dptr(XX, f, (p, p)), _dptr(XD, f, (p, p)),
                                 _dptr(M, f, (p, p)), _dptr(out, f), pr, _stream(stream)),
            "gsi_linesearch")
+
+
+def pp_step(C, B, Gam, Z, XX, K, beta, M, Knext, out, cluster=True, stream=None):
+    """The df64 p x p step in the solver's two launches (gsi_pp_step)."""
+    import torch
+    p = C.shape[0]
+    f = torch.float64
+    _check(lib().gsi_pp_step(p, _dptr(C, f, (p, p)), _dptr(B, f, (p, p)), _dptr(Gam, f, (p, p)),
+                             _dptr(Z, f, (p, p)), _dptr(XX, f, (p, p)), _dptr(K, f, (p, p)), float(beta),
+                             _dptr(M, f, (p, p)), _dptr(Knext, f, (p, p)), _dptr(out, f), 1 if cluster else 0,
+                             _stream(stream)), "gsi_pp_step")
 
 
 def retract(t, M, X, D, Y, W, stream=None):
