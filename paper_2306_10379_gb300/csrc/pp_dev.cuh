@@ -50,7 +50,9 @@ struct PpCfg {
   static_assert(NC > 1 ? NT / 32 >= AW : NT / 32 > AW, "V needs warps (or ranks) of its own");
 };
 
-struct PpMat {  // a p x p input: df64, or float64 (then symmetrised where sym is set)
+// a p x p input: float64 (symmetrised where sym is set), and where f is set
+// the same in df64, which the df64 products then take
+struct PpMat {
   const float2* f;
   const double* d;
   int sym;
@@ -77,7 +79,7 @@ constexpr int PP_CTL = 1024 + 64;  // float2: control words, then the partial do
 
 struct PpSh {  // small tables, shared memory
   double al[128], be[128], ga[128], ze[128], sv[128];
-  float2 alf[128], bef[128], gaf[128], zef[128];  // the same in df64
+  float2 alf[128], bef[128], gaf[128], zef[128], svf[128];  // the same in df64
   float2 lam[2][130];
   float2 cs[64];
   float red[32];
@@ -834,11 +836,11 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
       stop = 1e-30f * tot * UP * UP;
       if (off > 1e-27f * tot) {
         // K_ij = F_ij / (lambda_j - lambda_i) leaves F of the order |F| |K|,
-        // without a sweep of its m - 1 dependent rounds. Up to |K| = 3e-4,
-        // I + K + K^2 / 2 is orthogonal to |K|^4 / 4 = 2e-15, and float32
-        // carries K^2 to 6e-15.
-        // Up to |K| = 0.1 (single small gaps) the pairs' exact angles and an
-        // orthogonalisation of the result still replace the sweeps.
+        // without a sweep of its m - 1 dependent rounds. Up to |K| = 2e-4,
+        // I + K + K^2 / 2 with K^2 in df64 is orthogonal to |K|^4 / 4 = 4e-16.
+        // Up to |K| = 0.07 (single small gaps) the pairs' exact angles and an
+        // orthogonalisation of the result (which leaves |K|^12 / 200) still
+        // replace the sweeps.
         // Angles below 1e-8 are I + K to working accuracy. K is made exactly
         // skew from the upper half of F: the halves differ by rounding,
         // which over a small gap would leave V off orthogonal. Small gaps
@@ -860,7 +862,7 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
             }
         kmax = pp_bmax<P>(kmax);
         kf = pp_bsum<P>(kf);
-        word = first_order && pass > 0 && kmax <= 1e-8f ? 2 : kf <= 1e-7f ? 3 : kf <= 1e-2f ? 4 : 1;
+        word = first_order && pass > 0 && kmax <= 1e-8f ? 2 : kf <= 4e-8f ? 3 : kf <= 5e-3f ? 4 : 1;
       }
     }
     word = publish(c.Td, word, word >= 2 ? 2 : 0);
@@ -881,9 +883,15 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
         for (int j = c.cl; j < p; j += P::CL) pp_sf(c.Af)[i * lda + j] = c.ldm(c.Td + i * c.ld + j).x;
       pp_sync<P>();  // every rank has read Td before its rows are replaced
       pp_each(c, [&](int i, int j) {
-        float t = 0.f;
-        for (int k = 0; k < p; ++k) t = fmaf(pp_sf(c.Af)[i * lda + k], pp_sf(c.Af)[k * lda + j], t);
-        c.mat(c.Td)[i * c.ld + j] = two_sum(pp_sf(c.Af)[i * lda + j], 0.5f * t);
+        float h = 0.f, e = 0.f;
+        for (int k = 0; k < p; ++k) {
+          const float x = pp_sf(c.Af)[i * lda + k], y = pp_sf(c.Af)[k * lda + j], pr = __fmul_rn(x, y);
+          const float2 t = two_sum(h, pr);
+          h = t.x;
+          e = __fadd_rn(e, __fadd_rn(t.y, __fmaf_rn(x, y, -pr)));
+        }
+        c.mat(c.Td)[i * c.ld + j] =
+            df_add(make_float2(pp_sf(c.Af)[i * lda + j], 0.f), two_sum(0.5f * h, 0.5f * e));
       });
       pp_sync<P>();
     }
@@ -910,10 +918,17 @@ __device__ void pp_eig(const PpCtx<P>& c, bool first_order, double* diag) {
   }
 }
 
+__device__ __forceinline__ float2 df_div(float2 a, float2 b) {
+  const float q1 = __fdiv_rn(a.x, b.x);
+  const float p = __fmul_rn(q1, b.x);
+  const float e = __fmaf_rn(q1, b.y, __fmaf_rn(q1, b.x, -p));
+  const float2 r = df_add(a, make_float2(-p, -e));
+  return fast_two_sum(q1, __fdiv_rn(__fadd_rn(r.x, r.y), b.x));
+}
+
 // M = V [diag(s^-1/2) + F o Df] V^T for S' = diag(s) + F in c.Ud, df64 into
 // c.Ud and float64 into M; status (0, or 5 if some s_i is not positive) in
-// sh->flag of every CTA. F is rounding-level, so its divided differences are
-// taken in float32.
+// sh->flag of every CTA.
 template <class P>
 __device__ void pp_inv_sqrt(const PpCtx<P>& c, double* M) {
   PpSh* const sh = pp_sh();
@@ -932,6 +947,7 @@ __device__ void pp_inv_sqrt(const PpCtx<P>& c, double* M) {
       // numerically singular: below the df64 rounding level of the largest
       bad = bad || !(s > 1e-13 * mx) || !isfinite(s);
       sh->sv[i] = s > 0.0 ? sqrt(s) : 1.0;
+      sh->svf[i] = df_from_double(sh->sv[i]);
     }
     bad = __any_sync(0xffffffffu, bad);
     if (c.tid == 0) sh->flag = bad ? 5 : 0;
@@ -943,9 +959,8 @@ __device__ void pp_inv_sqrt(const PpCtx<P>& c, double* M) {
     if (i == j) {
       v = df_from_double(1.0 / sh->sv[i]);
     } else {
-      const float ri = (float)sh->sv[i], rj = (float)sh->sv[j];
-      const float2 f = c.mat(c.Ud)[i * c.ld + j];
-      v = make_float2(-((__fadd_rn(f.x, f.y) / ri) / rj) / (ri + rj), 0.f);
+      const float2 ri = sh->svf[i], rj = sh->svf[j];
+      v = df_div(df_div(df_div(pp_neg(c.mat(c.Ud)[i * c.ld + j]), ri), rj), df_add(ri, rj));
     }
     c.mat(c.Ud)[i * c.ld + j] = v;
   });
@@ -972,14 +987,6 @@ __device__ __forceinline__ void pp_load(const PpCtx<P>& c, const PpMat& a, int d
 }
 
 // ---- the exact step of Alg. 3 ------------------------------------------------
-
-__device__ __forceinline__ float2 df_div(float2 a, float2 b) {
-  const float q1 = __fdiv_rn(a.x, b.x);
-  const float p = __fmul_rn(q1, b.x);
-  const float e = __fmaf_rn(q1, b.y, __fmaf_rn(q1, b.x, -p));
-  const float2 r = df_add(a, make_float2(-p, -e));
-  return fast_two_sum(q1, __fdiv_rn(__fadd_rn(r.x, r.y), b.x));
-}
 
 __device__ __forceinline__ bool df_less(float2 a, float2 b) { return a.x < b.x || (a.x == b.x && a.y < b.y); }
 
@@ -1365,15 +1372,15 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
   pp_sync<P>();
   const double t = P::NC == 1 ? sh->t : __ldcg(reinterpret_cast<const double*>(c.gws + c.ctl + 2));
   const long long t3 = clock64();
-  // S' = V^T S V with S = XX + t (XD + XD^T) + t^2 B
-  const float2 td = df_from_double(t), tt = df_from_double(t * t);
+  // S' = V^T S V with S = XX + t (XD + XD^T) + t^2 B, summed in float64
   auto elem = [&](const PpMat& g, int i, int j) {
-    return g.f ? g.f[i * p + j]
-               : df_from_double(g.sym ? 0.5 * (g.d[i * p + j] + g.d[j * p + i]) : g.d[i * p + j]);
+    return g.sym ? 0.5 * (g.d[i * p + j] + g.d[j * p + i]) : g.d[i * p + j];
   };
-  pp_load(c, a.XX, c.Ud, [&](int i, int j, float2 v) {
-    const float2 xd = df_add(c.ldm(c.Bd + i * c.ld + j), c.ldm(c.Bd + j * c.ld + i));
-    return df_add(df_add(v, df_mul(td, xd)), df_mul(tt, elem(a.B, i, j)));
+  pp_each(c, [&](int i, int j) {
+    // X^T D as the caller holds it, where it was given
+    const double xd = a.XD.d ? a.XD.d[i * p + j] + a.XD.d[j * p + i]
+                             : df_to_double(c.ldm(c.Bd + i * c.ld + j)) + df_to_double(c.ldm(c.Bd + j * c.ld + i));
+    c.mat(c.Ud)[i * c.ld + j] = df_from_double(fma(t, xd, elem(a.XX, i, j)) + t * t * elem(a.B, i, j));
   });
   pp_sync<P>();
   pp_mm(c, c.Ud, false, c.Vd, false, c.Td);
@@ -1382,17 +1389,34 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
   pp_sync<P>();
   pp_inv_sqrt(c, a.M);
   if (lead) out[3] = (double)sh->flag;
-  if (a.Kd) {  // K_next = X_new^T D = M (X^T D + t D^T D)
+  if (a.Kd) {
+    // K_next = X_new^T D = M (X^T D + t D^T D) in float64: it goes into the
+    // next direction and X^T D with no correction after it. The operands
+    // leave df64 once (a conversion costs as much as a multiply-add): T =
+    // X^T D + t B in the space of T, from there staged for NC > 1, the rows
+    // of M in that of V (the strip of X).
+    double *T = reinterpret_cast<double*>(c.mat(c.Td)), *Mr;
     pp_each(c, [&](int i, int j) {
-      c.mat(c.Td)[i * c.ld + j] = df_add(c.mat(c.Bd)[i * c.ld + j], df_mul(td, elem(a.B, i, j)));
+      T[i * p + j] = fma(t, elem(a.B, i, j), df_to_double(c.mat(c.Bd)[i * c.ld + j]));
     });
-    pp_sync<P>();
-    pp_mm(c, c.Ud, false, c.Td, false, c.Bd);
-    pp_sync<P>();
+    if constexpr (P::NC == 1) {
+      Mr = reinterpret_cast<double*>(pp_s2(c.Vd));
+    } else {
+      pp_sync<P>();
+      const double* const Tg = T;
+      T = reinterpret_cast<double*>(pp_s2(c.sY));
+      Mr = reinterpret_cast<double*>(pp_s2(c.sX));
+      for (int e = c.tid; e < p * p; e += P::NT) T[e] = __ldcg(Tg + e);
+    }
+    pp_each(c, [&](int i, int j) { Mr[(i - c.r0) * p + j] = df_to_double(c.mat(c.Ud)[i * c.ld + j]); });
+    __syncthreads();
     pp_each(c, [&](int i, int j) {
-      const float2 v = c.mat(c.Bd)[i * c.ld + j];
-      a.Kd[i * p + j] = df_to_double(v);
-      if (a.Kf) a.Kf[i * p + j] = v;
+      const double* const mr = Mr + (i - c.r0) * p;
+      double v = 0.0;
+#pragma unroll 4
+      for (int k = 0; k < p; ++k) v = fma(mr[k], T[k * p + j], v);
+      a.Kd[i * p + j] = v;
+      if (a.Kf) a.Kf[i * p + j] = df_from_double(v);
     });
   }
   if (lead) {

@@ -393,10 +393,11 @@ gsi_status op_rowinf(gsi_ctx* c, const void* Rb) {
   return s;
 }
 
-// a p x p input of the df64 step: the df64 copy where there is one
+// a p x p input of the df64 step, with its df64 copy where there is one (B and
+// XX are exactly symmetric then)
 PpMat pp_in(gsi_ctx* c, const double* G) {
   float2* f = pp_df(c, G);
-  return f ? PpMat{f, nullptr, 0} : PpMat{nullptr, G, 1};
+  return PpMat{f, G, f ? 0 : 1};
 }
 
 // The df64 p x p step (PpArgs, pp_dev.cuh): mode 1 with B; mode 2 with B,

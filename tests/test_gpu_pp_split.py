@@ -1,6 +1,7 @@
 """The df64 p x p step in the two launches of the solver: both forms of the
-eigenbasis for 32 < p <= 64 (one CTA, which large n takes, and a cluster) and
-spectra of B whose gaps put the corrections K on either side of their limits."""
+eigenbasis for 32 < p <= 64 (one CTA, which large n takes, and a cluster),
+spectra of B whose gaps put the corrections K on either side of their limits,
+and the next K = M (X^T D + t B), which is a float64 product."""
 import numpy as np
 import pytest
 
@@ -78,6 +79,27 @@ def test_gaps_around_the_limits(torch_cuda, p, cluster, lo):
     XD = (np.eye(p) - XX) @ C
     S = XX + t * (XD + XD.T) + t * t * B
     _check_polar(M, 0.5 * (S + S.T), p)
+
+
+@pytest.mark.parametrize("p,cluster", [(1, False), (4, False), (8, False), (15, False), (16, False), (17, False),
+                                       (32, False), (33, False), (64, False), (64, True), (65, True), (128, True)])
+def test_next_k_is_a_float64_product(torch_cuda, p, cluster):
+    rng = np.random.default_rng(p)
+    X, A, C, R, D = _problem(p, "plain", rng)
+    B, Gam, Z, XX = _grams(X, A, D, R)
+    K = 1e-3 * rng.standard_normal((p, p))
+    beta = 0.7
+    M, Kn, o = _step(torch_cuda, C, B, Gam, Z, XX, K, beta, cluster)
+    L = np.longdouble
+    E = np.eye(p, dtype=L) - 0.5 * (XX + XX.T).astype(L)
+    XD = E @ (C.astype(L) + L(beta) * K.astype(L))
+    T = XD + L(o[0]) * (0.5 * (B + B.T)).astype(L)
+    ref = M.astype(L) @ T
+    # p float64 additions; X^T D = (I - XX)(C + beta K) carries df64 rounding
+    # of the (rounding-level) I - XX
+    size = np.abs(M) @ np.abs(T).astype(np.float64)
+    xd = np.abs(M) @ (np.abs(E).astype(np.float64) @ (np.abs(C) + beta * np.abs(K)))
+    assert np.all(np.abs(Kn - ref) <= (p + 3) * 2.0 ** -53 * size + (p + 4) * 2.0 ** -45 * xd)
 
 
 @pytest.mark.parametrize("p", [33, 64])
