@@ -796,8 +796,10 @@ gsi_status gsi_warm_loss_grad(int32_t batch, int32_t m, int32_t p, const int64_t
   void* ws = nullptr;
   GSI_CUDA_TRY(cudaMallocAsync(&ws, warm_ws_bytes(batch, m, p), st));
   const gsi_status s = loss_grad(batch, m, p, S_rowptr, S_colidx, S_val, C, Bt, SC_scratch, loss, dC, gscale, ws, st);
-  GSI_CUDA_TRY(cudaFreeAsync(ws, st));
-  return s;
+  const cudaError_t fe = cudaFreeAsync(ws, st);
+  GSI_TRY(s);
+  GSI_CUDA_TRY(fe);
+  return GSI_OK;
 }
 
 gsi_status gsi_warm_train_step(gsi_mlp* n, int32_t batch, const float* x, int32_t m, int32_t p,
@@ -805,29 +807,33 @@ gsi_status gsi_warm_train_step(gsi_mlp* n, int32_t batch, const float* x, int32_
                                const float* Bt, double lr, double* mean_loss) {
   if (!n || !x || !Bt || batch < 1 || batch > n->max_batch || p < 1 || p > 64 || (int64_t)m * p != n->dout)
     return GSI_ERR_ARG;
+  // a captured step gets a buffer of the graph's own: the kept one is
+  // replaced by a later, larger step, which a replay would not learn of
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  GSI_CUDA_TRY(cudaStreamIsCapturing(n->st, &cap));
   const size_t need = warm_ws_bytes(batch, m, p);
-  void *ws = n->loss_ws, *tmp = nullptr;
-  if (need > n->loss_ws_bytes) {
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    GSI_CUDA_TRY(cudaStreamIsCapturing(n->st, &cap));
-    if (cap != cudaStreamCaptureStatusNone) {  // recorded: a buffer of the graph's own
-      GSI_CUDA_TRY(cudaMallocAsync(&tmp, need, n->st));
-      ws = tmp;
-    } else {  // kept for later steps; grown on the first of a size
-      GSI_CUDA_TRY(cudaStreamSynchronize(n->st));
-      if (n->loss_ws) cudaFree(n->loss_ws);
+  void *ws = nullptr, *tmp = nullptr;
+  if (cap != cudaStreamCaptureStatusNone) {
+    GSI_CUDA_TRY(cudaMallocAsync(&tmp, need, n->st));
+    ws = tmp;
+  } else {
+    if (need > n->loss_ws_bytes) {  // stream-ordered: earlier steps on n->st may still use the old one
+      void* old = n->loss_ws;
       n->loss_ws = nullptr;
       n->loss_ws_bytes = 0;
-      const cudaError_t e = cudaMalloc(&n->loss_ws, need);
-      if (e != cudaSuccess) return cuda_status(e);
+      if (old) GSI_CUDA_TRY(cudaFreeAsync(old, n->st));
+      GSI_CUDA_TRY(cudaMallocAsync(&n->loss_ws, need, n->st));
       n->loss_ws_bytes = need;
-      ws = n->loss_ws;
     }
+    ws = n->loss_ws;
   }
-  GSI_TRY(mlp_forward(n, batch, x, n->out));
-  GSI_TRY(loss_grad(batch, m, p, S_rowptr, S_colidx, S_val, n->out, Bt, n->sc_buf, n->loss, n->dout_buf,
-                    1.f / batch, ws, n->st));
-  if (tmp) GSI_CUDA_TRY(cudaFreeAsync(tmp, n->st));
+  gsi_status ls = mlp_forward(n, batch, x, n->out);
+  if (ls == GSI_OK)
+    ls = loss_grad(batch, m, p, S_rowptr, S_colidx, S_val, n->out, Bt, n->sc_buf, n->loss, n->dout_buf, 1.f / batch,
+                   ws, n->st);
+  const cudaError_t fe = tmp ? cudaFreeAsync(tmp, n->st) : cudaSuccess;
+  GSI_TRY(ls);
+  GSI_CUDA_TRY(fe);
   GSI_TRY(mlp_backward(n, batch, x, n->dout_buf));
   GSI_TRY(mlp_adam(n, lr, 0.9, 0.999, 1e-8));
   if (mean_loss) {

@@ -1,0 +1,63 @@
+"""The warm-start network where a call can go wrong without a wrong size: a
+captured training step that outlives a larger one."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def _mass(torch, nc):
+    """P^T P of the bilinear prolongation is close to this tensor product (CSR, CUDA)."""
+    T = np.diag(np.full(nc, 2.0 / 3.0)) + np.diag(np.full(nc - 1, 1.0 / 6.0), 1) + np.diag(np.full(nc - 1, 1.0 / 6.0), -1)
+    S = np.kron(T, T)
+    r, c = np.nonzero(S)
+    rp = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=nc * nc))])
+    return S, tuple(torch.as_tensor(v, device="cuda")
+                    for v in (rp.astype(np.int64), c.astype(np.int32), S[r, c].astype(np.float64)))
+
+
+def test_captured_step_after_a_larger_one(torch_cuda):
+    """Warm-up, a captured step, a larger eager step, then a replay: the
+    replay's gradients are those of an eager step from the same weights."""
+    import ctypes
+    torch = torch_cuda
+    from paper_2306_10379_gb300 import gsi
+    nc, p, hid, big, small = 6, 4, 64, 48, 3
+    m = nc * nc
+    S, csr = _mass(torch, nc)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x = torch.randn(big, 16, generator=g, device="cuda")
+    Bt = torch.randn(big, m, p, generator=g, device="cuda") / m
+    w0 = 0.2 * np.random.default_rng(5).standard_normal(gsi.mlp_num_params(16, hid, m * p)).astype(np.float32)
+    st = torch.cuda.Stream()
+    st.wait_stream(torch.cuda.current_stream())
+    net = gsi.MLP(16, hid, m * p, w0, max_batch=big, stream=st)
+    xs, bs = x[:small].contiguous(), Bt[:small].contiguous()
+    st.wait_stream(torch.cuda.current_stream())
+
+    def enqueue():
+        f = gsi._f32
+        s = gsi.lib().gsi_warm_train_step(net._ctx, small, f(xs), m, p, gsi._dptr(csr[0], torch.int64),
+                                          gsi._dptr(csr[1], torch.int32), gsi._dptr(csr[2], torch.float64), f(bs),
+                                          ctypes.c_double(1e-3), None)
+        assert s == gsi.GSI_OK
+
+    with torch.cuda.stream(st):
+        net.train_step(xs, csr, bs, m, p, 1e-3)
+        graph = torch.cuda.CUDAGraph()
+        graph.capture_begin()
+        enqueue()
+        graph.capture_end()
+        net.train_step(x, csr, Bt, m, p, 1e-3)  # needs a larger scratch
+        for _ in range(3):
+            prm = gsi.MLP.flatten(net.params())
+            graph.replay()
+            st.synchronize()
+            got = net.grads()
+            ref_net = gsi.MLP(16, hid, m * p, prm, max_batch=big, stream=st)
+            ref_net.train_step(xs, csr, bs, m, p, 1e-3)
+            ref = ref_net.grads()
+            for k in ref:
+                assert np.all(np.isfinite(got[k])) and np.array_equal(got[k], ref[k]), k
+            net.train_step(x, csr, Bt, m, p, 1e-3)
+    del graph
