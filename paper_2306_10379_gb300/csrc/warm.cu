@@ -386,6 +386,8 @@ __global__ void __launch_bounds__(WT) warm_gram_kernel(int m, int p, const int64
 // 1/sqrt(d) in float64 from a float32 seed: the pipe's own root and division
 // are serial chains of many slow operations
 __device__ __forceinline__ double w_rsqrt(double d) {
+  const double up = d < 2.2250738585072014e-308 ? 18014398509481984.0 : 1.0;  // subnormal: times 2^54
+  d *= up;
   const int ex = ((__double2hiint(d) >> 20) & 0x7ff) - 1023;
   const int h = ex >= 0 ? ex / 2 : -((1 - ex) / 2);              // floor(ex / 2)
   const double sc = __hiloint2double((1023 - 2 * h) << 20, 0);   // d sc in [1, 4)
@@ -393,13 +395,15 @@ __device__ __forceinline__ double w_rsqrt(double d) {
   double y = (double)rsqrtf((float)x);
   y = y * fma(-0.5 * x, y * y, 1.5);
   y = y * fma(-0.5 * x, y * y, 1.5);
-  return y * __hiloint2double((1023 - h) << 20, 0);
+  return y * __hiloint2double((1023 - h + (up == 1.0 ? 0 : 27)) << 20, 0);
 }
 
 // Dynamic shared memory: 5 p^2 + p doubles. A1 = G N^{-1} and A2 = N^{-1} Q
-// N^{-1} (float32, 2 p^2 per sample) are NaN where N is not positive definite.
+// N^{-1}: float32, 2 p^2 per sample. status: 1 where N is not positive
+// definite (a loss can be NaN for other reasons), else 0.
 __global__ void __launch_bounds__(WT) warm_alg_kernel(int p, int nblk, const double* __restrict__ part,
-                                                      double* __restrict__ loss, float* __restrict__ Aall) {
+                                                      double* __restrict__ loss, float* __restrict__ Aall,
+                                                      int32_t* __restrict__ status) {
   extern __shared__ __align__(16) double wsm[];
   __shared__ int bad;
   __shared__ double trw[WT / 32];
@@ -508,19 +512,21 @@ __global__ void __launch_bounds__(WT) warm_alg_kernel(int p, int nblk, const dou
     double t = 0.0;
     for (int w = 0; w < WT / 32; ++w) t += trw[w];
     loss[s] = ok ? (double)p - t : NAN;
+    status[s] = bad;
   }
 }
 
 __global__ void __launch_bounds__(WT) warm_dc_kernel(int m, int p, const float* __restrict__ Btall,
                                                      const float* __restrict__ SCall,
-                                                     const float* __restrict__ Aall, const double* __restrict__ loss,
+                                                     const float* __restrict__ Aall,
+                                                     const int32_t* __restrict__ status,
                                                      float* __restrict__ dCall, float sc) {
   extern __shared__ __align__(16) float w_sm[];  // A1, A2, then 32 rows of Bt and SC at a time
   const int tid = threadIdx.x, q = p * p;
   float *a1 = w_sm, *a2 = a1 + q, *bt = a2 + q, *st = bt + 32 * p;
   const float* A = Aall + (size_t)blockIdx.y * 2 * q;
   for (int e = tid; e < 2 * q; e += WT) a1[e] = A[e];
-  const bool ok = !isnan(loss[blockIdx.y]);
+  const bool ok = status[blockIdx.y] == 0;
   const int64_t off = (int64_t)blockIdx.y * m * p;
   const int r0 = blockIdx.x * WR, r1 = min(m, r0 + WR);
   for (int b0 = r0; b0 < r1; b0 += 32) {
@@ -562,10 +568,10 @@ __global__ void __launch_bounds__(WT) warm_dc_kernel(int m, int p, const float* 
 size_t warm_alg_smem(int p) { return ((size_t)5 * p * p + p) * sizeof(double); }
 size_t warm_gram_smem(int p) { return (size_t)3 * WR * ((p + 3) & ~3) * sizeof(float); }
 size_t warm_dc_smem(int p) { return ((size_t)2 * p * p + 64 * p) * sizeof(float); }
-// partial Grams (float64), then A1 and A2 of every sample
+// partial Grams (float64), then A1 and A2 and the status of every sample
 size_t warm_ws_bytes(int batch, int m, int p) {
   const size_t nblk = (m + WR - 1) / WR, q = (size_t)p * p;
-  return (size_t)batch * (nblk * 2 * q * sizeof(double) + 2 * q * sizeof(float));
+  return (size_t)batch * (nblk * 2 * q * sizeof(double) + 2 * q * sizeof(float) + sizeof(int32_t));
 }
 
 }  // namespace
@@ -680,6 +686,7 @@ gsi_status loss_grad(int batch, int m, int p, const int64_t* Srp, const int32_t*
   const int nblk = (m + WR - 1) / WR;
   double* part = reinterpret_cast<double*>(ws);
   float* A = reinterpret_cast<float*>(part + (size_t)batch * nblk * 2 * p * p);
+  int32_t* status = reinterpret_cast<int32_t*>(A + (size_t)batch * 2 * p * p);
   GSI_CUDA_TRY(ensure_dyn_smem((const void*)warm_gram_kernel, (int)warm_gram_smem(p)));
   GSI_CUDA_TRY(ensure_dyn_smem((const void*)warm_alg_kernel, (int)warm_alg_smem(p)));
   GSI_CUDA_TRY(ensure_dyn_smem((const void*)warm_dc_kernel, (int)warm_dc_smem(p)));
@@ -691,9 +698,9 @@ gsi_status loss_grad(int batch, int m, int p, const int64_t* Srp, const int32_t*
     float* Ab = A + (size_t)b0 * 2 * p * p;
     warm_gram_kernel<<<dim3(nblk, nb), WT, warm_gram_smem(p), st>>>(m, p, Srp, Sci, Sv, C + o, Bt + o, SC + o, pt);
     GSI_LAUNCH_CHECK();
-    warm_alg_kernel<<<nb, WT, warm_alg_smem(p), st>>>(p, nblk, pt, loss + b0, Ab);
+    warm_alg_kernel<<<nb, WT, warm_alg_smem(p), st>>>(p, nblk, pt, loss + b0, Ab, status + b0);
     GSI_LAUNCH_CHECK();
-    warm_dc_kernel<<<dim3(nblk, nb), WT, warm_dc_smem(p), st>>>(m, p, Bt + o, SC + o, Ab, loss + b0, dC + o,
+    warm_dc_kernel<<<dim3(nblk, nb), WT, warm_dc_smem(p), st>>>(m, p, Bt + o, SC + o, Ab, status + b0, dC + o,
                                                                -2.f * gscale);
     GSI_LAUNCH_CHECK();
   }

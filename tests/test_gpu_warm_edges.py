@@ -1,5 +1,6 @@
 """The warm-start network where a call can go wrong without a wrong size: a
-captured training step that outlives a larger one."""
+captured training step that outlives a larger one, and samples whose data or
+whose N are bad."""
 import numpy as np
 import pytest
 
@@ -61,3 +62,29 @@ def test_captured_step_after_a_larger_one(torch_cuda):
                 assert np.all(np.isfinite(got[k])) and np.array_equal(got[k], ref[k]), k
             net.train_step(x, csr, Bt, m, p, 1e-3)
     del graph
+
+
+@pytest.mark.parametrize("what", ["nan", "inf"])
+def test_bad_samples(torch_cuda, what):
+    """dC = 0 only where N is not positive definite: NaN or infinity in a
+    sample's Bt shows in its loss and gradient; the other samples are as without it."""
+    torch = torch_cuda
+    from paper_2306_10379_gb300 import gsi
+    nc, p, batch = 5, 4, 4
+    m = nc * nc
+    S, csr = _mass(torch, nc)
+    g = torch.Generator(device="cuda").manual_seed(6)
+    C = torch.randn(batch, m, p, generator=g, device="cuda")
+    Bt = torch.randn(batch, m, p, generator=g, device="cuda") / m
+    C[3, :, 1] = 0.0  # N singular
+    loss0, dC0 = gsi.warm_loss_grad(C, csr, Bt, m, p)
+    Bt[1, 7, 2] = float(what)
+    loss, dC = gsi.warm_loss_grad(C, csr, Bt, m, p)
+    for s in (0, 2):
+        assert torch.equal(loss[s], loss0[s]) and torch.equal(dC[s], dC0[s]) and bool(torch.isfinite(dC[s]).all())
+    assert not bool(torch.isfinite(loss[1]))
+    # G = Bt^T C is not finite in a whole row, so no row of dC can be
+    assert not bool(torch.isfinite(dC[1]).any())
+    for q in (loss0, loss):
+        assert bool(torch.isnan(q[3]))
+    assert bool((dC0[3] == 0).all()) and bool((dC[3] == 0).all())
