@@ -296,7 +296,9 @@ constexpr int WT = 256;
 constexpr int WR = 128;  // rows of a block, a multiple of 32
 constexpr int WNZ = 1536;  // entries of S staged per block (bilinear elements: 9 a row)
 
-// acc += a x with a split in two floats: float64-class in float32 arithmetic
+// acc += a x with a split in two floats: 2^-46 of the terms in float32
+// arithmetic, for a sum that is rounded to float32 (C's range decides its
+// overflow and underflow as long as |a| lies in [2^-100, 2^60))
 __device__ __forceinline__ void w_mac(float& h, float& e, float2 a, float x) {
   const float p = __fmul_rn(a.x, x);
   const float pe = __fmaf_rn(a.x, x, -p);
@@ -323,11 +325,20 @@ __global__ void __launch_bounds__(WT) warm_gram_kernel(int m, int p, const int64
   const float* C = Call + off;
   const int r0 = blockIdx.x * WR, nr = min(WR, m - r0);
   const int64_t k0 = Srp[r0], kn = min((int64_t)WNZ, Srp[r0 + nr] - k0);
+  // float64 compares are slow: the exponent field decides
+  auto in_range = [](double v) {
+    const uint32_t hi = (uint32_t)__double2hiint(v) & 0x7fffffffu;
+    return (hi | (uint32_t)__double2loint(v)) == 0u || hi - ((1023u - 100u) << 20) < (160u << 20);
+  };
+  bool range = true;
   for (int k = tid; k < kn; k += WT) {
-    sval[k] = df_from_double(Sv[k0 + k]);
+    const double v = Sv[k0 + k];
+    range = range && in_range(v);
+    sval[k] = df_from_double(v);
     scol[k] = Sci[k0 + k];
   }
-  __syncthreads();
+  for (int64_t k = kn + tid; k < Srp[r0 + nr] - k0; k += WT) range = range && in_range(Sv[k0 + k]);
+  const bool pairs = __syncthreads_and(range);
   for (int e = tid; e < WR * pp; e += WT) {
     const int r = e / pp, c = e - r * pp;
     const bool ok = r < nr && c < p;
@@ -345,6 +356,15 @@ __global__ void __launch_bounds__(WT) warm_gram_kernel(int m, int p, const int64
     ss[e] = sc;
     if (ok) SCall[off + (int64_t)(r0 + r) * p + c] = sc;
   }
+  if (!pairs)  // some value beyond a pair's range: S C again, in float64
+    for (int e = tid; e < WR * pp; e += WT) {
+      const int r = e / pp, c = e - r * pp;
+      if (r >= nr || c >= p) continue;
+      double a = 0.0;
+      for (int64_t k = Srp[r0 + r]; k < Srp[r0 + r + 1]; ++k) a += Sv[k] * (double)C[(int64_t)Sci[k] * p + c];
+      ss[e] = (float)a;
+      SCall[off + (int64_t)(r0 + r) * p + c] = (float)a;
+    }
   __syncthreads();
   // N = C^T SC and G = Bt^T C: a thread forms 4 x 2 entries
   const int ti = pp / 4, tj = (p + 1) / 2;
@@ -386,16 +406,15 @@ __global__ void __launch_bounds__(WT) warm_gram_kernel(int m, int p, const int64
 // 1/sqrt(d) in float64 from a float32 seed: the pipe's own root and division
 // are serial chains of many slow operations
 __device__ __forceinline__ double w_rsqrt(double d) {
-  const double up = d < 2.2250738585072014e-308 ? 18014398509481984.0 : 1.0;  // subnormal: times 2^54
-  d *= up;
   const int ex = ((__double2hiint(d) >> 20) & 0x7ff) - 1023;
+  if (ex == -1023) return 1.0 / sqrt(d);  // subnormal
   const int h = ex >= 0 ? ex / 2 : -((1 - ex) / 2);              // floor(ex / 2)
   const double sc = __hiloint2double((1023 - 2 * h) << 20, 0);   // d sc in [1, 4)
   const double x = d * sc;
   double y = (double)rsqrtf((float)x);
   y = y * fma(-0.5 * x, y * y, 1.5);
   y = y * fma(-0.5 * x, y * y, 1.5);
-  return y * __hiloint2double((1023 - h + (up == 1.0 ? 0 : 27)) << 20, 0);
+  return y * __hiloint2double((1023 - h) << 20, 0);
 }
 
 // Dynamic shared memory: 5 p^2 + p doubles. A1 = G N^{-1} and A2 = N^{-1} Q

@@ -1,6 +1,6 @@
 """The warm-start network where a call can go wrong without a wrong size: a
 captured training step that outlives a larger one, and samples whose data or
-whose N are bad."""
+whose N are bad, and operators far from one in scale."""
 import numpy as np
 import pytest
 
@@ -88,3 +88,41 @@ def test_bad_samples(torch_cuda, what):
     for q in (loss0, loss):
         assert bool(torch.isnan(q[3]))
     assert bool((dC0[3] == 0).all()) and bool((dC[3] == 0).all())
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-42, 1e42, 1e-150])
+def test_scaled_operator(torch_cuda, scale):
+    """S of any float64 scale: N = C^T S C in range, loss and dC C^T unchanged
+    by S -> a S, C -> C / sqrt(a) (a power of two), Bt as it is scaled."""
+    torch = torch_cuda
+    from paper_2306_10379_gb300 import gsi
+    nc, p, batch = 7, 5, 3
+    m = nc * nc
+    a = 2.0 ** (2 * round(np.log2(scale) / 2))
+    c = 2.0 ** np.clip(round(np.log2(1.0 / a) / 2), -60, 60)  # C stays a float32, and C^T S C too
+    rng = np.random.default_rng(8)
+    S, csr = _mass(torch, nc)
+    S = S * (1.0 + 0.1 * rng.random(S.shape))  # 53-bit values
+    S = 0.5 * (S + S.T)
+    r, col = np.nonzero(S)
+    sv = torch.as_tensor(a * S[r, col], device="cuda")
+    C = (c * rng.standard_normal((batch, m, p))).astype(np.float32)
+    Bt = (rng.standard_normal((batch, m, p)) / (m * c)).astype(np.float32)
+    loss, dC = gsi.warm_loss_grad(torch.as_tensor(C, device="cuda"), (csr[0], csr[1], sv),
+                                  torch.as_tensor(Bt, device="cuda"), m, p)
+    for s in range(batch):
+        c64, b64 = C[s].astype(np.float64), Bt[s].astype(np.float64)
+        SC = (a * S) @ c64
+        if np.abs(SC).max() < 1e-30:  # S C underflows in float32: N is zero, not positive definite
+            assert np.isnan(float(loss[s])) and bool((dC[s] == 0).all())
+            continue
+        N, G = c64.T @ SC, b64.T @ c64
+        Ni = np.linalg.inv(0.5 * (N + N.T))
+        Q = G.T @ G
+        # as test_gpu_warm_shapes: N and G carry float32 sums of 32 terms
+        eps = 40 * 2.0 ** -24 * np.linalg.cond(N)
+        tr = np.trace(Ni @ Q)
+        assert abs(float(loss[s]) - (p - tr)) <= eps * max(p, tr)
+        d = -2.0 * (b64 @ (G @ Ni) - SC @ (Ni @ Q @ Ni))
+        assert np.linalg.norm(dC[s].cpu().numpy() - d) <= eps * max(np.linalg.norm(b64) * np.linalg.norm(G @ Ni),
+                                                                   np.linalg.norm(d))
