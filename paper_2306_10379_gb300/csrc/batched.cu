@@ -1673,14 +1673,11 @@ gsi_status gsi_batched_create(int32_t nprob, const int32_t* n, const int32_t* p,
   CK(cuda_status_ok(cudaMemset(b->Km, 0, (size_t)pp * sizeof(double))));
   {
     b->small_smem = pp_smem(pmax, 1);
-    CK(cuda_status_ok(cudaFuncSetAttribute(b_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)b->small_smem)));
-    CK(cuda_status_ok(cudaFuncSetAttribute(b_gram_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)sizeof(GramSm<1>))));
-    CK(cuda_status_ok(cudaFuncSetAttribute(b_gram_kernel<NG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)sizeof(GramSm<NG>))));
-    CK(cuda_status_ok(cudaFuncSetAttribute(b_retract_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)sizeof(RowSm<2>))));
+    // only ever raised: batches of other widths share the kernels
+    CK(cuda_status_ok(ensure_dyn_smem((const void*)b_small_kernel, (int)b->small_smem)));
+    CK(cuda_status_ok(ensure_dyn_smem((const void*)b_gram_kernel<1>, (int)sizeof(GramSm<1>))));
+    CK(cuda_status_ok(ensure_dyn_smem((const void*)b_gram_kernel<NG>, (int)sizeof(GramSm<NG>))));
+    CK(cuda_status_ok(ensure_dyn_smem((const void*)b_retract_kernel, (int)sizeof(RowSm<2>))));
   }
   CK(set_tiles(b, 2048, 4, 4));
   CK(start(b));
