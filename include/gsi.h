@@ -529,8 +529,8 @@ gsi_status gsi_batched_get_tiles(gsi_batch* b, int32_t* tile_max, int32_t* ctas_
 gsi_status gsi_batched_last_plan(gsi_batch* b, int32_t* ntiles, int32_t* tile_prob,
                                  int32_t* tile_row0, int32_t* tile_rows, int32_t capacity);
 /* Autotuner: times npasses passes from the start for every candidate tile
- * shape (tile_max 256..4096, 2/4/8 CTAs per SM, 1/2/4 tiles per CTA), keeps
- * the fastest and restarts the batch from X0. Outputs may be NULL. */
+ * shape (tile_max 256..4096, 2/4/8 CTAs per SM, 1/2 tiles per CTA; every tile has
+ * a CTA, so 8 x 2 also stands for the default's 4 x 4), keeps the fastest and restarts the batch from X0. Outputs may be NULL. */
 gsi_status gsi_batched_tune(gsi_batch* b, int32_t npasses, int32_t* tile_max, int32_t* ctas_per_sm,
                             int32_t* tiles_per_cta, double* ms_per_pass);
 /* Back to the orthonormalised X0. */

@@ -1751,7 +1751,7 @@ gsi_status gsi_batched_tune(gsi_batch* b, int32_t npasses, int32_t* tile_max, in
   if (!b || npasses < 1) return GSI_ERR_ARG;
   static const int cand_rows[] = {256, 512, 1024, 2048, 4096};
   static const int cand_ctas[] = {2, 4, 8};
-  static const int cand_tpc[] = {1, 2, 4};
+  static const int cand_tpc[] = {1, 2};
   cudaEvent_t e0, e1;
   GSI_CUDA_TRY(cudaEventCreate(&e0));
   GSI_CUDA_TRY(cudaEventCreate(&e1));
