@@ -185,11 +185,12 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;\n" 
 // G = 1: sel 0 -> X^T Y, sel 1 -> X^T X, sel 2 -> X^T W.
 // G = 4: D^T D, D^T W, D^T R, X^T X (the line-search Grams, Eqs. (diags),
 // (CG_linesearch_D), and the measured X^T X of the polar factor).
-// D^T D, X^T X and D^T W (W = A D explicitly) are symmetric: their upper half
-// is formed, and mirrored. X^T Y is formed in full: Y follows A X by a
-// recursion, and X^T D = (I - X^T X)(C + beta K) takes C to be the symmetric
-// part of X^T Y exactly (mirrored, X^T X - I grew from 5e-13 to 2.5e-12 over
-// a solve). A thread owns 4 x 4 output blocks -- columns 2b, 2b+1,
+// D^T D and X^T X are symmetric: their upper half is formed, and mirrored.
+// D^T W is symmetric as far as A is: formed in full, and averaged with its
+// transpose by the reduction, as the single-problem solver does. X^T Y is
+// formed in full too: Y follows A X by a recursion, and X^T D = (I - X^T X)(C +
+// beta K) takes C to be the symmetric part of X^T Y exactly (mirrored,
+// X^T X - I grew from 5e-13 to 2.5e-12 over a solve). A thread owns 4 x 4 output blocks -- columns 2b, 2b+1,
 // p/2 + 2b, p/2 + 2b + 1, which keeps its 16-byte loads of a row free of bank
 // conflicts -- over the rows s, s + S, ... of a staged chunk; chunks are
 // double-buffered with cp.async. At p = 32, which is where the multiply-adds
@@ -201,7 +202,8 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;\n" 
 // tenth): 48 problems of 2048..65536 rows, p in {4, 8, 16, 32}, together
 // 1.6e6 rows, take 880 us for G = 4 (2 x 2 blocks, full products and TwoProd
 // + TwoSum throughout: 1770) and 400 us for G = 1 (465).
-constexpr int GT = 192;     // 172 blocks of 4 x 4 at p = 32, G = 4
+template <int G>
+constexpr int GT = G == 4 ? 224 : 192;  // threads: 200 and 64 blocks of 4 x 4 at p = 32
 constexpr int kGE = 512;    // most elements of an array per chunk
 
 template <int G>
@@ -209,9 +211,9 @@ struct GramSm {
   static constexpr int NA = G == 4 ? 4 : 2;
   union {
     float4 st[2][NA][kGE / 2];
-    double red[GT * 16];  // at the end: [row group][entry of the block][block]
+    double red[GT<G> * 16];  // at the end: [row group][entry of the block][block]
   };
-  float wmax[NA][GT / 32][PMAX], wsum[NA][GT / 32][PMAX];
+  float wmax[NA][GT<G> / 32][PMAX], wsum[NA][GT<G> / 32][PMAX];
   float cf[NA][PMAX], cg[NA][PMAX];
 };
 
@@ -219,10 +221,10 @@ template <int G, int P>
 __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const BProb& pr, int sel,
                                           GramSm<G>& sm) {
   constexpr int U = P >= 4 ? 4 : 2, NB = P / U, SYM = NB * (NB + 1) / 2;
-  constexpr int UNITS = (G == 4 ? 3 * SYM : 0) + NB * NB;
-  constexpr int S = GT / UNITS, RC = (G == 4 && P == 32 ? kGE / 2 : kGE) / P, H4 = P / 2, NA = GramSm<G>::NA;
+  constexpr int UNITS = G == 4 ? 2 * SYM + 2 * NB * NB : NB * NB;  // D^T D, D^T W, D^T R, X^T X or one full product
+  constexpr int T = GT<G>, S = T / UNITS, RC = (G == 4 && P == 32 ? kGE / 2 : kGE) / P, H4 = P / 2, NA = GramSm<G>::NA;
   constexpr bool OFFSET = G == 4 && P == 32;
-  static_assert(S >= 1 && GT % H4 == 0 && NA * P <= GT, "thread mapping");
+  static_assert(S >= 1 && T % H4 == 0 && NA * P <= T, "thread mapping");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nload = G == 4 ? 4 : (sel == 1 ? 1 : 2);
   const float2* src[NA];
@@ -241,10 +243,10 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
     g = 0;
     if (G == 4) {
       if (unit >= SYM) g = 1, unit -= SYM;
-      if (g == 1 && unit >= SYM) g = 2, unit -= SYM;
+      if (g == 1 && unit >= NB * NB) g = 2, unit -= NB * NB;
       if (g == 2 && unit >= NB * NB) g = 3, unit -= NB * NB;
     }
-    if (G == 1 || g == 2) {
+    if (G == 1 || g == 1 || g == 2) {
       bi = unit / NB;
       bj = unit % NB;
     } else {
@@ -268,7 +270,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
     const int64_t off = pr.boff + (int64_t)(tl.row0 + c0) * P;
     for (int a = 0; a < nload; ++a) {
       const float4* g4 = reinterpret_cast<const float4*>(src[a] + off);
-      for (int i = tid; i < cnt; i += GT) cp16(&sm.st[buf][a][i], g4 + i);
+      for (int i = tid; i < cnt; i += T) cp16(&sm.st[buf][a][i], g4 + i);
     }
   };
   __syncthreads();  // the last tile's sums have been read
@@ -282,7 +284,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
     // the chunk's column maxima and column sums of |.|
     for (int a = 0; OFFSET && a < nload; ++a) {
       float m0 = 0.f, m1 = 0.f, t0 = 0.f, t1 = 0.f;
-      for (int i = tid; i < rows * H4; i += GT) {
+      for (int i = tid; i < rows * H4; i += T) {
         const float4 v = sm.st[buf][a][i];
         m0 = fmaxf(m0, fabsf(v.x));
         m1 = fmaxf(m1, fabsf(v.z));
@@ -307,7 +309,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
       const int a = tid / P, c = tid % P;
       float m = 0.f, t = 0.f;
 #pragma unroll
-      for (int w = 0; w < GT / 32; ++w) {
+      for (int w = 0; w < T / 32; ++w) {
         m = fmaxf(m, sm.wmax[a][w][c]);
         t += sm.wsum[a][w][c];
       }
@@ -371,7 +373,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
   }
   __syncthreads();
   double* out = d.parts + tl.part;
-  for (int k = tid; k < UNITS * U * U; k += GT) {
+  for (int k = tid; k < UNITS * U * U; k += T) {
     double v = 0.0;
     for (int z = 0; z < S; ++z) v += sm.red[z * U * U * UNITS + k];
     int gk, bik, bjk;
@@ -379,7 +381,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
     decode(k % UNITS, gk, bik, bjk);
     const int i = col(bik, q / U), j = col(bjk, q % U);
     out[gk * P * P + i * P + j] = v;
-    if (bik != bjk && G == 4 && gk != 2) out[gk * P * P + j * P + i] = v;
+    if (bik != bjk && G == 4 && gk != 1 && gk != 2) out[gk * P * P + j * P + i] = v;
   }
 }
 
@@ -1420,7 +1422,7 @@ gsi_status launch_pass(gsi_batch* b, cudaStream_t s, int32_t use_cond) {
   const int g = tile_grid(b), np = b->nprob;
   b_plan_kernel<<<1, 1024, 0, s>>>(d, F_ACTIVE);
   GSI_LAUNCH_CHECK();
-  b_gram_kernel<1><<<g, GT, sizeof(GramSm<1>), s>>>(d, F_ACTIVE, 0);  // C = X^T Y
+  b_gram_kernel<1><<<g, GT<1>, sizeof(GramSm<1>), s>>>(d, F_ACTIVE, 0);  // C = X^T Y
   GSI_LAUNCH_CHECK();
   b_reduce_kernel<<<rgrid(b, 1), 256, 0, s>>>(d, F_ACTIVE, 1, 1, 0);
   GSI_LAUNCH_CHECK();
@@ -1438,7 +1440,7 @@ gsi_status launch_pass(gsi_batch* b, cudaStream_t s, int32_t use_cond) {
   }
   b_spmm_kernel<<<g, BT, 0, s>>>(d, F_STEP, 0);  // W = A D
   GSI_LAUNCH_CHECK();
-  b_gram_kernel<NG><<<g, GT, sizeof(GramSm<NG>), s>>>(d, F_STEP, 0);
+  b_gram_kernel<NG><<<g, GT<NG>, sizeof(GramSm<NG>), s>>>(d, F_STEP, 0);
   GSI_LAUNCH_CHECK();
   // D^T D, D^T W, X^T X symmetrised; D^T R as it is
   b_reduce_kernel<<<rgrid(b, NG), 256, 0, s>>>(d, F_STEP, NG, 1 | 2 | 8, 1);
@@ -1465,7 +1467,7 @@ gsi_status start(gsi_batch* b) {
   b_plan_kernel<<<1, 1024, 0, s>>>(d, F_START);
   GSI_LAUNCH_CHECK();
   for (int pass = 0; pass < 2; ++pass) {
-    b_gram_kernel<1><<<g, GT, sizeof(GramSm<1>), s>>>(d, F_START, 1);  // X^T X
+    b_gram_kernel<1><<<g, GT<1>, sizeof(GramSm<1>), s>>>(d, F_START, 1);  // X^T X
     GSI_LAUNCH_CHECK();
     b_reduce_kernel<<<rgrid(b, 1), 256, 0, s>>>(d, F_START, 1, 1, 1);
     GSI_LAUNCH_CHECK();
@@ -1863,7 +1865,7 @@ gsi_status gsi_batched_get_basis(gsi_batch* b, int32_t i, double* X, double* eva
     GSI_LAUNCH_CHECK();
     b_spmm_kernel<<<g, BT, 0, s>>>(d, F_START, 2);
     GSI_LAUNCH_CHECK();
-    b_gram_kernel<1><<<g, GT, sizeof(GramSm<1>), s>>>(d, F_START, 2);
+    b_gram_kernel<1><<<g, GT<1>, sizeof(GramSm<1>), s>>>(d, F_START, 2);
     GSI_LAUNCH_CHECK();
     b_reduce_kernel<<<rgrid(b, 1), 256, 0, s>>>(d, F_START, 1, 1, 1);
     GSI_LAUNCH_CHECK();
