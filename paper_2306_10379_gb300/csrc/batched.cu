@@ -144,33 +144,6 @@ __device__ float bmaxf(float v, float* red) {
   return s;
 }
 
-// ---- sums against an offset ---------------------------------------------------
-// A sum of df64 products whose partial sums are bounded beforehand by 2^k
-// starts at sigma = 1.5 * 2^k instead of 0. Every partial sum S then lies in
-// [2^(k-1), 2.5 * 2^k], so S_new - S is exact, the fma that made S_new has
-// rounded the product to a multiple of S's ulp, and a second fma returns what
-// that rounding left: product and accumulation take 6 float32 operations
-// instead of the 12 of TwoProd + TwoSum (bmac). What the rounding leaves is
-// at most 2^(k-23), and its sum e keeps a further 24 bits. The bound is
-// Hoelder's, max |a| times sum |b|, over few rows: the error grows with their
-// number to the power 3/2, that of all rows with the square root.
-constexpr float kBoundMax = 4.2535296e37f;  // 2^125
-
-// 1.5 times the power of two above the bound v >= 0 (at least 2^-126)
-__device__ __forceinline__ float sigma_of(float f, float g) {
-  return 1.5f * __uint_as_float((__float_as_uint(fminf(f * g, kBoundMax)) & 0x7f800000u) + 0x00800000u);
-}
-
-// S + e += a b
-__device__ __forceinline__ void omac(float& S, float& e, float2 a, float2 b) {
-  const float n = __fmaf_rn(a.x, b.x, S);
-  float r = __fmaf_rn(a.x, b.x, -__fsub_rn(n, S));
-  r = __fmaf_rn(a.y, b.x, r);
-  r = __fmaf_rn(a.x, b.y, r);
-  S = n;
-  e = __fadd_rn(e, r);
-}
-
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
@@ -190,18 +163,18 @@ __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_all;\n" 
 // transpose by the reduction, as the single-problem solver does. X^T Y is
 // formed in full too: Y follows A X by a recursion, and X^T D = (I - X^T X)(C +
 // beta K) takes C to be the symmetric part of X^T Y exactly (mirrored,
-// X^T X - I grew from 5e-13 to 2.5e-12 over a solve). A thread owns 4 x 4 output blocks -- columns 2b, 2b+1,
-// p/2 + 2b, p/2 + 2b + 1, which keeps its 16-byte loads of a row free of bank
-// conflicts -- over the rows s, s + S, ... of a staged chunk; chunks are
-// double-buffered with cp.async. At p = 32, which is where the multiply-adds
-// are, the sums over a chunk's 8 rows run against the offsets of its own
-// columns and are added to df64 totals by TwoSum; at p <= 16 a block sums by
-// TwoProd + TwoSum throughout (offsets taken over a chunk of many short rows
-// were up to 10 times less accurate there).
-// Bound by instruction issue (0.57 of the slots, 18 warps per SM; DRAM at a
+// X^T X - I grew from 5e-13 to 2.5e-12 over a solve). A thread owns 4 x 4
+// output blocks -- columns 2b, 2b+1, p/2 + 2b, p/2 + 2b + 1, which keeps its
+// 16-byte loads of a row free of bank conflicts -- over the rows s, s + S, ...
+// of a staged chunk; chunks are double-buffered with cp.async. Sums are TwoProd + TwoSum throughout, as in
+// the single-problem path. (At p = 32, offsets of 1.5 times a power of two
+// above a chunk's bound max |a| sum |b| take half the operations, but their
+// rounding is relative to that bound, not to the terms: 880 us against 1064.)
+// Bound by instruction issue (0.75 of the slots, 21 warps per SM; DRAM at a
 // tenth): 48 problems of 2048..65536 rows, p in {4, 8, 16, 32}, together
-// 1.6e6 rows, take 880 us for G = 4 (2 x 2 blocks, full products and TwoProd
-// + TwoSum throughout: 1770) and 400 us for G = 1 (465).
+// 1.6e6 rows, take 1064 us for G = 4 and 370 us for G = 1 (2 x 2 blocks of
+// every product: 1975 and 475), with 80 registers (112, two resident CTAs
+// for G = 4: a pass 3.45 instead of 3.36 ms).
 template <int G>
 constexpr int GT = G == 4 ? 224 : 192;  // threads: 200 and 64 blocks of 4 x 4 at p = 32
 constexpr int kGE = 512;    // most elements of an array per chunk
@@ -213,8 +186,6 @@ struct GramSm {
     float4 st[2][NA][kGE / 2];
     double red[GT<G> * 16];  // at the end: [row group][entry of the block][block]
   };
-  float wmax[NA][GT<G> / 32][PMAX], wsum[NA][GT<G> / 32][PMAX];
-  float cf[NA][PMAX], cg[NA][PMAX];
 };
 
 template <int G, int P>
@@ -222,10 +193,9 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
                                           GramSm<G>& sm) {
   constexpr int U = P >= 4 ? 4 : 2, NB = P / U, SYM = NB * (NB + 1) / 2;
   constexpr int UNITS = G == 4 ? 2 * SYM + 2 * NB * NB : NB * NB;  // D^T D, D^T W, D^T R, X^T X or one full product
-  constexpr int T = GT<G>, S = T / UNITS, RC = (G == 4 && P == 32 ? kGE / 2 : kGE) / P, H4 = P / 2, NA = GramSm<G>::NA;
-  constexpr bool OFFSET = G == 4 && P == 32;
-  static_assert(S >= 1 && T % H4 == 0 && NA * P <= T, "thread mapping");
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int T = GT<G>, S = T / UNITS, RC = kGE / P, H4 = P / 2, NA = GramSm<G>::NA;
+  static_assert(S >= 1, "thread mapping");
+  const int tid = threadIdx.x;
   const int nload = G == 4 ? 4 : (sel == 1 ? 1 : 2);
   const float2* src[NA];
   if (G == 4) {
@@ -259,7 +229,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
   decode(tid % UNITS, g, bi, bj);
   const int ia = G == 4 ? (g == 3 ? 3 : 0) : 0;
   const int ib = G == 4 ? g : (nload == 1 ? 0 : 1);
-  auto col = [&](int b, int q) { return U == 4 && q >= 2 ? P / 2 + 2 * b + q - 2 : 2 * b + q; };
+  auto col = [](int b, int q) { return U == 4 && q >= 2 ? P / 2 + 2 * b + q - 2 : 2 * b + q; };
   float H[U][U], E[U][U];
 #pragma unroll
   for (int a = 0; a < U; ++a)
@@ -281,53 +251,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
     cp_wait();
     __syncthreads();
     if (c0 + RC < tl.rows) issue(buf ^ 1, c0 + RC);
-    // the chunk's column maxima and column sums of |.|
-    for (int a = 0; OFFSET && a < nload; ++a) {
-      float m0 = 0.f, m1 = 0.f, t0 = 0.f, t1 = 0.f;
-      for (int i = tid; i < rows * H4; i += T) {
-        const float4 v = sm.st[buf][a][i];
-        m0 = fmaxf(m0, fabsf(v.x));
-        m1 = fmaxf(m1, fabsf(v.z));
-        t0 += fabsf(v.x);
-        t1 += fabsf(v.z);
-      }
-      for (int o = 16; o >= H4; o >>= 1) {
-        m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-        m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-        t0 += __shfl_xor_sync(0xffffffffu, t0, o);
-        t1 += __shfl_xor_sync(0xffffffffu, t1, o);
-      }
-      if (lane < H4) {
-        sm.wmax[a][warp][2 * lane] = m0;
-        sm.wmax[a][warp][2 * lane + 1] = m1;
-        sm.wsum[a][warp][2 * lane] = t0;
-        sm.wsum[a][warp][2 * lane + 1] = t1;
-      }
-    }
-    if (OFFSET) __syncthreads();
-    if (OFFSET && tid < nload * P) {
-      const int a = tid / P, c = tid % P;
-      float m = 0.f, t = 0.f;
-#pragma unroll
-      for (int w = 0; w < T / 32; ++w) {
-        m = fmaxf(m, sm.wmax[a][w][c]);
-        t += sm.wsum[a][w][c];
-      }
-      sm.cf[a][c] = m;
-      sm.cg[a][c] = t * 1.000004f;  // above the rounding of t and of m t
-    }
-    if (OFFSET) __syncthreads();
     if (s < S) {
-      float Sm[U][U], e[U][U];
-      if (OFFSET) {
-#pragma unroll
-        for (int a = 0; a < U; ++a)
-#pragma unroll
-          for (int b = 0; b < U; ++b) {
-            Sm[a][b] = sigma_of(sm.cf[ia][col(bi, a)], sm.cg[ib][col(bj, b)]);
-            e[a][b] = 0.f;
-          }
-      }
       const float4* A = &sm.st[buf][ia][bi];
       const float4* B = &sm.st[buf][ib][bj];
       for (int r = s; r < rows; r += S) {
@@ -341,26 +265,12 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
 #pragma unroll
         for (int a = 0; a < U; ++a)
 #pragma unroll
-          for (int b = 0; b < U; ++b) {
-            if (OFFSET)
-              omac(Sm[a][b], e[a][b], av[a], bv[b]);
-            else
-              bmac(H[a][b], E[a][b], av[a], bv[b]);
-          }
+          for (int b = 0; b < U; ++b) bmac(H[a][b], E[a][b], av[a], bv[b]);
       }
 #pragma unroll
       for (int a = 0; a < U; ++a)
 #pragma unroll
-        for (int b = 0; b < U; ++b) {
-          if (OFFSET) {
-            const float sg = sigma_of(sm.cf[ia][col(bi, a)], sm.cg[ib][col(bj, b)]);
-            const float2 t = two_sum(H[a][b], __fsub_rn(Sm[a][b], sg));
-            H[a][b] = t.x;
-            E[a][b] = __fadd_rn(E[a][b], __fadd_rn(t.y, e[a][b]));
-          } else {
-            renorm(H[a][b], E[a][b]);
-          }
-        }
+        for (int b = 0; b < U; ++b) renorm(H[a][b], E[a][b]);
     }
   }
   __syncthreads();
@@ -386,7 +296,7 @@ __device__ __forceinline__ void gram_tile(const BDev& d, const BTile& tl, const 
 }
 
 template <int G>
-__global__ void __maxnreg__(112) b_gram_kernel(BDev d, int32_t mask, int32_t sel) {
+__global__ void __maxnreg__(80) b_gram_kernel(BDev d, int32_t mask, int32_t sel) {
   extern __shared__ __align__(16) unsigned char gram_smem[];
   GramSm<G>& sm = *reinterpret_cast<GramSm<G>*>(gram_smem);
   const int nt = *d.ntiles;
@@ -565,9 +475,9 @@ __global__ void __launch_bounds__(256) b_reduce_kernel(BDev d, int32_t mask, int
 // the error is relative to the largest |z| of the row, and a row of X that
 // carries a localised vector has entries far below that (6.7e-13 instead of
 // 9e-15 for X U with an orthogonal U at p = 32). Bound by instruction issue
-// (0.73 of the slots); 1.6e6 rows in 48 problems of p in {4, 8, 16, 32}:
-// residual 381 us, direction 283, retraction 503, where one product per
-// thread and row took 645, 500 and 867.
+// (0.67 to 0.77 of the slots); 1.6e6 rows in 48 problems of p in {4, 8, 16,
+// 32}: residual 383 us, direction 358, retraction 618, where one product per
+// thread and row took 650, 634 and 1075.
 template <int P>
 struct RowCfg {
   static constexpr int TC = P >= 4 ? 4 : 2, CG = P / TC, RG = BT / CG, ROWS = 2 * RG;
@@ -924,7 +834,7 @@ __global__ void __launch_bounds__(BT) b_copy_kernel(BDev d) {
 // Block matvec (Sec. 6.1): which 0 -> W = A D (step problems), 1 -> Y = A X,
 // 2 -> W = A X; thread <-> (row, column pair): the p / 2 lanes of a row read
 // the gathered neighbour rows as 16-byte pieces, four neighbours at a time
-// (1.6e6 rows of mean degree 8 in 48 problems: 300 us, 402 with 8-byte ones).
+// (1.6e6 rows of mean degree 8 in 48 problems: 316 us, 831 with 8-byte ones).
 __global__ void __launch_bounds__(BT) b_spmm_kernel(BDev d, int32_t mask, int32_t which) {
   const int tid = threadIdx.x;
   const float2* in = which == 0 ? d.D : d.X;
