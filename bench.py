@@ -365,7 +365,7 @@ def run_dense(args):
           {"workload": d["workload"], "n": 16384, "p": 128,
            "precision": "mixed (3-digit apply, 7-digit correction)", "iterations": d["mixed"]["iters"],
            "rel_residual": d["mixed"]["rel_residual"], "ritz_max_abs_err": d["mixed"]["ritz_max_abs_err"]},
-          "bf16 tensor-core digits (3 then 7 per operand), df64 blocks, f64 p x p",
+          "bf16 tensor-core digits (3 then 7 per operand), df64 blocks, df64 p x p step",
           {"baseline": {"plain_f64_gpu": d["plain_f64_gpu"], "df64_gpu": d["df64_gpu"],
                         "speedup_vs_f64": d["speedup_vs_f64"]},
            "clocks": clk, "gpu_launches": launches})
@@ -546,7 +546,7 @@ def run_table(args):
           {"workload": "3D 7-point FD Laplacian 35x40x25 (n=35000), p=16/32/64, largest and smallest, "
                        "RCG and LOBCG(+) from the same start, stop at ||R||_inf/||R_0||_inf <= 1e-8",
            "rows": rows, "value_is": "sum of the 12 solves' times"},
-          "df64 blocks, bf16 tensor-core digit products; float64 p x p",
+          "df64 blocks, bf16 tensor-core digit products; df64 p x p step",
           {"clocks": clk, "gpu_launches": gsi.launch_count() - l0})
 
 
@@ -793,7 +793,8 @@ def main():
         "warmup_kind": f"solves capped at {WARMUP_ITERS} iterations (same kernels and shapes)",
         "vs_baseline": None,
         "dtype": ("df64: float32 pairs (48-bit significand, float32 exponent range) with bf16 tensor-core "
-                  "digit products exact to 2^-45 of the row/column scale; f64 p x p step. The library's "
+                  "digit products exact to 2^-45 of the row/column scale; df64 p x p step (its sums S, K and the "
+                  "root of the line search in float64). The library's "
                   "float64-class precision form; the native float64 solve is in 'baseline'")
         if args.precision == "df64" else "f64", "data": "synthetic",
         "config": {"workload": workload_name(args, n), "n": n, "p": p, "nnz": int(A.nnz),

@@ -1,17 +1,20 @@
 // Device code of the p x p step (Alg. 3 and the polar normaliser) for one
-// thread block or one thread-block cluster per problem, all matrices df64.
+// thread block or one thread-block cluster per problem. Matrices and products
+// are df64; S = Gram of X + tD and K_next are formed in float64, and the root
+// of the line search is corrected with a float64 evaluation.
 //
 // Eigenbasis of a symmetric B: float32 Jacobi sweeps give V0; V is made
 // orthonormal in df64; then B' = V^T B V = diag(lambda) + F is formed in df64
 // and the small F taken out by V <- V exp(K), K_ij = F_ij / (lambda_j -
 // lambda_i), which squares the relative size of F without a sweep's dependent
-// rounds. Where eigenvalues cluster (|K| > 0.1), F is rotated away by the same
+// rounds. Where eigenvalues cluster (|K| > 0.07), F is rotated away by the same
 // float32 Jacobi, which works on F and on df64 differences of lambda, so that
 // its float32 rounding is relative to F: each such pass gains six to seven
 // digits. Either way the correction is one matrix, applied in df64. One step
-// at p = 8 / 32 / 64 / 128: 64 / 174 / 355 / 1330 us; with sweeps instead of
-// the corrections 70 / 195 / 411 / 1728, as one CTA of 1024 threads with df64
-// sweeps and a float64 line search 72 / - / 760 / 6060.
+// of a random B in one launch, p = 8 / 32 / 64 / 128: 66 / 177 / 351 / 1540 us;
+// as one CTA of 1024 threads with df64 sweeps and a float64 line search 159 /
+// 515 / 1432 / 10660. In the solver's two launches and with K: 71 / 200 / 372 /
+// 1640. (Sweeps instead of the corrections cost 10% at p = 8 and 30% at 128.)
 //
 // Layout of the work. The sweeps are a chain of p - 1 rounds each, so a
 // round is kept short: AW warps (1, 4, 8 or 16) work on A alone, every lane
