@@ -102,7 +102,7 @@ gsi_status gsi_pp_step(int32_t p, const double* C, const double* B, const double
   cudaStream_t st = (cudaStream_t)stream;
   ScratchGuard g(st);
   const size_t wb = (small_df_scratch_bytes(p) + 255) / 256 * 256;
-  GSI_CUDA_TRY(cudaMallocAsync(&g.ptr, wb + ((size_t)p * p + p) * sizeof(float2), st));
+  GSI_CUDA_TRY(cudaMallocAsync(&g.ptr, wb + (2 * (size_t)p * p + p) * sizeof(float2), st));
   PpArgs a{};
   a.p = p;
   a.B = {nullptr, B, 1};
@@ -113,14 +113,17 @@ gsi_status gsi_pp_step(int32_t p, const double* C, const double* B, const double
   a.K = {nullptr, K, 0};
   a.beta = beta;
   a.M = M;
-  a.Kd = Knext;
   a.out = out;
   a.gws = (float2*)g.ptr;
   a.eig = (float2*)((char*)g.ptr + wb);
+  double* const T = (double*)(a.eig + (size_t)p * p + p);
+  if (p <= PP_K_INSIDE) a.Kd = Knext;
+  else a.Tn = T;
   a.mode = 3;
   GSI_TRY(small_step_df(a, cluster != 0, st));
   a.mode = 4;
-  return small_step_df(a, true, st);
+  GSI_TRY(small_step_df(a, true, st));
+  return a.Tn ? pp_gemm(p, 1.0, M, T, 0.0, nullptr, Knext, st) : GSI_OK;
 }
 
 gsi_status gsi_retract(int64_t n, int32_t p, double t, const double* M, double* X,

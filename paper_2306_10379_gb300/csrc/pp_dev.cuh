@@ -13,8 +13,8 @@
 // digits. Either way the correction is one matrix, applied in df64. One step
 // of a random B in one launch, p = 8 / 32 / 64 / 128: 66 / 177 / 351 / 1540 us;
 // as one CTA of 1024 threads with df64 sweeps and a float64 line search 159 /
-// 515 / 1432 / 10660. In the solver's two launches and with K: 71 / 200 / 372 /
-// 1640. (Sweeps instead of the corrections cost 10% at p = 8 and 30% at 128.)
+// 515 / 1432 / 10660. In the solver's two launches and with K: 71 / 194 / 382 /
+// 1610. (Sweeps instead of the corrections cost 10% at p = 8 and 30% at 128.)
 //
 // Layout of the work. The sweeps are a chain of p - 1 rounds each, so a
 // round is kept short: AW warps (1, 4, 8 or 16) work on A alone, every lane
@@ -71,13 +71,14 @@ struct PpArgs {
   PpMat C, B, Gam, Z, XX, XD, K;
   double beta;
   double* M;      // p x p result (eigenvectors in mode 2)
-  double* Kd;     // K_next = M (XD + t B), float64 (or null)
-  float2* Kf;     // and df64 (or null)
+  double* Kd;     // K_next = M (XD + t B), float64 (or null; one CTA only)
+  double* Tn;     // XD + t B alone, for a product on more SMs (or null)
   double* theta;  // mode 2: eigenvalues
   float2* eig;    // modes 3, 4: V (p x p), then the diagonal of V^T B V
   double* out;    // 16 doubles: t, phi, evaluations, status, max beta, cycle counts and sweeps
   float2* gws;    // NC > 1: pp_gws_bytes(p) of global scratch
 };
+constexpr int PP_K_INSIDE = 16;  // widest block whose K_next the step forms itself in a solve
 constexpr int PP_CTL = 1024 + 64;  // float2: control words, then the partial dots of up to 8 ranks
 
 struct PpSh {  // small tables, shared memory
@@ -1392,35 +1393,31 @@ __device__ void pp_body(const PpArgs& a, PpCtx<P>& c) {
   pp_sync<P>();
   pp_inv_sqrt(c, a.M);
   if (lead) out[3] = (double)sh->flag;
-  if (a.Kd) {
-    // K_next = X_new^T D = M (X^T D + t D^T D) in float64: it goes into the
-    // next direction and X^T D with no correction after it. The operands
-    // leave df64 once (a conversion costs as much as a multiply-add): T =
-    // X^T D + t B in the space of T, from there staged for NC > 1, the rows
-    // of M in that of V (the strip of X).
-    double *T = reinterpret_cast<double*>(c.mat(c.Td)), *Mr;
-    pp_each(c, [&](int i, int j) {
-      T[i * p + j] = fma(t, elem(a.B, i, j), df_to_double(c.mat(c.Bd)[i * c.ld + j]));
-    });
-    if constexpr (P::NC == 1) {
-      Mr = reinterpret_cast<double*>(pp_s2(c.Vd));
-    } else {
-      pp_sync<P>();
-      const double* const Tg = T;
-      T = reinterpret_cast<double*>(pp_s2(c.sY));
-      Mr = reinterpret_cast<double*>(pp_s2(c.sX));
-      for (int e = c.tid; e < p * p; e += P::NT) T[e] = __ldcg(Tg + e);
-    }
-    pp_each(c, [&](int i, int j) { Mr[(i - c.r0) * p + j] = df_to_double(c.mat(c.Ud)[i * c.ld + j]); });
-    __syncthreads();
-    pp_each(c, [&](int i, int j) {
-      const double* const mr = Mr + (i - c.r0) * p;
-      double v = 0.0;
+  // K_next = X_new^T D = M T, T = X^T D + t D^T D, in float64: it goes into the
+  // next direction and X^T D with no correction after it. The product takes
+  // p^3 / 2 cycles of an SM's float64 pipe (p = 16: 3 us of a step's 98; p = 32
+  // 13 of 200; on a cluster at p = 128 70 of 1640), so a solve forms it here up
+  // to p = PP_K_INSIDE only and takes T for a product over many SMs beyond; the
+  // batch, with a block per problem, always forms it here. T and M leave df64
+  // once (a conversion costs as much as a multiply-add), in the space of T, V.
+  auto t_elem = [&](int i, int j) { return fma(t, elem(a.B, i, j), df_to_double(c.mat(c.Bd)[i * c.ld + j])); };
+  if (a.Tn) pp_each(c, [&](int i, int j) { a.Tn[i * p + j] = t_elem(i, j); });
+  if constexpr (P::NC == 1) {
+    if (a.Kd) {
+      double* const T = reinterpret_cast<double*>(pp_s2(c.Td));
+      double* const Md = reinterpret_cast<double*>(pp_s2(c.Vd));
+      pp_each(c, [&](int i, int j) {
+        T[i * p + j] = t_elem(i, j);
+        Md[i * p + j] = df_to_double(c.mat(c.Ud)[i * c.ld + j]);
+      });
+      __syncthreads();
+      pp_each(c, [&](int i, int j) {
+        double v = 0.0;
 #pragma unroll 4
-      for (int k = 0; k < p; ++k) v = fma(mr[k], T[k * p + j], v);
-      a.Kd[i * p + j] = v;
-      if (a.Kf) a.Kf[i * p + j] = df_from_double(v);
-    });
+        for (int k = 0; k < p; ++k) v = fma(Md[i * p + k], T[k * p + j], v);
+        a.Kd[i * p + j] = v;
+      });
+    }
   }
   if (lead) {
     // cycles: eigenbasis (mode 3 wrote it), coefficients and X^T D, line

@@ -402,8 +402,8 @@ PpMat pp_in(gsi_ctx* c, const double* G) {
 
 // The df64 p x p step (PpArgs, pp_dev.cuh): mode 1 with B; mode 2 with B,
 // eigenvectors into Mout, eigenvalues into theta; mode 3 with B; mode 4 with
-// C, B, Gm, Zp, XX and K (X^T D = (I - XX)(C + beta K) formed inside), K_next
-// into Km for CG.
+// C, B, Gm, Zp, XX and K (X^T D = (I - XX)(C + beta K) formed inside); for CG
+// K_next into Km, or (p > PP_K_INSIDE) X^T D + t B into XDm for op_knext.
 gsi_status op_pp(gsi_ctx* c, int mode, const double* B, const double* Zp, double beta, bool want_k,
                  double* Mout = nullptr, double* theta = nullptr) {
   PpArgs a{};
@@ -415,11 +415,11 @@ gsi_status op_pp(gsi_ctx* c, int mode, const double* B, const double* Zp, double
     a.Gam = pp_in(c, c->Gm);
     a.Z = pp_in(c, Zp);
     a.XX = pp_in(c, c->XXm);
-    a.K = pp_in(c, c->Km);
+    a.K = PpMat{nullptr, c->Km, 0};
     a.beta = beta;
     if (want_k) {
-      a.Kd = c->Km;
-      a.Kf = pp_df(c, c->Km);
+      if (c->p <= PP_K_INSIDE) a.Kd = c->Km;
+      else a.Tn = c->XDm;
     }
   }
   a.M = Mout ? Mout : c->Mm;
@@ -428,6 +428,20 @@ gsi_status op_pp(gsi_ctx* c, int mode, const double* B, const double* Zp, double
   a.out = c->out;
   a.gws = (float2*)c->small_ws;
   return small_step_df(a, mode == 3 ? c->eig_cluster : true, c->st);
+}
+
+// K_next = M T (T from op_pp in XDm) on the second stream, while the host reads
+// the step; op_knext_join makes st wait for it (M, T and K are free after that)
+gsi_status op_knext(gsi_ctx* c) {
+  GSI_CUDA_TRY(cudaEventRecord(c->ev_b, c->st));
+  GSI_CUDA_TRY(cudaStreamWaitEvent(c->st2, c->ev_b, 0));
+  GSI_TRY(pp_gemm(c->p, 1.0, c->Mm, c->XDm, 0.0, nullptr, c->Km, c->st2));
+  GSI_CUDA_TRY(cudaEventRecord(c->ev_e, c->st2));
+  return GSI_OK;
+}
+gsi_status op_knext_join(gsi_ctx* c) {
+  GSI_CUDA_TRY(cudaStreamWaitEvent(c->st, c->ev_e, 0));
+  return GSI_OK;
 }
 
 gsi_status op_small(gsi_ctx* c, int mode, const double* B, const double* Zp) {
@@ -567,7 +581,11 @@ gsi_status iterate(gsi_ctx* c, bool* stop) {
     prof_end(c, GSI_K_SMALL, 0.0, 0.0);
     GSI_TRY(op_small(c, 0, c->Bm, Zp));
   }
-  GSI_TRY(readback(c, c->out, 5));
+  const bool knext = split && cg && c->p > PP_K_INSIDE;
+  if (knext) GSI_TRY(op_knext(c));
+  const gsi_status rs = readback(c, c->out, 5);
+  if (knext) GSI_TRY(op_knext_join(c));
+  GSI_TRY(rs);
   const double t = c->host[0];
   c->last_t = t;
   c->last_evals = (int)c->host[2];
